@@ -1,14 +1,19 @@
-"""ctypes binding of libqsgd.so: the same entry points as include/qsgd.h, argument marshalling
-only. PyTorch supplies device memory and the CUDA stream; every step of the path runs in the
-library's kernels. There is no CPU fallback: a missing library or a missing device raises.
+"""Binding of libqsgd.so: the same entry points as include/qsgd.h, argument marshalling only. The calls
+that a training loop makes every step go through the native module (csrc/python_binding.cpp), size
+queries, plans and test hooks through ctypes. PyTorch supplies device memory and the CUDA stream; every
+step of the path runs in the library's kernels. There is no CPU fallback: a missing library or a missing
+device raises.
 """
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_HERE, "libqsgd.so")
+_NATIVE_PATH = os.path.join(_HERE, "_qsgd_native.so")
 
 NORM_L2, NORM_MAX = 0, 1
 CODE_FIXED, CODE_ELIAS, CODE_ELIAS_DENSE = 0, 1, 2
@@ -114,20 +119,28 @@ def lib():
     return _lib
 
 
+class _Native:
+    """Stands in for the native module until the first call loads it."""
+
+    def __getattr__(self, name):
+        global _native
+        if not os.path.exists(_NATIVE_PATH):
+            raise QsgdError("_qsgd_native.so is not built; run paper_1610_02132_b200.build.build()")
+        lib()                                             # the library it is linked against: its own message if missing
+        loader = importlib.machinery.ExtensionFileLoader("_qsgd_native", _NATIVE_PATH)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_qsgd_native", loader))
+        loader.exec_module(module)
+        module.set_error(QsgdError)
+        _native = module
+        return getattr(module, name)
+
+
+_native = _Native()
+
+
 def _check(st):
     if st != 0:
         raise QsgdError("qsgd status %d: %s" % (st, lib().qsgd_status_string(st).decode()))
-
-
-def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
-
-
-def _require_cuda(t, name):
-    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous()):
-        raise QsgdError("%s must be a contiguous CUDA tensor" % name)
 
 
 def qsgd_message_capacity(n, bucket, s, code_kind):
@@ -182,15 +195,8 @@ def qsgd_profile_collect():
 def qsgd_encode(g, bucket, s, norm_kind, code_kind, seed, step, worker, out, out_bits,
                 workspace=None, status_dev=None, stream=None, n=None):
     """Encode g (fp32 CUDA tensor) into `out` (uint8 CUDA tensor); see include/qsgd.h."""
-    _require_cuda(g, "g")
-    _require_cuda(out, "out")
-    _require_cuda(out_bits, "out_bits")
-    _require_cuda(status_dev, "status_dev")
-    n = g.numel() if n is None else n
-    ws = None if workspace is None else C.c_void_p(workspace.data_ptr())
-    _check(lib().qsgd_encode(g.data_ptr(), n, bucket, s, norm_kind, code_kind, seed, step, worker,
-                             out.data_ptr(), out.numel() * out.element_size(),
-                             out_bits.data_ptr(), ws, status_dev.data_ptr(), _stream(stream)))
+    _check(_native.encode(g, n, bucket, s, norm_kind, code_kind, seed, step, worker, out, out_bits, workspace,
+                          status_dev, stream))
 
 
 def qsgd_static_scratch_bytes():
@@ -203,44 +209,15 @@ def qsgd_encode_elias_static(g, bucket, s, norm_kind, code_kind, seed, step, wor
     library, so this call allocates nothing (for callers that may not allocate device memory when
     they encode). Same results as qsgd_encode; sizes beyond the built-in scratch raise. Calls
     that overlap on the GPU share the scratch and must be serialised by the caller."""
-    _require_cuda(g, "g")
-    _require_cuda(out, "out")
-    _require_cuda(out_bits, "out_bits")
-    _require_cuda(status_dev, "status_dev")
-    _check(lib().qsgd_encode_elias_static(g.data_ptr(), g.numel(), bucket, s, norm_kind, code_kind,
-                                          seed, step, worker, out.data_ptr(),
-                                          out.numel() * out.element_size(), out_bits.data_ptr(),
-                                          status_dev.data_ptr(), _stream(stream)))
-
-
-def _ptr_array(tensors):
-    arr = (C.c_void_p * len(tensors))()
-    for i, t in enumerate(tensors):
-        arr[i] = t if isinstance(t, int) else t.data_ptr()
-    return arr
-
-
-def _u64_array(values):
-    if values is None:
-        return None
-    return (C.c_uint64 * len(values))(*[int(v) for v in values])
+    _check(_native.encode_static(g, bucket, s, norm_kind, code_kind, seed, step, worker, out, out_bits, status_dev,
+                                 stream))
 
 
 def qsgd_decode_accumulate(msgs, tables, n, bucket, s, code_kind, acc, status_dev, stream=None,
                            payload_bytes=None):
     """acc <- ascending-k sum of the decoded messages; msgs / tables: lists of CUDA tensors
     (or raw device addresses); payload_bytes: optional list of payload lengths (read bound)."""
-    _require_cuda(acc, "acc")
-    mp = _ptr_array(msgs)
-    tp = None if tables is None else _ptr_array(tables)
-    _check(lib().qsgd_decode_accumulate(mp, tp, _u64_array(payload_bytes), len(msgs), n, bucket, s, code_kind,
-                                        acc.data_ptr(), status_dev.data_ptr(), _stream(stream)))
-
-
-def _msg_bytes(msgs, msg_bytes):
-    if msg_bytes is not None:
-        return _u64_array(msg_bytes)
-    return _u64_array([m.numel() * m.element_size() for m in msgs])
+    _check(_native.decode(False, msgs, tables, payload_bytes, n, bucket, s, code_kind, acc, None, status_dev, stream))
 
 
 def qsgd_decode_accumulate_packed(msgs, infos, n, bucket, s, code_kind, acc, status_dev, stream=None,
@@ -248,35 +225,21 @@ def qsgd_decode_accumulate_packed(msgs, infos, n, bucket, s, code_kind, acc, sta
     """As qsgd_decode_accumulate, for messages as Encode left them: infos[k] is the CUDA tensor (or
     device address) of message k's four info words; the tables are found on the device. msg_bytes
     defaults to the sizes of the message tensors."""
-    _require_cuda(acc, "acc")
-    ip = None if infos is None else _ptr_array(infos)
-    _check(lib().qsgd_decode_accumulate_packed(_ptr_array(msgs), ip, _msg_bytes(msgs, msg_bytes), len(msgs), n,
-                                               bucket, s, code_kind, acc.data_ptr(), status_dev.data_ptr(),
-                                               _stream(stream)))
+    _check(_native.decode(True, msgs, infos, msg_bytes, n, bucket, s, code_kind, acc, None, status_dev, stream))
 
 
 def qsgd_decode_sgd_step_packed(msgs, infos, n, bucket, s, code_kind, x, eta, status_dev, stream=None,
                                 msg_bytes=None):
-    _require_cuda(x, "x")
-    ip = None if infos is None else _ptr_array(infos)
-    _check(lib().qsgd_decode_sgd_step_packed(_ptr_array(msgs), ip, _msg_bytes(msgs, msg_bytes), len(msgs), n,
-                                             bucket, s, code_kind, x.data_ptr(), eta, status_dev.data_ptr(),
-                                             _stream(stream)))
+    _check(_native.decode(True, msgs, infos, msg_bytes, n, bucket, s, code_kind, x, eta, status_dev, stream))
 
 
 def qsgd_sgd_step(x, acc, eta, K, stream=None):
-    _require_cuda(x, "x")
-    _require_cuda(acc, "acc")
-    _check(lib().qsgd_sgd_step(x.data_ptr(), acc.data_ptr(), eta, K, x.numel(), _stream(stream)))
+    _check(_native.sgd_step(x, acc, eta, K, stream))
 
 
 def qsgd_decode_sgd_step(msgs, tables, n, bucket, s, code_kind, x, eta, status_dev, stream=None,
                          payload_bytes=None):
-    _require_cuda(x, "x")
-    mp = _ptr_array(msgs)
-    tp = None if tables is None else _ptr_array(tables)
-    _check(lib().qsgd_decode_sgd_step(mp, tp, _u64_array(payload_bytes), len(msgs), n, bucket, s, code_kind,
-                                      x.data_ptr(), eta, status_dev.data_ptr(), _stream(stream)))
+    _check(_native.decode(False, msgs, tables, payload_bytes, n, bucket, s, code_kind, x, eta, status_dev, stream))
 
 
 # ------------------------------- per-tensor policy -------------------------------------------
@@ -308,6 +271,7 @@ class Policy:
         self.struct = PolicyStruct(self.dev["bucket_src"].data_ptr(), self.dev["bucket_len"].data_ptr(), nb,
                                    self.dev["raw_src"].data_ptr(), self.dev["raw_start"].data_ptr(), ns, nr,
                                    self.n, quads.value)
+        self.address = C.addressof(self.struct)
 
 
 def qsgd_policy_message_capacity(plan, s, code_kind):
@@ -318,40 +282,32 @@ def qsgd_policy_workspace_bytes(plan, s, code_kind):
     return int(lib().qsgd_policy_workspace_bytes(C.byref(plan.struct), plan.bucket, s, code_kind))
 
 
+def _covered(t, name, plan):
+    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous()):
+        raise QsgdError("%s must be a contiguous CUDA tensor" % name)
+    if t.numel() != plan.n:
+        raise QsgdError("%s has %d elements, the plan covers %d" % (name, t.numel(), plan.n))
+
+
 def qsgd_policy_encode(g, plan, s, norm_kind, code_kind, seed, step, worker, out, out_bits, workspace=None,
                        status_dev=None, stream=None):
-    _require_cuda(g, "g")
-    _require_cuda(out, "out")
-    _require_cuda(out_bits, "out_bits")
-    _require_cuda(status_dev, "status_dev")
-    if g.numel() != plan.n:
-        raise QsgdError("g has %d elements, the plan covers %d" % (g.numel(), plan.n))
-    ws = None if workspace is None else C.c_void_p(workspace.data_ptr())
-    _check(lib().qsgd_policy_encode(g.data_ptr(), C.byref(plan.struct), plan.bucket, s, norm_kind, code_kind, seed,
-                                    step, worker, out.data_ptr(), out.numel() * out.element_size(),
-                                    out_bits.data_ptr(), ws, status_dev.data_ptr(), _stream(stream)))
+    _covered(g, "g", plan)
+    _check(_native.policy_encode(g, plan.address, plan.bucket, s, norm_kind, code_kind, seed, step, worker, out,
+                                 out_bits, workspace, status_dev, stream))
 
 
 def qsgd_policy_decode_accumulate(msgs, tables, plan, s, code_kind, acc, status_dev, stream=None,
                                   payload_bytes=None):
-    _require_cuda(acc, "acc")
-    if acc.numel() != plan.n:
-        raise QsgdError("acc has %d elements, the plan covers %d" % (acc.numel(), plan.n))
-    mp = _ptr_array(msgs)
-    tp = None if tables is None else _ptr_array(tables)
-    _check(lib().qsgd_policy_decode_accumulate(mp, tp, _u64_array(payload_bytes), len(msgs), C.byref(plan.struct), plan.bucket, s, code_kind,
-                                               acc.data_ptr(), status_dev.data_ptr(), _stream(stream)))
+    _covered(acc, "acc", plan)
+    _check(_native.policy_decode(msgs, tables, payload_bytes, plan.address, plan.bucket, s, code_kind, acc, None,
+                                 status_dev, stream))
 
 
 def qsgd_policy_decode_sgd_step(msgs, tables, plan, s, code_kind, x, eta, status_dev, stream=None,
                                 payload_bytes=None):
-    _require_cuda(x, "x")
-    if x.numel() != plan.n:
-        raise QsgdError("x has %d elements, the plan covers %d" % (x.numel(), plan.n))
-    mp = _ptr_array(msgs)
-    tp = None if tables is None else _ptr_array(tables)
-    _check(lib().qsgd_policy_decode_sgd_step(mp, tp, _u64_array(payload_bytes), len(msgs), C.byref(plan.struct), plan.bucket, s, code_kind,
-                                             x.data_ptr(), eta, status_dev.data_ptr(), _stream(stream)))
+    _covered(x, "x", plan)
+    _check(_native.policy_decode(msgs, tables, payload_bytes, plan.address, plan.bucket, s, code_kind, x, eta,
+                                 status_dev, stream))
 
 
 # ------------------------------- conveniences (allocation only) -----------------------------

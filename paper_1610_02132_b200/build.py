@@ -1,11 +1,15 @@
-"""Builds libqsgd.so (the C-ABI library with the sm_100a kernels) in-tree with nvcc."""
+"""Builds libqsgd.so (the C-ABI library with the sm_100a kernels, nvcc) and _qsgd_native.so (its Python
+binding, g++ against the torch headers) in-tree."""
 import glob
 import os
 import subprocess
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libqsgd.so")
+NATIVE = os.path.join(_HERE, "_qsgd_native.so")
+NATIVE_SRC = os.path.join(CSRC, "python_binding.cpp")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC", "--cudart", "shared", "--threads", "0"]
@@ -15,23 +19,51 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def _stale():
-    if not os.path.exists(LIB):
+def _stale(target, deps):
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + \
-        glob.glob(os.path.join(_HERE, "..", "include", "*.h"))
+    t = os.path.getmtime(target)
     return any(os.path.getmtime(p) > t for p in deps)
 
 
-def build(force=False, verbose=False):
+def _headers():
+    return glob.glob(os.path.join(_HERE, "..", "include", "*.h"))
+
+
+def build_library(force=False, verbose=False):
     """Compile every kernel for sm_100a into libqsgd.so; returns the library path."""
-    if force or _stale():
+    if force or _stale(LIB, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + _headers()):
         nvcc = os.environ.get("NVCC", "nvcc")
         tmp = LIB + ".tmp%d" % os.getpid()
         cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", tmp] + sources()
         subprocess.check_call(cmd)
         os.replace(tmp, LIB)
+    return LIB
+
+
+def build_native(force=False):
+    """Compile the Python binding; it finds libqsgd.so beside itself and torch's libraries by rpath."""
+    if force or _stale(NATIVE, [NATIVE_SRC] + _headers()):
+        import torch
+        from torch.utils import cpp_extension
+        tmp = NATIVE + ".tmp%d" % os.getpid()
+        inc = cpp_extension.include_paths("cuda") + [sysconfig.get_paths()["include"]]
+        libdirs = cpp_extension.library_paths("cuda")
+        cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+               "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)]
+        cmd += ["-isystem" + p for p in inc] + [NATIVE_SRC, "-o", tmp]
+        cmd += ["-L" + _HERE, "-l:libqsgd.so", "-Wl,-rpath,$ORIGIN"]
+        cmd += ["-L" + p for p in libdirs] + ["-Wl,-rpath," + libdirs[0]]
+        cmd += ["-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+        subprocess.check_call(cmd)
+        os.replace(tmp, NATIVE)
+    return NATIVE
+
+
+def build(force=False, verbose=False):
+    """Builds whatever is out of date; returns the path of libqsgd.so."""
+    build_library(force, verbose)
+    build_native(force)
     return LIB
 
 
