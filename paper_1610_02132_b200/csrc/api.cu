@@ -36,6 +36,31 @@ ScopedKernel::~ScopedKernel() {
   }
 }
 
+static int device_attribute(cudaDeviceAttr which, std::atomic<int>* known, int* out) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return (int)e;
+  if (dev < 0 || dev >= kMaxDevices) return (int)cudaErrorInvalidDevice;
+  int v = known[dev].load(std::memory_order_relaxed);
+  if (!v) {
+    e = cudaDeviceGetAttribute(&v, which, dev);
+    if (e != cudaSuccess) return (int)e;
+    known[dev].store(v, std::memory_order_relaxed);
+  }
+  *out = v;
+  return 0;
+}
+
+int device_sms(int* sms_out) {
+  static std::atomic<int> known[kMaxDevices];
+  return device_attribute(cudaDevAttrMultiProcessorCount, known, sms_out);
+}
+
+int device_shared_memory(int* bytes_out) {
+  static std::atomic<int> known[kMaxDevices];
+  return device_attribute(cudaDevAttrMaxSharedMemoryPerBlockOptin, known, bytes_out);
+}
+
 static const char* const kKernelNames[kKernCount] = {
     "quantize_fixed", "quantize_tail", "decode_fixed", "sgd_step", "elias_length",
     "elias_scatter", "decode_elias", "decode_elias_sparse", "raw_gather", "raw_decode"};

@@ -144,4 +144,25 @@ __device__ __forceinline__ void store_span16(const OutSpan& sp, const float (&ac
   }
 }
 
+// The same for 8 values.
+template <bool FUSED>
+__device__ __forceinline__ void store_span8(const OutSpan& sp, const float (&acc)[8], float c) {
+  if (sp.valid == 8u && (reinterpret_cast<uintptr_t>(sp.ptr) & 15u) == 0) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      float4 r = make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+      if (FUSED) {
+        const float4 x = *reinterpret_cast<const float4*>(sp.ptr + 4 * j);
+        r.x = __fsub_rn(x.x, __fmul_rn(c, r.x)); r.y = __fsub_rn(x.y, __fmul_rn(c, r.y));
+        r.z = __fsub_rn(x.z, __fmul_rn(c, r.z)); r.w = __fsub_rn(x.w, __fmul_rn(c, r.w));
+      }
+      *reinterpret_cast<float4*>(sp.ptr + 4 * j) = r;
+    }
+  } else {
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if ((uint32_t)e < sp.valid) sp.ptr[e] = FUSED ? __fsub_rn(sp.ptr[e], __fmul_rn(c, acc[e])) : acc[e];
+  }
+}
+
 }  // namespace qsgd

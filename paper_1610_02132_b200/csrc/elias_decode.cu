@@ -1,11 +1,36 @@
 // Decode-and-aggregate, Elias path, optionally fused with the SGD step (Section 3.1, end of
 // "Efficient Coding of Gradients": scale first, then the codes of the nonzeros in index order;
-// Appendix A.2 decoder; Algorithm 1 for the sum and the step): the choice among the decoders. Whole-bucket and ranged field rebuilding live in elias_decode_fields.cu, the
-// nonzero-driven decoder of the sparse regime in elias_decode_sparse.cu, the general fallback in
-// elias_decode_slow.cu; what they share is in elias_decode.cuh.
+// Appendix A.2 decoder; Algorithm 1 for the sum and the step): the choice among the decoders. Those with a
+// lane per string (whole-bucket and ranged field rebuilding, byte codes) live in elias_decode_fields.cu, the
+// one with a team of lanes per string in elias_decode_teams.cu, the nonzero-driven decoder of the sparse
+// regime in elias_decode_sparse.cu; what they share is in elias_decode.cuh.
 #include "elias_decode.cuh"
 
 namespace qsgd {
+
+namespace {
+
+// Coordinates x peers up to which the sparse-regime decoder is not considered beside the teams: one launch
+// less, and a string's latency decides (n = 2^20, d = 4096, s = 1, K = 8: 16.7 against 31.4 us; at 2^22 41.0
+// against 33.9).
+constexpr uint64_t kSmallWork = 8ull << 20;
+
+// A lane per string, or a team of lanes? A lane per string is the cheaper reading (a team reads its string
+// almost twice) but needs strings enough for the GPU, and short ones, whose rows leave room for many
+// warps. Measured lines (us, a lane against a team): 16 K strings of d = 512, s = 15: 66 / 34, 65 K: 85 /
+// 107; 32 K of d = 128, s = 3: 28 / 26, 262 K: 37 / 60; s = 255:
+// 16 K of d = 512 118 / 74, 524 K 1974 / 1744, but
+// 2 M of d = 128 1488 / 1751. From d = 1024 on a lane's string is long enough to decide the time by itself
+// (2 K strings of d = 4096: 280 / 23; 32 K: 1849 / 568), except where hundreds of lanes per SM read
+// nearly empty ones (65 K with s = 3: 252 / 313). Code'_s has a symbol per coordinate: always teams.
+bool use_teams(uint64_t B, uint32_t K, uint32_t d, uint32_t s, bool dense) {
+  const uint64_t strings = B * K;
+  if (dense || K > 32u) return true;
+  if (d >= 1024u) return s > 3u || strings <= (48u << 10);
+  return strings <= (40u << 10) || (s > 15u && d >= 512u);
+}
+
+}  // namespace
 
 int launch_decode_elias(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d, uint32_t s,
                         bool dense, float* acc_or_x, bool fused, float eta, uint32_t* status_dev,
@@ -26,28 +51,18 @@ int launch_decode_elias(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
     else payload_bits += 8ull * (uint64_t)(t - w);
   }
   const bool host_sparse = sizes_known && payload_bits < (uint64_t)K * B * (32ull + d / 4u);
+  FieldParams f;
+  f.peers = peers; f.K = K; f.n = n; f.d = d; f.s = s; f.B = B;
+  f.out = acc_or_x; f.c = eta / (float)K; f.status = status_dev; f.map = map;
+  const bool teams = use_teams(B, K, d, s, dense);
   bool sparse = false;
-  {
-    FieldParams f;
-    f.peers = peers; f.K = K; f.n = n; f.d = d; f.s = s;
-    f.B = B;
-    f.out = acc_or_x; f.c = eta / (float)K; f.status = status_dev; f.map = map;
-    bool handled = false;
-    int st = 0;
-    if (!dense && (host_sparse || !sizes_known))
-      st = launch_elias_sparse(peers, K, n, d, s, acc_or_x, fused, f.c, status_dev, !sizes_known, map, stream, &sparse);
+  if (!dense && (host_sparse || !sizes_known) && !(teams && n * K <= kSmallWork)) {
+    const int st = launch_elias_sparse(peers, K, n, d, s, acc_or_x, fused, f.c, status_dev, !sizes_known, map, stream, &sparse);
     if (st) return st;
     if (sparse && sizes_known) return 0;                    // the host chose the sparse-regime kernel
-    f.defer_sparse = sparse ? 1u : 0u;
-    st = launch_elias_fields(f, dense, fused, stream, &handled);
-    if (handled || st) return st;
   }
-  EliasDecodeParams p;
-  p.peers = peers; p.K = K; p.Kc = K; p.n = n; p.d = d; p.s = s;
-  p.B = (n + d - 1) / d;
-  p.out = acc_or_x; p.c = eta / (float)K; p.status = status_dev; p.warp_bytes = 0;
-  p.defer_sparse = sparse ? 1u : 0u; p.map = map;
-  return launch_elias_slow(p, dense, fused, stream);
+  f.defer_sparse = sparse ? 1u : 0u;
+  return teams ? launch_elias_teams(f, dense, fused, stream) : launch_elias_fields(f, fused, stream);
 }
 
 }  // namespace qsgd

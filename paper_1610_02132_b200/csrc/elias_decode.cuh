@@ -8,22 +8,6 @@
 
 namespace qsgd {
 
-struct EliasDecodeParams {
-  PeerSet peers;
-  uint32_t K;
-  uint32_t Kc;         // peers per pass (scratch holds Kc x d codes)
-  uint64_t n;
-  uint32_t d;
-  uint32_t s;
-  uint64_t B;
-  float* out;          // acc (overwritten) or x (updated in place)
-  float c;             // eta / K
-  uint32_t* status;
-  uint32_t warp_bytes; // shared memory per warp
-  uint32_t defer_sparse;  // a sparse-regime kernel was launched beside this one
-  BucketMap map;       // where the buckets live in `out` (per-tensor policy), or no map
-};
-
 // Work split of the sparse-regime decoder (elias_decode_sparse.cu): a warp owns G <= 32 / Kpad
 // buckets and walks each in ranges of R positions; a (bucket, peer) list holds the C entries of one
 // range. Fewer buckets per warp (some lanes idle) spread a small problem over more warps: the parse
@@ -219,22 +203,6 @@ __device__ __forceinline__ void fill_elias_lut(uint16_t* lut) {
   }
 }
 
-// One Elias integer from the window: table hit in the common case, group loop otherwise.
-__device__ __forceinline__ bool read_int(BitSrc& src, const uint16_t* lut, uint32_t skip, uint32_t& value,
-                                         uint32_t& used) {
-  // `skip` (0 or 1) bits in front of the code are dropped together with it
-  const uint32_t e = lut[(src.hi << skip) >> (32 - kLutBits)];
-  if (e) {
-    const uint32_t nb = (e >> 8) + skip;
-    value = e & 0xFFu;
-    src.drop(nb);
-    used += nb;
-    return true;
-  }
-  if (skip) { src.drop(1); used += 1; }
-  return src.elias(value, used);
-}
-
 struct SparseParams {
   PeerSet peers;
   uint32_t K;
@@ -273,6 +241,68 @@ __device__ __forceinline__ bool elias_from_window(uint32_t w, uint32_t& value, u
   len = c0 ? (c1 ? (c2 ? 3u + l2 + l3 : 3u + l2) : 3u) : 1u;
   return !(c0 & c1 & c2 & c3);
 }
+
+// The same code by its first 7 bits, which fix the lengths of all its groups: no code takes a slower path
+// than another, so lanes with different codes stay together. The closing 0 is left to the symbol behind:
+// "body" below is the code without it. Entry i describes the code that starts with the 7 bits i: x holds
+// the bits in front of the value (bits 0-4), the right shift that leaves the value (8-15) and the body's
+// length (16-23); y is 1 for the code of 1, whose body is empty, and is what the shift then brings in.
+__device__ __forceinline__ uint2 code_entry(uint32_t i) {
+  if (!(i & 64u)) return make_uint2(32u << 8, 1u);
+  uint32_t prefix = 0, m = 2;                      // m: bit length of the value
+  const uint32_t n1 = 2u | ((i >> 5) & 1u);
+  if (i & 16u) {                                   // a second group, n1 + 1 bits
+    const uint32_t rest = 4u - n1;                 // bits of i behind it: 2 or 1
+    const uint32_t n2 = (i & 31u) >> rest;
+    prefix = 2; m = n1 + 1u;
+    if ((i >> (rest - 1u)) & 1u) { prefix += m; m = n2 + 1u; }     // and a third, n2 + 1 bits
+  }
+  return make_uint2(prefix | (32u - m) << 8 | (prefix + m) << 16, 0u);
+}
+constexpr uint32_t kCodeEntries = 128;
+
+// The value of the code at the top of w (below 2^16), and the length of its body.
+__device__ __forceinline__ uint32_t code_value(uint32_t w, uint2 e) {
+  return __funnelshift_rc(__funnelshift_l(0u, w, e.x), e.y, __byte_perm(e.x, 0u, 0x4441));
+}
+__device__ __forceinline__ uint32_t code_body(uint2 e) { return __byte_perm(e.x, 0u, 0x4442); }
+
+// What stands behind a gap's body, by its next 9 bits: the closing 0, the sign and the level code of a level
+// <= min(s, 15). Entry: level | negative << 4 | bits << 8, or 0 when they hold no such thing.
+constexpr uint32_t kTailBits = 9, kTailEntries = 1u << kTailBits;
+
+__device__ __forceinline__ uint32_t tail_entry(uint32_t i, uint32_t s) {
+  uint32_t level, len;
+  const bool ok = !(i >> 8) && elias_from_window((i & 127u) << 25, level, len) && len <= 7u && level <= s && level <= 15u;
+  return ok ? level | ((i >> 3) & 16u) | ((len + 2u) << 8) : 0u;
+}
+
+// Three words of a payload: w0 holds bit `bp`, `edge` is the first bit of w1, w2 is on its way. Bits are
+// counted from the word that open() was given a bit of. The words may lie in global or in shared memory.
+struct Window {
+  const uint32_t* wp;     // the word behind w2
+  uint32_t w0, w1, w2;
+  uint32_t bp, edge;
+  __device__ __forceinline__ void open(const uint32_t* words, uint64_t bit) {
+    wp = words + (bit >> 5);
+    w0 = wp[0]; w1 = wp[1]; w2 = wp[2];
+    wp += 3;
+    bp = (uint32_t)(bit & 31u);
+    edge = 32u;
+  }
+  __device__ __forceinline__ uint32_t peek() const { return __funnelshift_l(w1, w0, bp); }   // 32 bits from bp on
+  // 32 bits from `ahead` <= 32 bits behind bp on
+  __device__ __forceinline__ uint32_t peek_at(uint32_t ahead) const {
+    const uint32_t b = bp + ahead;
+    return b >= edge ? __funnelshift_l(w2, w1, b) : __funnelshift_l(w1, w0, b);
+  }
+  // At most 32 bits. No word is fetched on account of bits at or behind `end`, so that the reads stay
+  // within two words of the word that holds the string's end.
+  __device__ __forceinline__ void drop(uint32_t bits, uint32_t end) {
+    bp += bits;
+    if (bp >= edge && bp < end) { w0 = w1; w1 = w2; w2 = *wp; ++wp; edge += 32u; }
+  }
+};
 
 constexpr uint32_t kNoEntry = 0xFFFFFFFFu;           // entries are position | level << 16 | negative << 31
 
@@ -332,10 +362,9 @@ __device__ __forceinline__ uint32_t advance(LaneParse& st, uint32_t rend, uint32
   return n;
 }
 
-// Launchers of the three decoders. `handled` / `launched` report whether a kernel was started (a
-// shape can be outside a decoder's reach); the return value is 0 or a cudaError_t.
-int launch_elias_slow(EliasDecodeParams& p, bool dense, bool fused, cudaStream_t stream);
-int launch_elias_fields(FieldParams& p, bool dense, bool fused, cudaStream_t stream, bool* handled);
+// Launchers of the decoders; 0 or a cudaError_t. `launched`: whether the sparse-regime kernel takes the shape.
+int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream);     // Code_s, at most 32 peers
+int launch_elias_teams(const FieldParams& p, bool dense, bool fused, cudaStream_t stream);
 int launch_elias_sparse(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d, uint32_t s, float* out, bool fused,
                         float c, uint32_t* status, bool check_regime, const BucketMap& map, cudaStream_t stream,
                         bool* launched);

@@ -10,40 +10,17 @@
 // and sign bitmap -- for the bucket in shared memory. Phase 2 (apply): exactly the fixed-width
 // decoder's inner loop, reading the fields from shared memory: every lane takes 16 coordinates
 // and adds the peers in ascending k, which fixes the summation order however phase 1 was
-// scheduled. Shapes whose fields do not fit in shared memory go to the
-// decoder of elias_decode_slow.cu.
+// scheduled. Which shapes come here and which are read by teams of lanes: use_teams in elias_decode.cu.
 #include "elias_decode.cuh"
 
 namespace qsgd {
 
 namespace {
 
-// Dense code: the next kDenseBits stream bits usually hold two or three whole (sign, Elias(level + 1))
-// symbols (2, 4, 4, 7 bits for levels 0 .. 3). Entry: symbols held (0 .. 3) | their total length << 2 |
-// (level | negative << 3) << (6 + 4 j) for symbol j; only levels <= min(s, 7) are listed.
-constexpr uint32_t kDenseBits = 10;
-
-__device__ __forceinline__ void fill_dense_lut(uint32_t* lut, uint32_t s) {
-  for (uint32_t i = threadIdx.x; i < (1u << kDenseBits); i += blockDim.x) {
-    uint32_t w = i << (32 - kDenseBits), used = 0, held = 0, entry = 0;
-    while (held < 3u && used + 2u <= kDenseBits) {
-      const uint32_t neg = w >> 31;
-      uint32_t v, len;
-      if (!elias_from_window(w << 1, v, len) || used + 1u + len > kDenseBits || v - 1u > min(s, 7u)) break;
-      entry |= ((v - 1u) | (neg << 3)) << (6u + 4u * held);
-      w <<= 1u + len;
-      used += 1u + len;
-      ++held;
-    }
-    lut[i] = held | (used << 2) | entry;
-  }
-}
-
-template <int LB, bool DENSE>
+template <int LB>
 __device__ __forceinline__ uint32_t parse_to_fields(const PeerSet& peers, uint32_t k, uint64_t b,
                                                     uint64_t B, uint32_t db, uint32_t d, uint32_t s,
-                                                    const uint16_t* lut, const uint32_t* dense_lut,
-                                                    uint32_t* __restrict__ row, float* A_out) {
+                                                    const uint16_t* lut, uint32_t* __restrict__ row, float* A_out) {
   *A_out = 0.f;
   const StringRef ref = string_ref(peers, k, b, B, db);
   if (ref.err) return ref.err;
@@ -54,109 +31,57 @@ __device__ __forceinline__ uint32_t parse_to_fields(const PeerSet& peers, uint32
   uint32_t* srow = row + ((d * LB) >> 5);            // sign bitmap of this peer row
   uint32_t used = 0, err = 0;
   // The row is zero and only this lane writes it, so fields are OR-ed in place.
-  if (DENSE) {
-    // every coordinate is coded, in order: level and sign words fill up in registers and are stored
-    // whole; up to three symbols per table lookup, one by the definition's decoder otherwise
-    uint32_t lw = 0u, sg = 0u;
-    auto put = [&](uint32_t c, uint32_t level, uint32_t neg) {
-      lw |= level << ((c * LB) & 31);
-      sg |= (level ? neg : 0u) << (c & 31);
-      if ((((c + 1u) * LB) & 31u) == 0u) { row[(c * LB) >> 5] = lw; lw = 0u; }
-      if (((c + 1u) & 31u) == 0u) { srow[c >> 5] = sg; sg = 0u; }
-    };
-    uint32_t c = 0;
-    while (c < db) {
+  uint32_t at = 0xFFFFFFFFu;                        // position of the previous nonzero (-1)
+  while (used < total) {
+    // One refill leaves >= 33 bits: enough for a table-decoded triple (<= 12 + 1 + 12 bits).
+    src.refill();
+    uint32_t gap, level, neg;
+    const uint32_t e1 = lut[src.hi >> (32 - kLutBits)];
+    if (e1) {
+      gap = e1 & 0xFFu;
+      src.drop(e1 >> 8);
+      used += e1 >> 8;
+    } else {
+      if (!src.elias(gap, used)) { err = QSGD_DEV_OVERRUN; break; }
       src.refill();
-      const uint32_t e = dense_lut[src.hi >> (32 - kDenseBits)];
-      const uint32_t held = e & 3u;
-      if (held != 0u && c + held <= db) {
-        put(c, (e >> 6) & 7u, (e >> 9) & 1u);
-        if (held > 1u) put(c + 1u, (e >> 10) & 7u, (e >> 13) & 1u);
-        if (held > 2u) put(c + 2u, (e >> 14) & 7u, (e >> 17) & 1u);
-        const uint32_t len = (e >> 2) & 15u;
-        src.drop(len);
-        used += len;
-        c += held;
-        if (used > total) { err = QSGD_DEV_OVERRUN; break; }
-        continue;
-      }
-      const uint32_t neg = src.hi >> 31;
-      uint32_t v, len;
-      const bool ok = elias_from_window(src.hi << 1, v, len);
-      src.drop(len + 1u);
-      used += len + 1u;
-      if (!ok || used > total) { err = QSGD_DEV_OVERRUN; break; }
-      if (v - 1u > s) { err = QSGD_DEV_LEVEL; break; }
-      put(c, v - 1u, neg);
-      ++c;
     }
-    if (!err) {
-      if ((db * LB) & 31u) row[(db * LB) >> 5] = lw;          // a last word that did not fill up
-      if (db & 31u) srow[db >> 5] = sg;
-      if (used != total) err = QSGD_DEV_OVERRUN;
+    neg = src.hi >> 31;
+    const uint32_t e2 = lut[(src.hi << 1) >> (32 - kLutBits)];
+    if (e2) {
+      level = e2 & 0xFFu;
+      src.drop((e2 >> 8) + 1u);
+      used += (e2 >> 8) + 1u;
+    } else {
+      src.drop(1);
+      used += 1;
+      if (!src.elias(level, used)) { err = QSGD_DEV_OVERRUN; break; }
     }
-  } else {
-    uint32_t at = 0xFFFFFFFFu;                        // position of the previous nonzero (-1)
-    while (used < total) {
-      // One refill leaves >= 33 bits: enough for a table-decoded triple (<= 12 + 1 + 12 bits).
-      src.refill();
-      uint32_t gap, level, neg;
-      const uint32_t e1 = lut[src.hi >> (32 - kLutBits)];
-      if (e1) {
-        gap = e1 & 0xFFu;
-        src.drop(e1 >> 8);
-        used += e1 >> 8;
-      } else {
-        if (!src.elias(gap, used)) { err = QSGD_DEV_OVERRUN; break; }
-        src.refill();
-      }
-      neg = src.hi >> 31;
-      const uint32_t e2 = lut[(src.hi << 1) >> (32 - kLutBits)];
-      if (e2) {
-        level = e2 & 0xFFu;
-        src.drop((e2 >> 8) + 1u);
-        used += (e2 >> 8) + 1u;
-      } else {
-        src.drop(1);
-        used += 1;
-        if (!src.elias(level, used)) { err = QSGD_DEV_OVERRUN; break; }
-      }
-      at += gap;
-      if (at >= db || level - 1u >= s || used > total) {     // one rarely taken branch for all three checks
-        err = at >= db ? QSGD_DEV_POSITION : 0u;
-        err |= level - 1u >= s ? QSGD_DEV_LEVEL : 0u;
-        err |= used > total ? QSGD_DEV_OVERRUN : 0u;
-        break;
-      }
-      row[(at * LB) >> 5] |= level << ((at * LB) & 31);
-      srow[at >> 5] |= neg << (at & 31);
+    at += gap;
+    if (at >= db || level - 1u >= s || used > total) {     // one rarely taken branch for all three checks
+      err = at >= db ? QSGD_DEV_POSITION : 0u;
+      err |= level - 1u >= s ? QSGD_DEV_LEVEL : 0u;
+      err |= used > total ? QSGD_DEV_OVERRUN : 0u;
+      break;
     }
+    row[(at * LB) >> 5] |= level << ((at * LB) & 31);
+    srow[at >> 5] |= neg << (at & 31);
   }
   return err;
 }
 
-template <int LB, bool DENSE, bool FUSED, bool SINGLE>
+template <bool FUSED>
 __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_constant__ FieldParams p) {
+  constexpr int LB = 8;
   extern __shared__ __align__(16) uint32_t fsm[];
-  __shared__ __align__(16) float xi_tab[LB == 8 ? 256 * 32 : 32];
-  __shared__ uint16_t elias_lut[DENSE ? 1u : (1u << kLutBits)];
-  __shared__ uint32_t dense_lut[DENSE ? (1u << kDenseBits) : 1u];
+  __shared__ __align__(16) float xi_tab[256 * 32];
+  __shared__ uint16_t elias_lut[1u << kLutBits];
   chain_wait();                                   // the messages come from the kernels ahead
-  if (!DENSE && p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
+  if (p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   const float sf = (float)p.s;
-  float lut0 = 0.f;
-  if (DENSE) fill_dense_lut(dense_lut, p.s);
-  else fill_elias_lut(elias_lut);
-  if (LB == 8) {
-    for (uint32_t i = tid; i < 256 * 32; i += blockDim.x) xi_tab[i] = __fdiv_rn((float)(i >> 5), sf);
-  }
+  fill_elias_lut(elias_lut);
+  for (uint32_t i = tid; i < 256 * 32; i += blockDim.x) xi_tab[i] = __fdiv_rn((float)(i >> 5), sf);
   __syncthreads();
-  if (LB != 8) {
-    const uint32_t level = lane & ((1u << LB) - 1u), neg = (lane >> LB) & 1u;
-    const float q = __fdiv_rn((float)level, sf);
-    lut0 = neg ? -q : q;
-  }
   const uint8_t* tab_lane = reinterpret_cast<const uint8_t*>(xi_tab) + 4 * lane;
 
   const uint32_t warp_words = p.G * p.bucket_words;
@@ -172,19 +97,14 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
     for (uint32_t q = lane; q < (warp_words >> 2); q += 32) reinterpret_cast<uint4*>(mine)[q] = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
     // ---- phase 1: one lane per (bucket, peer) ------------------------------------------------
-    for (uint32_t k = pk; k < p.K; k += 32) {
-      const uint64_t b = b0 + pg;
-      if (pg < p.G && b < p.B) {
-        uint32_t* bucket = mine + pg * p.bucket_words;
-        const uint64_t base = b * p.d;
-        const uint32_t db = (uint32_t)min((uint64_t)p.d, p.n - base);
-        float A;
-        const uint32_t st = parse_to_fields<LB, DENSE>(p.peers, k, b, p.B, db, p.d,
-                                                       p.s, elias_lut, dense_lut, bucket + k * p.row_words, &A);
-        reinterpret_cast<float*>(bucket + p.K * p.row_words)[k] = A;
-        if (st) atomicOr(p.status, st);
-      }
-      if (p.Kpad < 32) break;
+    if (pk < p.K && pg < p.G && b0 + pg < p.B) {
+      uint32_t* bucket = mine + pg * p.bucket_words;
+      const uint32_t db = (uint32_t)min((uint64_t)p.d, p.n - (b0 + pg) * p.d);
+      float A;
+      const uint32_t st = parse_to_fields<LB>(p.peers, pk, b0 + pg, p.B, db, p.d, p.s, elias_lut,
+                                              bucket + pk * p.row_words, &A);
+      reinterpret_cast<float*>(bucket + p.K * p.row_words)[pk] = A;
+      if (st) atomicOr(p.status, st);
     }
     __syncwarp();
     // ---- phase 2: the fixed-width decoder's inner loop over the rebuilt fields ----------------
@@ -208,21 +128,10 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
         if (live) {
           A = scales[k];
           sb = (row[level_words + (c >> 5)] >> (c & 31)) & 0xFFFFu;
-          if (LB == 8) {
-            const uint4 t = *reinterpret_cast<const uint4*>(row + (c >> 2));
-            w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
-          } else if (LB == 4) {
-            const uint2 t = *reinterpret_cast<const uint2*>(row + (c >> 3));
-            w[0] = t.x; w[1] = t.y;
-          } else if (LB == 2) {
-            w[0] = row[c >> 4];
-          } else {
-            w[0] = (row[c >> 5] >> (c & 31)) & 0xFFFFu;
-          }
+          const uint4 t = *reinterpret_cast<const uint4*>(row + (c >> 2));
+          w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
         }
-        if (LB == 8) add_peer_tab(acc, w, sb, tab_lane, A);
-        else if (SINGLE) add_peer_lut<LB, true>(acc, w, sb, __fmul_rn(__shfl_sync(0xffffffffu, A, 0), lut0), A);
-        else add_peer_lut<LB, false>(acc, w, sb, lut0, A);
+        add_peer_tab(acc, w, sb, tab_lane, A);
       }
       if (live) {
         if (p.map.src) store_span16<FUSED>(out_span(p.out, p.map, b, c, p.d, p.n, 16u), acc, p.c);
@@ -233,89 +142,66 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
   }
 }
 
-template <int LB, bool DENSE>
-int launch_fields(FieldParams& p, bool fused, cudaStream_t stream, bool* handled) {
-  *handled = false;
-  int dev = 0, max_smem = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const uint32_t level_words = (p.d * LB) >> 5, sign_words = p.d >> 5;
+int launch_fields(FieldParams& p, bool fused, cudaStream_t stream) {
+  static KernelSite site[2];
+  int max_smem = 0;
+  const int st0 = device_shared_memory(&max_smem);
+  if (st0) return st0;
+  const uint32_t level_words = p.d >> 2, sign_words = p.d >> 5;
   p.row_words = (level_words + sign_words + 3u) & ~3u;
   p.bucket_words = (p.K * p.row_words + p.K + 3u) & ~3u;
   uint32_t kpad = 1;
-  while (kpad < p.K && kpad < 32) kpad <<= 1;
+  while (kpad < p.K) kpad <<= 1;
   p.Kpad = kpad;
-  uint32_t G = p.K <= 32 ? 32 / kpad : 1;
+  uint32_t G = 32 / kpad;
   while (G > 1 && (size_t)G * p.bucket_words * 4 > (16u << 10)) G >>= 1;
   p.G = G;
   const size_t per_warp = (size_t)G * p.bucket_words * 4;
-  const size_t budget = (size_t)max_smem - (LB == 8 ? 32768 : 128) - 8192 - 1024;
   // Warps per CTA: the count that leaves the most warps resident on an SM. The code table and the
   // level table are per CTA, the fields per warp; the parse is latency-bound, so warps are what counts.
-  const size_t per_cta = (LB == 8 ? 32768 : 128) + 8192 + 1024;
+  const size_t per_cta = 32768 + 8192 + 1024, budget = (size_t)max_smem - per_cta;
   const size_t per_sm = 227u << 10;
-  int warps = 0, best = 0;
+  int warps = 1, best = 0;
   for (int w = 1; w <= 10; ++w) {
     if ((size_t)w * per_warp > budget) break;
     const int resident = (int)(per_sm / ((size_t)w * per_warp + per_cta)) * w;
     if (resident > best) { best = resident; warps = w; }
   }
-  if (warps == 0) return 0;                                      // caller falls back to the slow kernel
-  const bool single = p.d >= 512 && (p.d & (p.d - 1)) == 0 && LB != 8;
-  void (*kern)(FieldParams);
-  if (fused) kern = single ? decode_elias_fields_kernel<LB, DENSE, true, true> : decode_elias_fields_kernel<LB, DENSE, true, false>;
-  else kern = single ? decode_elias_fields_kernel<LB, DENSE, false, true> : decode_elias_fields_kernel<LB, DENSE, false, false>;
+  auto kern = fused ? decode_elias_fields_kernel<true> : decode_elias_fields_kernel<false>;
   const size_t smem = (size_t)warps * per_warp;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return (int)e;
-  int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, smem);
-  if (e != cudaSuccess) return (int)e;
-  if (occ < 1) occ = 1;
+  int sms = 0, occ = 0;
+  const int st = site[fused ? 1 : 0].lookup_dynamic(kern, warps * 32, smem, &sms, &occ);
+  if (st) return st;
   const uint64_t groups = (p.B + G - 1) / G;
   const uint64_t want = (groups + warps - 1) / warps;
   const uint64_t cap = (uint64_t)sms * occ;
-  const uint32_t grid = (uint32_t)(want < cap ? want : cap);
-  {
-    ScopedKernel sk(kKernDecodeElias, stream);
-    const cudaError_t le = launch_chained(kern, grid, warps * 32, smem, stream, p);
-    if (le != cudaSuccess) return (int)le;
-  }
-  *handled = true;
-  return (int)cudaGetLastError();
+  ScopedKernel sk(kKernDecodeElias, stream);
+  return (int)launch_chained(kern, (uint32_t)(want < cap ? want : cap), warps * 32, smem, stream, p);
 }
 
 // ------------------------------------------------------------------------------------------------
-// Field-rebuilding decoder for long buckets (d >= 1024): the same two phases, but a bucket is
+// Field-rebuilding decoder for long buckets (d >= 1024) of few levels (s <= 3), where strings are many and
+// nearly empty (use_teams in elias_decode.cu draws the line): the same two phases, but a bucket is
 // walked in ranges of 512 positions. A lane keeps its place in its string between ranges (bit
 // window, position, one decoded entry that lies past the range), so shared memory holds the fields
 // of one range only and as many warps fit on an SM as for d = 512; with whole-bucket fields a CTA
 // of d = 4096 is down to one or two warps.
 // ------------------------------------------------------------------------------------------------
-template <int LB, bool DENSE, bool FUSED>
+template <int LB, bool FUSED>
 __global__ void __launch_bounds__(128) decode_elias_ranged_kernel(const __grid_constant__ FieldParams p) {
   constexpr uint32_t kR = 512;                                  // positions per range = one warp pass of phase 2
   constexpr uint32_t kLevelWords = kR * LB / 32, kRowWords = kLevelWords + kR / 32;
   extern __shared__ __align__(16) uint32_t fsm[];
-  __shared__ __align__(16) float xi_tab[LB == 8 ? 256 * 32 : 32];
-  __shared__ uint32_t dense_lut[DENSE ? (1u << kDenseBits) : 1u];
-  if (DENSE) fill_dense_lut(dense_lut, p.s);
   chain_wait();                                   // the messages come from the kernels ahead
-  if (!DENSE && p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
+  if (p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   const float sf = (float)p.s;
   float lut0 = 0.f;
-  if (LB == 8) {
-    for (uint32_t i = tid; i < 256 * 32; i += blockDim.x) xi_tab[i] = __fdiv_rn((float)(i >> 5), sf);
-  }
-  __syncthreads();
-  if (LB != 8) {
+  {
     const uint32_t level = lane & ((1u << LB) - 1u), neg = (lane >> LB) & 1u;
     const float q = __fdiv_rn((float)level, sf);
     lut0 = neg ? -q : q;
   }
-  const uint8_t* tab_lane = reinterpret_cast<const uint8_t*>(xi_tab) + 4 * lane;
 
   // per warp: G * K rows of kRowWords (level fields, then sign bits, of one range) | 32 scales
   const uint32_t rows_words = p.G * p.K * kRowWords;
@@ -355,56 +241,11 @@ __global__ void __launch_bounds__(128) decode_elias_ranged_kernel(const __grid_c
       // ---- phase 1: this lane's entries of the range, OR-ed into its zeroed row ----------------
       if (readable) {
         uint32_t* srow = row + kLevelWords;
-        if (DENSE) {
-          // every coordinate is coded, in order: level and sign words fill up in registers and are
-          // stored whole (the row is zero, and a range starts on a word boundary)
-          const uint32_t lim = min(rend, db), cnt = lim > rbeg ? lim - rbeg : 0u;
-          uint32_t lw = 0u, sg = 0u;
-          auto put = [&](uint32_t pos, uint32_t level, uint32_t neg) {
-            lw |= level << ((pos * LB) & 31);
-            sg |= (level ? neg : 0u) << (pos & 31);
-            if ((((pos + 1u) * LB) & 31u) == 0u) { row[(pos * LB) >> 5] = lw; lw = 0u; }
-            if (((pos + 1u) & 31u) == 0u) { srow[pos >> 5] = sg; sg = 0u; }
-          };
-          uint32_t pos = 0;
-          while (pos < cnt && st.err == 0u) {
-            st.src.refill();
-            const uint32_t e = dense_lut[st.src.hi >> (32 - kDenseBits)];
-            const uint32_t held = e & 3u;
-            if (held != 0u && pos + held <= cnt) {            // two or three symbols at once (or one)
-              put(pos, (e >> 6) & 7u, (e >> 9) & 1u);
-              if (held > 1u) put(pos + 1u, (e >> 10) & 7u, (e >> 13) & 1u);
-              if (held > 2u) put(pos + 2u, (e >> 14) & 7u, (e >> 17) & 1u);
-              const uint32_t len = (e >> 2) & 15u;
-              st.src.drop(len);
-              st.used += len;
-              pos += held;
-              if (st.used > st.total) st.err = QSGD_DEV_OVERRUN;
-              continue;
-            }
-            // one symbol by the definition's decoder: a level above 7, or fewer coordinates left
-            // in the range than the entry holds
-            const uint32_t neg = st.src.hi >> 31;
-            uint32_t v, len;
-            const bool ok = elias_from_window(st.src.hi << 1, v, len);
-            st.src.drop(len + 1u);
-            st.used += len + 1u;
-            if (!ok || st.used > st.total) st.err = QSGD_DEV_OVERRUN;
-            else if (v - 1u > p.s) st.err = QSGD_DEV_LEVEL;
-            else put(pos, v - 1u, neg);
-            ++pos;
-          }
-          if (st.err == 0u && cnt) {                        // a last word that did not fill up
-            if ((cnt * LB) & 31u) row[(cnt * LB) >> 5] = lw;
-            if (cnt & 31u) srow[cnt >> 5] = sg;
-          }
-        } else {
-          advance(st, rend, 0xFFFFFFFFu, db, p.s, [&](uint32_t, uint32_t en) {
-            const uint32_t pos = (en & 0xFFFFu) - rbeg;
-            row[(pos * LB) >> 5] |= ((en >> 16) & 0xFFu) << ((pos * LB) & 31);
-            srow[pos >> 5] |= (en >> 31) << (pos & 31);
-          });
-        }
+        advance(st, rend, 0xFFFFFFFFu, db, p.s, [&](uint32_t, uint32_t en) {
+          const uint32_t pos = (en & 0xFFFFu) - rbeg;
+          row[(pos * LB) >> 5] |= ((en >> 16) & 0xFFu) << ((pos * LB) & 31);
+          srow[pos >> 5] |= (en >> 31) << (pos & 31);
+        });
       }
       __syncwarp();
       // ---- phase 2: one warp pass per bucket over the range's fields, ascending k ---------------
@@ -425,20 +266,13 @@ __global__ void __launch_bounds__(128) decode_elias_ranged_kernel(const __grid_c
           const float Ak = scales[g * p.Kpad + k];
           if (live) {
             sb = (rk[kLevelWords + (cl >> 5)] >> (cl & 31)) & 0xFFFFu;
-            if (LB == 8) {
-              const uint4 t = *reinterpret_cast<const uint4*>(rk + (cl >> 2));
-              w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
-            } else if (LB == 4) {
-              const uint2 t = *reinterpret_cast<const uint2*>(rk + (cl >> 3));
-              w[0] = t.x; w[1] = t.y;
-            } else if (LB == 2) {
+            if (LB == 2) {
               w[0] = rk[cl >> 4];
             } else {
               w[0] = (rk[cl >> 5] >> (cl & 31)) & 0xFFFFu;
             }
           }
-          if (LB == 8) add_peer_tab(acc, w, sb, tab_lane, live ? Ak : 0.f);
-          else add_peer_lut<LB, true>(acc, w, sb, __fmul_rn(Ak, lut0), Ak);
+          add_peer_lut<LB, true>(acc, w, sb, __fmul_rn(Ak, lut0), Ak);
         }
         if (live) {
           if (p.map.src) store_span16<FUSED>(out_span(p.out, p.map, b, c, p.d, p.n, 16u), acc, p.c);
@@ -454,13 +288,9 @@ __global__ void __launch_bounds__(128) decode_elias_ranged_kernel(const __grid_c
   }
 }
 
-template <int LB, bool DENSE>
-int launch_ranged(FieldParams& p, bool fused, cudaStream_t stream, bool* handled) {
-  *handled = false;
-  if (p.K > 32u) return 0;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+template <int LB>
+int launch_ranged(FieldParams& p, bool fused, cudaStream_t stream) {
+  static KernelSite site[2];
   constexpr uint32_t kRowWords = 512u * LB / 32u + 16u;
   uint32_t kpad = 1;
   while (kpad < p.K) kpad <<= 1;
@@ -468,25 +298,16 @@ int launch_ranged(FieldParams& p, bool fused, cudaStream_t stream, bool* handled
   p.G = 32u / kpad;
   const size_t per_warp = ((size_t)p.G * p.K * kRowWords + 32u) * 4;   // at most 18.6 KB
   const int warps = 4;
-  auto kern = fused ? decode_elias_ranged_kernel<LB, DENSE, true> : decode_elias_ranged_kernel<LB, DENSE, false>;
+  auto kern = fused ? decode_elias_ranged_kernel<LB, true> : decode_elias_ranged_kernel<LB, false>;
   const size_t smem = (size_t)warps * per_warp;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return (int)e;
-  int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, smem);
-  if (e != cudaSuccess) return (int)e;
-  if (occ < 1) occ = 1;
+  int sms = 0, occ = 0;
+  const int st = site[fused ? 1 : 0].lookup_dynamic(kern, warps * 32, smem, &sms, &occ);
+  if (st) return st;
   const uint64_t groups = (p.B + p.G - 1) / p.G;
   const uint64_t want = (groups + warps - 1) / warps;
   const uint64_t cap = (uint64_t)sms * occ;
-  const uint32_t grid = (uint32_t)(want < cap ? want : cap);
-  {
-    ScopedKernel sk(kKernDecodeElias, stream);
-    const cudaError_t le = launch_chained(kern, grid, warps * 32, smem, stream, p);
-    if (le != cudaSuccess) return (int)le;
-  }
-  *handled = true;
-  return (int)cudaGetLastError();
+  ScopedKernel sk(kKernDecodeElias, stream);
+  return (int)launch_chained(kern, (uint32_t)(want < cap ? want : cap), warps * 32, smem, stream, p);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -705,72 +526,49 @@ __global__ void __launch_bounds__(512) decode_elias_bytes_kernel(const __grid_co
   }
 }
 
-int launch_bytes(FieldParams& p, bool fused, cudaStream_t stream, bool* handled) {
-  *handled = false;
-  if (p.K > 32u) return 0;
-  int dev = 0, max_smem = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+int launch_bytes(FieldParams& p, bool fused, cudaStream_t stream) {
+  static KernelSite site[4];
+  int max_smem = 0;
+  const int st0 = device_shared_memory(&max_smem);
+  if (st0) return st0;
   uint32_t kpad = 1;
   while (kpad < p.K) kpad <<= 1;
   p.Kpad = kpad;
   p.G = 32u / kpad;
   const uint32_t R = p.d <= kByteRange ? p.d : kByteRange;
   p.range = R;
-  const size_t per_warp = (size_t)p.G * p.K * (R + kRowPad) + 128u;
+  const size_t per_warp = (size_t)p.G * p.K * (R + kRowPad) + 128u;     // at most 8.8 KB
   const size_t per_cta = 8192 + 512 + 1024;                     // the two code tables + slack
   const size_t budget = (size_t)max_smem - per_cta;
   const size_t per_sm = 227u << 10;
-  int warps = 0, best = 0;
+  int warps = 1, best = 0;
   for (int w = 1; w <= 16; ++w) {
     if ((size_t)w * per_warp > budget) break;
     const int resident = (int)(per_sm / ((size_t)w * per_warp + per_cta)) * w;
     if (resident > best) { best = resident; warps = w; }
   }
-  if (warps == 0) return 0;
   const bool single = (p.d & 255u) == 0;                        // every range is 256 long: a pass of 32 lanes x 8 stays inside one bucket
   void (*kern)(FieldParams);
   if (fused) kern = single ? decode_elias_bytes_kernel<true, true> : decode_elias_bytes_kernel<true, false>;
   else kern = single ? decode_elias_bytes_kernel<false, true> : decode_elias_bytes_kernel<false, false>;
   const size_t smem = (size_t)warps * per_warp;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return (int)e;
-  int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, smem);
-  if (e != cudaSuccess) return (int)e;
-  if (occ < 1) occ = 1;
+  int sms = 0, occ = 0;
+  const int st = site[(fused ? 2 : 0) + (single ? 1 : 0)].lookup_dynamic(kern, warps * 32, smem, &sms, &occ);
+  if (st) return st;
   const uint64_t groups = (p.B + p.G - 1) / p.G;
   const uint64_t want = (groups + warps - 1) / warps;
   const uint64_t cap = (uint64_t)sms * occ;
-  const uint32_t grid = (uint32_t)(want < cap ? want : cap);
-  {
-    ScopedKernel sk(kKernDecodeElias, stream);
-    const cudaError_t le = launch_chained(kern, grid, warps * 32, smem, stream, p);
-    if (le != cudaSuccess) return (int)le;
-  }
-  *handled = true;
-  return (int)cudaGetLastError();
-}
-
-
-template <int LB>
-int launch_fields_lb(FieldParams& p, bool dense, bool fused, cudaStream_t stream, bool* handled) {
-  if (!dense && LB != 8 && p.d < 1024u && p.K <= 32u) return launch_bytes(p, fused, stream, handled);
-  if (p.d >= 1024u && p.K <= 32u)       // long buckets: fields of one range at a time
-    return dense ? launch_ranged<LB, true>(p, fused, stream, handled) : launch_ranged<LB, false>(p, fused, stream, handled);
-  return dense ? launch_fields<LB, true>(p, fused, stream, handled) : launch_fields<LB, false>(p, fused, stream, handled);
+  ScopedKernel sk(kKernDecodeElias, stream);
+  return (int)launch_chained(kern, (uint32_t)(want < cap ? want : cap), warps * 32, smem, stream, p);
 }
 
 }  // namespace
 
-int launch_elias_fields(FieldParams& p, bool dense, bool fused, cudaStream_t stream, bool* handled) {
-  switch (level_bits_for(p.s)) {
-    case 1: return launch_fields_lb<1>(p, dense, fused, stream, handled);
-    case 2: return launch_fields_lb<2>(p, dense, fused, stream, handled);
-    case 4: return launch_fields_lb<4>(p, dense, fused, stream, handled);
-    default: return launch_fields_lb<8>(p, dense, fused, stream, handled);
-  }
+int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream) {
+  const uint32_t lb = level_bits_for(p.s);
+  if (lb == 8u) return launch_fields(p, fused, stream);
+  if (p.d < 1024u) return launch_bytes(p, fused, stream);
+  return lb == 1u ? launch_ranged<1>(p, fused, stream) : launch_ranged<2>(p, fused, stream);    // s <= 3 (use_teams)
 }
 
 }  // namespace qsgd

@@ -219,9 +219,10 @@ int launch_elias_sparse(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
                         bool* launched) {
   *launched = false;
   if (K > 32u) return 0;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  static KernelSite site[2];
+  int sms = 0;
+  const int st0 = device_sms(&sms);
+  if (st0) return st0;
   SparseParams p;
   p.peers = peers; p.K = K; p.n = n; p.d = d; p.s = s;
   p.B = (n + d - 1) / d;
@@ -247,12 +248,9 @@ int launch_elias_sparse(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
   }
   auto kern = fused ? decode_elias_sparse_kernel<true> : decode_elias_sparse_kernel<false>;
   const size_t smem = (size_t)warps * per_warp;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return (int)e;
   int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, smem);
-  if (e != cudaSuccess) return (int)e;
-  if (occ < 1) occ = 1;
+  const int st = site[fused ? 1 : 0].lookup_dynamic(kern, warps * 32, smem, &sms, &occ);
+  if (st) return st;
   const uint64_t groups = (p.B + p.sh.G - 1) / p.sh.G;
   const uint64_t want = (groups + warps - 1) / warps;
   const uint64_t cap = (uint64_t)sms * occ;
@@ -263,7 +261,7 @@ int launch_elias_sparse(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
     if (le != cudaSuccess) return (int)le;
   }
   *launched = true;
-  return (int)cudaGetLastError();
+  return 0;
 }
 
 }  // namespace qsgd

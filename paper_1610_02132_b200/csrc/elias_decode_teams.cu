@@ -1,0 +1,469 @@
+// Decode-and-aggregate, Elias path, for problems with too few strings to give every lane of the GPU one of
+// its own: a team of up to 32 lanes shares a string. (Section 3.1 for the string, Appendix A.2 and A.3 for
+// the codes, Algorithm 1 for the sum and the step.)
+//
+// A string can only be read front to back, but a reader that starts at the wrong bit usually falls into
+// step with the right one after a few symbols (the self-synchronisation of variable-length codes used for
+// parallel Huffman decoding: Weissenberger & Schmidt, ICPP 2018). Lane t of a team owns the t-th part of
+// the string's bits. It starts kWarmUp bits ahead of its part, reads up to the first symbol that starts in
+// it, then reads its part through, counting positions. Its start is right when it is where lane t - 1
+// ended; where it is not, the lane reads its part again from there, and so on until all agree. Lane 0 is
+// right from the start and every round makes at least one more lane right, so T rounds always suffice
+// (the time of reading the string by one lane); two or three are the rule. A scan of the counts gives
+// every lane the position its part starts at, and a last reading writes one code per coordinate (level,
+// sign) into the string's row in shared memory. Then all threads add the rows in ascending k.
+//
+// Latency is what counts here: one string of 4096 dense symbols read by one lane is 300 us, whatever else
+// the GPU does.
+#include <type_traits>
+
+#include "elias_decode.cuh"
+
+namespace qsgd {
+
+namespace {
+
+constexpr uint32_t kThreads = 256;
+constexpr uint32_t kWarmUp = 64;                  // bits: 75-95 % of the starts are then right
+constexpr uint32_t kLeastPart = 64;               // bits of a string that are worth a lane
+constexpr uint32_t kDenseBits = 10;
+constexpr uint32_t kRowPad = 16;                  // bytes between rows: teams at similar positions use other banks
+
+constexpr uint32_t kLanesPerSm = 1024;            // lanes that fill an SM well enough
+constexpr size_t kMostBytes = 108u << 10;         // shared memory of a CTA: two of them fit on an SM
+
+// One code per coordinate: level | negative << kSignShift. s <= 15: 5 bits, the lane index of the value in a
+// shuffle table; s <= 127: 8 bits; else 9 bits, in 16.
+enum CodeWidth { kNibble = 0, kByte = 1, kWide = 2 };
+template <int WIDTH> struct CodeOf {
+  using type = uint8_t;
+  static constexpr uint32_t kSignShift = WIDTH == kNibble ? 4u : 7u;
+};
+template <> struct CodeOf<kWide> {
+  using type = uint16_t;
+  static constexpr uint32_t kSignShift = 8u;
+};
+
+struct TeamParams {
+  PeerSet peers;
+  uint32_t K;
+  uint32_t Kc;            // peers per pass
+  uint64_t n;
+  uint32_t d;
+  uint32_t s;
+  uint64_t B;
+  float* out;             // acc (overwritten) or x (updated in place)
+  float c;                // eta / K
+  uint32_t* status;
+  uint32_t T;             // lanes per string, a power of two
+  uint32_t buckets;       // per CTA and pass
+  uint32_t row_bytes;
+  uint32_t share;         // bytes of staging per peer
+  uint32_t defer_sparse;  // a sparse-regime kernel was launched beside this one
+  BucketMap map;
+};
+
+// Where in its row the code of a position lies. The lanes of a team write at positions a fixed distance
+// apart (128 with 4096 coordinates and 32 lanes: one bank for all), so the pieces that the sum reads at
+// once (8 codes) are permuted inside each block of 128 bytes by the number of the block.
+template <int WIDTH>
+__device__ __forceinline__ uint32_t place(uint32_t pos) {       // in bytes
+  if (WIDTH == kWide) { const uint32_t a = 2u * pos; return a ^ ((a >> 3) & 0x70u); }
+  return pos ^ ((pos >> 4) & 0x78u);
+}
+
+struct Tables {
+  uint2 code[kCodeEntries];
+  // Code_s, s <= 15: what follows a gap (tail_entry). Code'_s: what the next 10 bits hold, up to three
+  // symbols of levels <= 7: their codes in bytes 0, 1 and 2 (kWide: level | negative << 7), their length in
+  // byte 3, bits 0-3, their number in bits 4-5; 0 when they hold none
+  uint32_t symbol[1 << kDenseBits];
+};
+
+// Reads symbols from bit `from` to the first one that starts at or behind bit `until` (both counted from
+// bit 0 of words[0]; `end`: first bit behind the string). Returns where that is; *sum: the gaps or, in the
+// dense code, the symbols passed. What is no symbol (the reader is out of step, or the string is
+// malformed) still moves it on.
+template <bool DENSE, int WIDTH>
+__device__ __forceinline__ uint32_t walk(const Tables& tab, const uint32_t* words, uint32_t from, uint32_t until,
+                                         uint32_t end, uint32_t* sum) {
+  *sum = 0;
+  if (from >= until) return from;
+  Window in;
+  in.open(words, from);
+  const uint32_t origin = from & ~31u;
+  const uint32_t stop = until - origin, last = end - origin;
+  uint32_t n = 0;
+  while (in.bp < stop) {
+    const uint32_t w = in.peek();
+    if (DENSE) {
+      const uint32_t e = tab.symbol[w >> (32 - kDenseBits)];
+      if (e && in.bp + kDenseBits <= stop) {
+        in.drop((e >> 24) & 15u, last);
+        n += e >> 28;
+      } else {
+        in.drop(code_body(tab.code[(w << 1) >> 25]) + 2u, last);
+        ++n;
+      }
+    } else {
+      const uint2 e = tab.code[w >> 25];
+      const uint32_t body = code_body(e);
+      n += code_value(w, e);
+      if (WIDTH == kNibble) {
+        const uint32_t tail = tab.symbol[(w << body) >> (32 - kTailBits)];
+        in.drop(tail ? body + (tail >> 8) : body + 1u, last);
+      } else {
+        const uint32_t y = in.peek_at(body) << 2;
+        in.drop(body, last);
+        in.drop(code_body(tab.code[y >> 25]) + 3u, last);
+      }
+    }
+  }
+  *sum = n;
+  return origin + in.bp;
+}
+
+// The last reading: the same part, every check, one code per coordinate into the row. `at`: position of
+// the last nonzero in front of the part (Code_s) or the part's first position (Code'_s).
+template <bool DENSE, int WIDTH>
+__device__ __forceinline__ uint32_t emit(const Tables& tab, const uint32_t* words, uint32_t from, uint32_t until,
+                                         uint32_t end, uint32_t at, uint32_t db, uint32_t s, uint8_t* row) {
+  using Code = typename CodeOf<WIDTH>::type;
+  auto put = [&](uint32_t pos, uint32_t code) { *reinterpret_cast<Code*>(row + place<WIDTH>(pos)) = (Code)code; };
+  constexpr uint32_t kSignShift = CodeOf<WIDTH>::kSignShift;
+  if (from >= until) return 0u;
+  Window in;
+  in.open(words, from);
+  const uint32_t origin = from & ~31u;
+  const uint32_t stop = until - origin, last = end - origin;
+  uint32_t bad = 0;
+  while (in.bp < stop) {
+    const uint32_t w = in.peek();
+    if (DENSE) {
+      const uint32_t e = tab.symbol[w >> (32 - kDenseBits)], held = e >> 28;
+      if (e && in.bp + kDenseBits <= stop && at + held <= db) {
+        if (WIDTH == kWide) {
+#pragma unroll
+          for (uint32_t j = 0; j < 3; ++j)
+            if (j < held) put(at + j, ((e >> (8u * j)) & 7u) | ((e >> (8u * j)) & 0x80u) << 1);
+        } else {
+          put(at, e);
+          if (held > 1u) put(at + 1u, e >> 8);
+          if (held > 2u) put(at + 2u, e >> 16);
+        }
+        in.drop((e >> 24) & 15u, last);
+        at += held;
+        continue;
+      }
+      const uint32_t x = w << 1;
+      const uint2 c = tab.code[x >> 25];
+      const uint32_t level = code_value(x, c) - 1u, body = code_body(c);
+      bad |= x << body;                           // the closing bit
+      if (level > s) return QSGD_DEV_LEVEL;
+      if (at >= db) return QSGD_DEV_OVERRUN;      // more symbols than coordinates
+      put(at, level | (level ? (w >> 31) << kSignShift : 0u));
+      ++at;
+      in.drop(body + 2u, last);
+    } else {
+      const uint2 e = tab.code[w >> 25];
+      const uint32_t body = code_body(e);
+      at += code_value(w, e);
+      if (WIDTH == kNibble) {
+        const uint32_t y = w << body, tail = tab.symbol[y >> (32 - kTailBits)];
+        if (tail == 0u) return y >> 31 ? QSGD_DEV_OVERRUN : in.bp + body + 2u > last ? QSGD_DEV_OVERRUN : QSGD_DEV_LEVEL;
+        if (at >= db) return QSGD_DEV_POSITION;
+        put(at, tail);
+        in.drop(body + (tail >> 8), last);
+      } else {
+        const uint32_t y = in.peek_at(body), z = y << 2;
+        const uint2 c = tab.code[z >> 25];
+        const uint32_t level = code_value(z, c), lb = code_body(c);
+        bad |= y | (z << lb);                     // the two closing bits
+        if (at >= db) return QSGD_DEV_POSITION;
+        if (level > s) return QSGD_DEV_LEVEL;
+        put(at, level | (((y >> 30) & 1u) << kSignShift));
+        in.drop(body, last);
+        in.drop(lb + 3u, last);
+      }
+    }
+  }
+  return bad >> 31 ? QSGD_DEV_OVERRUN : 0u;
+}
+
+// Reads a part in kMarks pieces and keeps where each piece ended, so that a lane that has to read its part
+// again from another bit can stop at the first mark where it falls into step with its first reading.
+constexpr uint32_t kMarks = 4;
+constexpr uint32_t kLeastPiece = 96;      // bits
+struct Marks {
+  uint32_t pos[kMarks];       // first symbol at or behind the mark
+  uint32_t sum[kMarks];       // positions from the part's start up to there
+};
+
+template <bool DENSE, int WIDTH>
+__device__ __forceinline__ void read_part(const Tables& tab, const uint32_t* words, uint32_t start, uint32_t lo,
+                                          uint32_t hi, uint32_t end, bool again, Marks& m) {
+  const uint32_t piece = max((hi - lo + kMarks - 1u) / kMarks, kLeastPiece);
+  uint32_t pos = start, sum = 0;
+#pragma unroll
+  for (uint32_t q = 0; q < kMarks; ++q) {
+    uint32_t n;
+    pos = walk<DENSE, WIDTH>(tab, words, pos, q == kMarks - 1u ? hi : min(lo + (q + 1u) * piece, hi), end, &n);
+    sum += n;
+    if (again && pos == m.pos[q]) {                 // in step from here on: the rest differs by the count only
+      const uint32_t more = sum - m.sum[q];
+#pragma unroll
+      for (uint32_t r = 0; r < kMarks; ++r)
+        if (r >= q) m.sum[r] += more;
+      return;
+    }
+    m.pos[q] = pos;
+    m.sum[q] = sum;
+  }
+}
+
+template <bool DENSE, int WIDTH, bool FUSED>
+__global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __grid_constant__ TeamParams p) {
+  using Code = typename CodeOf<WIDTH>::type;
+  constexpr uint32_t kLevels = 1u << CodeOf<WIDTH>::kSignShift;
+  extern __shared__ __align__(16) uint8_t tsm[];
+  __shared__ Tables tab;
+  __shared__ float xi[2 * kLevels];                     // +-(level / s) by code
+  const uint32_t tid = threadIdx.x, lane = tid & 31;
+  const float sf = (float)p.s;
+  for (uint32_t i = tid; i < kCodeEntries; i += kThreads) tab.code[i] = code_entry(i);
+  if (DENSE) {
+    for (uint32_t i = tid; i < (1u << kDenseBits); i += kThreads) {
+      uint32_t w = i << (32 - kDenseBits), used = 0, held = 0, entry = 0;
+      while (held < 3u && used + 2u <= kDenseBits) {
+        uint32_t v, len;
+        if (!elias_from_window(w << 1, v, len) || used + 1u + len > kDenseBits || v - 1u > min(p.s, 7u)) break;
+        entry |= ((v - 1u) | (v > 1u ? (w >> 31) << (WIDTH == kNibble ? 4 : 7) : 0u)) << (8u * held);
+        w <<= 1u + len;
+        used += 1u + len;
+        ++held;
+      }
+      tab.symbol[i] = held ? entry | (used << 24) | (held << 28) : 0u;
+    }
+  } else if (WIDTH == kNibble) {
+    for (uint32_t i = tid; i < kTailEntries; i += kThreads) tab.symbol[i] = tail_entry(i, p.s);
+  }
+  for (uint32_t i = tid; i < 2u * kLevels; i += kThreads) {
+    const float q = __fdiv_rn((float)(i & (kLevels - 1u)), sf);
+    xi[i] = i & kLevels ? -q : q;
+  }
+
+  // rows[bucket][peer] of one pass over the peers | their strings | with several passes, the sums so far |
+  // the scales
+  const uint32_t most = p.buckets * p.Kc;
+  uint8_t* strings = tsm + (size_t)most * p.row_bytes;
+  float* sums = reinterpret_cast<float*>(strings + (size_t)p.Kc * p.share);
+  float* scales = sums + (p.Kc < p.K ? p.buckets * p.d : 0u);
+  const uint32_t T = p.T, t = lane & (T - 1u), team = tid / T, teams = kThreads / T;
+  const uint64_t groups = (p.B + p.buckets - 1) / p.buckets;
+  chain_wait();                                         // the messages come from the kernels ahead
+  if (!DENSE && p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
+
+  for (uint64_t grp = blockIdx.x; grp < groups; grp += gridDim.x) {
+    const uint64_t b0 = grp * p.buckets;
+    const uint32_t nb = (uint32_t)min((uint64_t)p.buckets, p.B - b0);
+    for (uint32_t k0 = 0; k0 < p.K; k0 += p.Kc) {
+      const uint32_t kc = min(p.Kc, p.K - k0), rows = p.buckets * kc;
+      // ---- peer k's strings of these buckets are one stretch of its payload: a warp copies it --------
+      // (a stretch that its table makes longer than the share is read where it is)
+      for (uint32_t k = tid >> 5; k < kc && p.share; k += kThreads >> 5) {
+        PeerTable pt;
+        if (!peer_table(p.peers, k0 + k, p.B, &pt)) continue;
+        const uint64_t from = __ldg(pt.table + b0) >> 7, to = (__ldg(pt.table + b0 + nb) + 127u) >> 7;   // 16-byte units
+        const uint64_t all = __ldg(pt.table + p.B);
+        if (all > pt.cap_bits || from > to || to * 128u > align16((all + 7u) / 8u) * 8u || (to - from + 1u) * 16u > p.share) continue;
+        const uint4* src = reinterpret_cast<const uint4*>(p.peers.payload[k0 + k]) + from;
+        uint4* dst = reinterpret_cast<uint4*>(strings + (size_t)k * p.share);
+        for (uint32_t i = lane; i <= (uint32_t)(to - from); i += 32) dst[i] = __ldg(src + i);   // and 16 bytes behind it
+      }
+      for (uint32_t i = tid; i < rows * (p.row_bytes >> 4); i += kThreads)
+        reinterpret_cast<uint4*>(tsm)[i] = make_uint4(0u, 0u, 0u, 0u);
+      __syncthreads();
+
+      // ---- the strings, one per team and pass -------------------------------------------------------
+      for (uint32_t j0 = 0; j0 < rows; j0 += teams) {
+        const uint32_t j = j0 + team;
+        const uint32_t g = j / kc, k = j - g * kc;         // k: in this pass
+        const uint64_t b = b0 + g;
+        const bool mine = j < rows && g < nb;
+        StringRef ref;
+        ref.words = nullptr; ref.lo = 0; ref.total = 0; ref.err = 0;
+        uint32_t db = 0;
+        const uint32_t* words = nullptr;
+        if (mine) {
+          db = (uint32_t)min((uint64_t)p.d, p.n - b * p.d);
+          ref = string_ref(p.peers, k0 + k, b, p.B, db);
+          if (!ref.err) {
+            PeerTable pt;
+            peer_table(p.peers, k0 + k, p.B, &pt);
+            const uint64_t from = __ldg(pt.table + b0) >> 7, to = (__ldg(pt.table + b0 + nb) + 127u) >> 7;
+            // the copy holds this string whole, whatever the table says about its neighbours
+            const bool copied = from <= to && to * 128u <= align16((__ldg(pt.table + p.B) + 7u) / 8u) * 8u &&
+                                (to - from + 1u) * 16u <= p.share && from * 128u <= ref.lo && ref.lo + 32u + ref.total <= to * 128u;
+            words = copied ? reinterpret_cast<const uint32_t*>(strings + (size_t)k * p.share) + ((ref.lo >> 5) - from * 4u)
+                           : ref.words + (ref.lo >> 5);
+          }
+        }
+        const bool reads = mine && ref.err == 0u;
+        const uint32_t first = (uint32_t)(ref.lo & 31u) + 32u, end = first + ref.total;   // bits behind the scale
+        // parts of equal length, not shorter than kLeastPart
+        const uint32_t per = max((ref.total + T - 1u) / T, kLeastPart);
+        const uint32_t lo = min(first + t * per, end), hi = t == T - 1u ? end : min(lo + per, end);
+        uint32_t start = lo;
+        Marks m;
+#pragma unroll
+        for (uint32_t q = 0; q < kMarks; ++q) { m.pos[q] = lo; m.sum[q] = 0u; }
+        if (reads) {
+          if (t == 0u) {
+            Window in;
+            in.open(words, first - 32u);
+            scales[j] = __uint_as_float(in.peek());
+          } else if (lo < end) {
+            uint32_t skipped;
+            start = walk<DENSE, WIDTH>(tab, words, lo - min(kWarmUp, lo - first), lo, end, &skipped);
+          }
+          read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, false, m);
+        } else if (j < rows && t == 0u) {
+          scales[j] = 0.f;
+        }
+        for (;;) {
+          const uint32_t before = __shfl_up_sync(0xffffffffu, m.pos[kMarks - 1u], 1, (int)T);
+          const bool again = t != 0u && before != start;
+          if (!__any_sync(0xffffffffu, again)) break;
+          if (again) {
+            start = before;
+            read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, true, m);
+          }
+        }
+        const uint32_t sum = m.sum[kMarks - 1u], stop = m.pos[kMarks - 1u];
+        uint32_t upto = sum;                              // positions passed by the lanes up to this one
+        for (uint32_t o = 1; o < T; o <<= 1) {
+          const uint32_t q = __shfl_up_sync(0xffffffffu, upto, o, (int)T);
+          if (t >= o) upto += q;
+        }
+        uint32_t err = ref.err;
+        if (reads) {
+          uint8_t* row = tsm + (size_t)j * p.row_bytes;
+          const uint32_t at = upto - sum - (DENSE ? 0u : 1u);
+          err |= emit<DENSE, WIDTH>(tab, words, start, hi, end, at, db, p.s, row);
+          // a string must end exactly where the table says and, in the dense code, hold every coordinate
+          if (t == T - 1u && (stop != end || (DENSE && upto != db))) err |= QSGD_DEV_OVERRUN;
+        }
+        if (err) atomicOr(p.status, err);
+      }
+      __syncthreads();
+
+      // ---- ascending-k sum; a thread takes 8 coordinates per pass ------------------------------------
+      const uint32_t slots_per_bucket = p.d >> 3, slots = nb * slots_per_bucket;
+      for (uint32_t s0 = 0; s0 < slots; s0 += kThreads) {
+        const uint32_t slot = s0 + tid;
+        const uint32_t g = slot / slots_per_bucket, c = (slot - g * slots_per_bucket) << 3;
+        const uint64_t b = b0 + g;
+        const bool live = slot < slots && b * p.d + c < p.n;
+        if (!__any_sync(0xffffffffu, live)) continue;
+        const uint32_t gg = live ? g : 0u, cc = live ? c : 0u;
+        const uint8_t* codes = tsm + (size_t)gg * kc * p.row_bytes + place<WIDTH>(cc);
+        const float* sc = scales + gg * kc;
+        float4* carry = reinterpret_cast<float4*>(sums + gg * p.d + cc);
+        float acc[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+        if (k0) {                                         // the peers of the passes before, added by this thread
+          const float4 u = carry[0], v = carry[1];
+          acc[0] = u.x; acc[1] = u.y; acc[2] = u.z; acc[3] = u.w;
+          acc[4] = v.x; acc[5] = v.y; acc[6] = v.z; acc[7] = v.w;
+        }
+        if (WIDTH == kWide) {
+          for (uint32_t k = 0; k < kc; ++k) {
+            const uint4 q = *reinterpret_cast<const uint4*>(codes + k * p.row_bytes);
+            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+            const float Ak = sc[k];
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+              acc[2 * h] = __fadd_rn(acc[2 * h], __fmul_rn(Ak, xi[w[h] & 0xFFFFu]));
+              acc[2 * h + 1] = __fadd_rn(acc[2 * h + 1], __fmul_rn(Ak, xi[w[h] >> 16]));
+            }
+          }
+        } else {
+          const float lut = WIDTH == kNibble ? xi[lane] : 0.f;
+#pragma unroll 2
+          for (uint32_t k = 0; k < kc; ++k) {
+            const uint2 q = *reinterpret_cast<const uint2*>(codes + k * p.row_bytes);
+            const float Ak = sc[k];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const uint32_t code = (e < 4 ? q.x : q.y) >> (8 * (e & 3));
+              acc[e] = __fadd_rn(acc[e], __fmul_rn(Ak, WIDTH == kNibble ? shfl_f(lut, code) : xi[code & 0xFFu]));
+            }
+          }
+        }
+        if (!live) continue;
+        if (k0 + kc < p.K) {
+          carry[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+          carry[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+        } else {
+          store_span8<FUSED>(out_span(p.out, p.map, b, c, p.d, p.n, 8u), acc, p.c);
+        }
+      }
+      __syncthreads();                                    // the rows are free again
+    }
+  }
+}
+
+template <bool DENSE, int WIDTH>
+int launch_width(TeamParams& p, bool fused, size_t smem, cudaStream_t stream) {
+  static KernelSite site[2];
+  auto kern = fused ? decode_elias_teams_kernel<DENSE, WIDTH, true> : decode_elias_teams_kernel<DENSE, WIDTH, false>;
+  int sms = 0, occ = 0;
+  const int st = site[fused ? 1 : 0].lookup_dynamic(kern, kThreads, smem, &sms, &occ);
+  if (st) return st;
+  const uint64_t groups = (p.B + p.buckets - 1) / p.buckets, cap = (uint64_t)sms * occ;
+  ScopedKernel sk(kKernDecodeElias, stream);
+  return (int)launch_chained(kern, (uint32_t)(groups < cap ? groups : cap), kThreads, smem, stream, p);
+}
+
+}  // namespace
+
+int launch_elias_teams(const FieldParams& f, bool dense, bool fused, cudaStream_t stream) {
+  TeamParams p;
+  p.peers = f.peers; p.K = f.K; p.n = f.n; p.d = f.d; p.s = f.s; p.B = f.B; p.out = f.out; p.c = f.c;
+  p.status = f.status; p.map = f.map; p.defer_sparse = f.defer_sparse;
+  const int width = f.s <= 15u ? kNibble : f.s <= 127u ? kByte : kWide;
+  p.row_bytes = ((p.d * (width == kWide ? 2u : 1u) + 127u) & ~127u) + kRowPad;
+  // room for strings of up to 6, 9 or 14 bits per coordinate (what max-norm scales and normal values
+  // need at s = 15, 63 and 255)
+  const uint32_t bits = width == kNibble ? 6u : width == kByte ? 9u : 14u;
+  auto share = [&](uint32_t buckets) { return (uint32_t)align16((buckets * (p.d * bits + 32ull) + 7u) / 8u) + 32u; };
+  auto bytes = [&](uint32_t buckets, uint32_t peers) {
+    return (size_t)peers * (buckets * (p.row_bytes + 4ull) + share(buckets)) + (peers < p.K ? buckets * p.d * 4ull : 0ull);
+  };
+  // all peers at once, or (long buckets and many peers) in as few passes as shared memory allows
+  uint32_t passes = 1;
+  while (bytes(1, (p.K + passes - 1) / passes) > kMostBytes) ++passes;
+  p.Kc = (p.K + passes - 1) / passes;
+  int sms = 0;
+  const int st = device_sms(&sms);
+  if (st) return st;
+  const uint64_t strings = p.B * p.K, lanes = (uint64_t)sms * kLanesPerSm;
+  // Lanes per string: as many as fill the GPU, but not more than the strings are likely to have work for
+  // (96 bits a lane at 3, 5 or 9 bits per coordinate). Then as many buckets to a CTA as occupy its threads,
+  // within 64 KB, and if that does not occupy them more lanes per string after all.
+  p.T = 32;
+  while (p.T > 1u && p.T * 96u > p.d * (width == kNibble ? 3u : width == kByte ? 5u : 9u)) p.T >>= 1;
+  while (p.T > 1u && strings * p.T > lanes) p.T >>= 1;
+  p.buckets = 1;
+  while (p.buckets * 2u * p.Kc * p.T <= kThreads && p.buckets * 2u <= p.B && bytes(p.buckets * 2u, p.Kc) <= (64u << 10)) p.buckets *= 2u;
+  while (p.T < 32u && p.buckets * p.Kc * p.T * 2u <= kThreads) p.T <<= 1;
+  p.share = share(p.buckets);
+  const size_t smem = align16(bytes(p.buckets, p.Kc));
+#define QSGD_RUN(D, W) launch_width<D, W>(p, fused, smem, stream)
+  if (dense) return width == kNibble ? QSGD_RUN(true, kNibble) : width == kByte ? QSGD_RUN(true, kByte) : QSGD_RUN(true, kWide);
+  return width == kNibble ? QSGD_RUN(false, kNibble) : width == kByte ? QSGD_RUN(false, kByte) : QSGD_RUN(false, kWide);
+#undef QSGD_RUN
+}
+
+}  // namespace qsgd

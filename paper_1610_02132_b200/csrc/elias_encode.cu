@@ -13,7 +13,8 @@
 //      with coalesced stores; only the first and last word of a CTA's range, which it may share
 //      with its neighbours, are merged with atomicOr in global memory.
 // A bucket is handled by a team of d / 64 lanes (at most a warp, at least one lane), so that the
-// sequential walk over a lane's nonzeros is long enough to amortise the team's scans.
+// sequential walk over a lane's nonzeros is long enough to amortise the team's scans. Small problems and
+// bucket sizes that are no power of two take the tile kernels below instead (use_tiles).
 #include <mutex>
 
 #include "elias_common.cuh"
@@ -38,11 +39,9 @@ struct Teams {
   uint32_t nbc;               // buckets per CTA
 };
 
-Teams make_teams(uint32_t d) {
+Teams make_teams(uint32_t d) {        // d a power of two, at least 64: lanes get whole blocks of 64
   Teams t;
-  const bool pow2 = (d & (d - 1)) == 0;
-  t.lpb = 32;
-  if (pow2) { t.lpb = d / 64; if (t.lpb < 1) t.lpb = 1; if (t.lpb > 32) t.lpb = 32; }
+  t.lpb = d / 64 > 32u ? 32u : d / 64;
   t.seg = d / t.lpb;
   t.nbc = kWarps * (32 / t.lpb);
   return t;
@@ -57,15 +56,33 @@ struct EliasWs {
   size_t bytes;
 };
 
+// Which pair of length and scatter kernels? The tile kernels (a thread has 16 coordinates) finish a small
+// problem sooner; the team kernels (a lane walks 64 or more) do less per coordinate. Whole encodes measured
+// both ways on three input families, teams against tiles (us): Code_s with s <= 15 16.7 / 16.0 at n = 2^21,
+// 19.2 / 20.4 at 3 * 2^20; s = 255 35 to 47 / 27 to 31 at 3 * 2^20, 44 / 44 at 6 * 2^20; Code'_s with d = 512
+// 29 / 28 at 2^22, 36 / 39 at 6 * 2^20, with d = 4096 (128 coordinates a lane) 56 / 49 at 2^23. Bucket sizes
+// whose lanes would not get whole 64-coordinate blocks always take the tiles (978 / 280 us at n = 2^25,
+// d = 96).
+inline bool use_tiles(uint64_t n, uint32_t d, uint32_t s, bool dense) {
+  if ((d & (d - 1u)) || d < 64u) return true;
+  const uint64_t m = dense ? (d > 1024u ? 12u : 4u) : s > 15u ? 6u : 2u;
+  return n <= m << 20;
+}
+
+constexpr uint32_t kTileCoords = 16u * kThreads;      // a tile: whole buckets, at most this many coordinates
+inline uint32_t tile_buckets(uint32_t d) { return kTileCoords / d; }
+
 EliasWs carve(uint8_t* ws, uint64_t n, uint32_t d, uint32_t s) {
   const FixedLayout L = make_fixed_layout(n, d, s);
-  const Teams tm = make_teams(d);
+  const bool teams = (d & (d - 1u)) == 0 && d >= 64u;
+  const Teams tm = teams ? make_teams(d) : Teams{1u, d, tile_buckets(d)};
   EliasWs w;
   size_t o = 0;
   w.fixed = ws + o; o += align16(L.total);
   w.len = reinterpret_cast<uint32_t*>(ws + o); o += align16(4 * L.B);
   w.lane_rec = reinterpret_cast<uint32_t*>(ws + o); o += align16(4 * L.B * tm.lpb);
-  const uint64_t ctas = (L.B + tm.nbc - 1) / tm.nbc;
+  const uint32_t run = tm.nbc < tile_buckets(d) ? tm.nbc : tile_buckets(d);    // buckets per CTA of either kind
+  const uint64_t ctas = (L.B + run - 1) / run;
   w.cta_sums = reinterpret_cast<uint64_t*>(ws + o); o += align16(8 * (ctas + 1));
   w.ctrl = reinterpret_cast<Ctrl*>(ws + o); o += align16(sizeof(Ctrl));
   w.bytes = o;
@@ -103,13 +120,6 @@ __device__ __forceinline__ uint32_t tab_code(const uint32_t* tab, uint32_t k, ui
   return ((((e & 0xFFu) << m) | k) << 1) ^ (e >> 16);
 }
 
-// Level field c of a bucket whose level fields start at word pointer lwb.
-template <int LB>
-__device__ __forceinline__ uint32_t level_at(const uint32_t* __restrict__ lwb, uint32_t c) {
-  const uint32_t bit = c * LB;
-  return (__ldg(lwb + (bit >> 5)) >> (bit & 31)) & ((1u << LB) - 1u);
-}
-
 // Bit j of the result is set iff field j of the level word is nonzero (32 / LB fields).
 template <int LB>
 __device__ __forceinline__ uint32_t nonzero_mask(uint32_t w) {
@@ -133,54 +143,6 @@ __device__ __forceinline__ uint32_t nonzero_mask(uint32_t w) {
   y = (y | (y >> 1)) & 0x01010101u;
   y = (y | (y >> 7)) & 0x00030003u;
   return (y | (y >> 14)) & 0xFu;
-}
-
-// Walks the nonzero levels of bucket-relative coordinates [c_lo, c_hi) in index order and
-// calls visit(position, level). When the range starts on a 32-coordinate boundary (every
-// power-of-two bucket size) it is processed in blocks of 64 coordinates: the nonzero fields of a
-// block are first condensed into a 64-bit mask, so the visiting loop runs once per nonzero of
-// the lane and not once per (word, most loaded lane) pair. Otherwise words are walked one by one.
-template <int LB, typename F>
-__device__ __forceinline__ void for_each_nonzero(const uint32_t* __restrict__ lwb, uint32_t c_lo,
-                                                 uint32_t c_hi, F&& visit) {
-  constexpr uint32_t kMask = (1u << LB) - 1u;
-  constexpr uint32_t kFields = 32u / LB;           // fields per word
-  if ((c_lo & 31u) == 0u) {
-    for (uint32_t c0 = c_lo; c0 < c_hi; c0 += 64u) {
-      const uint32_t* wp = lwb + ((c0 * LB) >> 5);
-      unsigned long long m = 0ull;
-#pragma unroll
-      for (uint32_t j = 0; j < 2u * LB; ++j) {
-        const uint32_t w = (c0 + j * kFields < c_hi) ? __ldg(wp + j) : 0u;
-        m |= (unsigned long long)nonzero_mask<LB>(w) << (j * kFields);
-      }
-      while (m) {
-        const uint32_t pos = c0 + (uint32_t)__ffsll((long long)m) - 1u;
-        m &= m - 1ull;
-        if (pos < c_hi) {
-          const uint32_t bit = pos * LB;
-          visit(pos, (__ldg(lwb + (bit >> 5)) >> (bit & 31u)) & kMask);
-        }
-      }
-    }
-    return;
-  }
-  uint32_t c = c_lo;
-  while (c < c_hi) {
-    const uint32_t bit = c * LB;
-    const uint32_t sh = bit & 31u;
-    uint32_t w = __ldg(lwb + (bit >> 5)) >> sh;
-    const uint32_t fields = (32u - sh) / LB;
-    const uint32_t cnt = min(fields, c_hi - c);
-    if (cnt * LB < 32u) w &= (1u << (cnt * LB)) - 1u;
-    while (w) {
-      const uint32_t fb = ((uint32_t)__ffs((int)w) - 1u) & ~(uint32_t)(LB - 1);   // first bit of the field
-      const uint32_t level = (w >> fb) & kMask;
-      visit(c + fb / LB, level);
-      w &= ~(kMask << fb);
-    }
-    c += cnt;
-  }
 }
 
 struct LaneSummary {
@@ -241,75 +203,72 @@ __device__ __forceinline__ uint32_t gap_code_bits(unsigned long long m) {
   return bits;
 }
 
-// whole_blocks: the lanes' ranges are multiples of 64 coordinates, so every level word this lane
-// reads holds only its own coordinates (or, in the last bucket, coordinates past the end of the vector).
+// The same for the 16 coordinates of a small problem's thread: gaps of at most 15.
+__device__ __forceinline__ uint32_t gap_code_bits16(uint32_t m) {
+  uint32_t prev = 0u, P = m << 1;
+  uint32_t bits = (uint32_t)__popc(m & P);
+  prev = P; P = P | (m << 2) | (P << 2);
+  bits += 3u * (uint32_t)__popc(m & P & ~prev);
+  prev = P; P = P | (m << 4) | (P << 4);
+  bits += 6u * (uint32_t)__popc(m & P & ~prev);
+  prev = P; P = P | (m << 8) | (P << 8);
+  return bits + 7u * (uint32_t)__popc(m & P & ~prev);
+}
+
+// The lanes' ranges are multiples of 64 coordinates, so every level word this lane reads holds only its
+// own coordinates (or, in the last bucket, coordinates past the end of the vector).
 template <int LB>
 __device__ __forceinline__ LaneSummary summarize_sparse(const uint32_t* tab, const uint32_t* __restrict__ lwb,
-                                                        uint32_t c_lo, uint32_t c_hi, bool whole_blocks) {
+                                                        uint32_t c_lo, uint32_t c_hi) {
+  // Blocks of 64 coordinates, no loop over the nonzeros: code lengths come from counting. Fields
+  // past the end of the vector are zero in the fixed-width layout, so a ragged c_hi needs no mask
+  // beyond not reading words that start past it.
   LaneSummary s{0u, -1, -1};
-  if (whole_blocks) {
-    // Blocks of 64 coordinates, no loop over the nonzeros: code lengths come from counting. Fields
-    // past the end of the vector are zero in the fixed-width layout, so a ragged c_hi needs no mask
-    // beyond not reading words that start past it.
-    constexpr uint32_t kFields = 32u / LB;
-    for (uint32_t c0 = c_lo; c0 < c_hi; c0 += 64u) {
-      const uint32_t* wp = lwb + ((c0 * LB) >> 5);
-      unsigned long long m = 0ull;
-      uint32_t bits = 0;
+  constexpr uint32_t kFields = 32u / LB;
+  for (uint32_t c0 = c_lo; c0 < c_hi; c0 += 64u) {
+    const uint32_t* wp = lwb + ((c0 * LB) >> 5);
+    unsigned long long m = 0ull;
+    uint32_t bits = 0;
 #pragma unroll
-      for (uint32_t j = 0; j < 2u * LB; ++j) {
-        const uint32_t w = (c0 + j * kFields < c_hi) ? __ldg(wp + j) : 0u;
-        m |= (unsigned long long)nonzero_mask<LB>(w) << (j * kFields);
-        bits += level_code_bits<LB>(w);
-      }
-      if (m) {
-        const int32_t lowest = (int32_t)c0 + __ffsll((long long)m) - 1;
-        if (s.first < 0) s.first = lowest;
-        else bits += tab_len(tab, (uint32_t)(lowest - s.last));          // gap across two blocks of this lane
-        s.last = (int32_t)c0 + 63 - __clzll((long long)m);
-        s.bits += bits + gap_code_bits(m);
-      }
+    for (uint32_t j = 0; j < 2u * LB; ++j) {
+      const uint32_t w = (c0 + j * kFields < c_hi) ? __ldg(wp + j) : 0u;
+      m |= (unsigned long long)nonzero_mask<LB>(w) << (j * kFields);
+      bits += level_code_bits<LB>(w);
     }
-    return s;
+    if (m) {
+      const int32_t lowest = (int32_t)c0 + __ffsll((long long)m) - 1;
+      if (s.first < 0) s.first = lowest;
+      else bits += tab_len(tab, (uint32_t)(lowest - s.last));          // gap across two blocks of this lane
+      s.last = (int32_t)c0 + 63 - __clzll((long long)m);
+      s.bits += bits + gap_code_bits(m);
+    }
   }
-  for_each_nonzero<LB>(lwb, c_lo, c_hi, [&](uint32_t pos, uint32_t level) {
-    const bool is_first = s.first < 0;
-    const uint32_t gap_bits = tab_len(tab, is_first ? 1u : pos - (uint32_t)s.last);
-    s.first = is_first ? (int32_t)pos : s.first;
-    s.bits += (is_first ? 0u : gap_bits) + 1u + tab_len(tab, level);
-    s.last = (int32_t)pos;
-  });
   return s;
 }
 
-// whole_blocks as above: whole level words are loaded once and their fields taken from the register
-// (fields past the end of the vector are zero in the fixed-width layout but are not coordinates: the
-// count stops at c_hi).
+// Whole level words are loaded once and their fields taken from the register (fields past the end of the
+// vector are zero in the fixed-width layout but are not coordinates: the count stops at c_hi).
 template <int LB>
 __device__ __forceinline__ uint32_t summarize_dense(const uint32_t* tab, const uint32_t* __restrict__ lwb,
-                                                    uint32_t c_lo, uint32_t c_hi, bool whole_blocks) {
+                                                    uint32_t c_lo, uint32_t c_hi) {
   uint32_t bits = 0;
-  if (whole_blocks) {
-    constexpr uint32_t kFields = 32u / LB, kMask = (1u << LB) - 1u;
-    for (uint32_t c0 = c_lo; c0 < c_hi; c0 += 64u) {
-      const uint32_t* wp = lwb + ((c0 * LB) >> 5);
+  constexpr uint32_t kFields = 32u / LB, kMask = (1u << LB) - 1u;
+  for (uint32_t c0 = c_lo; c0 < c_hi; c0 += 64u) {
+    const uint32_t* wp = lwb + ((c0 * LB) >> 5);
 #pragma unroll
-      for (uint32_t j = 0; j < 2u * LB; ++j) {
-        const uint32_t cw = c0 + j * kFields;                 // first coordinate of this word
-        if (cw >= c_hi) break;
-        const uint32_t w = __ldg(wp + j);
-        const uint32_t cnt = min(kFields, c_hi - cw);
-        if (cnt == kFields) {
+    for (uint32_t j = 0; j < 2u * LB; ++j) {
+      const uint32_t cw = c0 + j * kFields;                 // first coordinate of this word
+      if (cw >= c_hi) break;
+      const uint32_t w = __ldg(wp + j);
+      const uint32_t cnt = min(kFields, c_hi - cw);
+      if (cnt == kFields) {
 #pragma unroll
-          for (uint32_t f = 0; f < kFields; ++f) bits += 1u + tab_len(tab, ((w >> (f * LB)) & kMask) + 1u);
-        } else {
-          for (uint32_t f = 0; f < cnt; ++f) bits += 1u + tab_len(tab, ((w >> (f * LB)) & kMask) + 1u);
-        }
+        for (uint32_t f = 0; f < kFields; ++f) bits += 1u + tab_len(tab, ((w >> (f * LB)) & kMask) + 1u);
+      } else {
+        for (uint32_t f = 0; f < cnt; ++f) bits += 1u + tab_len(tab, ((w >> (f * LB)) & kMask) + 1u);
       }
     }
-    return bits;
   }
-  for (uint32_t c = c_lo; c < c_hi; ++c) bits += 1u + tab_len(tab, level_at<LB>(lwb, c) + 1u);
   return bits;
 }
 
@@ -348,14 +307,14 @@ struct BucketParams {
 template <int LB, bool DENSE>
 __device__ __forceinline__ uint32_t lane_bits(const uint32_t* tab, const uint32_t* __restrict__ lwb, uint32_t lpb,
                                               uint32_t c_lo, uint32_t c_hi, uint32_t tl, bool live,
-                                              bool whole_blocks, int32_t* prev_out) {
+                                              int32_t* prev_out) {
   uint32_t bits = 0;
   int32_t prev = -1;
   if (DENSE) {
-    if (live) bits = summarize_dense<LB>(tab, lwb, c_lo, c_hi, whole_blocks);
+    if (live) bits = summarize_dense<LB>(tab, lwb, c_lo, c_hi);
   } else {
     LaneSummary s{0u, -1, -1};
-    if (live) s = summarize_sparse<LB>(tab, lwb, c_lo, c_hi, whole_blocks);
+    if (live) s = summarize_sparse<LB>(tab, lwb, c_lo, c_hi);
     prev = prev_nonzero_before_lane(s.last, tl, lpb);
     bits = s.bits + (s.first >= 0 ? tab_len(tab, (uint32_t)(s.first - prev)) : 0u);
   }
@@ -461,7 +420,7 @@ __global__ void __launch_bounds__(kThreads) elias_length_kernel(const BucketPara
   const uint32_t c_lo = min(tl * p.seg, db), c_hi = min(c_lo + p.seg, db);
   const uint32_t* lwb = p.level + ((base * LB) >> 5);            // the bucket's first level word
   int32_t prev;
-  const uint32_t bits = lane_bits<LB, DENSE>(tab, lwb, p.lpb, c_lo, c_hi, tl, live, (p.seg & 63u) == 0u, &prev);
+  const uint32_t bits = lane_bits<LB, DENSE>(tab, lwb, p.lpb, c_lo, c_hi, tl, live, &prev);
   if (live) lane_rec[b * p.lpb + tl] = bits | ((uint32_t)(prev + 1) << 16);   // reused by the scatter
   const uint32_t L = team_sum(bits, p.lpb);
   if (live && tl == 0) len[b] = L;
@@ -483,6 +442,22 @@ __global__ void __launch_bounds__(kThreads) elias_length_kernel(const BucketPara
   if (is_last) {
     __threadfence();
     scan_cta_sums(cta_sums, sa.ctas, p.B, sa.out_capacity, sa.ctrl, sa.out_bits, sa.status_dev, sa.out);
+  }
+}
+
+// Whole code words (code | length << 16) of the integers met most: every level, and gaps below 64.
+template <int LB>
+struct CodeWords {
+  uint32_t level[1u << LB];
+  uint32_t gap[64];
+};
+template <int LB>
+__device__ __forceinline__ void fill_code_words(CodeWords<LB>& words) {
+  for (uint32_t k = threadIdx.x; k < (1u << LB) + 64u; k += kThreads) {
+    const uint32_t v = k < (1u << LB) ? k : k - (1u << LB);
+    uint32_t ln = 0;
+    const uint32_t code = v ? elias_code(v, &ln) : 0u;
+    (k < (1u << LB) ? words.level[v] : words.gap[v]) = code | (ln << 16);
   }
 }
 
@@ -519,18 +494,9 @@ __global__ void __launch_bounds__(kThreads) elias_scatter_kernel(const BucketPar
   extern __shared__ uint32_t stage[];
   __shared__ uint32_t warp_sum[kWarps];
   __shared__ uint32_t tab[17];
-  // whole code words (code | length << 16) of the integers met most: every level, and gaps below 64
-  __shared__ uint32_t level_code[1u << LB];
-  __shared__ uint32_t gap_code[64];
+  __shared__ CodeWords<LB> words;
   fill_code_table(tab);
-  if (!DENSE) {
-    for (uint32_t k = threadIdx.x; k < (1u << LB) + 64u; k += kThreads) {
-      const uint32_t v = k < (1u << LB) ? k : k - (1u << LB);
-      uint32_t ln = 0;
-      const uint32_t code = v ? elias_code(v, &ln) : 0u;
-      (k < (1u << LB) ? level_code[v] : gap_code[v]) = code | (ln << 16);
-    }
-  }
+  if (!DENSE) fill_code_words<LB>(words);
   chain_wait();                                    // ctrl, lengths and sums come from the kernel ahead
   if (!ctrl->ok) return;
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -587,7 +553,7 @@ __global__ void __launch_bounds__(kThreads) elias_scatter_kernel(const BucketPar
     StageWriter bw;
     bw.begin(stage, lead + bucket_off + (linc - bits));
     if (tl == 0) bw.put(__float_as_uint(__ldg(p.A + b)), 32);
-    if (DENSE && (p.seg & 63u) == 0u) {
+    if (DENSE) {
       // ranges of whole 64-coordinate blocks: sign and level words are loaded once per block and word
       constexpr uint32_t kFields = 32u / LB, kMask = (1u << LB) - 1u;
       for (uint32_t c0 = c_lo; c0 < c_hi; c0 += 64u) {
@@ -607,15 +573,8 @@ __global__ void __launch_bounds__(kThreads) elias_scatter_kernel(const BucketPar
           }
         }
       }
-    } else if (DENSE) {
-      for (uint32_t c = c_lo; c < c_hi; ++c) {
-        const uint32_t sg = (__ldg(swb + (c >> 5)) >> (c & 31)) & 1u;
-        uint32_t ln;
-        const uint32_t code = tab_code(tab, level_at<LB>(lwb, c) + 1u, &ln);
-        bw.put((sg << ln) | code, ln + 1);
-      }
-    } else if ((p.seg & 63u) == 0u) {
-      // Ranges of whole 64-coordinate blocks (every power-of-two d >= 64): the block's nonzero mask
+    } else {
+      // ranges of whole 64-coordinate blocks: the block's nonzero mask
       // and sign bits sit in registers, code words come whole from the two tables.
       constexpr uint32_t kFields = 32u / LB, kMask = (1u << LB) - 1u;
       for (uint32_t c0 = c_lo; c0 < c_hi; c0 += 64u) {
@@ -636,13 +595,13 @@ __global__ void __launch_bounds__(kThreads) elias_scatter_kernel(const BucketPar
           const uint32_t gap = pos - (uint32_t)prev;
           uint32_t gcode, gl;
           if (gap < 64u) {
-            const uint32_t e = gap_code[gap];
+            const uint32_t e = words.gap[gap];
             gcode = e & 0xFFFFu;
             gl = e >> 16;
           } else {
             gcode = tab_code(tab, gap, &gl);
           }
-          const uint32_t e = level_code[level];
+          const uint32_t e = words.level[level];
           const uint32_t ll = e >> 16;
           const uint32_t lcode = (e & 0xFFFFu) | ((uint32_t)((signs >> off) & 1ull) << ll);
           if (gl + ll + 1u <= 32u) {                     // gap, sign and level in one piece (the rule)
@@ -654,21 +613,6 @@ __global__ void __launch_bounds__(kThreads) elias_scatter_kernel(const BucketPar
           prev = (int32_t)pos;
         }
       }
-    } else {
-      for_each_nonzero<LB>(lwb, c_lo, c_hi, [&](uint32_t pos, uint32_t level) {
-        uint32_t gl, ll;
-        const uint32_t gcode = tab_code(tab, pos - (uint32_t)prev, &gl);
-        const uint32_t sg = (__ldg(swb + (pos >> 5)) >> (pos & 31)) & 1u;
-        uint32_t lcode = tab_code(tab, level, &ll);
-        lcode |= sg << ll;
-        if (gl + ll + 1u <= 32u) {                     // gap, sign and level in one piece (the rule)
-          bw.put((gcode << (ll + 1u)) | lcode, gl + ll + 1u);
-        } else {
-          bw.put(gcode, gl);
-          bw.put(lcode, ll + 1u);
-        }
-        prev = (int32_t)pos;
-      });
     }
     bw.finish();
   }
@@ -684,6 +628,253 @@ __global__ void __launch_bounds__(kThreads) elias_scatter_kernel(const BucketPar
   }
 }
 
+// ---- 2. and 4. for small problems --------------------------------------------------------------------
+// The kernels above give a lane 64 coordinates or more, which is what makes them cheap per coordinate; on a
+// problem that does not fill the GPU their time is that serial walk (13 to 22 us of scatter whatever n up
+// to 10^6). Here a thread takes 16 coordinates, a CTA a tile of whole buckets of at most 4096
+// coordinates, and what a lane needs of its predecessors (the last nonzero of its bucket, the bits in
+// front of it) comes from scans over the CTA. Three times the instructions per coordinate of a sparse
+// bucket, a quarter of the chain.
+
+// What one thread holds of its 16 coordinates.
+template <int LB>
+struct Piece {
+  static constexpr int kWords = LB == 8 ? 4 : LB == 4 ? 2 : 1;
+  uint32_t level[kWords];     // 16 fields of LB bits
+  uint32_t sign;              // 16 bits
+  uint32_t c0;                // position of the first in its bucket
+  uint32_t bucket;            // bucket in the tile
+  uint32_t count;             // coordinates that exist: 0 .. 16
+};
+
+template <int LB>
+__device__ __forceinline__ uint32_t piece_level(const Piece<LB>& q, uint32_t j) {   // j is a constant after unrolling
+  return (q.level[(j * LB) >> 5] >> ((j * LB) & 31u)) & ((1u << LB) - 1u);
+}
+
+template <int LB>
+__device__ __forceinline__ Piece<LB> load_piece(const BucketParams& p) {
+  Piece<LB> q;
+  const uint32_t local = threadIdx.x * 16u;               // first coordinate in the tile
+  const uint32_t tile = p.nbc * p.d;
+  const uint64_t i0 = (uint64_t)blockIdx.x * tile + local;
+  q.bucket = local / p.d;
+  q.c0 = local - q.bucket * p.d;
+  q.count = local < tile && i0 < p.n ? (uint32_t)min((uint64_t)16u, p.n - i0) : 0u;
+  q.sign = 0u;
+#pragma unroll
+  for (int j = 0; j < Piece<LB>::kWords; ++j) q.level[j] = 0u;
+  if (q.count) {                                          // fields past the end of the vector are zero
+    const uint64_t slot = i0 >> 4;
+    q.sign = __ldg(reinterpret_cast<const uint16_t*>(p.sign) + slot);
+    if (LB == 8) {
+      const uint4 w = __ldg(reinterpret_cast<const uint4*>(p.level) + slot);
+      q.level[0] = w.x; q.level[1] = w.y; q.level[2] = w.z; q.level[3] = w.w;
+    } else if (LB == 4) {
+      const uint2 w = __ldg(reinterpret_cast<const uint2*>(p.level) + slot);
+      q.level[0] = w.x; q.level[1] = w.y;
+    } else if (LB == 2) {
+      q.level[0] = __ldg(p.level + slot);
+    } else {
+      q.level[0] = __ldg(reinterpret_cast<const uint16_t*>(p.level) + slot);
+    }
+  }
+  return q;
+}
+
+// Bit j: level j is nonzero.
+template <int LB>
+__device__ __forceinline__ uint32_t piece_mask(const Piece<LB>& q) {
+  uint32_t m = 0;
+#pragma unroll
+  for (int j = 0; j < Piece<LB>::kWords; ++j) m |= nonzero_mask<LB>(q.level[j]) << (j * (32 / LB));
+  return m;
+}
+
+// Scans over the CTA, one barrier each: the largest key, or the sum, in front of this thread (0 for the
+// first).
+__device__ __forceinline__ uint32_t cta_max_before(uint32_t key, uint32_t* warp_slots) {
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, key, o);
+    if (lane >= (uint32_t)o) key = max(key, t);
+  }
+  if (lane == 31) warp_slots[warp] = key;
+  __syncthreads();
+  uint32_t before = __shfl_up_sync(0xffffffffu, key, 1);
+  if (lane == 0) before = 0u;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w)
+    if ((uint32_t)w < warp) before = max(before, warp_slots[w]);
+  return before;
+}
+__device__ __forceinline__ uint32_t cta_sum_before(uint32_t v, uint32_t* warp_slots, uint32_t* total) {
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= (uint32_t)o) inc += t;
+  }
+  if (lane == 31) warp_slots[warp] = inc;
+  __syncthreads();
+  uint32_t before = inc - v, all = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    if ((uint32_t)w < warp) before += warp_slots[w];
+    all += warp_slots[w];
+  }
+  *total = all;
+  return before;
+}
+
+// Last nonzero of the piece's bucket in front of the piece (-1: none). One CTA barrier.
+template <int LB>
+__device__ __forceinline__ int32_t nonzero_before(const Piece<LB>& q, uint32_t mask, uint32_t* warp_slots) {
+  // bucket number above position + 1: the largest key in front is the nearest nonzero, if of this bucket
+  const uint32_t at = mask ? q.c0 + 32u - (uint32_t)__clz((int)mask) : 0u;
+  const uint32_t before = cta_max_before((q.bucket + 1u) << 13 | at, warp_slots);
+  return before >> 13 == q.bucket + 1u ? (int32_t)(before & 8191u) - 1 : -1;
+}
+
+// Bits of the piece's part of its bucket's string (with the scale's 32 where the bucket starts).
+template <int LB, bool DENSE>
+__device__ __forceinline__ uint32_t piece_bits(const uint32_t* tab, const Piece<LB>& q, uint32_t mask, int32_t prev) {
+  uint32_t bits = q.count && q.c0 == 0u ? 32u : 0u;
+  if (DENSE) {
+#pragma unroll
+    for (uint32_t j = 0; j < 16; ++j)
+      if (j < q.count) bits += 1u + tab_len(tab, piece_level<LB>(q, j) + 1u);
+    return bits;
+  }
+  if (mask) {
+#pragma unroll
+    for (int j = 0; j < Piece<LB>::kWords; ++j) bits += level_code_bits<LB>(q.level[j]);
+    bits += gap_code_bits16(mask);
+    bits += tab_len(tab, q.c0 + (uint32_t)__ffs((int)mask) - 1u - (uint32_t)prev);
+  }
+  return bits;
+}
+
+template <int LB, bool DENSE>
+__global__ void __launch_bounds__(kThreads) elias_tile_length_kernel(const BucketParams p, uint64_t* cta_sums, const ScanArgs sa) {
+  __shared__ uint32_t slots[2][kWarps];
+  __shared__ uint32_t is_last;
+  __shared__ uint32_t tab[17];
+  fill_code_table(tab);
+  __syncthreads();
+  chain_wait();                                    // the fields come from the kernel ahead
+  const Piece<LB> q = load_piece<LB>(p);
+  const uint32_t mask = DENSE ? 0u : piece_mask<LB>(q);
+  const int32_t prev = DENSE ? -1 : nonzero_before<LB>(q, mask, slots[0]);
+  uint32_t total;
+  cta_sum_before(piece_bits<LB, DENSE>(tab, q, mask, prev), slots[1], &total);
+  if (threadIdx.x == 0) {
+    cta_sums[blockIdx.x] = total;
+    __threadfence();
+    is_last = atomicAdd(&sa.ctrl->arrived, 1u) == gridDim.x - 1u ? 1u : 0u;
+  }
+  __syncthreads();
+  if (is_last) {
+    __threadfence();
+    scan_cta_sums(cta_sums, sa.ctas, p.B, sa.out_capacity, sa.ctrl, sa.out_bits, sa.status_dev, sa.out);
+  }
+}
+
+// Assembles the piece's codes at bit `bit` of the CTA's staging words.
+template <int LB, bool DENSE>
+__device__ __forceinline__ void emit_piece(const uint32_t* tab, const CodeWords<LB>& words, uint32_t* stage, uint32_t bit,
+                                           const Piece<LB>& q, uint32_t mask, int32_t prev, float A) {
+  StageWriter bw;
+  bw.begin(stage, bit);
+  if (q.c0 == 0u) bw.put(__float_as_uint(A), 32);
+  if (DENSE) {
+#pragma unroll
+    for (uint32_t j = 0; j < 16; ++j) {
+      if (j >= q.count) break;
+      uint32_t ln;
+      const uint32_t code = tab_code(tab, piece_level<LB>(q, j) + 1u, &ln);
+      bw.put((((q.sign >> j) & 1u) << ln) | code, ln + 1u);
+    }
+  } else {
+while (mask) {                                 // once per nonzero of the busiest lane
+      const uint32_t j = (uint32_t)__ffs((int)mask) - 1u;
+      mask &= mask - 1u;
+      const uint32_t pos = q.c0 + j, gap = pos - (uint32_t)prev;
+      uint32_t level, gcode, gl;
+      if (LB == 8) {
+        const uint32_t lo = j & 4u ? q.level[1 % Piece<LB>::kWords] : q.level[0];
+        const uint32_t hi = j & 4u ? q.level[3 % Piece<LB>::kWords] : q.level[2 % Piece<LB>::kWords];
+        level = ((j & 8u ? hi : lo) >> (8u * (j & 3u))) & 0xFFu;
+      } else if (LB == 4) {
+        level = (q.level[j >> 3 ? 1 % Piece<LB>::kWords : 0] >> (4u * (j & 7u))) & 15u;
+      } else {
+        level = (q.level[0] >> (LB * j)) & ((1u << LB) - 1u);
+      }
+      if (gap < 64u) {
+        const uint32_t e = words.gap[gap];
+        gcode = e & 0xFFFFu;
+        gl = e >> 16;
+      } else {
+        gcode = tab_code(tab, gap, &gl);
+      }
+      const uint32_t e = words.level[level], ll = e >> 16;
+      const uint32_t lcode = (e & 0xFFFFu) | (((q.sign >> j) & 1u) << ll);
+      if (gl + ll + 1u <= 32u) {                   // gap, sign and level in one piece (the rule)
+        bw.put((gcode << (ll + 1u)) | lcode, gl + ll + 1u);
+      } else {
+        bw.put(gcode, gl);
+        bw.put(lcode, ll + 1u);
+      }
+      prev = (int32_t)pos;
+    }
+  }
+  bw.finish();
+}
+
+template <int LB, bool DENSE>
+__global__ void __launch_bounds__(kThreads) elias_tile_scatter_kernel(const BucketParams p, const uint64_t* __restrict__ cta_start,
+                                                                     const Ctrl* __restrict__ ctrl, uint8_t* __restrict__ out) {
+  extern __shared__ uint32_t stage[];
+  __shared__ uint32_t slots[2][kWarps];
+  __shared__ uint32_t tab[17];
+  __shared__ CodeWords<LB> words;
+  fill_code_table(tab);
+  if (!DENSE) fill_code_words<LB>(words);
+  chain_wait();                                    // ctrl and sums come from the kernel ahead
+  if (!ctrl->ok) return;
+  const uint64_t start = __ldg(cta_start + blockIdx.x), stop = __ldg(cta_start + blockIdx.x + 1);
+  const Piece<LB> q = load_piece<LB>(p);
+  const uint64_t b = (uint64_t)blockIdx.x * p.nbc + q.bucket;
+  const bool opens = q.count && q.c0 == 0u;        // this piece opens its bucket's string
+  const float A = opens ? __ldg(p.A + b) : 0.f;
+  const uint32_t lead = (uint32_t)(start & 31);    // bits of the first word owned by the previous CTA
+  const uint32_t span = (uint32_t)(stop - start);
+  const uint32_t nwords = (lead + span + 31) >> 5;
+  for (uint32_t j = threadIdx.x; j < nwords; j += kThreads) stage[j] = 0u;
+  __syncthreads();                                 // staging zeroed, table there
+  const uint32_t mask = DENSE ? 0u : piece_mask<LB>(q);
+  const int32_t prev = DENSE ? -1 : nonzero_before<LB>(q, mask, slots[0]);
+  uint32_t total;
+  const uint32_t bits = piece_bits<LB, DENSE>(tab, q, mask, prev);
+  const uint32_t before = cta_sum_before(bits, slots[1], &total);
+  if (opens) {
+    uint64_t* table = reinterpret_cast<uint64_t*>(out + ctrl->payload_bytes);
+    table[b] = start + before;
+    if (b == p.B - 1) table[p.B] = stop;           // the last bucket ends its CTA's run
+  }
+  if (bits) emit_piece<LB, DENSE>(tab, words, stage, lead + before, q, mask, prev, A);
+  __syncthreads();
+  uint32_t* gw = reinterpret_cast<uint32_t*>(out) + (start >> 5);
+  const bool last_shared = ((lead + span) & 31) != 0;
+  for (uint32_t j = threadIdx.x; j < nwords; j += kThreads) {
+    const uint32_t v = stage[j];
+    if ((j == 0 && lead != 0) || (j == nwords - 1 && last_shared)) atomicOr(gw + j, v);
+    else gw[j] = v;
+  }
+}
+
 uint32_t host_elias_len(uint32_t k) {
   uint32_t len = 1;
   while (k > 1) {
@@ -695,9 +886,33 @@ uint32_t host_elias_len(uint32_t k) {
   return len;
 }
 
+// Staging: the longest legal strings of a CTA's buckets, plus the shared lead-in word.
+template <bool DENSE>
+size_t stage_bytes(uint32_t buckets, uint32_t d, uint32_t s) {
+  const uint32_t per = DENSE ? 1 + host_elias_len(s + 1) : 2 + host_elias_len(s);
+  const size_t run_bits = (size_t)buckets * (32 + (size_t)d * per);
+  return ((run_bits + 31) / 32 + 4) * 4;
+}
+
 template <int LB, bool DENSE>
 int run_pipeline(BucketParams& bp, const EliasWs& w, uint32_t s, uint8_t* out, size_t out_capacity,
                  uint64_t* out_bits, uint32_t* status_dev, cudaStream_t stream) {
+  if (use_tiles(bp.n, bp.d, s, DENSE)) {
+    bp.lpb = 0; bp.seg = 16; bp.nbc = tile_buckets(bp.d);
+    const uint64_t ctas = (bp.B + bp.nbc - 1) / bp.nbc;
+    ScanArgs sa;
+    sa.ctas = ctas; sa.out_capacity = out_capacity; sa.ctrl = w.ctrl; sa.out_bits = out_bits;
+    sa.status_dev = status_dev; sa.out = out;
+    {
+      ScopedKernel sk(kKernEliasLength, stream);
+      const cudaError_t e = launch_chained(elias_tile_length_kernel<LB, DENSE>, (uint32_t)ctas, kThreads, 0, stream, bp,
+                                           w.cta_sums, sa);
+      if (e != cudaSuccess) return (int)e;
+    }
+    ScopedKernel sk(kKernEliasScatter, stream);
+    return (int)launch_chained(elias_tile_scatter_kernel<LB, DENSE>, (uint32_t)ctas, kThreads, stage_bytes<DENSE>(bp.nbc, bp.d, s),
+                               stream, bp, w.cta_sums, w.ctrl, out);
+  }
   const Teams tm = make_teams(bp.d);
   bp.lpb = tm.lpb; bp.seg = tm.seg; bp.nbc = tm.nbc;
   const uint64_t ctas = (bp.B + tm.nbc - 1) / tm.nbc;
@@ -711,10 +926,7 @@ int run_pipeline(BucketParams& bp, const EliasWs& w, uint32_t s, uint8_t* out, s
     if (e != cudaSuccess) return (int)e;
   }
   {
-    // staging: the longest legal strings of a CTA's buckets, plus the shared lead-in word
-    const uint32_t per = DENSE ? 1 + host_elias_len(s + 1) : 2 + host_elias_len(s);
-    const size_t run_bits = (size_t)tm.nbc * (32 + (size_t)bp.d * per);
-    const size_t smem = ((run_bits + 31) / 32 + 4) * 4;
+    const size_t smem = stage_bytes<DENSE>(tm.nbc, bp.d, s);
     auto kern = elias_scatter_kernel<LB, DENSE>;
     if (smem > 48 * 1024) {
       cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -7,6 +7,7 @@
 #include <utility>
 #include <stdint.h>
 
+#include <map>
 #include <mutex>
 
 #include "../../include/qsgd.h"
@@ -159,6 +160,10 @@ enum KernelId {
   kKernEliasScatter, kKernDecodeElias, kKernDecodeEliasSparse, kKernRawGather, kKernRawDecode, kKernCount
 };
 
+// SM count of the current device, and the most shared memory a CTA can have (looked up once per device).
+int device_sms(int* sms_out);
+int device_shared_memory(int* bytes_out);
+
 // Launch facts of one kernel that belong to a device, not to the process: the opt-in to more than
 // 48 KB of dynamic shared memory, the SM count and the resident CTAs per SM. Looked up once per
 // device, with that device current, under a lock; one instance per kernel (a function-local static).
@@ -166,9 +171,11 @@ constexpr int kMaxDevices = 64;
 
 struct KernelSite {
   std::mutex mu;
+  std::map<uint64_t, int> occ_by_smem[kMaxDevices];   // lookup_dynamic: threads << 32 | bytes -> resident CTAs
   bool ready[kMaxDevices] = {};
   int sms[kMaxDevices] = {};
   int occ[kMaxDevices] = {};
+  int opted[kMaxDevices] = {};   // dynamic shared memory the kernel may use so far
 
   template <class Kernel>
   int lookup(Kernel kern, int threads, size_t smem, int* sms_out, int* occ_out) {
@@ -192,6 +199,38 @@ struct KernelSite {
     }
     *sms_out = sms[dev];
     *occ_out = occ[dev];
+    return 0;
+  }
+
+  // The same for a kernel whose shared memory depends on the problem: the opt-in is raised as needed and
+  // the residency of every size met so far is kept (a few dozen at most: sizes follow K and d).
+  template <class Kernel>
+  int lookup_dynamic(Kernel kern, int threads, size_t smem, int* sms_out, int* occ_out) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return (int)e;
+    if (dev < 0 || dev >= kMaxDevices) return (int)cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lk(mu);
+    const uint64_t key = (uint64_t)threads << 32 | smem;
+    auto it = occ_by_smem[dev].find(key);
+    if (it == occ_by_smem[dev].end()) {
+      if (!sms[dev]) {
+        e = cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return (int)e;
+      }
+      if ((int)smem > opted[dev]) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return (int)e;
+        opted[dev] = (int)smem;
+      }
+      int o = 0;
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, threads, smem);
+      if (e != cudaSuccess) return (int)e;
+      if (occ_by_smem[dev].size() > 512) occ_by_smem[dev].clear();
+      it = occ_by_smem[dev].emplace(key, o > 0 ? o : 1).first;
+    }
+    *sms_out = sms[dev];
+    *occ_out = it->second;
     return 0;
   }
 };

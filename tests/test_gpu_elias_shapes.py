@@ -1,0 +1,87 @@
+"""Elias Encode and Decode at the edges of their dispatch rules: problems read by teams of lanes (parts of a
+string shorter and longer than a lane's least part, peers in several passes, codes on which a reader that
+starts out of step stays out of step) and encoded in tiles (tiles of whole buckets, sizes around a tile, both
+sides of the line to the team kernels). Bit for bit against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_1610_02132_b200 import inputs as I
+from parity_util import decode_parity, encode_parity
+
+pytestmark = pytest.mark.gpu
+
+L2, MAX = O.NORM_L2, O.NORM_MAX
+ELIAS, DENSE = O.CODE_ELIAS, O.CODE_ELIAS_DENSE
+
+
+def run(n, d, s, norm, code, K, make=None):
+    make = make or (lambda w: I.gaussian(n, 1.0, seed=50 + w))
+    msgs, infos = [], []
+    for w in range(K):
+        m, info = encode_parity(make(w), d, s, norm, code, 7, 3, w)
+        msgs.append(m)
+        infos.append(info)
+    x0 = I.gaussian(n, 1.0, seed=9)
+    decode_parity(msgs, infos, n, d, s, code, eta=0.05, x0=x0)
+    decode_parity(msgs, infos, n, d, s, code, eta=-0.05, x0=x0, tables_first=True)
+
+
+@pytest.mark.parametrize("n,d,s,norm,code,K", [
+    (32, 32, 1, L2, ELIAS, 1), (31, 32, 15, MAX, DENSE, 2),              # one string, shorter than a part
+    (4096, 4096, 64, L2, DENSE, 8), (4064, 4064, 63, L2, DENSE, 3),      # 32 lanes a string
+    (3 * 4096 + 5, 4096, 15, MAX, ELIAS, 5), (5 * 1024 + 1, 1024, 127, MAX, ELIAS, 17),
+    (2 * 4096 + 77, 4096, 255, MAX, ELIAS, 17), (4096 + 40, 4096, 255, MAX, DENSE, 33),   # several passes over the peers
+    (2 * 4096, 4096, 15, MAX, ELIAS, 64), (3000, 992, 128, L2, ELIAS, 40),
+    (70 * 96 + 11, 96, 255, L2, ELIAS, 5), (1000, 160, 31, L2, DENSE, 4),
+])
+def test_teams(n, d, s, norm, code, K):
+    run(n, d, s, norm, code, K)
+
+
+@pytest.mark.parametrize("code,s,value", [(DENSE, 1, 0.0), (DENSE, 1, 1.0), (ELIAS, 1, 1.0), (ELIAS, 255, 1.0)])
+def test_teams_out_of_step(code, s, value):
+    """Strings of one repeated symbol (all levels 0, or every level s at gap 1): a lane that starts inside a
+    symbol never falls into step and every part has to be read again from its predecessor's end."""
+    n, d = 2 * 4096 + 100, 4096
+
+    def make(w):
+        g = np.full(n, value, np.float32)
+        g[::d] = 1.0 + w
+        return g
+    run(n, d, s, MAX, code, 3, make)
+
+
+@pytest.mark.parametrize("n,d,s,K", [(40 * 512 * 128, 512, 15, 8), (40 * 512 * 128 + 512, 512, 15, 8),
+                                     (48 * 1024 * 1024 + 1, 1024, 3, 1), (2 ** 20, 4096, 1, 8), (2 ** 20 + 4096, 4096, 1, 8)])
+def test_lines_between_decoders(n, d, s, K):
+    """Both sides of the lines between a lane and a team per string and between one and two launches, against
+    the sum of the messages decoded one by one (K = 1 goes through another decoder or another split)."""
+    import paper_1610_02132_b200 as Q
+    msgs, infos = [], []
+    for w in range(K):
+        g = I.sparse_laplace_device(n, seed=w) if s == 1 else I.gaussian_device(n, 1.0, seed=w)
+        out, bits, st = Q.encode_alloc(g, d, s, L2, ELIAS, 7, 0, w)
+        msgs.append(out)
+        infos.append(bits)
+    status = Q.new_status()
+    acc = torch.empty(n, device="cuda")
+    Q.qsgd_decode_accumulate_packed(msgs, infos, n, d, s, ELIAS, acc, status)
+    fixed, ref = [], torch.empty(n, device="cuda")
+    for w in range(K):
+        g = I.sparse_laplace_device(n, seed=w) if s == 1 else I.gaussian_device(n, 1.0, seed=w)
+        fixed.append(Q.encode_alloc(g, d, s, L2, O.CODE_FIXED, 7, 0, w)[0])
+    Q.qsgd_decode_accumulate_packed(fixed, None, n, d, s, O.CODE_FIXED, ref, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert torch.equal(acc.view(torch.int32), ref.view(torch.int32))
+
+
+@pytest.mark.parametrize("n,d,s,code", [
+    (1, 32, 15, ELIAS), (4095, 32, 3, ELIAS), (4096, 64, 1, ELIAS), (4097, 512, 15, ELIAS), (42 * 96 + 1, 96, 255, ELIAS),
+    (2 * 4032, 2016, 15, DENSE), (2 ** 21, 512, 15, ELIAS), (2 ** 21 + 1, 512, 15, ELIAS),
+    (2 ** 21 + 37, 480, 7, ELIAS), (2 ** 22 + 5, 4096, 64, DENSE), (2 ** 22 + 5, 128, 255, ELIAS),
+])
+def test_tiles(n, d, s, code):
+    encode_parity(I.gaussian_mixture(n, seed=3), d, s, MAX, code, 7, 1, 2)
