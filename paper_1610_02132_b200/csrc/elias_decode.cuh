@@ -364,6 +364,7 @@ __device__ __forceinline__ uint32_t advance(LaneParse& st, uint32_t rend, uint32
 
 // Launchers of the decoders; 0 or a cudaError_t. `launched`: whether the sparse-regime kernel takes the shape.
 int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream);     // Code_s, at most 32 peers
+int launch_elias_ring(const FieldParams& p, bool fused, cudaStream_t stream);                  // ... and s <= 15
 int launch_elias_teams(const FieldParams& p, bool dense, bool fused, cudaStream_t stream);
 int launch_elias_sparse(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d, uint32_t s, float* out, bool fused,
                         float c, uint32_t* status, bool check_regime, const BucketMap& map, cudaStream_t stream,
