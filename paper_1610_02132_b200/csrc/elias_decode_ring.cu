@@ -167,3 +167,293 @@ __device__ __forceinline__ void add_mul2(unsigned long long& acc, unsigned long 
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(t) : "l"(a), "l"(b), "l"(m0));
   asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc) : "l"(t));
 }
+
+template <bool FUSED>
+__global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(const __grid_constant__ RingParams p) {
+  extern __shared__ __align__(16) uint8_t ring_shared[];
+  __shared__ uint32_t tab[2u * kTabWords];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  for (uint32_t i = tid; i < 2u * kTabWords; i += blockDim.x) tab[i] = ring_entry(i & (kTabWords - 1u), i >= kTabWords, p.s);
+  const uint32_t G = 32u / p.Kpad, g = lane / p.Kpad, k = lane % p.Kpad, rows = G * p.K;
+  float lut0;
+  {
+    const float q = __fdiv_rn((float)(lane & 15u), (float)p.s);
+    lut0 = lane & 16u ? -q : q;
+  }
+  // per warp: rows of kRing bytes | 32 lanes' pieces of their streams | slots x 32 scales. Position q of lane l's
+  // row is byte q ^ 4 l of the row, so that lanes at the same position are in different banks.
+  uint8_t* mine = ring_shared + ((256u - (shared_address(ring_shared) & 255u)) & 255u) + (size_t)warp * p.warp_bytes;
+  for (uint32_t i = lane; i < p.warp_bytes / 16u; i += 32) reinterpret_cast<uint4*>(mine)[i] = make_uint4(0u, 0u, 0u, 0u);
+  const uint32_t shared_mine = shared_address(mine);
+  const uint32_t stage = shared_mine + rows * kRing + lane * kStage;
+  float2* scales = reinterpret_cast<float2*>(mine + rows * kRing + 32u * kStage);   // each twice: operands of packed products
+  const bool walker = k < p.K;
+  const uint32_t ring = shared_mine + (walker ? g * p.K + k : 0u) * kRing;          // 256-aligned
+  const uint32_t cell = ring | lane * 4u;                                            // address of q: (q & 255) ^ cell
+  chain_wait();                                   // the messages come from the kernels ahead
+  if (p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
+  __syncthreads();
+
+  const uint64_t first_of_warp = ((uint64_t)blockIdx.x * nwarps + warp) * G * p.run;
+  const uint64_t first = first_of_warp + (uint64_t)g * p.run;             // the run's first bucket
+  const uint32_t nb = first < p.B ? (uint32_t)min((uint64_t)p.run, p.B - first) : 0u;
+  const unsigned long long m0 = pack2(p.minus_zero, p.minus_zero);
+  const uint32_t most = __reduce_max_sync(0xffffffffu, nb * p.d);         // positions of the warp's longest run
+
+  // ---- the peer's table; the end of the string after the current one is always on its way -----------
+  const uint64_t* table = nullptr;
+  uint64_t all = 0, hi = 0, ahead = 0;
+  uint32_t err = 0;
+  uint32_t b = nb;                                // buckets opened so far
+  if (walker && nb) {
+    PeerTable pt;
+    if (peer_table(p.peers, k, p.B, &pt)) {
+      b = 0;
+      table = pt.table + first;
+      all = __ldg(pt.table + p.B);
+      hi = __ldg(table);
+      ahead = __ldg(table + 1);
+      if (all > pt.cap_bits) all = 0;             // a payload that ends past its bound: no string passes
+    } else {
+      err = QSGD_DEV_TABLE;                       // nothing of this message is read
+    }
+  }
+  // The stream: bits are counted from the 16-byte piece that it was entered in. Pieces [0, pieces) of it have been
+  // asked for, of pieces_all that the payload has; bits up to `ready` are there. The window: w0 holds bit bp, edge is
+  // the first bit of w1, next the place of the word behind w2.
+  const uint4* stream = nullptr;
+  uint32_t pieces = 0, pieces_all = 0, ready = 0;
+  uint32_t w0 = 0, w1 = 0, w2 = 0, bp = 0, edge = 32, next = 0, end = 0;
+  uint32_t at = 0xFFFFFFFFu;                      // last position passed
+  uint32_t stop = 0;                              // first position behind the bucket
+  uint32_t state = 0;                             // 0 or kStateBit
+  bool live = false;                              // inside a string
+  enum { kAway, kAsked, kThere } where = kAway;   // the window: not at the next string; its bits asked for; at it
+  auto drop = [&](uint32_t bits) {                // at most 32
+    bp += bits;
+    if (bp >= edge) { w0 = w1; w1 = w2; w2 = load_word(stage + (next & (kStage - 1u))); next += 4u; edge += 32u; }
+  };
+
+  // ---- this lane's part in adding up: 4 positions of a run, from `off_sum` on in every step ----------
+  const uint32_t quads = p.step >> 2, passes = (G * quads + 31u) >> 5;      // quads per run and step: 16 or 32
+  const uint32_t off_sum = (lane & (quads - 1u)) << 2;
+  uint32_t bucket_sum = 0, in_bucket = 0;         // bucket of the run, and place in it, of position `consumed`
+
+  for (uint32_t consumed = 0; consumed < most; consumed += p.step) {
+    const uint32_t goal = consumed + p.step;
+    // ---- every lane reads on until it has passed `goal` ---------------------------------------------
+    bool stuck = false;
+    for (;;) {
+      copies_done();
+      ready = pieces == pieces_all ? 0x7FFFFFFFu : pieces * 128u;
+      // a lane short of the goal is at the end of a string or at something the table does not cover, or its bits
+      // have not been there
+      const bool is_short = (live || b < nb) && (int32_t)at < (int32_t)goal - 1;
+      const bool over = live && (int32_t)(at + (state ? 1u : 0u) - stop) >= 0;
+      if (__any_sync(0xffffffffu, over || (is_short && (!live || bp >= end || stuck)))) {
+        if (over) {                               // went past the bucket: take it back
+          for (uint32_t q = stop; q != at + 1u; ++q) store_byte((q & (kRing - 1u)) ^ cell, 0u);
+          err |= QSGD_DEV_POSITION;
+          live = false;
+          where = kAway;
+        } else if (live && stuck && bp < end && (int32_t)(at + 1u - consumed) < (int32_t)kRing &&
+                   (int32_t)(ready - bp) >= kAhead) {
+          const SlowStep sl = slow_entry(__funnelshift_l(w1, w0, bp), end - bp, at, stop, p.s, state != 0u);
+          if (sl.err) {
+            err |= sl.err;
+            live = false;
+            where = kAway;
+          } else {
+            if (state) store_byte((sl.at & (kRing - 1u)) ^ cell, sl.code);
+            at = sl.at;
+            state = sl.state ? kStateBit : 0u;
+            drop(sl.used);
+          }
+        }
+        if (live && bp >= end) {                  // through: it must end exactly where the table says
+          if (bp != end || state) { err |= QSGD_DEV_OVERRUN; where = kAway; }
+          live = false;
+        }
+        if (!live) { end = bp; at = b * p.d - 1u; }
+        if (!live && b < nb && (int32_t)(b * p.d - consumed) < (int32_t)kRing) {      // the next one
+          const uint64_t lo = hi;
+          const uint32_t db = (uint32_t)min((uint64_t)p.d, p.n - (first + b) * p.d);
+          uint32_t fault = 0;
+          if (ahead < lo || ahead - lo < 32ull || ahead > all) fault = QSGD_DEV_TABLE;
+          else if (ahead - lo > 32ull + 40ull * db) fault = QSGD_DEV_OVERRUN;
+          if (!fault && where == kAway) {         // enter the stream there
+            stream = reinterpret_cast<const uint4*>(p.peers.payload[k]) + (lo >> 7);
+            pieces_all = (uint32_t)(((all + 127ull) >> 7) - (lo >> 7));
+            pieces = 0;
+            bp = end = (uint32_t)(lo & 127u);
+            ready = 0;
+            where = kAsked;
+          }
+          if (fault || (int32_t)(ready - bp) >= kAhead + 32) {
+            float A = 0.f;
+            if (fault) {                          // nothing of this string is read
+              err |= fault;
+              where = kAway;
+              at = (b + 1u) * p.d - 1u;
+            } else {
+              if (where == kAsked) {
+                next = (bp >> 5) * 4u;
+                w0 = load_word(stage + (next & (kStage - 1u)));
+                w1 = load_word(stage + ((next + 4u) & (kStage - 1u)));
+                w2 = load_word(stage + ((next + 8u) & (kStage - 1u)));
+                next += 12u;
+                edge = (bp & ~31u) + 32u;
+                where = kThere;
+              }
+              end = bp + (uint32_t)(ahead - lo);
+              A = __uint_as_float(__funnelshift_l(w1, w0, bp));
+              drop(32u);
+              stop = b * p.d + db;
+              state = 0u;
+              live = true;
+            }
+            scales[(b & (p.slots - 1u)) * 32u + lane] = make_float2(A, A);
+            hi = ahead;
+            ++b;
+            if (b < nb) ahead = __ldg(table + b + 1);
+          }
+        }
+      }
+      if (where != kAway)                         // ask for what there is room for
+        while (pieces < pieces_all && pieces < (bp >> 7) + kChunks) {
+          copy16(stage + ((pieces * 16u) & (kStage - 1u)), stream + pieces);
+          ++pieces;
+        }
+      // the burst: all lanes together, until none that can go on is short of the goal
+      int32_t until = (int32_t)(consumed + kRing - 2u * kMostAdvance);      // of `at`: room for two entries
+      const uint32_t last = ready ? min(end, ready - (uint32_t)kAhead + 1u) : 0u;        // first bit to stop at
+      for (;;) {
+        const bool go = (int32_t)at < until && (int32_t)(last - bp) > 0;
+        if (!__any_sync(0xffffffffu, go && (int32_t)at < (int32_t)goal - 1)) break;
+        if (go) {
+          // bits behind the string's end read as ones: no code is complete with them
+          uint32_t w = __funnelshift_l(w1, w0, bp) | __funnelshift_rc(0xFFFFFFFFu, 0u, end - bp);
+          const uint32_t e = table_entry(tab, w, state);
+          store_byte((__dp4a(e, 0x00010000u, at) & (kRing - 1u)) ^ cell, e >> 4);
+          at += e >> 26;
+          if (e & 15u) store_byte((at & (kRing - 1u)) ^ cell, e >> 9);
+          w <<= e & 15u;
+          const uint32_t f = table_entry(tab, w, e & kStateBit);
+          store_byte((__dp4a(f, 0x00010000u, at) & (kRing - 1u)) ^ cell, f >> 4);
+          at += f >> 26;
+          if (f & 15u) store_byte((at & (kRing - 1u)) ^ cell, f >> 9);
+          else until = INT32_MIN;                                           // nothing for the table here
+          state = f & kStateBit;
+          drop((e & 15u) + (f & 15u));
+        }
+      }
+      stuck = until == INT32_MIN;
+      if (!__any_sync(0xffffffffu, ((live || b < nb) && (int32_t)at < (int32_t)goal - 1) ||
+                                       (live && (int32_t)(at + (state ? 1u : 0u) - stop) >= 0)))
+        break;
+    }
+    __syncwarp();
+
+    // ---- ascending-k sums of positions [consumed, goal) of each run, 4 a lane ---------------------------
+    uint32_t bq = bucket_sum, c = in_bucket + off_sum;
+    while (c >= p.d) { c -= p.d; ++bq; }
+    const uint32_t q = consumed + off_sum;
+    for (uint32_t pass = 0; pass < passes; ++pass) {
+      const uint32_t gq = (pass * 32u + lane) / quads;
+      const uint32_t gr = gq < G ? gq : 0u;
+      const uint64_t run_first = first_of_warp + (uint64_t)gr * p.run;
+      OutSpan sp;
+      sp.ptr = p.out; sp.valid = 0u;
+      if (gq < G && bq < p.run) {
+        if (p.map.src) {
+          if (run_first + bq < p.B) sp = out_span(p.out, p.map, run_first + bq, c, p.d, p.n, 4u);
+        } else {                                  // buckets follow one another: position q of the run is simply there
+          const uint64_t i = run_first * p.d + q;
+          sp.ptr = p.out + i;
+          sp.valid = i < p.n ? (uint32_t)min((uint64_t)4u, p.n - i) : 0u;
+        }
+      }
+      const bool whole = sp.valid == 4u && (reinterpret_cast<uintptr_t>(sp.ptr) & 15u) == 0;
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (FUSED && whole) x = *reinterpret_cast<const float4*>(sp.ptr);
+      const uint32_t row0 = shared_mine + gr * p.K * kRing, pos = (q & (kRing - 1u)) ^ (gr * p.Kpad * 4u);
+      const float2* sc = scales + (bq & (p.slots - 1u)) * 32u + gr * p.Kpad;
+      unsigned long long a01 = 0ull, a23 = 0ull;
+#pragma unroll 4
+      for (uint32_t kk = 0; kk < p.K; ++kk) {
+        const uint32_t w = load_word(row0 + kk * kRing + (pos ^ (kk * 4u)));
+        const unsigned long long AA = *reinterpret_cast<const unsigned long long*>(sc + kk);
+        add_mul2(a01, AA, pack2(shfl_f(lut0, w), shfl_f(lut0, w >> 8)), m0);
+        add_mul2(a23, AA, pack2(shfl_f(lut0, w >> 16), shfl_f(lut0, w >> 24)), m0);
+      }
+      if (sp.valid) {
+        float v[4];
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(v[0]), "=f"(v[1]) : "l"(a01));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(v[2]), "=f"(v[3]) : "l"(a23));
+        if (whole) {
+          float4 o = make_float4(v[0], v[1], v[2], v[3]);
+          if (FUSED) {
+            o.x = __fsub_rn(x.x, __fmul_rn(p.c, o.x)); o.y = __fsub_rn(x.y, __fmul_rn(p.c, o.y));
+            o.z = __fsub_rn(x.z, __fmul_rn(p.c, o.z)); o.w = __fsub_rn(x.w, __fmul_rn(p.c, o.w));
+          }
+          *reinterpret_cast<float4*>(sp.ptr) = o;
+        } else {
+#pragma unroll
+          for (uint32_t e = 0; e < 4; ++e)
+            if (e < sp.valid) sp.ptr[e] = FUSED ? __fsub_rn(sp.ptr[e], __fmul_rn(p.c, v[e])) : v[e];
+        }
+      }
+    }
+    in_bucket += p.step;
+    while (in_bucket >= p.d) { in_bucket -= p.d; ++bucket_sum; }
+    __syncwarp();
+    // ---- zeros back: each lane its own row, 16 bytes at a time, starting at different banks ------------
+    if (walker) {
+      const uint32_t from = ((consumed & (kRing - 1u)) ^ cell) & ~63u;
+      for (uint32_t h = 0; h < p.step; h += 64u)
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i) zero_quad((from ^ h) | (((i + lane) & 3u) << 4));
+    }
+    __syncwarp();
+  }
+  copies_done();
+  if (live && (bp != end || state)) err |= QSGD_DEV_OVERRUN;      // a string must end exactly where the table says
+  if (err) atomicOr(p.status, err);
+}
+
+}  // namespace
+
+int launch_elias_ring(const FieldParams& f, bool fused, cudaStream_t stream) {
+  static KernelSite site[2];
+  RingParams p;
+  p.peers = f.peers; p.K = f.K; p.n = f.n; p.d = f.d; p.s = f.s; p.B = f.B; p.out = f.out; p.c = f.c; p.minus_zero = -0.f;
+  p.status = f.status; p.map = f.map; p.defer_sparse = f.defer_sparse;
+  p.Kpad = 1;
+  while (p.Kpad < p.K) p.Kpad <<= 1;
+  const uint32_t G = 32u / p.Kpad;
+  p.step = G == 1u ? 128u : 64u;
+  p.slots = 2;
+  while (p.slots < kRing / p.d + 2u) p.slots <<= 1;
+  p.warp_bytes = G * p.K * kRing + 32u * kStage + p.slots * 256u;
+  p.warp_bytes = (p.warp_bytes + 255u) & ~255u;
+  int sms = 0, most_shared = 0, occ = 0;
+  int st = device_sms(&sms);
+  if (!st) st = device_shared_memory(&most_shared);
+  if (st) return st;
+  uint32_t warps = ((uint32_t)most_shared - 2u * kStateBit - 2048u) / p.warp_bytes;
+  if (warps > kMaxWarps) warps = kMaxWarps;
+  // one run of consecutive buckets per lane group, all of the same length, in one wave
+  const uint64_t groups = (uint64_t)sms * warps * G;
+  p.run = (uint32_t)((p.B + groups - 1) / groups);
+  const uint64_t need = (p.B + (uint64_t)p.run * G - 1) / ((uint64_t)p.run * G);      // warps with work
+  const uint32_t per_sm = (uint32_t)((need + sms - 1) / sms);
+  if (per_sm < warps) warps = per_sm < 8u ? 8u : per_sm;
+  const size_t smem = (size_t)warps * p.warp_bytes + 1024u;
+  auto kern = fused ? decode_elias_ring_kernel<true> : decode_elias_ring_kernel<false>;
+  st = site[fused ? 1 : 0].lookup_dynamic(kern, (int)warps * 32, smem, &sms, &occ);
+  if (st) return st;
+  ScopedKernel sk(kKernDecodeElias, stream);
+  return (int)launch_chained(kern, (uint32_t)((need + warps - 1) / warps), warps * 32u, smem, stream, p);
+}
+
+}  // namespace qsgd
