@@ -4,6 +4,7 @@
 // lane per string (whole-bucket and ranged field rebuilding, byte codes) live in elias_decode_fields.cu, the
 // one with a team of lanes per string in elias_decode_teams.cu, the nonzero-driven decoder of the sparse
 // regime in elias_decode_sparse.cu; what they share is in elias_decode.cuh.
+#include <cstdlib>
 #include "elias_decode.cuh"
 
 namespace qsgd {
@@ -62,6 +63,7 @@ int launch_decode_elias(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
     if (sparse && sizes_known) return 0;                    // the host chose the sparse-regime kernel
   }
   f.defer_sparse = sparse ? 1u : 0u;
+  if (getenv("QRING") && !dense && s <= 15u && K <= 32u) return launch_elias_ring(f, fused, stream);
   return teams ? launch_elias_teams(f, dense, fused, stream) : launch_elias_fields(f, fused, stream);
 }
 
