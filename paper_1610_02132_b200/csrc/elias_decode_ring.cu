@@ -26,6 +26,7 @@ constexpr uint32_t kBits = 12;                         // stream bits per lookup
 constexpr uint32_t kTabWords = 1u << kBits;            // entries per state
 constexpr uint32_t kStateBit = 4u << kBits;            // byte offset of the second state's table: also its bit in an entry
 constexpr uint32_t kRing = 256;                        // positions (bytes) per lane
+constexpr uint32_t kStep = 128;                        // positions added up at a time
 constexpr uint32_t kMostAdvance = 63;                  // positions per entry of the table
 constexpr uint32_t kChunks = 4;                        // 16-byte pieces of the stream that a lane has in shared memory
 constexpr uint32_t kStage = 16u * kChunks;             // bytes of them
@@ -33,16 +34,10 @@ constexpr int32_t kAhead = 128;                        // bits (one piece) that 
 constexpr uint32_t kMaxWarps = 20;
 
 // Table entry: bits 0-3 stream bits used (0: nothing here for the table), 4-8 first byte, 9-13 second byte (what
-// stands above either is ignored by the shuffles), kStateBit next state, byte 2 place of the first byte, 26-31
-// place of the second = how far the entry goes, both from the last position passed. Where there is no second
-// byte its place is the first one's again, with the same value, or one that is still zero, with 0: both stores
-// are always made. An entry for nothing puts its first byte, 0, in front of everything.
-struct EntryBits {
-  uint32_t used, c1, c2, next, p1, p2;
-  __device__ __forceinline__ uint32_t pack() const {
-    return used | c1 << 4 | c2 << 9 | (next ? kStateBit : 0u) | p1 << 16 | p2 << 26;
-  }
-};
+// stands above either is ignored by the shuffles), kStateBit next state, 15 and 24 whether there is a first and
+// a second byte, byte 2 place of the first byte, 26-31 place of the second = how far the entry goes, both from
+// the last position passed.
+constexpr uint32_t kFirst = 1u << 15, kSecond = 1u << 24;
 
 // Sign and level at the top of w, `room` bits of which are there: level | negative << 4, and its length (0: none).
 __device__ __forceinline__ uint32_t tail_at(uint32_t w, uint32_t room, uint32_t s, uint32_t* len) {
@@ -53,38 +48,24 @@ __device__ __forceinline__ uint32_t tail_at(uint32_t w, uint32_t room, uint32_t 
 }
 
 __device__ __forceinline__ uint32_t ring_entry(uint32_t i, bool tail_first, uint32_t s) {
-  uint32_t w = i << (32u - kBits), room = kBits;
-  EntryBits e{0u, 0u, 0u, tail_first ? 1u : 0u, 0u, 0u};
-  const uint32_t stuck = (tail_first ? kStateBit : 0u) | 1u << 16;
+  uint32_t w = i << (32u - kBits), room = kBits, used = 0;
+  const uint32_t stuck = tail_first ? kStateBit : 0u;
   uint32_t gap = 1, len;
   if (!tail_first) {
     if (!elias_from_window(w, gap, len) || len > room || gap > kMostAdvance) return stuck;
-    w <<= len; room -= len; e.used = len;
-    uint32_t tl;
-    tail_at(w, room, s, &tl);
-    if (tl == 0u) {                                    // a gap alone: stop in front of its position
-      if (gap == 1u) return stuck;
-      e.next = 1u; e.p1 = gap; e.p2 = gap - 1u;
-      return e.pack();
-    }
+    w <<= len; room -= len; used = len;
   }
-  e.c1 = tail_at(w, room, s, &len);
-  if (len == 0u) return stuck;
-  w <<= len; room -= len; e.used += len;
-  e.next = 0u; e.p1 = gap; e.p2 = gap; e.c2 = e.c1;
+  const uint32_t c1 = tail_at(w, room, s, &len);
+  if (len == 0u)                                       // a gap alone: stop in front of its position
+    return tail_first || gap == 1u ? stuck : used | kStateBit | (gap - 1u) << 26;
+  w <<= len; room -= len; used += len;
+  const uint32_t first = c1 << 4 | kFirst | gap << 16;
   uint32_t gap2;
-  if (!elias_from_window(w, gap2, len) || len > room || gap + gap2 > kMostAdvance) return e.pack();
-  w <<= len; room -= len;
-  uint32_t tl;
-  const uint32_t c2 = tail_at(w, room, s, &tl);
-  e.used += len;
-  if (tl) {
-    e.used += tl; e.c2 = c2; e.p2 = gap + gap2;
-  } else {                                             // the second gap alone
-    e.next = 1u; e.p2 = gap + gap2 - 1u;
-    if (gap2 > 1u) e.c2 = 0u;
-  }
-  return e.pack();
+  if (!elias_from_window(w, gap2, len) || len > room || gap + gap2 > kMostAdvance) return used | first | gap << 26;
+  w <<= len; room -= len; used += len;
+  const uint32_t c2 = tail_at(w, room, s, &len);
+  if (len == 0u) return used | first | kStateBit | (gap + gap2 - 1u) << 26;       // the second gap alone
+  return (used + len) | first | c2 << 9 | kSecond | (gap + gap2) << 26;
 }
 
 __device__ __forceinline__ uint32_t table_entry(const uint32_t* tab, uint32_t w, uint32_t state) {
@@ -102,10 +83,8 @@ struct RingParams {
   uint64_t B;
   float* out;             // acc (overwritten) or x (updated in place)
   float c;                // eta / K
-  float minus_zero;       // -0
   uint32_t* status;
   uint32_t run;           // buckets per run
-  uint32_t step;          // positions added up at a time: 64 or 128
   uint32_t slots;         // scales kept per lane, a power of two: the buckets that a ring can touch
   uint32_t warp_bytes;
   uint32_t defer_sparse;  // a sparse-regime kernel was launched beside this one
@@ -120,6 +99,9 @@ __device__ __forceinline__ uint32_t load_word(uint32_t addr) {
   uint32_t v;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
   return v;
+}
+__device__ __forceinline__ void load_words(uint32_t addr, uint32_t& a, uint32_t& b) {
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(addr) : "memory");
 }
 // 16 bytes from global to shared memory, in the background; and the wait for all of this thread's.
 __device__ __forceinline__ void copy16(uint32_t addr, const void* from) {
@@ -154,21 +136,8 @@ __device__ __noinline__ SlowStep slow_entry(uint32_t w, uint32_t left, uint32_t 
   return r;
 }
 
-__device__ __forceinline__ unsigned long long pack2(float a, float b) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-// Two products and two sums, each rounded to nearest. The product is an fma with -0 that the compiler cannot see
-// (`m0`, from the kernel's parameters): a mul.rn.f32x2 in front of an add.rn.f32x2 was contracted.
-__device__ __forceinline__ void add_mul2(unsigned long long& acc, unsigned long long a, unsigned long long b,
-                                         unsigned long long m0) {
-  unsigned long long t;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(t) : "l"(a), "l"(b), "l"(m0));
-  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc) : "l"(t));
-}
-
-template <bool FUSED>
+// V: coordinates a lane adds up at a time: 8, or 4 where a warp has only one run.
+template <bool FUSED, uint32_t V>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(const __grid_constant__ RingParams p) {
   extern __shared__ __align__(16) uint8_t ring_shared[];
   __shared__ uint32_t tab[2u * kTabWords];
@@ -181,15 +150,15 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
     lut0 = lane & 16u ? -q : q;
   }
   // per warp: rows of kRing bytes | 32 lanes' pieces of their streams | slots x 32 scales. Position q of lane l's
-  // row is byte q ^ 4 l of the row, so that lanes at the same position are in different banks.
+  // row is byte q ^ 8 l of the row, so that lanes at the same position are in different banks.
   uint8_t* mine = ring_shared + ((256u - (shared_address(ring_shared) & 255u)) & 255u) + (size_t)warp * p.warp_bytes;
   for (uint32_t i = lane; i < p.warp_bytes / 16u; i += 32) reinterpret_cast<uint4*>(mine)[i] = make_uint4(0u, 0u, 0u, 0u);
   const uint32_t shared_mine = shared_address(mine);
   const uint32_t stage = shared_mine + rows * kRing + lane * kStage;
-  float2* scales = reinterpret_cast<float2*>(mine + rows * kRing + 32u * kStage);   // each twice: operands of packed products
+  float* scales = reinterpret_cast<float*>(mine + rows * kRing + 32u * kStage);
   const bool walker = k < p.K;
   const uint32_t ring = shared_mine + (walker ? g * p.K + k : 0u) * kRing;          // 256-aligned
-  const uint32_t cell = ring | lane * 4u;                                            // address of q: (q & 255) ^ cell
+  const uint32_t cell = ring | lane * 8u;                                            // address of q: (q & 255) ^ cell
   chain_wait();                                   // the messages come from the kernels ahead
   if (p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
   __syncthreads();
@@ -197,7 +166,6 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
   const uint64_t first_of_warp = ((uint64_t)blockIdx.x * nwarps + warp) * G * p.run;
   const uint64_t first = first_of_warp + (uint64_t)g * p.run;             // the run's first bucket
   const uint32_t nb = first < p.B ? (uint32_t)min((uint64_t)p.run, p.B - first) : 0u;
-  const unsigned long long m0 = pack2(p.minus_zero, p.minus_zero);
   const uint32_t most = __reduce_max_sync(0xffffffffu, nb * p.d);         // positions of the warp's longest run
 
   // ---- the peer's table; the end of the string after the current one is always on its way -----------
@@ -234,13 +202,13 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
     if (bp >= edge) { w0 = w1; w1 = w2; w2 = load_word(stage + (next & (kStage - 1u))); next += 4u; edge += 32u; }
   };
 
-  // ---- this lane's part in adding up: 4 positions of a run, from `off_sum` on in every step ----------
-  const uint32_t quads = p.step >> 2, passes = (G * quads + 31u) >> 5;      // quads per run and step: 16 or 32
-  const uint32_t off_sum = (lane & (quads - 1u)) << 2;
+  // ---- this lane's part in adding up: V positions of a run, from `off_sum` on in every step ----------
+  constexpr uint32_t kParts = kStep / V;          // lanes per run
+  const uint32_t off_sum = (lane & (kParts - 1u)) * V;
   uint32_t bucket_sum = 0, in_bucket = 0;         // bucket of the run, and place in it, of position `consumed`
 
-  for (uint32_t consumed = 0; consumed < most; consumed += p.step) {
-    const uint32_t goal = consumed + p.step;
+  for (uint32_t consumed = 0; consumed < most; consumed += kStep) {
+    const uint32_t goal = consumed + kStep;
     // ---- every lane reads on until it has passed `goal` ---------------------------------------------
     bool stuck = false;
     for (;;) {
@@ -312,7 +280,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
               state = 0u;
               live = true;
             }
-            scales[(b & (p.slots - 1u)) * 32u + lane] = make_float2(A, A);
+            scales[(b & (p.slots - 1u)) * 32u + lane] = A;
             hi = ahead;
             ++b;
             if (b < nb) ahead = __ldg(table + b + 1);
@@ -325,7 +293,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
           ++pieces;
         }
       // the burst: all lanes together, until none that can go on is short of the goal
-      int32_t until = (int32_t)(consumed + kRing - 2u * kMostAdvance);      // of `at`: room for two entries
+      int32_t until = (int32_t)(consumed + kRing - kMostAdvance);           // of `at`: room for an entry
       const uint32_t last = ready ? min(end, ready - (uint32_t)kAhead + 1u) : 0u;        // first bit to stop at
       for (;;) {
         const bool go = (int32_t)at < until && (int32_t)(last - bp) > 0;
@@ -334,17 +302,21 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
           // bits behind the string's end read as ones: no code is complete with them
           uint32_t w = __funnelshift_l(w1, w0, bp) | __funnelshift_rc(0xFFFFFFFFu, 0u, end - bp);
           const uint32_t e = table_entry(tab, w, state);
-          store_byte((__dp4a(e, 0x00010000u, at) & (kRing - 1u)) ^ cell, e >> 4);
+          if (e & kFirst) store_byte((__dp4a(e, 0x00010000u, at) & (kRing - 1u)) ^ cell, e >> 4);
           at += e >> 26;
-          if (e & 15u) store_byte((at & (kRing - 1u)) ^ cell, e >> 9);
-          w <<= e & 15u;
-          const uint32_t f = table_entry(tab, w, e & kStateBit);
-          store_byte((__dp4a(f, 0x00010000u, at) & (kRing - 1u)) ^ cell, f >> 4);
-          at += f >> 26;
-          if (f & 15u) store_byte((at & (kRing - 1u)) ^ cell, f >> 9);
-          else until = INT32_MIN;                                           // nothing for the table here
-          state = f & kStateBit;
-          drop((e & 15u) + (f & 15u));
+          if (e & kSecond) store_byte((at & (kRing - 1u)) ^ cell, e >> 9);
+          uint32_t used = e & 15u;
+          state = e & kStateBit;
+          if ((int32_t)at < until) {
+            const uint32_t f = table_entry(tab, w << used, state);
+            if (f & kFirst) store_byte((__dp4a(f, 0x00010000u, at) & (kRing - 1u)) ^ cell, f >> 4);
+            at += f >> 26;
+            if (f & kSecond) store_byte((at & (kRing - 1u)) ^ cell, f >> 9);
+            if ((f & 15u) == 0u) until = INT32_MIN;                         // nothing for the table here
+            used += f & 15u;
+            state = f & kStateBit;
+          }
+          drop(used);
         }
       }
       stuck = until == INT32_MIN;
@@ -354,65 +326,67 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
     }
     __syncwarp();
 
-    // ---- ascending-k sums of positions [consumed, goal) of each run, 4 a lane ---------------------------
+    // ---- ascending-k sums of positions [consumed, goal) of each run ------------------------------------
     uint32_t bq = bucket_sum, c = in_bucket + off_sum;
     while (c >= p.d) { c -= p.d; ++bq; }
     const uint32_t q = consumed + off_sum;
-    for (uint32_t pass = 0; pass < passes; ++pass) {
-      const uint32_t gq = (pass * 32u + lane) / quads;
-      const uint32_t gr = gq < G ? gq : 0u;
-      const uint64_t run_first = first_of_warp + (uint64_t)gr * p.run;
+    for (uint32_t gq = lane / kParts; gq < G; gq += 32u / kParts) {        // all lanes alike: 32 / kParts divides G
+      const uint64_t run_first = first_of_warp + (uint64_t)gq * p.run;
       OutSpan sp;
       sp.ptr = p.out; sp.valid = 0u;
-      if (gq < G && bq < p.run) {
+      if (bq < p.run) {
         if (p.map.src) {
-          if (run_first + bq < p.B) sp = out_span(p.out, p.map, run_first + bq, c, p.d, p.n, 4u);
+          if (run_first + bq < p.B) sp = out_span(p.out, p.map, run_first + bq, c, p.d, p.n, V);
         } else {                                  // buckets follow one another: position q of the run is simply there
           const uint64_t i = run_first * p.d + q;
           sp.ptr = p.out + i;
-          sp.valid = i < p.n ? (uint32_t)min((uint64_t)4u, p.n - i) : 0u;
+          sp.valid = i < p.n ? (uint32_t)min((uint64_t)V, p.n - i) : 0u;
         }
       }
-      const bool whole = sp.valid == 4u && (reinterpret_cast<uintptr_t>(sp.ptr) & 15u) == 0;
-      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (FUSED && whole) x = *reinterpret_cast<const float4*>(sp.ptr);
-      const uint32_t row0 = shared_mine + gr * p.K * kRing, pos = (q & (kRing - 1u)) ^ (gr * p.Kpad * 4u);
-      const float2* sc = scales + (bq & (p.slots - 1u)) * 32u + gr * p.Kpad;
-      unsigned long long a01 = 0ull, a23 = 0ull;
+      const bool whole = sp.valid == V && (reinterpret_cast<uintptr_t>(sp.ptr) & 15u) == 0;
+      float4 x[V / 4];
+      if (FUSED && whole)
+#pragma unroll
+        for (uint32_t h = 0; h < V / 4; ++h) x[h] = reinterpret_cast<const float4*>(sp.ptr)[h];
+      const uint32_t row0 = shared_mine + gq * p.K * kRing, pos = (q & (kRing - 1u)) ^ (gq * p.Kpad * 8u);
+      const float* sc = scales + (bq & (p.slots - 1u)) * 32u + gq * p.Kpad;
+      float acc[V];
+#pragma unroll
+      for (uint32_t e = 0; e < V; ++e) acc[e] = 0.f;
 #pragma unroll 4
       for (uint32_t kk = 0; kk < p.K; ++kk) {
-        const uint32_t w = load_word(row0 + kk * kRing + (pos ^ (kk * 4u)));
-        const unsigned long long AA = *reinterpret_cast<const unsigned long long*>(sc + kk);
-        add_mul2(a01, AA, pack2(shfl_f(lut0, w), shfl_f(lut0, w >> 8)), m0);
-        add_mul2(a23, AA, pack2(shfl_f(lut0, w >> 16), shfl_f(lut0, w >> 24)), m0);
-      }
-      if (sp.valid) {
-        float v[4];
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(v[0]), "=f"(v[1]) : "l"(a01));
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(v[2]), "=f"(v[3]) : "l"(a23));
-        if (whole) {
-          float4 o = make_float4(v[0], v[1], v[2], v[3]);
-          if (FUSED) {
-            o.x = __fsub_rn(x.x, __fmul_rn(p.c, o.x)); o.y = __fsub_rn(x.y, __fmul_rn(p.c, o.y));
-            o.z = __fsub_rn(x.z, __fmul_rn(p.c, o.z)); o.w = __fsub_rn(x.w, __fmul_rn(p.c, o.w));
-          }
-          *reinterpret_cast<float4*>(sp.ptr) = o;
-        } else {
+        uint32_t w[V / 4];
+        const uint32_t addr = row0 + kk * kRing + (pos ^ (kk * 8u));
+        if (V == 8) load_words(addr, w[0], w[V / 4 - 1]);
+        else w[0] = load_word(addr);
+        const float A = sc[kk];
 #pragma unroll
-          for (uint32_t e = 0; e < 4; ++e)
-            if (e < sp.valid) sp.ptr[e] = FUSED ? __fsub_rn(sp.ptr[e], __fmul_rn(p.c, v[e])) : v[e];
+        for (uint32_t e = 0; e < V; ++e) acc[e] = __fadd_rn(acc[e], __fmul_rn(A, shfl_f(lut0, w[e >> 2] >> (8u * (e & 3u)))));
+      }
+      if (whole) {
+#pragma unroll
+        for (uint32_t h = 0; h < V / 4; ++h) {
+          float4 o = make_float4(acc[4 * h], acc[4 * h + 1], acc[4 * h + 2], acc[4 * h + 3]);
+          if (FUSED) {
+            o.x = __fsub_rn(x[h].x, __fmul_rn(p.c, o.x)); o.y = __fsub_rn(x[h].y, __fmul_rn(p.c, o.y));
+            o.z = __fsub_rn(x[h].z, __fmul_rn(p.c, o.z)); o.w = __fsub_rn(x[h].w, __fmul_rn(p.c, o.w));
+          }
+          reinterpret_cast<float4*>(sp.ptr)[h] = o;
         }
+      } else if (sp.valid) {
+#pragma unroll
+        for (uint32_t e = 0; e < V; ++e)
+          if (e < sp.valid) sp.ptr[e] = FUSED ? __fsub_rn(sp.ptr[e], __fmul_rn(p.c, acc[e])) : acc[e];
       }
     }
-    in_bucket += p.step;
+    in_bucket += kStep;
     while (in_bucket >= p.d) { in_bucket -= p.d; ++bucket_sum; }
     __syncwarp();
     // ---- zeros back: each lane its own row, 16 bytes at a time, starting at different banks ------------
     if (walker) {
-      const uint32_t from = ((consumed & (kRing - 1u)) ^ cell) & ~63u;
-      for (uint32_t h = 0; h < p.step; h += 64u)
+      const uint32_t from = ((consumed & (kRing - 1u)) ^ cell) & ~(kStep - 1u);
 #pragma unroll
-        for (uint32_t i = 0; i < 4; ++i) zero_quad((from ^ h) | (((i + lane) & 3u) << 4));
+      for (uint32_t i = 0; i < kStep / 16u; ++i) zero_quad(from | (((i + lane) & (kStep / 16u - 1u)) << 4));
     }
     __syncwarp();
   }
@@ -424,17 +398,16 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
 }  // namespace
 
 int launch_elias_ring(const FieldParams& f, bool fused, cudaStream_t stream) {
-  static KernelSite site[2];
+  static KernelSite site[4];
   RingParams p;
-  p.peers = f.peers; p.K = f.K; p.n = f.n; p.d = f.d; p.s = f.s; p.B = f.B; p.out = f.out; p.c = f.c; p.minus_zero = -0.f;
+  p.peers = f.peers; p.K = f.K; p.n = f.n; p.d = f.d; p.s = f.s; p.B = f.B; p.out = f.out; p.c = f.c;
   p.status = f.status; p.map = f.map; p.defer_sparse = f.defer_sparse;
   p.Kpad = 1;
   while (p.Kpad < p.K) p.Kpad <<= 1;
   const uint32_t G = 32u / p.Kpad;
-  p.step = G == 1u ? 128u : 64u;
   p.slots = 2;
   while (p.slots < kRing / p.d + 2u) p.slots <<= 1;
-  p.warp_bytes = G * p.K * kRing + 32u * kStage + p.slots * 256u;
+  p.warp_bytes = G * p.K * kRing + 32u * kStage + p.slots * 128u;
   p.warp_bytes = (p.warp_bytes + 255u) & ~255u;
   int sms = 0, most_shared = 0, occ = 0;
   int st = device_sms(&sms);
@@ -449,8 +422,10 @@ int launch_elias_ring(const FieldParams& f, bool fused, cudaStream_t stream) {
   const uint32_t per_sm = (uint32_t)((need + sms - 1) / sms);
   if (per_sm < warps) warps = per_sm < 8u ? 8u : per_sm;
   const size_t smem = (size_t)warps * p.warp_bytes + 1024u;
-  auto kern = fused ? decode_elias_ring_kernel<true> : decode_elias_ring_kernel<false>;
-  st = site[fused ? 1 : 0].lookup_dynamic(kern, (int)warps * 32, smem, &sms, &occ);
+  void (*kern)(RingParams);
+  if (G == 1u) kern = fused ? decode_elias_ring_kernel<true, 4> : decode_elias_ring_kernel<false, 4>;
+  else kern = fused ? decode_elias_ring_kernel<true, 8> : decode_elias_ring_kernel<false, 8>;
+  st = site[(G == 1u ? 2 : 0) + (fused ? 1 : 0)].lookup_dynamic(kern, (int)warps * 32, smem, &sms, &occ);
   if (st) return st;
   ScopedKernel sk(kKernDecodeElias, stream);
   return (int)launch_chained(kern, (uint32_t)((need + warps - 1) / warps), warps * 32u, smem, stream, p);
