@@ -1,10 +1,10 @@
 // Decode-and-aggregate, Elias path, optionally fused with the SGD step (Section 3.1, end of
 // "Efficient Coding of Gradients": scale first, then the codes of the nonzeros in index order;
-// Appendix A.2 decoder; Algorithm 1 for the sum and the step): the choice among the decoders. Those with a
-// lane per string (whole-bucket and ranged field rebuilding, byte codes) live in elias_decode_fields.cu, the
-// one with a team of lanes per string in elias_decode_teams.cu, the nonzero-driven decoder of the sparse
-// regime in elias_decode_sparse.cu; what they share is in elias_decode.cuh.
-#include <cstdlib>
+// Appendix A.2 decoder; Algorithm 1 for the sum and the step): the choice among the decoders. The one that
+// reads streams of consecutive strings by table is in elias_decode_ring.cu (s <= 15), the one with a lane per
+// string for larger s in elias_decode_fields.cu, the one with a team of lanes per string in
+// elias_decode_teams.cu, the nonzero-driven decoder of the sparse regime in elias_decode_sparse.cu; what they
+// share is in elias_decode.cuh.
 #include "elias_decode.cuh"
 
 namespace qsgd {
@@ -16,19 +16,17 @@ namespace {
 // against 33.9).
 constexpr uint64_t kSmallWork = 8ull << 20;
 
-// A lane per string, or a team of lanes? A lane per string is the cheaper reading (a team reads its string
-// almost twice) but needs strings enough for the GPU, and short ones, whose rows leave room for many
-// warps. Measured lines (us, a lane against a team): 16 K strings of d = 512, s = 15: 66 / 34, 65 K: 85 /
-// 107; 32 K of d = 128, s = 3: 28 / 26, 262 K: 37 / 60; s = 255:
-// 16 K of d = 512 118 / 74, 524 K 1974 / 1744, but
-// 2 M of d = 128 1488 / 1751. From d = 1024 on a lane's string is long enough to decide the time by itself
-// (2 K strings of d = 4096: 280 / 23; 32 K: 1849 / 568), except where hundreds of lanes per SM read
-// nearly empty ones (65 K with s = 3: 252 / 313). Code'_s has a symbol per coordinate: always teams.
+// A lane per string (or stream of strings), or a team of lanes? A lane per string is the cheaper reading (a team
+// reads its string almost twice) but needs strings enough for the GPU's lanes. Measured lines (us, a lane against
+// a team). s <= 15: 16 K strings of d = 512 33 / 33, of d = 4096 (8 K of them) 168 / 114, 32 K of d = 4096 264 /
+// 563, 32 K of d = 128 19 / 26, 65 K of d = 512 43 / 107. s = 255: 16 K of d = 512 118 / 74, 524 K 1974 / 1744, but
+// 2 M of d = 128 1488 / 1751; from d = 1024 on always teams (131 K strings of d = 4096: 1559 / 493). Code'_s has
+// a symbol per coordinate: always teams.
 bool use_teams(uint64_t B, uint32_t K, uint32_t d, uint32_t s, bool dense) {
   const uint64_t strings = B * K;
   if (dense || K > 32u) return true;
-  if (d >= 1024u) return s > 3u || strings <= (48u << 10);
-  return strings <= (40u << 10) || (s > 15u && d >= 512u);
+  if (s <= 15u) return strings <= (12u << 10);
+  return d >= 512u || strings <= (40u << 10);
 }
 
 }  // namespace
@@ -63,8 +61,8 @@ int launch_decode_elias(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
     if (sparse && sizes_known) return 0;                    // the host chose the sparse-regime kernel
   }
   f.defer_sparse = sparse ? 1u : 0u;
-  if (getenv("QRING") && !dense && s <= 15u && K <= 32u) return launch_elias_ring(f, fused, stream);
-  return teams ? launch_elias_teams(f, dense, fused, stream) : launch_elias_fields(f, fused, stream);
+  if (teams) return launch_elias_teams(f, dense, fused, stream);
+  return s <= 15u ? launch_elias_ring(f, fused, stream) : launch_elias_fields(f, fused, stream);
 }
 
 }  // namespace qsgd

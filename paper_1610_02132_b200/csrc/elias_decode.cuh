@@ -121,7 +121,6 @@ struct FieldParams {
   uint32_t* status;
   uint32_t row_words;   // per peer row: d * lb / 32 level words, then d / 32 sign words (padded to 4)
   uint32_t bucket_words;  // K rows + K scales, padded to 4
-  uint32_t range;         // byte-code decoder: positions per range
   uint32_t defer_sparse;  // a sparse-regime kernel was launched beside this one
   BucketMap map;          // where the buckets live in `out` (per-tensor policy), or no map
 };
@@ -363,8 +362,8 @@ __device__ __forceinline__ uint32_t advance(LaneParse& st, uint32_t rend, uint32
 }
 
 // Launchers of the decoders; 0 or a cudaError_t. `launched`: whether the sparse-regime kernel takes the shape.
-int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream);     // Code_s, at most 32 peers
-int launch_elias_ring(const FieldParams& p, bool fused, cudaStream_t stream);                  // ... and s <= 15
+int launch_elias_ring(const FieldParams& p, bool fused, cudaStream_t stream);     // Code_s, s <= 15, at most 32 peers
+int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream);         // Code_s, s > 15, at most 32 peers
 int launch_elias_teams(const FieldParams& p, bool dense, bool fused, cudaStream_t stream);
 int launch_elias_sparse(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d, uint32_t s, float* out, bool fused,
                         float c, uint32_t* status, bool check_regime, const BucketMap& map, cudaStream_t stream,

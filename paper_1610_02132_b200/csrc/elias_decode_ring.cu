@@ -3,7 +3,7 @@
 // Appendix A.2 for the integer code; Algorithm 1 for the sum and the step.)
 //
 // A peer's strings of consecutive buckets are one stretch of its payload, so a lane reads one stream from
-// end to end, by background copies of 16 bytes into its own 64 bytes of shared memory: a load into a register
+// end to end, by background copies of 16 bytes into its own 128 bytes of shared memory: a load into a register
 // that a later instruction moves or shifts holds up the whole warp, whichever lane it was for (that, not the
 // instructions, was the time of reading: 300 of 360 us at n = 2^25). It writes one byte per nonzero -- level |
 // negative << 4, the lane index of +-(level / s) in a shuffle table -- into its ring of 256 positions in
@@ -28,7 +28,7 @@ constexpr uint32_t kStateBit = 4u << kBits;            // byte offset of the sec
 constexpr uint32_t kRing = 256;                        // positions (bytes) per lane
 constexpr uint32_t kStep = 128;                        // positions added up at a time
 constexpr uint32_t kMostAdvance = 63;                  // positions per entry of the table
-constexpr uint32_t kChunks = 4;                        // 16-byte pieces of the stream that a lane has in shared memory
+constexpr uint32_t kChunks = 8;                        // 16-byte pieces of the stream that a lane has in shared memory
 constexpr uint32_t kStage = 16u * kChunks;             // bytes of them
 constexpr int32_t kAhead = 128;                        // bits (one piece) that have to be there for a round of the burst
 constexpr uint32_t kMaxWarps = 20;
@@ -92,6 +92,15 @@ struct RingParams {
 };
 
 __device__ __forceinline__ uint32_t shared_address(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// The same and a load where `when` is nonzero, without a branch.
+__device__ __forceinline__ void store_byte_if(uint32_t when, uint32_t addr, uint32_t v) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.u8 [%1], %2;\n\t}" ::"r"(when), "r"(addr), "r"(v)
+               : "memory");
+}
+__device__ __forceinline__ void load_word_if(bool when, uint32_t& v, uint32_t addr) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p ld.shared.u32 %0, [%2];\n\t}" : "+r"(v) : "r"((uint32_t)when), "r"(addr)
+               : "memory");
+}
 __device__ __forceinline__ void store_byte(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.u8 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
@@ -142,6 +151,10 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
   extern __shared__ __align__(16) uint8_t ring_shared[];
   __shared__ uint32_t tab[2u * kTabWords];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  if (p.defer_sparse) {                           // standing down should cost little: before the table is made
+    chain_wait();
+    if (sparse_regime(p.peers, p.K, p.B, p.d)) return;
+  }
   for (uint32_t i = tid; i < 2u * kTabWords; i += blockDim.x) tab[i] = ring_entry(i & (kTabWords - 1u), i >= kTabWords, p.s);
   const uint32_t G = 32u / p.Kpad, g = lane / p.Kpad, k = lane % p.Kpad, rows = G * p.K;
   float lut0;
@@ -160,7 +173,6 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
   const uint32_t ring = shared_mine + (walker ? g * p.K + k : 0u) * kRing;          // 256-aligned
   const uint32_t cell = ring | lane * 8u;                                            // address of q: (q & 255) ^ cell
   chain_wait();                                   // the messages come from the kernels ahead
-  if (p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
   __syncthreads();
 
   const uint64_t first_of_warp = ((uint64_t)blockIdx.x * nwarps + warp) * G * p.run;
@@ -188,10 +200,10 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
   }
   // The stream: bits are counted from the 16-byte piece that it was entered in. Pieces [0, pieces) of it have been
   // asked for, of pieces_all that the payload has; bits up to `ready` are there. The window: w0 holds bit bp, edge is
-  // the first bit of w1, next the place of the word behind w2.
+  // the first bit of w1.
   const uint4* stream = nullptr;
   uint32_t pieces = 0, pieces_all = 0, ready = 0;
-  uint32_t w0 = 0, w1 = 0, w2 = 0, bp = 0, edge = 32, next = 0, end = 0;
+  uint32_t w0 = 0, w1 = 0, w2 = 0, bp = 0, edge = 32, end = 0;
   uint32_t at = 0xFFFFFFFFu;                      // last position passed
   uint32_t stop = 0;                              // first position behind the bucket
   uint32_t state = 0;                             // 0 or kStateBit
@@ -199,7 +211,18 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
   enum { kAway, kAsked, kThere } where = kAway;   // the window: not at the next string; its bits asked for; at it
   auto drop = [&](uint32_t bits) {                // at most 32
     bp += bits;
-    if (bp >= edge) { w0 = w1; w1 = w2; w2 = load_word(stage + (next & (kStage - 1u))); next += 4u; edge += 32u; }
+    const bool cross = bp >= edge;
+    w0 = cross ? w1 : w0;
+    w1 = cross ? w2 : w1;
+    load_word_if(cross, w2, stage + (((edge >> 3) + 8u) & (kStage - 1u)));        // the word behind w2
+    edge += cross ? 32u : 0u;
+  };
+  auto ask = [&]() {                              // for the pieces that there is room for
+    if (where != kAway)
+      while (pieces < pieces_all && pieces < (bp >> 7) + kChunks) {
+        copy16(stage + ((pieces * 16u) & (kStage - 1u)), stream + pieces);
+        ++pieces;
+      }
   };
 
   // ---- this lane's part in adding up: V positions of a run, from `off_sum` on in every step ----------
@@ -265,11 +288,10 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
               at = (b + 1u) * p.d - 1u;
             } else {
               if (where == kAsked) {
-                next = (bp >> 5) * 4u;
-                w0 = load_word(stage + (next & (kStage - 1u)));
-                w1 = load_word(stage + ((next + 4u) & (kStage - 1u)));
-                w2 = load_word(stage + ((next + 8u) & (kStage - 1u)));
-                next += 12u;
+                const uint32_t word = (bp >> 5) * 4u;
+                w0 = load_word(stage + (word & (kStage - 1u)));
+                w1 = load_word(stage + ((word + 4u) & (kStage - 1u)));
+                w2 = load_word(stage + ((word + 8u) & (kStage - 1u)));
                 edge = (bp & ~31u) + 32u;
                 where = kThere;
               }
@@ -287,43 +309,37 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
           }
         }
       }
-      if (where != kAway)                         // ask for what there is room for
-        while (pieces < pieces_all && pieces < (bp >> 7) + kChunks) {
-          copy16(stage + ((pieces * 16u) & (kStage - 1u)), stream + pieces);
-          ++pieces;
-        }
+      ask();
       // the burst: all lanes together, until none that can go on is short of the goal
       int32_t until = (int32_t)(consumed + kRing - kMostAdvance);           // of `at`: room for an entry
       const uint32_t last = ready ? min(end, ready - (uint32_t)kAhead + 1u) : 0u;        // first bit to stop at
       for (;;) {
         const bool go = (int32_t)at < until && (int32_t)(last - bp) > 0;
         if (!__any_sync(0xffffffffu, go && (int32_t)at < (int32_t)goal - 1)) break;
-        if (go) {
-          // bits behind the string's end read as ones: no code is complete with them
-          uint32_t w = __funnelshift_l(w1, w0, bp) | __funnelshift_rc(0xFFFFFFFFu, 0u, end - bp);
-          const uint32_t e = table_entry(tab, w, state);
-          if (e & kFirst) store_byte((__dp4a(e, 0x00010000u, at) & (kRing - 1u)) ^ cell, e >> 4);
-          at += e >> 26;
-          if (e & kSecond) store_byte((at & (kRing - 1u)) ^ cell, e >> 9);
-          uint32_t used = e & 15u;
-          state = e & kStateBit;
-          if ((int32_t)at < until) {
-            const uint32_t f = table_entry(tab, w << used, state);
-            if (f & kFirst) store_byte((__dp4a(f, 0x00010000u, at) & (kRing - 1u)) ^ cell, f >> 4);
-            at += f >> 26;
-            if (f & kSecond) store_byte((at & (kRing - 1u)) ^ cell, f >> 9);
-            if ((f & 15u) == 0u) until = INT32_MIN;                         // nothing for the table here
-            used += f & 15u;
-            state = f & kStateBit;
-          }
-          drop(used);
-        }
+        // (a lane that does not go on finds an entry for nothing)
+        // bits behind the string's end read as ones: no code is complete with them
+        const uint32_t w = __funnelshift_l(w1, w0, bp) | __funnelshift_rc(0xFFFFFFFFu, 0u, end - bp);
+        uint32_t e = table_entry(tab, w, state);
+        e = go ? e : state;
+        store_byte_if(e & kFirst, (__dp4a(e, 0x00010000u, at) & (kRing - 1u)) ^ cell, e >> 4);
+        at += e >> 26;
+        store_byte_if(e & kSecond, (at & (kRing - 1u)) ^ cell, e >> 9);
+        state = e & kStateBit;
+        uint32_t f = table_entry(tab, w << (e & 15u), state);
+        f = go && (int32_t)at < until ? f : state;
+        store_byte_if(f & kFirst, (__dp4a(f, 0x00010000u, at) & (kRing - 1u)) ^ cell, f >> 4);
+        at += f >> 26;
+        store_byte_if(f & kSecond, (at & (kRing - 1u)) ^ cell, f >> 9);
+        until = f & 15u ? until : INT32_MIN;      // nothing for the table here, or far enough
+        state = f & kStateBit;
+        drop((e & 15u) + (f & 15u));
       }
       stuck = until == INT32_MIN;
       if (!__any_sync(0xffffffffu, ((live || b < nb) && (int32_t)at < (int32_t)goal - 1) ||
                                        (live && (int32_t)(at + (state ? 1u : 0u) - stop) >= 0)))
         break;
     }
+    ask();                                        // they come while the warp adds up
     __syncwarp();
 
     // ---- ascending-k sums of positions [consumed, goal) of each run ------------------------------------

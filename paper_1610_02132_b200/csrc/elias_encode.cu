@@ -60,12 +60,13 @@ struct EliasWs {
 // problem sooner; the team kernels (a lane walks 64 or more) do less per coordinate. Whole encodes measured
 // both ways on three input families, teams against tiles (us): Code_s with s <= 15 16.7 / 16.0 at n = 2^21,
 // 19.2 / 20.4 at 3 * 2^20; s = 255 35 to 47 / 27 to 31 at 3 * 2^20, 44 / 44 at 6 * 2^20; Code'_s with d = 512
-// 29 / 28 at 2^22, 36 / 39 at 6 * 2^20, with d = 4096 (128 coordinates a lane) 56 / 49 at 2^23. Bucket sizes
+// 29 / 28 at 2^22, 36 / 39 at 6 * 2^20, with d = 4096 (128 coordinates a lane) 56 / 49 at 2^23,
+// 173 / 176 at 2^25. Bucket sizes
 // whose lanes would not get whole 64-coordinate blocks always take the tiles (978 / 280 us at n = 2^25,
 // d = 96).
 inline bool use_tiles(uint64_t n, uint32_t d, uint32_t s, bool dense) {
   if ((d & (d - 1u)) || d < 64u) return true;
-  const uint64_t m = dense ? (d > 1024u ? 12u : 4u) : s > 15u ? 6u : 2u;
+  const uint64_t m = dense ? (d > 1024u ? 20u : 4u) : s > 15u ? 6u : 2u;
   return n <= m << 20;
 }
 

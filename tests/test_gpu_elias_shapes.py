@@ -1,6 +1,7 @@
 """Elias Encode and Decode at the edges of their dispatch rules: problems read by teams of lanes (parts of a
 string shorter and longer than a lane's least part, peers in several passes, codes on which a reader that
-starts out of step stays out of step) and encoded in tiles (tiles of whole buckets, sizes around a tile, both
+starts out of step stays out of step), streams read by table (buckets shorter and longer than a ring, gaps that
+the table does not hold, malformed strings inside a stream) and encoded in tiles (tiles of whole buckets, sizes around a tile, both
 sides of the line to the team kernels). Bit for bit against the oracle."""
 import numpy as np
 import pytest
@@ -53,8 +54,59 @@ def test_teams_out_of_step(code, s, value):
     run(n, d, s, MAX, code, 3, make)
 
 
-@pytest.mark.parametrize("n,d,s,K", [(40 * 512 * 128, 512, 15, 8), (40 * 512 * 128 + 512, 512, 15, 8),
-                                     (48 * 1024 * 1024 + 1, 1024, 3, 1), (2 ** 20, 4096, 1, 8), (2 ** 20 + 4096, 4096, 1, 8)])
+@pytest.mark.parametrize("n,d,s,norm,K", [
+    (13000 * 32 + 5, 32, 15, MAX, 1), (6500 * 96 + 95, 96, 3, L2, 2), (3200 * 160, 160, 15, L2, 4), (1800 * 224 + 1, 224, 7, MAX, 8),
+    (1600 * 256 + 9, 256, 15, MAX, 8), (800 * 512 + 3, 512, 15, L2, 17), (500 * 1024 + 7, 1024, 1, MAX, 32), (1600 * 2048 + 2047, 2048, 15, L2, 9),
+])
+def test_streams(n, d, s, norm, K):
+    """A lane per (run of buckets, peer). Every other peer's strings have long gaps and empty buckets."""
+    def make(w):
+        if w % 2 == 0:
+            return I.gaussian(n, 1.0, seed=50 + w)
+        g = I.sparse_laplace(n, 1e-3, 0.3, seed=50 + w)
+        g[np.random.default_rng(w).random(n) < 0.97] = 0.0
+        g[n // 3: n // 3 + 3 * d] = 0.0
+        return g
+    run(n, d, s, norm, ELIAS, K, make)
+
+
+@pytest.mark.parametrize("d,K", [(32, 1), (512, 16), (1024, 24)])
+def test_malformed_streams(d, K):
+    """Streams with noise, strings cut short and offsets out of order in one peer's message: flagged, nothing
+    written out of bounds, and where only one string is bad the buckets of the others come out right."""
+    import paper_1610_02132_b200 as Q
+    B = 13000 // K + 1
+    n, s = B * d - d // 2, 3
+    good, info = O.encode(I.gaussian(n, 1.0, seed=4), d, s, MAX, ELIAS, 7, 0, 0)
+    table = O.message_table(good, info, n, d)
+    noise = good.copy()
+    noise[: info[1]] = np.random.default_rng(1).integers(0, 256, info[1], dtype=np.uint8)
+    cut, swapped, above = table.copy(), table.copy(), table.copy()
+    cut[B // 2] -= 3
+    swapped[[B // 3, B // 3 + 1]] = swapped[[B // 3 + 1, B // 3]]
+    above[-1] += 1 << 33
+    one = good.copy()                                          # a level above s in one string: its first sign and level all ones
+    lo = int(table[5]) + 32
+    for t in range(lo, min(lo + 24, int(table[6]))):
+        one[4 * (t // 32) + 3 - (t % 32) // 8] |= 1 << (7 - t % 8)
+    for msg, tab, only in ((noise, table, None), (good, cut, None), (good, swapped, None), (good, above, None), (one, table, 5)):
+        bufs = [torch.from_numpy(np.concatenate([m, np.zeros(64, np.uint8)])).cuda() for m in (msg, good)]
+        tabs = [torch.from_numpy(x.view(np.int64)).cuda() for x in (tab, table)]
+        order = [0] + [1] * (K - 1)
+        status = Q.new_status()
+        acc = torch.full((n + 256,), 7.0, device="cuda")
+        Q.qsgd_decode_accumulate([bufs[i] for i in order], [tabs[i] for i in order], n, d, s, ELIAS, acc[:n], status,
+                                 payload_bytes=[info[1]] * K)
+        torch.cuda.synchronize()
+        assert int(status.item()) != 0 and bool((acc[n:] == 7.0).all())
+        if only is not None:
+            ref = O.decode_accumulate([good] * K, [table] * K, n, d, s, ELIAS)[1]
+            same = acc[:n].cpu().numpy().view(np.uint32) == ref.view(np.uint32)
+            same[only * d: (only + 1) * d] = True
+            assert same.all()
+
+
+@pytest.mark.parametrize("n,d,s,K", [(1536 * 512, 512, 15, 8), (1536 * 512 + 1, 512, 15, 8), (2 ** 22, 128, 3, 2), (2 ** 25, 4096, 3, 2), (2 ** 20, 4096, 1, 8), (2 ** 20 + 4096, 4096, 1, 8)])
 def test_lines_between_decoders(n, d, s, K):
     """Both sides of the lines between a lane and a team per string and between one and two launches, against
     the sum of the messages decoded one by one (K = 1 goes through another decoder or another split)."""
