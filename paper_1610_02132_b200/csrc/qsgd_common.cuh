@@ -1,5 +1,4 @@
-// Shared device helpers of the QSGD kernels (sm_100a): Philox4x32-10, message layout,
-// bit-field helpers and the internal launch interface between the C ABI and the kernels.
+// Shared by the QSGD kernels (sm_100a): message layout and the internal launch interface between the C ABI and the kernels.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -45,45 +44,6 @@ __host__ __device__ inline FixedLayout make_fixed_layout(uint64_t n, uint32_t d,
   L.off_level = L.off_sign + align16(4 * L.sign_words);
   L.total = L.off_level + align16(4 * L.level_words);
   return L;
-}
-
-// ------------------------------------------------------------------------------------------
-// Philox4x32-10 (Salmon et al., SC'11). One call yields the uniforms of four consecutive
-// coordinates: counter = (q lo, q hi, step, worker) with q = i / 4, key = (seed lo, seed hi).
-// ------------------------------------------------------------------------------------------
-struct PhiloxKey { uint32_t k0, k1; };
-
-__device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
-                                               uint32_t k0, uint32_t k1) {
-  constexpr uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
-  constexpr uint32_t W0 = 0x9E3779B9u, W1 = 0xBB67AE85u;
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint32_t hi0 = __umulhi(M0, c0), lo0 = M0 * c0;
-    const uint32_t hi1 = __umulhi(M1, c2), lo1 = M1 * c2;
-    c0 = hi1 ^ c1 ^ k0;
-    c1 = lo1;
-    c2 = hi0 ^ c3 ^ k1;
-    c3 = lo0;
-    k0 += W0;
-    k1 += W1;
-  }
-  return make_uint4(c0, c1, c2, c3);
-}
-
-// Uniform in [0, 1 - 2^-24]: top 24 bits of a Philox word times 2^-24 (exact in fp32).
-__device__ __forceinline__ float u01_from_bits(uint32_t x) {
-  return __fmul_rn(__uint2float_rn(x >> 8), 5.9604644775390625e-08f);
-}
-
-// Level of one coordinate: min(floor((s * |v|) * r + u), s) with r = 1 / A (0 for a zero
-// bucket). Two multiplies and one add, each rounded to nearest, no contraction.
-__device__ __forceinline__ uint32_t quantize_level(float v, float r, float sf, uint32_t s,
-                                                   uint32_t rnd) {
-  const float t = __fmul_rn(__fmul_rn(sf, fabsf(v)), r);
-  const float c = __fadd_rn(t, u01_from_bits(rnd));
-  const uint32_t l = (uint32_t)__float2int_rz(c);
-  return min(l, s);
 }
 
 // ------------------------------------------------------------------------------------------

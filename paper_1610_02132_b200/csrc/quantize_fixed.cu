@@ -31,38 +31,15 @@
 //   * the sign bit "negative and level > 0" is the sign of fma(level, v, +0), shifted into the
 //     sign word with a funnel shift.
 // A generic kernel (any bucket size that is a multiple of 32) keeps the simple structure.
-#include <float.h>
-
 #include <atomic>
 
-#include "qsgd_common.cuh"
+#include "quantize.cuh"
 
 namespace qsgd {
 
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kTile = 4096;           // coordinates per tile
-
-struct QuantizeParams {
-  const float* g;
-  uint64_t n;
-  uint32_t d;
-  uint32_t s;
-  uint32_t tile_coords;   // generic kernel: coordinates per tile = whole buckets, <= kTile
-  uint64_t coord_base;    // generic kernel: first coordinate it is responsible for
-  uint32_t k0, k1, step, worker;
-  float* A_out;
-  uint32_t* sign_out;
-  uint32_t* level_out;
-  uint64_t B, sign_words, level_words;
-  uint64_t tiles;
-  uint32_t* status;
-  uint64_t* info;         // optional: the four message-info words of a fixed-width message
-  uint64_t total_bytes;
-  uint32_t* clear_word;   // optional: a word the kernel sets to zero (arrival counter of a later kernel)
-  BucketMap map;          // per-tensor policy: where each bucket lives in g, or no map
-};
+constexpr int kThreads = kQuantizeThreads;
 
 // ---------------------------------------------------------------------------------------------
 // PTX helpers: mbarrier and 1-D bulk copy global -> shared.
@@ -105,177 +82,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ float fma_rn(float a, float b, float c) {
-  float r;
-  asm("fma.rn.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-
-// ---------------------------------------------------------------------------------------------
-// Philox4x32-10 for the counter (q, 0, step, worker) with everything that does not depend on q
-// folded into kernel-uniform constants on the host: after round 0 two of the four words are
-// constants, which also makes one product of round 1 a constant. 37 instead of 40
-// multiply / xor instructions per block of four uniforms.
-// ---------------------------------------------------------------------------------------------
-struct PhiloxConsts {
-  uint32_t y0;        // worker ^ k1[0]
-  uint32_t z0;        // lo(M1 * step) ^ k0[1]
-  uint32_t z1;        // hi(M0 * x0) ^ k1[1],  x0 = hi(M1 * step) ^ k0[0]
-  uint32_t z2;        // lo(M0 * x0) ^ k1[2]
-  uint32_t k0_2;      // k0[2]
-  uint32_t k[7][2];   // round keys 3 .. 9
-};
-
-constexpr uint32_t kM0 = 0xD2511F53u, kM1 = 0xCD9E8D57u;
-
-__device__ __forceinline__ uint4 philox_q(uint32_t q, const PhiloxConsts& pc) {
-  // round 0: (q, 0, step, worker) -> (x0, l1, hi(M0 q) ^ y0, lo(M0 q))
-  uint64_t p0 = (uint64_t)kM0 * q;
-  uint32_t a2 = (uint32_t)(p0 >> 32) ^ pc.y0, a3 = (uint32_t)p0;
-  // round 1: (x0, l1, a2, a3) -> (hi(M1 a2) ^ z0, lo(M1 a2), a3 ^ z1, lo(M0 x0))
-  uint64_t p1 = (uint64_t)kM1 * a2;
-  uint32_t c0 = (uint32_t)(p1 >> 32) ^ pc.z0, c1 = (uint32_t)p1, c2 = a3 ^ pc.z1;
-  // round 2: c3 = lo(M0 x0) is folded into z2
-  p0 = (uint64_t)kM0 * c0;
-  p1 = (uint64_t)kM1 * c2;
-  c0 = (uint32_t)(p1 >> 32) ^ c1 ^ pc.k0_2;
-  c1 = (uint32_t)p1;
-  c2 = (uint32_t)(p0 >> 32) ^ pc.z2;
-  uint32_t c3 = (uint32_t)p0;
-  // rounds 3 .. 9: the high and low halves by separate multiplies (measured slightly faster than the
-  // 64-bit products here; the first rounds stay as they are, where it measured slower)
-#pragma unroll
-  for (int r = 0; r < 7; ++r) {
-    const uint32_t h0 = __umulhi(kM0, c0), l0 = kM0 * c0;
-    const uint32_t h1 = __umulhi(kM1, c2), l1 = kM1 * c2;
-    c0 = h1 ^ c1 ^ pc.k[r][0];
-    c1 = l1;
-    c2 = h0 ^ c3 ^ pc.k[r][1];
-    c3 = l0;
-  }
-  return make_uint4(c0, c1, c2, c3);
-}
-
-// The uniforms of the 16 coordinates of one thread (Philox blocks q0 .. q0 + 3) as fp32 bit
-// patterns m = word >> 8 (see quantize_one).
-__device__ __forceinline__ void philox_uniforms16(uint32_t q0, const PhiloxConsts& pc, float (&um)[16]) {
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const uint4 w = philox_q(q0 + b, pc);
-    um[4 * b] = __uint_as_float(w.x >> 8);
-    um[4 * b + 1] = __uint_as_float(w.y >> 8);
-    um[4 * b + 2] = __uint_as_float(w.z >> 8);
-    um[4 * b + 3] = __uint_as_float(w.w >> 8);
-  }
-}
-
-constexpr float kTwo23 = 8388608.0f;
-constexpr uint32_t kTwo23Bits = 0x4B000000u;
-
-constexpr float kTwo125 = 4.253529586511730793292182592897102643e+37f;
-
-// One coordinate. Returns the raw bits of 2^23 + level (level clamped to s when CLAMP); pushes the
-// sign bit into `sw`. `um` is the bit pattern m = top 24 Philox bits read as an fp32, i.e. m * 2^-149.
-// RAW_SIGN: push the sign bit of v as it is; the caller clears the signs of zero levels afterwards
-// with a mask derived from the packed level words (cheaper than two more operations per coordinate
-// when a word holds many fields).
-template <bool RAW_SIGN, bool CLAMP>
-__device__ __forceinline__ uint32_t quantize_one(float v, float r, float sf, float cap, float um,
-                                                 uint32_t& sw) {
-  const float t = __fmul_rn(__fmul_rn(sf, fabsf(v)), r);
-  const float c = fma_rn(um, kTwo125, t);                    // t + m * 2^-24, one rounding
-  float fl = __fadd_rd(c, kTwo23);                           // 2^23 + floor(c)
-  if (CLAMP) fl = fminf(fl, cap);                            // 2^23 + min(floor(c), s)
-  if (RAW_SIGN) {
-    sw = __funnelshift_l(__float_as_uint(v), sw, 1);
-  } else {
-    const float lf = __fsub_rn(fl, kTwo23);                 // the level as a float, exact
-    const float sv = fma_rn(lf, v, 0.0f);                   // sign set iff level > 0 and v < 0
-    sw = __funnelshift_l(__float_as_uint(sv), sw, 1);
-  }
-  return __float_as_uint(fl);
-}
-
-// Rounds and packs the 16 coordinates of a thread, highest first: level fields by Horner
-// multiply-adds on the raw float bits (the constant exponent bits are removed once per word),
-// sign bits by funnel shifts; signs of zero levels are cleared at the end.
-template <int LB, bool CLAMP>
-__device__ __forceinline__ void quantize16(const float (&v)[16], const float (&um)[16], float r, float sf,
-                                           float cap, uint32_t (&lw)[4], uint32_t& sw) {
-  sw = 0;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) lw[j] = 0u;                 // LB = 8: 4 words; 4: 2; 2: 1; 1: half
-#pragma unroll
-  for (int c4 = 3; c4 >= 0; --c4) {
-#pragma unroll
-    for (int e = 3; e >= 0; --e) {
-      const uint32_t bits = quantize_one<LB != 8, CLAMP>(v[4 * c4 + e], r, sf, cap, um[4 * c4 + e], sw);
-      if (LB == 8) lw[c4] = lw[c4] * 256u + bits;
-      else if (LB == 4) lw[c4 >> 1] = lw[c4 >> 1] * 16u + bits;
-      else if (LB == 2) lw[0] = lw[0] * 4u + bits;
-      else lw[0] = lw[0] * 2u + bits;
-    }
-  }
-  // remove the exponent bits that rode along: sum over the fields of 0x4B000000 << (LB * e)
-  if (LB == 8) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) lw[j] -= kTwo23Bits * 0x01010101u;
-  } else if (LB == 4) {
-    lw[0] -= kTwo23Bits * 0x11111111u;
-    lw[1] -= kTwo23Bits * 0x11111111u;
-  } else if (LB == 2) {
-    lw[0] -= kTwo23Bits * 0x55555555u;
-  } else {
-    lw[0] = (lw[0] - kTwo23Bits * 0xFFFFu) & 0xFFFFu;
-  }
-}
-
-// Bit e of the result is set iff level field e of the 16 coordinates packed in lw is nonzero.
-template <int LB>
-__device__ __forceinline__ uint32_t nonzero_fields16(const uint32_t (&lw)[4]) {
-  if (LB == 1) return lw[0] & 0xFFFFu;
-  if (LB == 2) {
-    uint32_t y = (lw[0] | (lw[0] >> 1)) & 0x55555555u;
-    y = (y | (y >> 1)) & 0x33333333u;
-    y = (y | (y >> 2)) & 0x0F0F0F0Fu;
-    y = (y | (y >> 4)) & 0x00FF00FFu;
-    return (y | (y >> 8)) & 0xFFFFu;
-  }
-  uint32_t m = 0;                                           // LB == 4: two words of eight fields
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    uint32_t y = lw[h] | (lw[h] >> 1);
-    y = (y | (y >> 2)) & 0x11111111u;
-    y = (y | (y >> 3)) & 0x03030303u;
-    y = (y | (y >> 6)) & 0x000F000Fu;
-    m |= ((y | (y >> 12)) & 0xFFu) << (8 * h);
-  }
-  return m;
-}
-
-// Stores the sign and level words of the 16 coordinates of every lane of a warp; `c` is the index
-// of the warp's chunk of 512 coordinates (complete chunks only: no bounds to check).
-template <int LB>
-__device__ __forceinline__ void store_chunk(uint32_t* sign_out, uint32_t* level_out, uint32_t c, uint32_t lane,
-                                            uint32_t sw, const uint32_t (&lw)[4]) {
-  {
-    uint32_t w = (sw & 0xFFFFu) << (16 * (lane & 1));
-    w |= __shfl_xor_sync(0xffffffffu, w, 1);
-    if ((lane & 1) == 0) sign_out[c * 16u + (lane >> 1)] = w;
-  }
-  if (LB == 8) {
-    *reinterpret_cast<uint4*>(level_out + ((size_t)c * 128u + lane * 4u)) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
-  } else if (LB == 4) {
-    *reinterpret_cast<uint2*>(level_out + ((size_t)c * 64u + lane * 2u)) = make_uint2(lw[0], lw[1]);
-  } else if (LB == 2) {
-    level_out[(size_t)c * 32u + lane] = lw[0];
-  } else {
-    uint32_t w = lw[0] << (16 * (lane & 1));
-    w |= __shfl_xor_sync(0xffffffffu, w, 1);
-    if ((lane & 1) == 0) level_out[c * 16u + (lane >> 1)] = w;
-  }
-}
-
 constexpr int kStages = 3;
 
 struct __align__(16) TileSmem {
@@ -304,10 +110,6 @@ struct FastParams {
   BucketMap map;            // per-tensor policy: where each bucket lives in g (quads set), or no map
   QuantizeParams tail;      // parameters of the extra CTA (used when gridDim.x > main_ctas)
 };
-
-template <int LB, int NORM, bool MAPPED>
-__device__ __forceinline__ void quantize_generic_tile(const QuantizeParams& p, uint32_t block, uint32_t nblocks,
-                                                      float* tile, float* part, float* s_rcp);
 
 // Producer side of one stage, called by all lanes of warp 0: start the bulk copies of tile t.
 // Ordinary case: lane 0 starts one copy of the whole tile. With a bucket map, lane j looks up
@@ -521,194 +323,6 @@ quantize_pow2_kernel(const __grid_constant__ FastParams p) {
       const uint64_t t = (uint64_t)blockIdx.x + (uint64_t)itj * grid;
       if (t < p.full_tiles) mbar_wait_bounded(&sm.full[itj % kStages], (itj / kStages) & 1, kDrainPolls);
     }
-  }
-}
-
-// ---------------------------------------------------------------------------------------------
-// Generic kernel: any bucket size that is a multiple of 32. One CTA per tile of whole buckets.
-// ---------------------------------------------------------------------------------------------
-constexpr int kGroupsPerThread = kTile / 8 / kThreads;  // 2
-constexpr int kMaxBucketsPerTile = kTile / 32;          // 128
-
-// One tile of the generic path. `block` / `nblocks` play the role of blockIdx / gridDim so that the
-// main kernel can run the ragged last tile in one extra CTA of its own grid.
-template <int LB, int NORM, bool MAPPED>
-__device__ __forceinline__ void quantize_generic_tile(const QuantizeParams& p, uint32_t block, uint32_t nblocks,
-                                                      float* tile, float* part, float* s_rcp) {
-  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint64_t t0 = p.coord_base + (uint64_t)block * p.tile_coords;   // first coordinate
-  if (block == 0 && tid == 0 && p.info) {
-    p.info[0] = 8 * p.total_bytes; p.info[1] = 0; p.info[2] = p.total_bytes; p.info[3] = 0;
-  }
-  if (block == 0 && tid == 0 && p.clear_word) *p.clear_word = 0u;
-  const uint64_t left = p.n - t0;
-  const uint32_t valid = left < p.tile_coords ? (uint32_t)left : p.tile_coords;
-  if (valid == 0) {                            // nothing left to encode: only the padding
-    if (tid < 4) {
-      if (p.B + tid < ((p.B + 3) & ~3ull)) p.A_out[p.B + tid] = 0.f;
-      if (p.sign_words + tid < ((p.sign_words + 3) & ~3ull)) p.sign_out[p.sign_words + tid] = 0u;
-      if (p.level_words + tid < ((p.level_words + 3) & ~3ull)) p.level_out[p.level_words + tid] = 0u;
-    }
-    return;
-  }
-
-  for (uint32_t i = tid * 4; i < p.tile_coords; i += kThreads * 4) {
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (MAPPED) {
-      // per-tensor policy: four coordinates of one bucket (d is a multiple of 32) from the
-      // bucket's own place; what lies behind the bucket's length is zero padding
-      if (i < valid) {
-        const uint32_t bi = i / p.d, c = i - bi * p.d;
-        const uint64_t b = t0 / p.d + bi;
-        const uint32_t L = __ldg(p.map.len + b);
-        const float* src = p.g + __ldg(p.map.src + b) + c;
-        if (c + 4 <= L && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
-          v = __ldcs(reinterpret_cast<const float4*>(src));
-        } else {
-          float t[4] = {0.f, 0.f, 0.f, 0.f};
-          for (uint32_t j = 0; j < 4 && c + j < L; ++j) t[j] = src[j];
-          v = make_float4(t[0], t[1], t[2], t[3]);
-        }
-      }
-    } else if (i + 4 <= valid) {
-      v = __ldcs(reinterpret_cast<const float4*>(p.g + t0 + i));
-    } else if (i < valid) {
-      float t[4] = {0.f, 0.f, 0.f, 0.f};
-      for (uint32_t j = 0; i + j < valid; ++j) t[j] = p.g[t0 + i + j];
-      v = make_float4(t[0], t[1], t[2], t[3]);
-    }
-    *reinterpret_cast<float4*>(tile + i) = v;
-  }
-  __syncthreads();
-
-  float v[kGroupsPerThread][8];
-  const uint32_t groups = p.tile_coords >> 3;
-#pragma unroll
-  for (int j = 0; j < kGroupsPerThread; ++j) {
-    const uint32_t grp = tid + j * kThreads;
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-    if (grp < groups) {
-      a = *reinterpret_cast<const float4*>(tile + grp * 8);
-      b = *reinterpret_cast<const float4*>(tile + grp * 8 + 4);
-    }
-    v[j][0] = a.x; v[j][1] = a.y; v[j][2] = a.z; v[j][3] = a.w;
-    v[j][4] = b.x; v[j][5] = b.y; v[j][6] = b.z; v[j][7] = b.w;
-    float acc = 0.f;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      if (NORM == QSGD_NORM_L2) acc = fmaf(v[j][e], v[j][e], acc);
-      else acc = fmaxf(acc, fabsf(v[j][e]));
-    }
-    if (grp < groups) part[grp] = acc;
-  }
-  __syncthreads();
-
-  const uint32_t nb = p.tile_coords / p.d;     // buckets in a full tile
-  const uint32_t gpb = p.d >> 3;               // groups per bucket
-  const uint64_t b0 = t0 / p.d;                // first bucket of the tile
-  for (uint32_t b = warp; b < nb; b += kThreads / 32) {
-    float A;
-    if (NORM == QSGD_NORM_L2) {
-      // fp32 partials of 8 squares each; redo in fp64 from the tile when they may have lost bits:
-      // a nonzero partial outside [8e-28, 1e30], or a bucket total below that range (a zero total
-      // too: squares below 1.4e-45 vanish in fp32 while the values do not in fp64)
-      double acc = 0.0;
-      bool shaky = false;
-      for (uint32_t j = lane; j < gpb; j += 32) {
-        const float q = part[b * gpb + j];
-        shaky |= !(q >= 8.0e-28f && q <= 1.0e30f) && q != 0.f;
-        acc += (double)q;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (__any_sync(0xffffffffu, shaky) || !(acc >= 8.0e-28)) {
-        acc = 0.0;
-        for (uint32_t i = lane; i < p.d; i += 32) {
-          const double x = (double)tile[b * p.d + i];
-          acc = fma(x, x, acc);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      }
-      A = __double2float_rn(__dsqrt_rn(acc));
-    } else {
-      float acc = 0.f;
-      for (uint32_t j = lane; j < gpb; j += 32) acc = fmaxf(acc, part[b * gpb + j]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc = fmaxf(acc, __shfl_xor_sync(0xffffffffu, acc, o));
-      A = acc;
-    }
-    if (!(A >= FLT_MIN)) A = 0.f;
-    if (lane == 0) {
-      s_rcp[b] = A > 0.f ? __frcp_rn(A) : 0.f;
-      if (b0 + b < p.B) p.A_out[b0 + b] = A;
-    }
-  }
-  __syncthreads();
-
-  const float sf = (float)p.s;
-#pragma unroll
-  for (int j = 0; j < kGroupsPerThread; ++j) {
-    const uint32_t grp = tid + j * kThreads;
-    const uint32_t bl = (grp * 8) / p.d;
-    const float r = (grp < groups) ? s_rcp[bl] : 0.f;
-    const uint64_t i0 = t0 + (uint64_t)grp * 8;
-    const uint64_t q = i0 >> 2;
-    const uint4 ra = philox4x32_10((uint32_t)q, (uint32_t)(q >> 32), p.step, p.worker, p.k0, p.k1);
-    const uint4 rb = philox4x32_10((uint32_t)(q + 1), (uint32_t)((q + 1) >> 32), p.step, p.worker,
-                                   p.k0, p.k1);
-    const uint32_t rnd[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
-    uint32_t lv[8];
-    uint32_t sb = 0;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      lv[e] = quantize_level(v[j][e], r, sf, p.s, rnd[e]);
-      sb |= (uint32_t)(lv[e] != 0 && v[j][e] < 0.f) << e;
-    }
-    uint32_t sw = sb << (8 * (lane & 3));
-    sw |= __shfl_xor_sync(0xffffffffu, sw, 1);
-    sw |= __shfl_xor_sync(0xffffffffu, sw, 2);
-    const uint64_t sidx = (t0 >> 5) + (grp >> 2);
-    if ((lane & 3) == 0 && grp < groups && sidx < p.sign_words) p.sign_out[sidx] = sw;
-
-    if (LB == 8) {
-      const uint32_t w0 = lv[0] | lv[1] << 8 | lv[2] << 16 | lv[3] << 24;
-      const uint32_t w1 = lv[4] | lv[5] << 8 | lv[6] << 16 | lv[7] << 24;
-      const uint64_t widx = (t0 >> 2) + (uint64_t)grp * 2;
-      if (grp < groups) {
-        if (widx + 1 < p.level_words) *reinterpret_cast<uint2*>(p.level_out + widx) = make_uint2(w0, w1);
-        else if (widx < p.level_words) p.level_out[widx] = w0;
-      }
-    } else if (LB == 4) {
-      uint32_t w = 0;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) w |= lv[e] << (4 * e);
-      const uint64_t widx = (t0 >> 3) + grp;
-      if (grp < groups && widx < p.level_words) p.level_out[widx] = w;
-    } else if (LB == 2) {
-      uint32_t w = 0;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) w |= lv[e] << (2 * e);
-      w <<= 16 * (lane & 1);
-      w |= __shfl_xor_sync(0xffffffffu, w, 1);
-      const uint64_t widx = (t0 >> 4) + (grp >> 1);
-      if ((lane & 1) == 0 && grp < groups && widx < p.level_words) p.level_out[widx] = w;
-    } else {
-      uint32_t w = 0;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) w |= lv[e] << e;
-      w <<= 8 * (lane & 3);
-      w |= __shfl_xor_sync(0xffffffffu, w, 1);
-      w |= __shfl_xor_sync(0xffffffffu, w, 2);
-      const uint64_t widx = (t0 >> 5) + (grp >> 2);
-      if ((lane & 3) == 0 && grp < groups && widx < p.level_words) p.level_out[widx] = w;
-    }
-  }
-
-  if (block == nblocks - 1 && tid < 4) {
-    if (p.B + tid < ((p.B + 3) & ~3ull)) p.A_out[p.B + tid] = 0.f;
-    if (p.sign_words + tid < ((p.sign_words + 3) & ~3ull)) p.sign_out[p.sign_words + tid] = 0u;
-    if (p.level_words + tid < ((p.level_words + 3) & ~3ull)) p.level_out[p.level_words + tid] = 0u;
   }
 }
 
@@ -1108,29 +722,12 @@ quantize_group_kernel(const __grid_constant__ FastParams p) {
 }
 
 template <int LB, int NORM, bool MAPPED>
-__global__ void __launch_bounds__(kThreads) quantize_generic_kernel(const QuantizeParams p) {
+__global__ void __launch_bounds__(kThreads, 6) quantize_generic_kernel(const QuantizeParams p) {
   __shared__ __align__(16) float tile[kTile];
   __shared__ float part[kTile / 8];
   __shared__ float s_rcp[kMaxBucketsPerTile];
   chain_wait();
   quantize_generic_tile<LB, NORM, MAPPED>(p, blockIdx.x, gridDim.x, tile, part, s_rcp);
-}
-
-PhiloxConsts make_philox_consts(uint64_t seed, uint32_t step, uint32_t worker) {
-  uint32_t k0[10], k1[10];
-  k0[0] = (uint32_t)seed; k1[0] = (uint32_t)(seed >> 32);
-  for (int r = 1; r < 10; ++r) { k0[r] = k0[r - 1] + 0x9E3779B9u; k1[r] = k1[r - 1] + 0xBB67AE85u; }
-  const uint64_t ps = (uint64_t)kM1 * step;
-  const uint32_t x0 = (uint32_t)(ps >> 32) ^ k0[0], l1 = (uint32_t)ps;
-  const uint64_t px = (uint64_t)kM0 * x0;
-  PhiloxConsts pc;
-  pc.y0 = worker ^ k1[0];
-  pc.z0 = l1 ^ k0[1];
-  pc.z1 = (uint32_t)(px >> 32) ^ k1[1];
-  pc.z2 = (uint32_t)px ^ k1[2];
-  pc.k0_2 = k0[2];
-  for (int r = 0; r < 7; ++r) { pc.k[r][0] = k0[r + 3]; pc.k[r][1] = k1[r + 3]; }
-  return pc;
 }
 
 std::atomic<uint32_t> g_poll_limit{kDrainPolls};
@@ -1182,7 +779,7 @@ int launch_cross(FastParams& fp, bool with_tail, cudaStream_t stream) {
 }
 
 template <int LB, int NORM>
-int launch_one(QuantizeParams& p, uint64_t seed, cudaStream_t stream) {
+int launch_one(QuantizeParams& p, cudaStream_t stream) {
   const uint32_t d = p.d;
   const bool pow2 = (d & (d - 1)) == 0;
   uint32_t full_tiles = 0;
@@ -1196,7 +793,7 @@ int launch_one(QuantizeParams& p, uint64_t seed, cudaStream_t stream) {
     while ((1u << fp.log2d) < d) ++fp.log2d;
     fp.A_out = p.A_out; fp.sign_out = p.sign_out; fp.level_out = p.level_out; fp.status = p.status;
     fp.info = p.info; fp.total_bytes = p.total_bytes; fp.clear_word = p.clear_word;
-    fp.pc = make_philox_consts(seed, p.step, p.worker);
+    fp.pc = p.pc;
     fp.map = p.map;
     // the ragged tail (fewer than 4096 coordinates) and the zero padding of the three regions go
     // to one extra CTA of the same launch; nothing to do when n is a multiple of the tile and
@@ -1233,9 +830,9 @@ int launch_one(QuantizeParams& p, uint64_t seed, cudaStream_t stream) {
 }
 
 template <int LB>
-int launch_lb(QuantizeParams& p, int norm_kind, uint64_t seed, cudaStream_t stream) {
-  return norm_kind == QSGD_NORM_L2 ? launch_one<LB, QSGD_NORM_L2>(p, seed, stream)
-                                   : launch_one<LB, QSGD_NORM_MAX>(p, seed, stream);
+int launch_lb(QuantizeParams& p, int norm_kind, cudaStream_t stream) {
+  return norm_kind == QSGD_NORM_L2 ? launch_one<LB, QSGD_NORM_L2>(p, stream)
+                                   : launch_one<LB, QSGD_NORM_MAX>(p, stream);
 }
 
 }  // namespace
@@ -1249,7 +846,7 @@ int launch_quantize_fixed(const float* g, uint64_t n, uint32_t d, uint32_t s, in
   p.g = g; p.n = n; p.d = d; p.s = s; p.map = map;
   p.tile_coords = (kTile / d) * d;
   p.coord_base = 0;
-  p.k0 = (uint32_t)seed; p.k1 = (uint32_t)(seed >> 32); p.step = step; p.worker = worker;
+  p.pc = make_philox_consts(seed, step, worker);
   p.A_out = reinterpret_cast<float*>(out);
   p.sign_out = reinterpret_cast<uint32_t*>(out + L.off_sign);
   p.level_out = reinterpret_cast<uint32_t*>(out + L.off_level);
@@ -1260,10 +857,10 @@ int launch_quantize_fixed(const float* g, uint64_t n, uint32_t d, uint32_t s, in
   p.total_bytes = L.total;
   p.clear_word = clear_word;
   switch (L.lb) {
-    case 1: return launch_lb<1>(p, norm_kind, seed, stream);
-    case 2: return launch_lb<2>(p, norm_kind, seed, stream);
-    case 4: return launch_lb<4>(p, norm_kind, seed, stream);
-    default: return launch_lb<8>(p, norm_kind, seed, stream);
+    case 1: return launch_lb<1>(p, norm_kind, stream);
+    case 2: return launch_lb<2>(p, norm_kind, stream);
+    case 4: return launch_lb<4>(p, norm_kind, stream);
+    default: return launch_lb<8>(p, norm_kind, stream);
   }
 }
 
