@@ -131,9 +131,10 @@ def test_lines_between_decoders(n, d, s, K):
 
 
 @pytest.mark.parametrize("n,d,s,code", [
-    (1, 32, 15, ELIAS), (4095, 32, 3, ELIAS), (4096, 64, 1, ELIAS), (4097, 512, 15, ELIAS), (42 * 96 + 1, 96, 255, ELIAS),
-    (2 * 4032, 2016, 15, DENSE), (2 ** 21, 512, 15, ELIAS), (2 ** 21 + 1, 512, 15, ELIAS),
-    (2 ** 21 + 37, 480, 7, ELIAS), (2 ** 22 + 5, 4096, 64, DENSE), (2 ** 22 + 5, 128, 255, ELIAS),
+    (1, 32, 15, ELIAS), (4095, 32, 3, ELIAS), (4096, 64, 1, ELIAS), (4097, 512, 15, ELIAS), (42 * 96, 96, 255, ELIAS), (42 * 96 + 1, 96, 255, ELIAS),
+    (2 * 4032, 2016, 15, DENSE), (3 * 4096, 4096, 64, DENSE), (4096000, 512, 15, ELIAS), (4096001, 512, 15, ELIAS), (1000 * 4032, 96, 7, ELIAS),
+    (1000 * 4032 + 1, 96, 7, ELIAS), (2 ** 22 + 5, 4096, 64, DENSE), (2 ** 22 + 5, 128, 255, ELIAS), (2 ** 22 + 5, 32, 15, ELIAS),
+    (2 ** 22 + 37, 480, 7, ELIAS), (2 ** 22 + 37, 2080, 3, DENSE), (7 * 2 ** 20 + 3, 160, 255, ELIAS),
 ])
 def test_tiles(n, d, s, code):
     encode_parity(I.gaussian_mixture(n, seed=3), d, s, MAX, code, 7, 1, 2)
