@@ -12,12 +12,12 @@ __device__ __forceinline__ float shfl_f(float v, uint32_t src) {
 
 // Adds peer k's 16 values to acc[]. SINGLE: the whole chunk lies in one bucket and `lut` is
 // already scaled by A; otherwise `lut` holds +-(level / s) and A is this lane's bucket scale.
-template <int LB, bool SINGLE, int WORDS = 2>
+template <int LB, bool SINGLE>
 __device__ __forceinline__ void add_peer_lut(float (&acc)[16], const uint32_t (&w)[4], uint32_t sb,
                                              float lut, float A) {
   if (LB == 4) {
 #pragma unroll
-    for (int h = 0; h < WORDS; ++h) {
+    for (int h = 0; h < 2; ++h) {
       const uint32_t word = w[h], s8 = sb >> (8 * h);
       const uint32_t ev = word & 0x0F0F0F0Fu, od = (word >> 4) & 0x0F0F0F0Fu;
       const uint32_t ie = (((s8 & 0x55u) * 0x00410410u) & 0x10101010u) | ev;   // coords 0,2,4,6
@@ -71,71 +71,21 @@ __device__ __forceinline__ void add_peer_lut(float (&acc)[16], const uint32_t (&
   }
 }
 
-// Reconstruction by arithmetic: A * (level / s), the quotient rounded to nearest as the definition has it, without a
-// table. With 1 / s = hi + lo in two floats, RN(level * hi + RN(level * lo)) is RN(level / s) for every s <= 255 and
-// level <= s (checked exhaustively in rational arithmetic). The level comes as the float 2^23 + level, made by one byte
-// permute. All steps work on pairs (f32x2).
-struct LevelQuotient {
-  unsigned long long hi, lo, klo, m23, m0;      // 1 / s; its rest; -2^23 * rest; -2^23; -0
-};
-
-__device__ __forceinline__ unsigned long long pair2(float a, float b) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-  unsigned long long r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-
-// `minus_zero` is -0 that the compiler cannot see (a kernel parameter): the product with A is an fma with it, because
-// ptxas contracts a mul.rn.f32x2 in front of an add.rn.f32x2.
-__device__ __forceinline__ LevelQuotient level_quotient(uint32_t s, float minus_zero) {
-  const float hi = __fdiv_rn(1.f, (float)s);
-  const float lo = __double2float_rn(1.0 / (double)s - (double)hi);
-  LevelQuotient q;
-  q.hi = pair2(hi, hi); q.lo = pair2(lo, lo);
-  q.klo = pair2(-8388608.f * lo, -8388608.f * lo); q.m23 = pair2(-8388608.f, -8388608.f);
-  q.m0 = pair2(minus_zero, minus_zero);
-  return q;
-}
-
-// acc += +-A * (level / s) for two coordinates: levels in bytes j0 of w0 and j1 of w1, signs in bits e and e + 1 of sb.
-__device__ __forceinline__ void add_level_pair(float& acc0, float& acc1, uint32_t w0, uint32_t j0, uint32_t w1, uint32_t j1, uint32_t sb,
-                                               uint32_t e, float A, const LevelQuotient& lq) {
-  const float f0 = __uint_as_float(__byte_perm(w0, 0x4B000000u, 0x7440u | j0));
-  const float f1 = __uint_as_float(__byte_perm(w1, 0x4B000000u, 0x7440u | j1));
-  const unsigned long long f = pair2(f0, f1);
-  const unsigned long long q = fma2(add2(f, lq.m23), lq.hi, fma2(f, lq.lo, lq.klo));
-  const float a0 = __uint_as_float(__float_as_uint(A) ^ ((sb << (31u - e)) & 0x80000000u));
-  const float a1 = __uint_as_float(__float_as_uint(A) ^ ((sb << (30u - e)) & 0x80000000u));
-  const unsigned long long r = add2(pair2(acc0, acc1), fma2(pair2(a0, a1), q, lq.m0));
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(acc0), "=f"(acc1) : "l"(r));
-}
-
-// 16 one-byte levels in w.
-__device__ __forceinline__ void add_peer_bytes(float (&acc)[16], const uint32_t (&w)[4], uint32_t sb, float A, const LevelQuotient& lq) {
+// LB = 8: table lookup of level / s in shared memory (entry l of lane t at word l * 32 + t).
+__device__ __forceinline__ void add_peer_tab(float (&acc)[16], const uint32_t (&w)[4], uint32_t sb,
+                                             const uint8_t* tab_lane, float A) {
 #pragma unroll
-  for (uint32_t h = 0; h < 4; ++h) {
-    add_level_pair(acc[4 * h], acc[4 * h + 1], w[h], 0, w[h], 1, sb, 4 * h, A, lq);
-    add_level_pair(acc[4 * h + 2], acc[4 * h + 3], w[h], 2, w[h], 3, sb, 4 * h + 2, A, lq);
+  for (int h = 0; h < 4; ++h) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t off = (j == 0 ? (w[h] << 7) : (w[h] >> (8 * j - 7))) & 0x7F80u;
+      const float xi = *reinterpret_cast<const float*>(tab_lane + off);
+      const uint32_t m = __float_as_uint(__fmul_rn(A, xi)) ^ ((sb << (31 - (4 * h + j))) & 0x80000000u);
+      acc[4 * h + j] = __fadd_rn(acc[4 * h + j], __uint_as_float(m));
+    }
   }
 }
 
-// Eight 4-bit levels of one word into acc[8 h ..].
-__device__ __forceinline__ void add_word_nibbles(float (&acc)[16], uint32_t word, uint32_t sb, int h, float A, const LevelQuotient& lq) {
-  const uint32_t ev = word & 0x0F0F0F0Fu, od = (word >> 4) & 0x0F0F0F0Fu;
-#pragma unroll
-  for (uint32_t j = 0; j < 4; ++j)
-    add_level_pair(acc[8 * h + 2 * j], acc[8 * h + 2 * j + 1], ev, j, od, j, sb, 8 * h + 2 * j, A, lq);
-}
 
 // Writes 16 accumulated values of one lane: acc as it is, or the SGD step x <- x - c * acc.
 template <bool FUSED>

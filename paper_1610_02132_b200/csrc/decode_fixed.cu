@@ -30,7 +30,6 @@ struct DecodeParams {
   uint32_t log2_chunks_per_bucket;   // valid when single_scale
   float* out;      // acc (overwritten) or x (updated in place)
   float c;         // eta / K (fused only)
-  float minus_zero;
   uint64_t chunks;
   BucketMap map;
 };
@@ -39,24 +38,21 @@ struct DecodeParams {
 // enough that the 16 running sums and the group's words stay in registers (measured per width).
 template <int LB> struct PeerUnroll { static constexpr int value = LB == 1 ? 3 : 4; };
 
-// How many of the two level words of a lane's 16 coordinates (4-bit levels) go by arithmetic.
-#ifndef QWA
-#define QWA 1
-#endif
-template <int LB> constexpr int kWordsByArithmetic = LB == 8 ? 4 : LB == 4 ? QWA : 0;
-
 template <int LB, bool FUSED, bool SINGLE>
 __global__ void __launch_bounds__(kThreads, 4) decode_fixed_kernel(const __grid_constant__ DecodeParams p) {
+  __shared__ __align__(16) float xi_tab[LB == 8 ? 256 * 32 : 32];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float sf = (float)p.s;
   float lut0 = 0.f;                                  // this lane's +-(level / s)
-  LevelQuotient lq;
-  if (kWordsByArithmetic<LB> > 0) lq = level_quotient(p.s, p.minus_zero);
-  if (LB != 8) {
+  if (LB == 8) {
+    for (uint32_t i = tid; i < 256 * 32; i += kThreads) xi_tab[i] = __fdiv_rn((float)(i >> 5), sf);
+    __syncthreads();
+  } else {
     const uint32_t level = lane & ((1u << LB) - 1u), neg = (lane >> LB) & 1u;
     const float q = __fdiv_rn((float)level, sf);
     lut0 = neg ? -q : q;
   }
+  const uint8_t* tab_lane = reinterpret_cast<const uint8_t*>(xi_tab) + 4 * lane;
   chain_wait();                                      // the messages come from the kernels ahead
 
   for (uint64_t ch = (uint64_t)blockIdx.x * kWarps + warp; ch < p.chunks; ch += (uint64_t)gridDim.x * kWarps) {
@@ -91,16 +87,9 @@ __global__ void __launch_bounds__(kThreads, 4) decode_fixed_kernel(const __grid_
           w[0] = __ldg(reinterpret_cast<const uint16_t*>(m + off_l));
         }
       }
-      if (LB == 8) {
-        add_peer_bytes(acc, w, sb, A, lq);
-      } else {
-        constexpr int kShuffled = 2 - kWordsByArithmetic<LB>;
-        if (SINGLE) add_peer_lut<LB, true, kShuffled>(acc, w, sb, __fmul_rn(__shfl_sync(0xffffffffu, A, 0), lut0), A);
-        else add_peer_lut<LB, false, kShuffled>(acc, w, sb, lut0, A);
-        if (LB == 4)
-#pragma unroll
-          for (int h = kShuffled; h < 2; ++h) add_word_nibbles(acc, w[h], sb, h, A, lq);
-      }
+      if (LB == 8) add_peer_tab(acc, w, sb, tab_lane, A);
+      else if (SINGLE) add_peer_lut<LB, true>(acc, w, sb, __fmul_rn(__shfl_sync(0xffffffffu, A, 0), lut0), A);
+      else add_peer_lut<LB, false>(acc, w, sb, lut0, A);
     }
 
     if (!live) continue;
@@ -164,7 +153,6 @@ int launch_decode_fixed(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
   p.off_sign = L.off_sign; p.off_level = L.off_level;
   p.K = K; p.n = n; p.d = d; p.s = s; p.out = acc_or_x; p.map = map;
   p.c = eta / (float)K;
-  p.minus_zero = -0.f;
   p.chunks = (n + kChunk - 1) / kChunk;
   // one scale per chunk when the bucket size is 512 * 2^j
   const bool single = d >= (uint32_t)kChunk && (d & (d - 1)) == 0;

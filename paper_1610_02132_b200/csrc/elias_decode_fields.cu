@@ -73,13 +73,16 @@ template <bool FUSED>
 __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_constant__ FieldParams p) {
   constexpr int LB = 8;
   extern __shared__ __align__(16) uint32_t fsm[];
+  __shared__ __align__(16) float xi_tab[256 * 32];
   __shared__ uint16_t elias_lut[1u << kLutBits];
   chain_wait();                                   // the messages come from the kernels ahead
   if (p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  const float sf = (float)p.s;
   fill_elias_lut(elias_lut);
+  for (uint32_t i = tid; i < 256 * 32; i += blockDim.x) xi_tab[i] = __fdiv_rn((float)(i >> 5), sf);
   __syncthreads();
-  const LevelQuotient lq = level_quotient(p.s, p.minus_zero);
+  const uint8_t* tab_lane = reinterpret_cast<const uint8_t*>(xi_tab) + 4 * lane;
 
   const uint32_t warp_words = p.G * p.bucket_words;
   uint32_t* mine = fsm + (size_t)warp * warp_words;
@@ -128,7 +131,7 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
           const uint4 t = *reinterpret_cast<const uint4*>(row + (c >> 2));
           w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
         }
-        add_peer_bytes(acc, w, sb, A, lq);
+        add_peer_tab(acc, w, sb, tab_lane, A);
       }
       if (live) {
         if (p.map.src) store_span16<FUSED>(out_span(p.out, p.map, b, c, p.d, p.n, 16u), acc, p.c);
@@ -156,7 +159,7 @@ int launch_fields(FieldParams& p, bool fused, cudaStream_t stream) {
   const size_t per_warp = (size_t)G * p.bucket_words * 4;
   // Warps per CTA: the count that leaves the most warps resident on an SM. The code table and the
   // level table are per CTA, the fields per warp; the parse is latency-bound, so warps are what counts.
-  const size_t per_cta = 8192 + 1024, budget = (size_t)max_smem - per_cta;
+  const size_t per_cta = 32768 + 8192 + 1024, budget = (size_t)max_smem - per_cta;
   const size_t per_sm = 227u << 10;
   int warps = 1, best = 0;
   for (int w = 1; w <= 10; ++w) {
