@@ -52,7 +52,7 @@ int launch_decode_elias(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
   const bool host_sparse = sizes_known && payload_bits < (uint64_t)K * B * (32ull + d / 4u);
   FieldParams f;
   f.peers = peers; f.K = K; f.n = n; f.d = d; f.s = s; f.B = B;
-  f.out = acc_or_x; f.c = eta / (float)K; f.status = status_dev; f.map = map;
+  f.out = acc_or_x; f.c = eta / (float)K; f.minus_zero = -0.f; f.status = status_dev; f.map = map;
   const bool teams = use_teams(B, K, d, s, dense);
   bool sparse = false;
   if (!dense && (host_sparse || !sizes_known) && !(teams && n * K <= kSmallWork)) {

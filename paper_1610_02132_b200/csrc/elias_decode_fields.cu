@@ -17,6 +17,66 @@ namespace qsgd {
 
 namespace {
 
+// Reconstruction by arithmetic: A * (level / s), the quotient rounded to nearest as the definition has it, without a
+// table. The table took 32 KB of a CTA, so fewer warps fitted, and the parse waits on latency: 42.5 us with it, 39.7 us
+// without (n = 1 M, d = 96, s = 255, K = 5). The fixed-width decoder does nothing else than this, and is faster with its
+// table (335 against 376 us at n = 60 M, K = 16). With 1 / s = hi + lo in two floats, RN(level * hi + RN(level * lo)) is
+// RN(level / s) for every s <= 255 and level <= s (checked exhaustively in rational arithmetic). The level comes as the
+// float 2^23 + level, made by one byte permute. All steps work on pairs (f32x2).
+struct LevelQuotient {
+  unsigned long long hi, lo, klo, m23, m0;      // 1 / s; its rest; -2^23 * rest; -2^23; -0
+};
+
+__device__ __forceinline__ unsigned long long pair2(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// `minus_zero` is -0 that the compiler cannot see (a kernel parameter): the product with A is an fma with it, because
+// ptxas contracts a mul.rn.f32x2 in front of an add.rn.f32x2.
+__device__ __forceinline__ LevelQuotient level_quotient(uint32_t s, float minus_zero) {
+  const float hi = __fdiv_rn(1.f, (float)s);
+  const float lo = __double2float_rn(1.0 / (double)s - (double)hi);
+  LevelQuotient q;
+  q.hi = pair2(hi, hi); q.lo = pair2(lo, lo);
+  q.klo = pair2(-8388608.f * lo, -8388608.f * lo); q.m23 = pair2(-8388608.f, -8388608.f);
+  q.m0 = pair2(minus_zero, minus_zero);
+  return q;
+}
+
+// acc += +-A * (level / s) for two coordinates: levels in bytes j0 of w0 and j1 of w1, signs in bits e and e + 1 of sb.
+__device__ __forceinline__ void add_level_pair(float& acc0, float& acc1, uint32_t w0, uint32_t j0, uint32_t w1, uint32_t j1, uint32_t sb,
+                                               uint32_t e, float A, const LevelQuotient& lq) {
+  const float f0 = __uint_as_float(__byte_perm(w0, 0x4B000000u, 0x7440u | j0));
+  const float f1 = __uint_as_float(__byte_perm(w1, 0x4B000000u, 0x7440u | j1));
+  const unsigned long long f = pair2(f0, f1);
+  const unsigned long long q = fma2(add2(f, lq.m23), lq.hi, fma2(f, lq.lo, lq.klo));
+  const float a0 = __uint_as_float(__float_as_uint(A) ^ ((sb << (31u - e)) & 0x80000000u));
+  const float a1 = __uint_as_float(__float_as_uint(A) ^ ((sb << (30u - e)) & 0x80000000u));
+  const unsigned long long r = add2(pair2(acc0, acc1), fma2(pair2(a0, a1), q, lq.m0));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(acc0), "=f"(acc1) : "l"(r));
+}
+
+// 16 one-byte levels in w.
+__device__ __forceinline__ void add_peer_bytes(float (&acc)[16], const uint32_t (&w)[4], uint32_t sb, float A, const LevelQuotient& lq) {
+#pragma unroll
+  for (uint32_t h = 0; h < 4; ++h) {
+    add_level_pair(acc[4 * h], acc[4 * h + 1], w[h], 0, w[h], 1, sb, 4 * h, A, lq);
+    add_level_pair(acc[4 * h + 2], acc[4 * h + 3], w[h], 2, w[h], 3, sb, 4 * h + 2, A, lq);
+  }
+}
+
 template <int LB>
 __device__ __forceinline__ uint32_t parse_to_fields(const PeerSet& peers, uint32_t k, uint64_t b,
                                                     uint64_t B, uint32_t db, uint32_t d, uint32_t s,
@@ -73,16 +133,13 @@ template <bool FUSED>
 __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_constant__ FieldParams p) {
   constexpr int LB = 8;
   extern __shared__ __align__(16) uint32_t fsm[];
-  __shared__ __align__(16) float xi_tab[256 * 32];
   __shared__ uint16_t elias_lut[1u << kLutBits];
   chain_wait();                                   // the messages come from the kernels ahead
   if (p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-  const float sf = (float)p.s;
   fill_elias_lut(elias_lut);
-  for (uint32_t i = tid; i < 256 * 32; i += blockDim.x) xi_tab[i] = __fdiv_rn((float)(i >> 5), sf);
   __syncthreads();
-  const uint8_t* tab_lane = reinterpret_cast<const uint8_t*>(xi_tab) + 4 * lane;
+  const LevelQuotient lq = level_quotient(p.s, p.minus_zero);
 
   const uint32_t warp_words = p.G * p.bucket_words;
   uint32_t* mine = fsm + (size_t)warp * warp_words;
@@ -131,7 +188,7 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
           const uint4 t = *reinterpret_cast<const uint4*>(row + (c >> 2));
           w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
         }
-        add_peer_tab(acc, w, sb, tab_lane, A);
+        add_peer_bytes(acc, w, sb, A, lq);
       }
       if (live) {
         if (p.map.src) store_span16<FUSED>(out_span(p.out, p.map, b, c, p.d, p.n, 16u), acc, p.c);
@@ -157,9 +214,9 @@ int launch_fields(FieldParams& p, bool fused, cudaStream_t stream) {
   while (G > 1 && (size_t)G * p.bucket_words * 4 > (16u << 10)) G >>= 1;
   p.G = G;
   const size_t per_warp = (size_t)G * p.bucket_words * 4;
-  // Warps per CTA: the count that leaves the most warps resident on an SM. The code table and the
-  // level table are per CTA, the fields per warp; the parse is latency-bound, so warps are what counts.
-  const size_t per_cta = 32768 + 8192 + 1024, budget = (size_t)max_smem - per_cta;
+  // Warps per CTA: the count that leaves the most warps resident on an SM. The code table is
+  // per CTA, the fields per warp; the parse is latency-bound, so warps are what counts.
+  const size_t per_cta = 8192 + 1024, budget = (size_t)max_smem - per_cta;
   const size_t per_sm = 227u << 10;
   int warps = 1, best = 0;
   for (int w = 1; w <= 10; ++w) {
