@@ -72,20 +72,47 @@ __device__ __forceinline__ uint32_t place(uint32_t pos) {       // in bytes
   return pos ^ ((pos >> 4) & 0x78u);
 }
 
+template <bool DENSE>
 struct Tables {
   uint2 code[kCodeEntries];
   // Code_s, s <= 15: what follows a gap (tail_entry). Code'_s: what the next 10 bits hold, up to three
   // symbols of levels <= 7: their codes in bytes 0, 1 and 2 (kWide: level | negative << 7), their length in
-  // byte 3, bits 0-3, their number in bits 4-5; 0 when they hold none
-  uint32_t symbol[1 << kDenseBits];
+  // byte 3, bits 0-3, their number in bits 6-7; 0 when they hold none
+  uint32_t symbol[DENSE ? 1u << kDenseBits : kTailEntries];
+  // Code'_s, the same for a reader that only counts: their length in bits 0-3, that of the first in bits 4-7, of the
+  // first two in bits 8-11 (15 where there is no symbol behind them), their number from bit 16 on
+  uint32_t count[DENSE ? 1u << kDenseBits : 1u];
 };
+
+// One symbol of the dense code by the general table: level and number of bits.
+__device__ __forceinline__ uint32_t dense_symbol(const uint2* code, uint32_t w, uint32_t* bits, uint32_t* closing) {
+  const uint32_t x = w << 1;
+  const uint2 c = code[x >> 25];
+  const uint32_t body = code_body(c);
+  *bits = body + 2u;
+  *closing = x << body;                           // top bit: has to be 0
+  return code_value(x, c) - 1u;
+}
+
+// Window::drop without a branch: the readers of the dense code are bound by the number of their instructions, and
+// lanes cross into a new word at different times.
+__device__ __forceinline__ void drop_even(Window& in, uint32_t bits, uint32_t end) {
+  in.bp += bits;
+  const bool cross = in.bp >= in.edge && in.bp < end;
+  in.w0 = cross ? in.w1 : in.w0;
+  in.w1 = cross ? in.w2 : in.w1;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p ld.u32 %0, [%2];\n\t}" : "+r"(in.w2) : "r"((uint32_t)cross), "l"(in.wp)
+               : "memory");
+  in.wp += cross ? 1 : 0;
+  in.edge += cross ? 32u : 0u;
+}
 
 // Reads symbols from bit `from` to the first one that starts at or behind bit `until` (both counted from
 // bit 0 of words[0]; `end`: first bit behind the string). Returns where that is; *sum: the gaps or, in the
 // dense code, the symbols passed. What is no symbol (the reader is out of step, or the string is
 // malformed) still moves it on.
 template <bool DENSE, int WIDTH>
-__device__ __forceinline__ uint32_t walk(const Tables& tab, const uint32_t* words, uint32_t from, uint32_t until,
+__device__ __forceinline__ uint32_t walk(const Tables<DENSE>& tab, const uint32_t* words, uint32_t from, uint32_t until,
                                          uint32_t end, uint32_t* sum) {
   *sum = 0;
   if (from >= until) return from;
@@ -94,18 +121,28 @@ __device__ __forceinline__ uint32_t walk(const Tables& tab, const uint32_t* word
   const uint32_t origin = from & ~31u;
   const uint32_t stop = until - origin, last = end - origin;
   uint32_t n = 0;
-  while (in.bp < stop) {
-    const uint32_t w = in.peek();
-    if (DENSE) {
-      const uint32_t e = tab.symbol[w >> (32 - kDenseBits)];
-      if (e && in.bp + kDenseBits <= stop) {
-        in.drop((e >> 24) & 15u, last);
-        n += e >> 28;
-      } else {
-        in.drop(code_body(tab.code[(w << 1) >> 25]) + 2u, last);
-        ++n;
+  if constexpr (DENSE) {
+    auto step = [&](uint32_t room) {              // room: bits up to `stop`, where that is less than an entry's
+      const uint32_t w = in.peek();
+      const uint32_t e = tab.count[w >> (32 - kDenseBits)];
+      uint32_t bits = e & 15u, held = e >> 16;
+      if (e == 0u) {
+        bits = code_body(tab.code[(w << 1) >> 25]) + 2u;
+        held = 1u;
+      } else if (room) {                          // only the symbols that start in front of it
+        const uint32_t one = (e >> 4) & 15u, two = (e >> 8) & 15u;
+        held = one >= room ? 1u : two >= room ? 2u : held;
+        bits = one >= room ? one : two >= room ? min(two, bits) : bits;
+        held = min(held, e >> 16);
       }
-    } else {
+      drop_even(in, bits, last);
+      n += held;
+    };
+    while (in.bp + kDenseBits <= stop) step(0u);
+    while (in.bp < stop) step(stop - in.bp);
+  } else {
+    while (in.bp < stop) {
+      const uint32_t w = in.peek();
       const uint2 e = tab.code[w >> 25];
       const uint32_t body = code_body(e);
       n += code_value(w, e);
@@ -123,15 +160,62 @@ __device__ __forceinline__ uint32_t walk(const Tables& tab, const uint32_t* word
   return origin + in.bp;
 }
 
+// The last reading of the dense code where a code is a byte. Codes are gathered in a word, and stored a word at a time.
+// A word that two lanes have codes for is the one's that its first code belongs to: that lane reads on until it has the
+// word, the others leave their part of it out. Which of the codes behind its part a lane has passed does not matter: the
+// lane that they belong to checks them.
+template <int WIDTH>
+__device__ __forceinline__ uint32_t emit_dense(const Tables<true>& tab, const uint32_t* words, uint32_t from, uint32_t until,
+                                               uint32_t end, uint32_t at, uint32_t db, uint32_t s, uint8_t* row) {
+  if (from >= until) return 0u;
+  Window in;
+  in.open(words, from);
+  const uint32_t origin = from & ~31u;
+  const uint32_t stop = until - origin, last = end - origin;
+  const uint32_t row_addr = (uint32_t)__cvta_generic_to_shared(row);
+  const uint32_t mine = (at + 3u) & ~3u, full = 8u * db;
+  uint32_t bad = 0, codes = 0;
+  uint32_t q = 8u * at;                           // eight times the next position
+  // the word under way is mine, has codes, and there are more
+  auto open_word = [&]() { return (q & 31u) != 0u && (q >> 3) > mine && q < full && in.bp < last; };
+  while (in.bp < stop || open_word()) {
+    const uint32_t w = in.peek();
+    const uint32_t e = tab.symbol[w >> (32 - kDenseBits)];
+    uint32_t bits = (e >> 24) & 15u, held = e >> 30, more = e & 0x00FFFFFFu;
+    if (e == 0u || q + 8u * held > full) {
+      uint32_t closing;
+      const uint32_t level = dense_symbol(tab.code, w, &bits, &closing);
+      bad |= closing;
+      if (level > s) return QSGD_DEV_LEVEL;
+      if (q >= full) return QSGD_DEV_OVERRUN;     // more symbols than coordinates
+      more = level | (level ? (w >> 31) << CodeOf<WIDTH>::kSignShift : 0u);
+      held = 1u;
+    }
+    drop_even(in, bits, last);
+    codes |= __funnelshift_l(0u, more, q);        // (the shift takes q mod 32)
+    const uint32_t over = __funnelshift_l(more, 0u, q);
+    const uint32_t next = q + 8u * held, pos = (q >> 3) & ~3u;
+    const bool whole = ((q ^ next) & 32u) != 0u;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.u32 [%1], %2;\n\t}" ::"r"((uint32_t)(whole && pos >= mine)),
+                 "r"(row_addr + place<WIDTH>(pos)), "r"(codes)
+                 : "memory");
+    codes = whole ? over : codes;
+    q = next;
+  }
+  if ((q & 31u) != 0u && (q >> 3) > mine) *reinterpret_cast<uint32_t*>(row + place<WIDTH>((q >> 3) & ~3u)) = codes;
+  return bad >> 31 ? QSGD_DEV_OVERRUN : 0u;
+}
+
 // The last reading: the same part, every check, one code per coordinate into the row. `at`: position of
 // the last nonzero in front of the part (Code_s) or the part's first position (Code'_s).
 template <bool DENSE, int WIDTH>
-__device__ __forceinline__ uint32_t emit(const Tables& tab, const uint32_t* words, uint32_t from, uint32_t until,
+__device__ __forceinline__ uint32_t emit(const Tables<DENSE>& tab, const uint32_t* words, uint32_t from, uint32_t until,
                                          uint32_t end, uint32_t at, uint32_t db, uint32_t s, uint8_t* row) {
   using Code = typename CodeOf<WIDTH>::type;
   auto put = [&](uint32_t pos, uint32_t code) { *reinterpret_cast<Code*>(row + place<WIDTH>(pos)) = (Code)code; };
   constexpr uint32_t kSignShift = CodeOf<WIDTH>::kSignShift;
   if (from >= until) return 0u;
+  if constexpr (DENSE && WIDTH != kWide) return emit_dense<WIDTH>(tab, words, from, until, end, at, db, s, row);
   Window in;
   in.open(words, from);
   const uint32_t origin = from & ~31u;
@@ -139,31 +223,24 @@ __device__ __forceinline__ uint32_t emit(const Tables& tab, const uint32_t* word
   uint32_t bad = 0;
   while (in.bp < stop) {
     const uint32_t w = in.peek();
-    if (DENSE) {
-      const uint32_t e = tab.symbol[w >> (32 - kDenseBits)], held = e >> 28;
+    if (DENSE) {                                  // (codes of two bytes)
+      const uint32_t e = tab.symbol[w >> (32 - kDenseBits)], held = e >> 30;
       if (e && in.bp + kDenseBits <= stop && at + held <= db) {
-        if (WIDTH == kWide) {
 #pragma unroll
-          for (uint32_t j = 0; j < 3; ++j)
-            if (j < held) put(at + j, ((e >> (8u * j)) & 7u) | ((e >> (8u * j)) & 0x80u) << 1);
-        } else {
-          put(at, e);
-          if (held > 1u) put(at + 1u, e >> 8);
-          if (held > 2u) put(at + 2u, e >> 16);
-        }
+        for (uint32_t j = 0; j < 3; ++j)
+          if (j < held) put(at + j, ((e >> (8u * j)) & 7u) | ((e >> (8u * j)) & 0x80u) << 1);
         in.drop((e >> 24) & 15u, last);
         at += held;
         continue;
       }
-      const uint32_t x = w << 1;
-      const uint2 c = tab.code[x >> 25];
-      const uint32_t level = code_value(x, c) - 1u, body = code_body(c);
-      bad |= x << body;                           // the closing bit
+      uint32_t bits, closing;
+      const uint32_t level = dense_symbol(tab.code, w, &bits, &closing);
+      bad |= closing;
       if (level > s) return QSGD_DEV_LEVEL;
       if (at >= db) return QSGD_DEV_OVERRUN;      // more symbols than coordinates
       put(at, level | (level ? (w >> 31) << kSignShift : 0u));
       ++at;
-      in.drop(body + 2u, last);
+      in.drop(bits, last);
     } else {
       const uint2 e = tab.code[w >> 25];
       const uint32_t body = code_body(e);
@@ -200,7 +277,7 @@ struct Marks {
 };
 
 template <bool DENSE, int WIDTH>
-__device__ __forceinline__ void read_part(const Tables& tab, const uint32_t* words, uint32_t start, uint32_t lo,
+__device__ __forceinline__ void read_part(const Tables<DENSE>& tab, const uint32_t* words, uint32_t start, uint32_t lo,
                                           uint32_t hi, uint32_t end, bool again, Marks& m) {
   const uint32_t piece = max((hi - lo + kMarks - 1u) / kMarks, kLeastPiece);
   uint32_t pos = start, sum = 0;
@@ -226,14 +303,14 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
   using Code = typename CodeOf<WIDTH>::type;
   constexpr uint32_t kLevels = 1u << CodeOf<WIDTH>::kSignShift;
   extern __shared__ __align__(16) uint8_t tsm[];
-  __shared__ Tables tab;
+  __shared__ Tables<DENSE> tab;
   __shared__ float xi[2 * kLevels];                     // +-(level / s) by code
   const uint32_t tid = threadIdx.x, lane = tid & 31;
   const float sf = (float)p.s;
   for (uint32_t i = tid; i < kCodeEntries; i += kThreads) tab.code[i] = code_entry(i);
   if (DENSE) {
     for (uint32_t i = tid; i < (1u << kDenseBits); i += kThreads) {
-      uint32_t w = i << (32 - kDenseBits), used = 0, held = 0, entry = 0;
+      uint32_t w = i << (32 - kDenseBits), used = 0, held = 0, entry = 0, upto = 0xFF0u;
       while (held < 3u && used + 2u <= kDenseBits) {
         uint32_t v, len;
         if (!elias_from_window(w << 1, v, len) || used + 1u + len > kDenseBits || v - 1u > min(p.s, 7u)) break;
@@ -241,8 +318,10 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
         w <<= 1u + len;
         used += 1u + len;
         ++held;
+        if (held < 3u) upto ^= (15u ^ used) << (4u * held);
       }
-      tab.symbol[i] = held ? entry | (used << 24) | (held << 28) : 0u;
+      tab.symbol[i] = held ? entry | (used << 24) | (held << 30) : 0u;
+      tab.count[i] = held ? upto | used | (held << 16) : 0u;
     }
   } else if (WIDTH == kNibble) {
     for (uint32_t i = tid; i < kTailEntries; i += kThreads) tab.symbol[i] = tail_entry(i, p.s);
