@@ -24,7 +24,7 @@ namespace qsgd {
 namespace {
 
 constexpr uint32_t kThreads = 256;
-constexpr uint32_t kWarmUp = 64;                  // bits: 75-95 % of the starts are then right
+template <bool DENSE> constexpr uint32_t kWarmUp = DENSE ? 96 : 64;      // bits: 75-98 % of the starts are then right
 constexpr uint32_t kLeastPart = 64;               // bits of a string that are worth a lane
 constexpr uint32_t kDenseBits = 10;
 constexpr uint32_t kRowPad = 16;                  // bytes between rows: teams at similar positions use other banks
@@ -66,8 +66,10 @@ struct TeamParams {
 // Where in its row the code of a position lies. The lanes of a team write at positions a fixed distance
 // apart (128 with 4096 coordinates and 32 lanes: one bank for all), so the pieces that the sum reads at
 // once (8 codes) are permuted inside each block of 128 bytes by the number of the block.
-template <int WIDTH>
+// (The dense code stores whole words, at places as irregular as the lengths of the parts: it needs no permutation.)
+template <bool DENSE, int WIDTH>
 __device__ __forceinline__ uint32_t place(uint32_t pos) {       // in bytes
+  if (DENSE && WIDTH != kWide) return pos;
   if (WIDTH == kWide) { const uint32_t a = 2u * pos; return a ^ ((a >> 3) & 0x70u); }
   return pos ^ ((pos >> 4) & 0x78u);
 }
@@ -75,12 +77,13 @@ __device__ __forceinline__ uint32_t place(uint32_t pos) {       // in bytes
 template <bool DENSE>
 struct Tables {
   uint2 code[kCodeEntries];
-  // Code_s, s <= 15: what follows a gap (tail_entry). Code'_s: what the next 10 bits hold, up to three
-  // symbols of levels <= 7: their codes in bytes 0, 1 and 2 (kWide: level | negative << 7), their length in
-  // byte 3, bits 0-3, their number in bits 6-7; 0 when they hold none
+  // Code_s, s <= 15: what follows a gap (tail_entry). Code'_s: what the next 10 bits hold, up to three symbols of
+  // levels <= 7: their length in bits 0-3, their number in bits 5-6, their codes in bytes 1, 2 and 3 (kWide: level |
+  // negative << 7); 0 when they hold none. Bit 4 is 0: an entry is a shift by its length as it is.
   uint32_t symbol[DENSE ? 1u << kDenseBits : kTailEntries];
-  // Code'_s, the same for a reader that only counts: their length in bits 0-3, that of the first in bits 4-7, of the
-  // first two in bits 8-11 (15 where there is no symbol behind them), their number from bit 16 on
+  // Code'_s, the same for a reader that only counts: their length in bits 0-3, that of the first in bits 5-8, of the
+  // first two in bits 9-12 (15 where there is no symbol behind them), their number from bit 16 on. The sum of three
+  // entries has the sum of the lengths in bits 0-4 and that of the numbers from bit 16 on.
   uint32_t count[DENSE ? 1u << kDenseBits : 1u];
 };
 
@@ -94,17 +97,12 @@ __device__ __forceinline__ uint32_t dense_symbol(const uint2* code, uint32_t w, 
   return code_value(x, c) - 1u;
 }
 
-// Window::drop without a branch: the readers of the dense code are bound by the number of their instructions, and
-// lanes cross into a new word at different times.
+// Window::drop without a branch: lanes cross into a new word at different times.
 __device__ __forceinline__ void drop_even(Window& in, uint32_t bits, uint32_t end) {
   in.bp += bits;
-  const bool cross = in.bp >= in.edge && in.bp < end;
-  in.w0 = cross ? in.w1 : in.w0;
-  in.w1 = cross ? in.w2 : in.w1;
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p ld.u32 %0, [%2];\n\t}" : "+r"(in.w2) : "r"((uint32_t)cross), "l"(in.wp)
-               : "memory");
-  in.wp += cross ? 1 : 0;
-  in.edge += cross ? 32u : 0u;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ge.u32 p, %5, %4;\n\tsetp.lt.and.u32 p, %5, %6, p;\n\t@p mov.u32 %0, %1;\n\t@p mov.u32 %1, %2;\n\t"
+               "@p ld.u32 %2, [%3];\n\t@p add.u64 %3, %3, 4;\n\t@p add.u32 %4, %4, 32;\n\t}"
+               : "+r"(in.w0), "+r"(in.w1), "+r"(in.w2), "+l"(in.wp), "+r"(in.edge) : "r"(in.bp), "r"(end) : "memory");
 }
 
 // Reads symbols from bit `from` to the first one that starts at or behind bit `until` (both counted from
@@ -122,22 +120,31 @@ __device__ __forceinline__ uint32_t walk(const Tables<DENSE>& tab, const uint32_
   const uint32_t stop = until - origin, last = end - origin;
   uint32_t n = 0;
   if constexpr (DENSE) {
+    auto single = [&](uint32_t w) { drop_even(in, code_body(tab.code[(w << 1) >> 25]) + 2u, last); ++n; };
     auto step = [&](uint32_t room) {              // room: bits up to `stop`, where that is less than an entry's
       const uint32_t w = in.peek();
       const uint32_t e = tab.count[w >> (32 - kDenseBits)];
+      if (e == 0u) { single(w); return; }
       uint32_t bits = e & 15u, held = e >> 16;
-      if (e == 0u) {
-        bits = code_body(tab.code[(w << 1) >> 25]) + 2u;
-        held = 1u;
-      } else if (room) {                          // only the symbols that start in front of it
-        const uint32_t one = (e >> 4) & 15u, two = (e >> 8) & 15u;
-        held = one >= room ? 1u : two >= room ? 2u : held;
+      if (room) {                                 // only the symbols that start in front of it
+        const uint32_t one = (e >> 5) & 15u, two = (e >> 9) & 15u;
         bits = one >= room ? one : two >= room ? min(two, bits) : bits;
-        held = min(held, e >> 16);
+        held = one >= room ? 1u : two >= room ? min(2u, held) : held;
       }
       drop_even(in, bits, last);
       n += held;
     };
+    while (in.bp + 3u * kDenseBits <= stop) {     // three entries to a window (an entry of 0 moves nothing)
+      uint32_t w = in.peek();
+      const uint32_t e0 = tab.count[w >> (32 - kDenseBits)];
+      w = __funnelshift_l(0u, w, e0);
+      const uint32_t e1 = tab.count[w >> (32 - kDenseBits)];
+      w = __funnelshift_l(0u, w, e1);
+      const uint32_t e2 = tab.count[w >> (32 - kDenseBits)], e = e0 + e1 + e2;
+      drop_even(in, e & 31u, last);
+      n += e >> 16;
+      if (e2 == 0u) single(in.peek());
+    }
     while (in.bp + kDenseBits <= stop) step(0u);
     while (in.bp < stop) step(stop - in.bp);
   } else {
@@ -162,8 +169,8 @@ __device__ __forceinline__ uint32_t walk(const Tables<DENSE>& tab, const uint32_
 
 // The last reading of the dense code where a code is a byte. Codes are gathered in a word, and stored a word at a time.
 // A word that two lanes have codes for is the one's that its first code belongs to: that lane reads on until it has the
-// word, the others leave their part of it out. Which of the codes behind its part a lane has passed does not matter: the
-// lane that they belong to checks them.
+// word, the others leave their part of it out. What a lane passes behind its part is checked by the lane that it belongs
+// to.
 template <int WIDTH>
 __device__ __forceinline__ uint32_t emit_dense(const Tables<true>& tab, const uint32_t* words, uint32_t from, uint32_t until,
                                                uint32_t end, uint32_t at, uint32_t db, uint32_t s, uint8_t* row) {
@@ -172,37 +179,57 @@ __device__ __forceinline__ uint32_t emit_dense(const Tables<true>& tab, const ui
   in.open(words, from);
   const uint32_t origin = from & ~31u;
   const uint32_t stop = until - origin, last = end - origin;
-  const uint32_t row_addr = (uint32_t)__cvta_generic_to_shared(row);
   const uint32_t mine = (at + 3u) & ~3u, full = 8u * db;
+  uint32_t addr = (uint32_t)__cvta_generic_to_shared(row) + (at & ~3u);      // of the word under way
   uint32_t bad = 0, codes = 0;
   uint32_t q = 8u * at;                           // eight times the next position
-  // the word under way is mine, has codes, and there are more
-  auto open_word = [&]() { return (q & 31u) != 0u && (q >> 3) > mine && q < full && in.bp < last; };
-  while (in.bp < stop || open_word()) {
-    const uint32_t w = in.peek();
-    const uint32_t e = tab.symbol[w >> (32 - kDenseBits)];
-    uint32_t bits = (e >> 24) & 15u, held = e >> 30, more = e & 0x00FFFFFFu;
-    if (e == 0u || q + 8u * held > full) {
-      uint32_t closing;
-      const uint32_t level = dense_symbol(tab.code, w, &bits, &closing);
-      bad |= closing;
-      if (level > s) return QSGD_DEV_LEVEL;
-      if (q >= full) return QSGD_DEV_OVERRUN;     // more symbols than coordinates
-      more = level | (level ? (w >> 31) << CodeOf<WIDTH>::kSignShift : 0u);
-      held = 1u;
+  auto gather = [&](uint32_t more, uint32_t eight) {                         // `eight` / 8 codes
+    codes |= __funnelshift_l(0u, more, q);        // (the shift takes q mod 32)
+    const uint32_t over = __funnelshift_l(more, 0u, q), next = q + eight;
+    // the word is whole, and it is mine
+    asm volatile("{\n\t.reg .pred p, m;\n\t.reg .u32 x;\n\txor.b32 x, %2, %3;\n\tand.b32 x, x, 32;\n\tsetp.ne.u32 p, x, 0;\n\t"
+                 "setp.ge.and.u32 m, %3, %4, p;\n\t@m st.shared.u32 [%1], %0;\n\t@p mov.u32 %0, %5;\n\t@p add.u32 %1, %1, 4;\n\t}"
+                 : "+r"(codes), "+r"(addr) : "r"(q), "r"(next), "r"(8u * mine + 32u), "r"(over) : "memory");
+    q = next;
+  };
+  auto single = [&](uint32_t w) {                 // one symbol, with every check
+    uint32_t bits, closing;
+    const uint32_t level = dense_symbol(tab.code, w, &bits, &closing);
+    bad |= closing;
+    if (level > s) return (uint32_t)QSGD_DEV_LEVEL;
+    if (q >= full) return (uint32_t)QSGD_DEV_OVERRUN;                        // more symbols than coordinates
+    gather(level | (level ? (w >> 31) << CodeOf<WIDTH>::kSignShift : 0u), 8u);
+    drop_even(in, bits, last);
+    return 0u;
+  };
+  while (in.bp + 3u * kDenseBits <= stop && q + 72u <= full) {               // three entries to a window
+    uint32_t w = in.peek(), bits = 0, e = 0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      e = tab.symbol[w >> (32 - kDenseBits)];
+      w = __funnelshift_l(0u, w, e);
+      bits += e & 15u;
+      gather(e >> 8, (e >> 2) & 24u);
     }
     drop_even(in, bits, last);
-    codes |= __funnelshift_l(0u, more, q);        // (the shift takes q mod 32)
-    const uint32_t over = __funnelshift_l(more, 0u, q);
-    const uint32_t next = q + 8u * held, pos = (q >> 3) & ~3u;
-    const bool whole = ((q ^ next) & 32u) != 0u;
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.u32 [%1], %2;\n\t}" ::"r"((uint32_t)(whole && pos >= mine)),
-                 "r"(row_addr + place<WIDTH>(pos)), "r"(codes)
-                 : "memory");
-    codes = whole ? over : codes;
-    q = next;
+    if (e == 0u) {
+      const uint32_t err = single(in.peek());
+      if (err) return err;
+    }
   }
-  if ((q & 31u) != 0u && (q >> 3) > mine) *reinterpret_cast<uint32_t*>(row + place<WIDTH>((q >> 3) & ~3u)) = codes;
+  // the rest; and on while the word under way is mine, has codes, and there are more
+  while (in.bp < stop || ((q & 31u) != 0u && (q >> 3) > mine && q < full && in.bp < last)) {
+    const uint32_t w = in.peek();
+    const uint32_t e = tab.symbol[w >> (32 - kDenseBits)], eight = (e >> 2) & 24u;
+    if (e == 0u || q + eight > full) {
+      const uint32_t err = single(w);
+      if (err) return err;
+    } else {
+      gather(e >> 8, eight);
+      drop_even(in, e & 15u, last);
+    }
+  }
+  if ((q & 31u) != 0u && (q >> 3) > mine) asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(codes) : "memory");
   return bad >> 31 ? QSGD_DEV_OVERRUN : 0u;
 }
 
@@ -212,7 +239,7 @@ template <bool DENSE, int WIDTH>
 __device__ __forceinline__ uint32_t emit(const Tables<DENSE>& tab, const uint32_t* words, uint32_t from, uint32_t until,
                                          uint32_t end, uint32_t at, uint32_t db, uint32_t s, uint8_t* row) {
   using Code = typename CodeOf<WIDTH>::type;
-  auto put = [&](uint32_t pos, uint32_t code) { *reinterpret_cast<Code*>(row + place<WIDTH>(pos)) = (Code)code; };
+  auto put = [&](uint32_t pos, uint32_t code) { *reinterpret_cast<Code*>(row + place<DENSE, WIDTH>(pos)) = (Code)code; };
   constexpr uint32_t kSignShift = CodeOf<WIDTH>::kSignShift;
   if (from >= until) return 0u;
   if constexpr (DENSE && WIDTH != kWide) return emit_dense<WIDTH>(tab, words, from, until, end, at, db, s, row);
@@ -224,12 +251,12 @@ __device__ __forceinline__ uint32_t emit(const Tables<DENSE>& tab, const uint32_
   while (in.bp < stop) {
     const uint32_t w = in.peek();
     if (DENSE) {                                  // (codes of two bytes)
-      const uint32_t e = tab.symbol[w >> (32 - kDenseBits)], held = e >> 30;
+      const uint32_t e = tab.symbol[w >> (32 - kDenseBits)], held = (e >> 5) & 3u;
       if (e && in.bp + kDenseBits <= stop && at + held <= db) {
 #pragma unroll
         for (uint32_t j = 0; j < 3; ++j)
-          if (j < held) put(at + j, ((e >> (8u * j)) & 7u) | ((e >> (8u * j)) & 0x80u) << 1);
-        in.drop((e >> 24) & 15u, last);
+          if (j < held) put(at + j, ((e >> (8u * j + 8u)) & 7u) | ((e >> (8u * j + 8u)) & 0x80u) << 1);
+        in.drop(e & 15u, last);
         at += held;
         continue;
       }
@@ -269,16 +296,19 @@ __device__ __forceinline__ uint32_t emit(const Tables<DENSE>& tab, const uint32_
 
 // Reads a part in kMarks pieces and keeps where each piece ended, so that a lane that has to read its part
 // again from another bit can stop at the first mark where it falls into step with its first reading.
-constexpr uint32_t kMarks = 4;
+template <bool DENSE> constexpr uint32_t kMarksOf = DENSE ? 2u : 4u;
 constexpr uint32_t kLeastPiece = 96;      // bits
+template <bool DENSE>
 struct Marks {
+  static constexpr uint32_t kMarks = kMarksOf<DENSE>;
   uint32_t pos[kMarks];       // first symbol at or behind the mark
   uint32_t sum[kMarks];       // positions from the part's start up to there
 };
 
 template <bool DENSE, int WIDTH>
 __device__ __forceinline__ void read_part(const Tables<DENSE>& tab, const uint32_t* words, uint32_t start, uint32_t lo,
-                                          uint32_t hi, uint32_t end, bool again, Marks& m) {
+                                          uint32_t hi, uint32_t end, bool again, Marks<DENSE>& m) {
+  constexpr uint32_t kMarks = kMarksOf<DENSE>;
   const uint32_t piece = max((hi - lo + kMarks - 1u) / kMarks, kLeastPiece);
   uint32_t pos = start, sum = 0;
 #pragma unroll
@@ -310,17 +340,17 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
   for (uint32_t i = tid; i < kCodeEntries; i += kThreads) tab.code[i] = code_entry(i);
   if (DENSE) {
     for (uint32_t i = tid; i < (1u << kDenseBits); i += kThreads) {
-      uint32_t w = i << (32 - kDenseBits), used = 0, held = 0, entry = 0, upto = 0xFF0u;
+      uint32_t w = i << (32 - kDenseBits), used = 0, held = 0, entry = 0, upto = 0xFFu << 5;
       while (held < 3u && used + 2u <= kDenseBits) {
         uint32_t v, len;
         if (!elias_from_window(w << 1, v, len) || used + 1u + len > kDenseBits || v - 1u > min(p.s, 7u)) break;
-        entry |= ((v - 1u) | (v > 1u ? (w >> 31) << (WIDTH == kNibble ? 4 : 7) : 0u)) << (8u * held);
+        entry |= ((v - 1u) | (v > 1u ? (w >> 31) << (WIDTH == kNibble ? 4 : 7) : 0u)) << (8u * held + 8u);
         w <<= 1u + len;
         used += 1u + len;
         ++held;
-        if (held < 3u) upto ^= (15u ^ used) << (4u * held);
+        if (held < 3u) upto ^= (15u ^ used) << (4u * held + 1u);
       }
-      tab.symbol[i] = held ? entry | (used << 24) | (held << 30) : 0u;
+      tab.symbol[i] = held ? entry | used | (held << 5) : 0u;
       tab.count[i] = held ? upto | used | (held << 16) : 0u;
     }
   } else if (WIDTH == kNibble) {
@@ -393,7 +423,8 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
         const uint32_t per = max((ref.total + T - 1u) / T, kLeastPart);
         const uint32_t lo = min(first + t * per, end), hi = t == T - 1u ? end : min(lo + per, end);
         uint32_t start = lo;
-        Marks m;
+        Marks<DENSE> m;
+        constexpr uint32_t kMarks = kMarksOf<DENSE>;
 #pragma unroll
         for (uint32_t q = 0; q < kMarks; ++q) { m.pos[q] = lo; m.sum[q] = 0u; }
         if (reads) {
@@ -403,7 +434,7 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
             scales[j] = __uint_as_float(in.peek());
           } else if (lo < end) {
             uint32_t skipped;
-            start = walk<DENSE, WIDTH>(tab, words, lo - min(kWarmUp, lo - first), lo, end, &skipped);
+            start = walk<DENSE, WIDTH>(tab, words, lo - min(kWarmUp<DENSE>, lo - first), lo, end, &skipped);
           }
           read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, false, m);
         } else if (j < rows && t == 0u) {
@@ -445,7 +476,7 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
         const bool live = slot < slots && b * p.d + c < p.n;
         if (!__any_sync(0xffffffffu, live)) continue;
         const uint32_t gg = live ? g : 0u, cc = live ? c : 0u;
-        const uint8_t* codes = tsm + (size_t)gg * kc * p.row_bytes + place<WIDTH>(cc);
+        const uint8_t* codes = tsm + (size_t)gg * kc * p.row_bytes + place<DENSE, WIDTH>(cc);
         const float* sc = scales + gg * kc;
         float4* carry = reinterpret_cast<float4*>(sums + gg * p.d + cc);
         float acc[8];
