@@ -14,7 +14,11 @@
 // sign) into the string's row in shared memory. Then all threads add the rows in ascending k.
 //
 // Latency is what counts here: one string of 4096 dense symbols read by one lane is 300 us, whatever else
-// the GPU does.
+// the GPU does. So the strings are read where they are, a word ahead of the need: a copy of them in shared memory costs
+// half of the resident warps (8 workers, n = 16.8 M, s = 64, d = 4096, dense code: 375 us with it, 283 without; Code_s
+// with d = 1024: 693 and 630; only the smallest problems, which leave most of the GPU idle, lose: 17.8 and 18.7 us at
+// n = 100 K). The rest is the number of instructions: the dense code is read three table entries to a window, for 10
+// instructions per symbol against 30 with one entry at a time (412 -> 279 us in all).
 #include <type_traits>
 
 #include "elias_decode.cuh"
@@ -27,6 +31,7 @@ constexpr uint32_t kThreads = 256;
 template <bool DENSE> constexpr uint32_t kWarmUp = DENSE ? 96 : 64;      // bits: 75-98 % of the starts are then right
 constexpr uint32_t kLeastPart = 64;               // bits of a string that are worth a lane
 constexpr uint32_t kDenseBits = 10;
+constexpr uint32_t kFewBits = 7;                  // bits per symbol of a string from which on a table entry rarely holds one
 constexpr uint32_t kRowPad = 16;                  // bytes between rows: teams at similar positions use other banks
 
 constexpr uint32_t kLanesPerSm = 1024;            // lanes that fill an SM well enough
@@ -58,7 +63,6 @@ struct TeamParams {
   uint32_t T;             // lanes per string, a power of two
   uint32_t buckets;       // per CTA and pass
   uint32_t row_bytes;
-  uint32_t share;         // bytes of staging per peer
   uint32_t defer_sparse;  // a sparse-regime kernel was launched beside this one
   BucketMap map;
 };
@@ -69,7 +73,7 @@ struct TeamParams {
 // (The dense code stores whole words, at places as irregular as the lengths of the parts: it needs no permutation.)
 template <bool DENSE, int WIDTH>
 __device__ __forceinline__ uint32_t place(uint32_t pos) {       // in bytes
-  if (DENSE && WIDTH != kWide) return pos;
+  if (DENSE) return WIDTH == kWide ? 2u * pos : pos;
   if (WIDTH == kWide) { const uint32_t a = 2u * pos; return a ^ ((a >> 3) & 0x70u); }
   return pos ^ ((pos >> 4) & 0x78u);
 }
@@ -78,12 +82,12 @@ template <bool DENSE>
 struct Tables {
   uint2 code[kCodeEntries];
   // Code_s, s <= 15: what follows a gap (tail_entry). Code'_s: what the next 10 bits hold, up to three symbols of
-  // levels <= 7: their length in bits 0-3, their number in bits 5-6, their codes in bytes 1, 2 and 3 (kWide: level |
-  // negative << 7); 0 when they hold none. Bit 4 is 0: an entry is a shift by its length as it is.
+  // levels <= 7 (kWide: two): their length in bits 0-3, their number in bits 5-6, their codes in bytes 1, 2 and 3
+  // (kWide: level | negative << 7); 0 when they hold none. Bit 4 is 0: an entry is a shift by its length as it is.
   uint32_t symbol[DENSE ? 1u << kDenseBits : kTailEntries];
-  // Code'_s, the same for a reader that only counts: their length in bits 0-3, that of the first in bits 5-8, of the
-  // first two in bits 9-12 (15 where there is no symbol behind them), their number from bit 16 on. The sum of three
-  // entries has the sum of the lengths in bits 0-4 and that of the numbers from bit 16 on.
+  // Code'_s, for a reader that only counts: up to three symbols of those 10 bits, or the one that they start. Their
+  // length in bits 0-4, that of the first of several in bits 8-11, of the first two of three in bits 12-15, their number
+  // from bit 20 on. Fields of three entries can be added.
   uint32_t count[DENSE ? 1u << kDenseBits : 1u];
 };
 
@@ -120,33 +124,25 @@ __device__ __forceinline__ uint32_t walk(const Tables<DENSE>& tab, const uint32_
   const uint32_t stop = until - origin, last = end - origin;
   uint32_t n = 0;
   if constexpr (DENSE) {
-    auto single = [&](uint32_t w) { drop_even(in, code_body(tab.code[(w << 1) >> 25]) + 2u, last); ++n; };
-    auto step = [&](uint32_t room) {              // room: bits up to `stop`, where that is less than an entry's
-      const uint32_t w = in.peek();
-      const uint32_t e = tab.count[w >> (32 - kDenseBits)];
-      if (e == 0u) { single(w); return; }
-      uint32_t bits = e & 15u, held = e >> 16;
-      if (room) {                                 // only the symbols that start in front of it
-        const uint32_t one = (e >> 5) & 15u, two = (e >> 9) & 15u;
-        bits = one >= room ? one : two >= room ? min(two, bits) : bits;
-        held = one >= room ? 1u : two >= room ? min(2u, held) : held;
-      }
-      drop_even(in, bits, last);
-      n += held;
-    };
-    while (in.bp + 3u * kDenseBits <= stop) {     // three entries to a window (an entry of 0 moves nothing)
+    auto look = [&](uint32_t w) { return tab.count[w >> (32 - kDenseBits)]; };
+    while (in.bp + 31u <= stop) {                 // three entries to a window
       uint32_t w = in.peek();
-      const uint32_t e0 = tab.count[w >> (32 - kDenseBits)];
+      const uint32_t e0 = look(w);
       w = __funnelshift_l(0u, w, e0);
-      const uint32_t e1 = tab.count[w >> (32 - kDenseBits)];
+      const uint32_t e1 = look(w), e01 = e0 + e1;
       w = __funnelshift_l(0u, w, e1);
-      const uint32_t e2 = tab.count[w >> (32 - kDenseBits)], e = e0 + e1 + e2;
+      uint32_t e = e01 + look(w);
+      // long symbols: what the window does not hold is left for the next
+      if ((e01 & 0xFFu) > 32u - kDenseBits || (e & 0xFFu) > 31u) e = (e01 & 0xFFu) > 31u ? e0 : e01;
       drop_even(in, e & 31u, last);
-      n += e >> 16;
-      if (e2 == 0u) single(in.peek());
+      n += e >> 20;
     }
-    while (in.bp + kDenseBits <= stop) step(0u);
-    while (in.bp < stop) step(stop - in.bp);
+    while (in.bp < stop) {                        // the symbols that start in front of it
+      const uint32_t e = look(in.peek()), room = stop - in.bp;
+      const uint32_t one = (e >> 8) & 15u, two = (e >> 12) & 15u;
+      drop_even(in, one >= room ? one : two >= room ? two : e & 31u, last);
+      n += one >= room ? 1u : two >= room ? 2u : e >> 20;
+    }
   } else {
     while (in.bp < stop) {
       const uint32_t w = in.peek();
@@ -167,82 +163,94 @@ __device__ __forceinline__ uint32_t walk(const Tables<DENSE>& tab, const uint32_
   return origin + in.bp;
 }
 
-// The last reading of the dense code where a code is a byte. Codes are gathered in a word, and stored a word at a time.
-// A word that two lanes have codes for is the one's that its first code belongs to: that lane reads on until it has the
-// word, the others leave their part of it out. What a lane passes behind its part is checked by the lane that it belongs
-// to.
+// The last reading of the dense code. Codes are gathered in a word, and stored a word at a time. A word that two lanes
+// have codes for is the one's that its first code belongs to: that lane reads on until it has the word, the others leave
+// their part of it out. What a lane passes behind its part is checked by the lane that it belongs to.
+// `few`: most symbols are too long for an entry of the table, which is then not asked for more than one at a time.
 template <int WIDTH>
 __device__ __forceinline__ uint32_t emit_dense(const Tables<true>& tab, const uint32_t* words, uint32_t from, uint32_t until,
-                                               uint32_t end, uint32_t at, uint32_t db, uint32_t s, uint8_t* row) {
+                                               uint32_t end, uint32_t at, uint32_t db, uint32_t s, bool few, uint8_t* row) {
+  constexpr uint32_t kBits = WIDTH == kWide ? 16u : 8u;
   if (from >= until) return 0u;
   Window in;
   in.open(words, from);
   const uint32_t origin = from & ~31u;
   const uint32_t stop = until - origin, last = end - origin;
-  const uint32_t mine = (at + 3u) & ~3u, full = 8u * db;
-  uint32_t addr = (uint32_t)__cvta_generic_to_shared(row) + (at & ~3u);      // of the word under way
+  const uint32_t full = kBits * db;
+  uint32_t q = kBits * at;                        // the next position, in bits of the row
+  const uint32_t mine = (q + 31u) & ~31u;
+  uint32_t addr = (uint32_t)__cvta_generic_to_shared(row) + (q >> 5) * 4u;   // of the word under way
   uint32_t bad = 0, codes = 0;
-  uint32_t q = 8u * at;                           // eight times the next position
-  auto gather = [&](uint32_t more, uint32_t eight) {                         // `eight` / 8 codes
+  auto gather = [&](uint32_t more, uint32_t width) {
     codes |= __funnelshift_l(0u, more, q);        // (the shift takes q mod 32)
-    const uint32_t over = __funnelshift_l(more, 0u, q), next = q + eight;
+    const uint32_t over = __funnelshift_l(more, 0u, q), next = q + width;
     // the word is whole, and it is mine
     asm volatile("{\n\t.reg .pred p, m;\n\t.reg .u32 x;\n\txor.b32 x, %2, %3;\n\tand.b32 x, x, 32;\n\tsetp.ne.u32 p, x, 0;\n\t"
                  "setp.ge.and.u32 m, %3, %4, p;\n\t@m st.shared.u32 [%1], %0;\n\t@p mov.u32 %0, %5;\n\t@p add.u32 %1, %1, 4;\n\t}"
-                 : "+r"(codes), "+r"(addr) : "r"(q), "r"(next), "r"(8u * mine + 32u), "r"(over) : "memory");
+                 : "+r"(codes), "+r"(addr) : "r"(q), "r"(next), "r"(mine + 32u), "r"(over) : "memory");
     q = next;
   };
+  auto entry = [&](uint32_t e) {                  // the codes of an entry; none of the entry 0
+    if (WIDTH == kWide) {
+      const uint32_t x = __byte_perm(e, 0u, 0x4241);
+      gather((x & 0x00070007u) | (x & 0x00800080u) << 1, (e >> 1) & 48u);
+    } else {
+      gather(e >> 8, (e >> 2) & 24u);
+    }
+  };
+  auto width_of = [&](uint32_t e) { return WIDTH == kWide ? (e >> 1) & 48u : (e >> 2) & 24u; };
   auto single = [&](uint32_t w) {                 // one symbol, with every check
     uint32_t bits, closing;
     const uint32_t level = dense_symbol(tab.code, w, &bits, &closing);
     bad |= closing;
     if (level > s) return (uint32_t)QSGD_DEV_LEVEL;
     if (q >= full) return (uint32_t)QSGD_DEV_OVERRUN;                        // more symbols than coordinates
-    gather(level | (level ? (w >> 31) << CodeOf<WIDTH>::kSignShift : 0u), 8u);
+    gather(level | (level ? (w >> 31) << CodeOf<WIDTH>::kSignShift : 0u), kBits);
     drop_even(in, bits, last);
     return 0u;
   };
-  while (in.bp + 3u * kDenseBits <= stop && q + 72u <= full) {               // three entries to a window
-    uint32_t w = in.peek(), bits = 0, e = 0;
+  if (!few) {
+    while (in.bp + 3u * kDenseBits <= stop && q + 96u <= full) {             // three entries to a window
+      uint32_t w = in.peek(), bits = 0, e = 0;
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      e = tab.symbol[w >> (32 - kDenseBits)];
-      w = __funnelshift_l(0u, w, e);
-      bits += e & 15u;
-      gather(e >> 8, (e >> 2) & 24u);
-    }
-    drop_even(in, bits, last);
-    if (e == 0u) {
-      const uint32_t err = single(in.peek());
-      if (err) return err;
+      for (int j = 0; j < 3; ++j) {
+        e = tab.symbol[w >> (32 - kDenseBits)];
+        w = __funnelshift_l(0u, w, e);
+        bits += e & 15u;
+        entry(e);
+      }
+      drop_even(in, bits, last);
+      if (e == 0u) {
+        const uint32_t err = single(in.peek());
+        if (err) return err;
+      }
     }
   }
   // the rest; and on while the word under way is mine, has codes, and there are more
-  while (in.bp < stop || ((q & 31u) != 0u && (q >> 3) > mine && q < full && in.bp < last)) {
+  while (in.bp < stop || ((q & 31u) != 0u && q > mine && q < full && in.bp < last)) {
     const uint32_t w = in.peek();
-    const uint32_t e = tab.symbol[w >> (32 - kDenseBits)], eight = (e >> 2) & 24u;
-    if (e == 0u || q + eight > full) {
+    const uint32_t e = few ? 0u : tab.symbol[w >> (32 - kDenseBits)];
+    if (e == 0u || q + width_of(e) > full) {
       const uint32_t err = single(w);
       if (err) return err;
     } else {
-      gather(e >> 8, eight);
+      entry(e);
       drop_even(in, e & 15u, last);
     }
   }
-  if ((q & 31u) != 0u && (q >> 3) > mine) asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(codes) : "memory");
+  if ((q & 31u) != 0u && q > mine) asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(codes) : "memory");
   return bad >> 31 ? QSGD_DEV_OVERRUN : 0u;
 }
 
-// The last reading: the same part, every check, one code per coordinate into the row. `at`: position of
-// the last nonzero in front of the part (Code_s) or the part's first position (Code'_s).
-template <bool DENSE, int WIDTH>
-__device__ __forceinline__ uint32_t emit(const Tables<DENSE>& tab, const uint32_t* words, uint32_t from, uint32_t until,
+// The last reading of Code_s: the same part, every check, one code per coordinate into the row. `at`: position of
+// the last nonzero in front of the part.
+template <int WIDTH>
+__device__ __forceinline__ uint32_t emit(const Tables<false>& tab, const uint32_t* words, uint32_t from, uint32_t until,
                                          uint32_t end, uint32_t at, uint32_t db, uint32_t s, uint8_t* row) {
   using Code = typename CodeOf<WIDTH>::type;
-  auto put = [&](uint32_t pos, uint32_t code) { *reinterpret_cast<Code*>(row + place<DENSE, WIDTH>(pos)) = (Code)code; };
+  auto put = [&](uint32_t pos, uint32_t code) { *reinterpret_cast<Code*>(row + place<false, WIDTH>(pos)) = (Code)code; };
   constexpr uint32_t kSignShift = CodeOf<WIDTH>::kSignShift;
   if (from >= until) return 0u;
-  if constexpr (DENSE && WIDTH != kWide) return emit_dense<WIDTH>(tab, words, from, until, end, at, db, s, row);
   Window in;
   in.open(words, from);
   const uint32_t origin = from & ~31u;
@@ -250,45 +258,25 @@ __device__ __forceinline__ uint32_t emit(const Tables<DENSE>& tab, const uint32_
   uint32_t bad = 0;
   while (in.bp < stop) {
     const uint32_t w = in.peek();
-    if (DENSE) {                                  // (codes of two bytes)
-      const uint32_t e = tab.symbol[w >> (32 - kDenseBits)], held = (e >> 5) & 3u;
-      if (e && in.bp + kDenseBits <= stop && at + held <= db) {
-#pragma unroll
-        for (uint32_t j = 0; j < 3; ++j)
-          if (j < held) put(at + j, ((e >> (8u * j + 8u)) & 7u) | ((e >> (8u * j + 8u)) & 0x80u) << 1);
-        in.drop(e & 15u, last);
-        at += held;
-        continue;
-      }
-      uint32_t bits, closing;
-      const uint32_t level = dense_symbol(tab.code, w, &bits, &closing);
-      bad |= closing;
-      if (level > s) return QSGD_DEV_LEVEL;
-      if (at >= db) return QSGD_DEV_OVERRUN;      // more symbols than coordinates
-      put(at, level | (level ? (w >> 31) << kSignShift : 0u));
-      ++at;
-      in.drop(bits, last);
+    const uint2 e = tab.code[w >> 25];
+    const uint32_t body = code_body(e);
+    at += code_value(w, e);
+    if (WIDTH == kNibble) {
+      const uint32_t y = w << body, tail = tab.symbol[y >> (32 - kTailBits)];
+      if (tail == 0u) return y >> 31 ? QSGD_DEV_OVERRUN : in.bp + body + 2u > last ? QSGD_DEV_OVERRUN : QSGD_DEV_LEVEL;
+      if (at >= db) return QSGD_DEV_POSITION;
+      put(at, tail);
+      in.drop(body + (tail >> 8), last);
     } else {
-      const uint2 e = tab.code[w >> 25];
-      const uint32_t body = code_body(e);
-      at += code_value(w, e);
-      if (WIDTH == kNibble) {
-        const uint32_t y = w << body, tail = tab.symbol[y >> (32 - kTailBits)];
-        if (tail == 0u) return y >> 31 ? QSGD_DEV_OVERRUN : in.bp + body + 2u > last ? QSGD_DEV_OVERRUN : QSGD_DEV_LEVEL;
-        if (at >= db) return QSGD_DEV_POSITION;
-        put(at, tail);
-        in.drop(body + (tail >> 8), last);
-      } else {
-        const uint32_t y = in.peek_at(body), z = y << 2;
-        const uint2 c = tab.code[z >> 25];
-        const uint32_t level = code_value(z, c), lb = code_body(c);
-        bad |= y | (z << lb);                     // the two closing bits
-        if (at >= db) return QSGD_DEV_POSITION;
-        if (level > s) return QSGD_DEV_LEVEL;
-        put(at, level | (((y >> 30) & 1u) << kSignShift));
-        in.drop(body, last);
-        in.drop(lb + 3u, last);
-      }
+      const uint32_t y = in.peek_at(body), z = y << 2;
+      const uint2 c = tab.code[z >> 25];
+      const uint32_t level = code_value(z, c), lb = code_body(c);
+      bad |= y | (z << lb);                     // the two closing bits
+      if (at >= db) return QSGD_DEV_POSITION;
+      if (level > s) return QSGD_DEV_LEVEL;
+      put(at, level | (((y >> 30) & 1u) << kSignShift));
+      in.drop(body, last);
+      in.drop(lb + 3u, last);
     }
   }
   return bad >> 31 ? QSGD_DEV_OVERRUN : 0u;
@@ -340,18 +328,24 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
   for (uint32_t i = tid; i < kCodeEntries; i += kThreads) tab.code[i] = code_entry(i);
   if (DENSE) {
     for (uint32_t i = tid; i < (1u << kDenseBits); i += kThreads) {
-      uint32_t w = i << (32 - kDenseBits), used = 0, held = 0, entry = 0, upto = 0xFFu << 5;
-      while (held < 3u && used + 2u <= kDenseBits) {
+      const uint32_t w = i << (32 - kDenseBits);
+      uint32_t used = 0, held = 0, ends = 0, codes = 0, small = 0, small_bits = 0;
+      while (held < 3u) {
+        const uint32_t x = w << used;
         uint32_t v, len;
-        if (!elias_from_window(w << 1, v, len) || used + 1u + len > kDenseBits || v - 1u > min(p.s, 7u)) break;
-        entry |= ((v - 1u) | (v > 1u ? (w >> 31) << (WIDTH == kNibble ? 4 : 7) : 0u)) << (8u * held + 8u);
-        w <<= 1u + len;
+        if (!elias_from_window(x << 1, v, len) || used + 1u + len > kDenseBits) break;
+        if (held) ends |= used << (4u * held + 4u);
         used += 1u + len;
+        if (small == held && held < (WIDTH == kWide ? 2u : 3u) && v - 1u <= min(p.s, 7u)) {
+          codes |= ((v - 1u) | (v > 1u ? (x >> 31) << (WIDTH == kNibble ? 4 : 7) : 0u)) << (8u * held + 8u);
+          small = held + 1u;
+          small_bits = used;
+        }
         ++held;
-        if (held < 3u) upto ^= (15u ^ used) << (4u * held + 1u);
       }
-      tab.symbol[i] = held ? entry | used | (held << 5) : 0u;
-      tab.count[i] = held ? upto | used | (held << 16) : 0u;
+      tab.symbol[i] = small ? codes | small_bits | (small << 5) : 0u;
+      // (a longer one than 22 bits is of no level <= 255)
+      tab.count[i] = held ? used | ends | (held << 20) : min(code_body(code_entry((w << 1) >> 25)) + 2u, 22u) | (1u << 20);
     }
   } else if (WIDTH == kNibble) {
     for (uint32_t i = tid; i < kTailEntries; i += kThreads) tab.symbol[i] = tail_entry(i, p.s);
@@ -361,11 +355,9 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
     xi[i] = i & kLevels ? -q : q;
   }
 
-  // rows[bucket][peer] of one pass over the peers | their strings | with several passes, the sums so far |
-  // the scales
+  // rows[bucket][peer] of one pass over the peers | with several passes, the sums so far | the scales
   const uint32_t most = p.buckets * p.Kc;
-  uint8_t* strings = tsm + (size_t)most * p.row_bytes;
-  float* sums = reinterpret_cast<float*>(strings + (size_t)p.Kc * p.share);
+  float* sums = reinterpret_cast<float*>(tsm + (size_t)most * p.row_bytes);
   float* scales = sums + (p.Kc < p.K ? p.buckets * p.d : 0u);
   const uint32_t T = p.T, t = lane & (T - 1u), team = tid / T, teams = kThreads / T;
   const uint64_t groups = (p.B + p.buckets - 1) / p.buckets;
@@ -377,18 +369,6 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
     const uint32_t nb = (uint32_t)min((uint64_t)p.buckets, p.B - b0);
     for (uint32_t k0 = 0; k0 < p.K; k0 += p.Kc) {
       const uint32_t kc = min(p.Kc, p.K - k0), rows = p.buckets * kc;
-      // ---- peer k's strings of these buckets are one stretch of its payload: a warp copies it --------
-      // (a stretch that its table makes longer than the share is read where it is)
-      for (uint32_t k = tid >> 5; k < kc && p.share; k += kThreads >> 5) {
-        PeerTable pt;
-        if (!peer_table(p.peers, k0 + k, p.B, &pt)) continue;
-        const uint64_t from = __ldg(pt.table + b0) >> 7, to = (__ldg(pt.table + b0 + nb) + 127u) >> 7;   // 16-byte units
-        const uint64_t all = __ldg(pt.table + p.B);
-        if (all > pt.cap_bits || from > to || to * 128u > align16((all + 7u) / 8u) * 8u || (to - from + 1u) * 16u > p.share) continue;
-        const uint4* src = reinterpret_cast<const uint4*>(p.peers.payload[k0 + k]) + from;
-        uint4* dst = reinterpret_cast<uint4*>(strings + (size_t)k * p.share);
-        for (uint32_t i = lane; i <= (uint32_t)(to - from); i += 32) dst[i] = __ldg(src + i);   // and 16 bytes behind it
-      }
       for (uint32_t i = tid; i < rows * (p.row_bytes >> 4); i += kThreads)
         reinterpret_cast<uint4*>(tsm)[i] = make_uint4(0u, 0u, 0u, 0u);
       __syncthreads();
@@ -406,16 +386,7 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
         if (mine) {
           db = (uint32_t)min((uint64_t)p.d, p.n - b * p.d);
           ref = string_ref(p.peers, k0 + k, b, p.B, db);
-          if (!ref.err) {
-            PeerTable pt;
-            peer_table(p.peers, k0 + k, p.B, &pt);
-            const uint64_t from = __ldg(pt.table + b0) >> 7, to = (__ldg(pt.table + b0 + nb) + 127u) >> 7;
-            // the copy holds this string whole, whatever the table says about its neighbours
-            const bool copied = from <= to && to * 128u <= align16((__ldg(pt.table + p.B) + 7u) / 8u) * 8u &&
-                                (to - from + 1u) * 16u <= p.share && from * 128u <= ref.lo && ref.lo + 32u + ref.total <= to * 128u;
-            words = copied ? reinterpret_cast<const uint32_t*>(strings + (size_t)k * p.share) + ((ref.lo >> 5) - from * 4u)
-                           : ref.words + (ref.lo >> 5);
-          }
+          if (!ref.err) words = ref.words + (ref.lo >> 5);
         }
         const bool reads = mine && ref.err == 0u;
         const uint32_t first = (uint32_t)(ref.lo & 31u) + 32u, end = first + ref.total;   // bits behind the scale
@@ -458,8 +429,8 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
         uint32_t err = ref.err;
         if (reads) {
           uint8_t* row = tsm + (size_t)j * p.row_bytes;
-          const uint32_t at = upto - sum - (DENSE ? 0u : 1u);
-          err |= emit<DENSE, WIDTH>(tab, words, start, hi, end, at, db, p.s, row);
+          if constexpr (DENSE) err |= emit_dense<WIDTH>(tab, words, start, hi, end, upto - sum, db, p.s, ref.total > kFewBits * db, row);
+          else err |= emit<WIDTH>(tab, words, start, hi, end, upto - sum - 1u, db, p.s, row);
           // a string must end exactly where the table says and, in the dense code, hold every coordinate
           if (t == T - 1u && (stop != end || (DENSE && upto != db))) err |= QSGD_DEV_OVERRUN;
         }
@@ -544,12 +515,8 @@ int launch_elias_teams(const FieldParams& f, bool dense, bool fused, cudaStream_
   p.status = f.status; p.map = f.map; p.defer_sparse = f.defer_sparse;
   const int width = f.s <= 15u ? kNibble : f.s <= 127u ? kByte : kWide;
   p.row_bytes = ((p.d * (width == kWide ? 2u : 1u) + 127u) & ~127u) + kRowPad;
-  // room for strings of up to 6, 9 or 14 bits per coordinate (what max-norm scales and normal values
-  // need at s = 15, 63 and 255)
-  const uint32_t bits = width == kNibble ? 6u : width == kByte ? 9u : 14u;
-  auto share = [&](uint32_t buckets) { return (uint32_t)align16((buckets * (p.d * bits + 32ull) + 7u) / 8u) + 32u; };
   auto bytes = [&](uint32_t buckets, uint32_t peers) {
-    return (size_t)peers * (buckets * (p.row_bytes + 4ull) + share(buckets)) + (peers < p.K ? buckets * p.d * 4ull : 0ull);
+    return (size_t)peers * (buckets * (p.row_bytes + 4ull)) + (peers < p.K ? buckets * p.d * 4ull : 0ull);
   };
   // all peers at once, or (long buckets and many peers) in as few passes as shared memory allows
   uint32_t passes = 1;
@@ -568,7 +535,6 @@ int launch_elias_teams(const FieldParams& f, bool dense, bool fused, cudaStream_
   p.buckets = 1;
   while (p.buckets * 2u * p.Kc * p.T <= kThreads && p.buckets * 2u <= p.B && bytes(p.buckets * 2u, p.Kc) <= (64u << 10)) p.buckets *= 2u;
   while (p.T < 32u && p.buckets * p.Kc * p.T * 2u <= kThreads) p.T <<= 1;
-  p.share = share(p.buckets);
   const size_t smem = align16(bytes(p.buckets, p.Kc));
 #define QSGD_RUN(D, W) launch_width<D, W>(p, fused, smem, stream)
   if (dense) return width == kNibble ? QSGD_RUN(true, kNibble) : width == kByte ? QSGD_RUN(true, kByte) : QSGD_RUN(true, kWide);

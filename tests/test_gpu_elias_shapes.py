@@ -36,6 +36,9 @@ def run(n, d, s, norm, code, K, make=None):
     (2 * 4096 + 77, 4096, 255, MAX, ELIAS, 17), (4096 + 40, 4096, 255, MAX, DENSE, 33),   # several passes over the peers
     (2 * 4096, 4096, 15, MAX, ELIAS, 64), (3000, 992, 128, L2, ELIAS, 40),
     (70 * 96 + 11, 96, 255, L2, ELIAS, 5), (1000, 160, 31, L2, DENSE, 4),
+    # the dense code by table and symbol by symbol, codes of 5, 8 and 9 bits, words that lanes share
+    (4096 + 33, 4096, 255, L2, DENSE, 3), (2 * 2048 + 1, 2048, 127, MAX, DENSE, 2), (999, 992, 15, L2, DENSE, 7),
+    (3 * 64 + 2, 64, 255, L2, DENSE, 9), (2 * 4096 - 1, 4096, 1, L2, DENSE, 4), (5 * 512 + 3, 512, 128, MAX, DENSE, 6),
 ])
 def test_teams(n, d, s, norm, code, K):
     run(n, d, s, norm, code, K)
