@@ -25,7 +25,7 @@ constexpr uint64_t kSmallWork = 8ull << 20;
 bool use_teams(uint64_t B, uint32_t K, uint32_t d, uint32_t s, bool dense) {
   const uint64_t strings = B * K;
   if (dense || K > 32u) return true;
-  if (s <= 15u) return strings <= (12u << 10);
+  if (s <= 15u) return strings <= (24u << 10);
   return d >= 512u || strings <= (40u << 10);
 }
 

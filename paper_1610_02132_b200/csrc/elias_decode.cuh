@@ -164,44 +164,7 @@ struct BitSrc {
     drop(nb);
     return v;
   }
-  // Definition A.1 decoder on the window; at most three groups (values < 2^16).
-  __device__ __forceinline__ bool elias(uint32_t& value, uint32_t& used) {
-    uint32_t N = 1;
-#pragma unroll
-    for (int it = 0; it < 3; ++it) {
-      if ((int32_t)hi >= 0) break;
-      const uint32_t nb = N + 1;
-      N = take(nb);
-      used += nb;
-    }
-    if ((int32_t)hi < 0) return false;
-    drop(1);
-    used += 1;
-    value = N;
-    return true;
-  }
 };
-
-// Lookup table for the recursive Elias code: entry i (the next 12 stream bits) holds
-// value | length << 8 when those bits start with a complete code of at most 12 bits (every value
-// below 64), else 0. Built once per CTA with the definition's decoder.
-constexpr uint32_t kLutBits = 12;
-
-__device__ __forceinline__ void fill_elias_lut(uint16_t* lut) {
-  for (uint32_t i = threadIdx.x; i < (1u << kLutBits); i += blockDim.x) {
-    uint32_t w = i << (32 - kLutBits), N = 1, used = 0;
-    bool ok = true;
-    for (int it = 0; it < 3 && (w >> 31); ++it) {
-      const uint32_t nb = N + 1;
-      if (used + nb > kLutBits) { ok = false; break; }
-      N = w >> (32 - nb);
-      w <<= nb;
-      used += nb;
-    }
-    ok = ok && !(w >> 31) && used + 1 <= kLutBits;
-    lut[i] = ok ? (uint16_t)(N | ((used + 1) << 8)) : (uint16_t)0;
-  }
-}
 
 struct SparseParams {
   PeerSet peers;
@@ -278,7 +241,7 @@ __device__ __forceinline__ uint32_t tail_entry(uint32_t i, uint32_t s) {
 }
 
 // Three words of a payload: w0 holds bit `bp`, `edge` is the first bit of w1, w2 is on its way. Bits are
-// counted from the word that open() was given a bit of. The words may lie in global or in shared memory.
+// counted from the word that open() was given a bit of.
 struct Window {
   const uint32_t* wp;     // the word behind w2
   uint32_t w0, w1, w2;
@@ -301,6 +264,13 @@ struct Window {
   __device__ __forceinline__ void drop(uint32_t bits, uint32_t end) {
     bp += bits;
     if (bp >= edge && bp < end) { w0 = w1; w1 = w2; w2 = *wp; ++wp; edge += 32u; }
+  }
+  // The same without a branch, for lanes that cross into a new word at different times.
+  __device__ __forceinline__ void drop_even(uint32_t bits, uint32_t end) {
+    bp += bits;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ge.u32 p, %5, %4;\n\tsetp.lt.and.u32 p, %5, %6, p;\n\t@p mov.u32 %0, %1;\n\t@p mov.u32 %1, %2;\n\t"
+                 "@p ld.global.u32 %2, [%3];\n\t@p add.u64 %3, %3, 4;\n\t@p add.u32 %4, %4, 32;\n\t}"
+                 : "+r"(w0), "+r"(w1), "+r"(w2), "+l"(wp), "+r"(edge) : "r"(bp), "r"(end) : "memory");
   }
 };
 

@@ -77,67 +77,52 @@ __device__ __forceinline__ void add_peer_bytes(float (&acc)[16], const uint32_t 
   }
 }
 
-template <int LB>
+// One lane, one string. Every code goes the same way (code_entry), so that lanes with different codes stay together, and
+// nothing is read back: a level is a byte, and the signs of 32 coordinates are gathered in a register.
 __device__ __forceinline__ uint32_t parse_to_fields(const PeerSet& peers, uint32_t k, uint64_t b,
                                                     uint64_t B, uint32_t db, uint32_t d, uint32_t s,
-                                                    const uint16_t* lut, uint32_t* __restrict__ row, float* A_out) {
+                                                    const uint2* code, uint32_t* __restrict__ row, float* A_out) {
   *A_out = 0.f;
   const StringRef ref = string_ref(peers, k, b, B, db);
   if (ref.err) return ref.err;
-  const uint32_t total = ref.total;
-  BitSrc src;
-  src.open(ref.words, ref.lo);
-  *A_out = __uint_as_float(src.take(32));
-  uint32_t* srow = row + ((d * LB) >> 5);            // sign bitmap of this peer row
-  uint32_t used = 0, err = 0;
-  // The row is zero and only this lane writes it, so fields are OR-ed in place.
-  uint32_t at = 0xFFFFFFFFu;                        // position of the previous nonzero (-1)
-  while (used < total) {
-    // One refill leaves >= 33 bits: enough for a table-decoded triple (<= 12 + 1 + 12 bits).
-    src.refill();
-    uint32_t gap, level, neg;
-    const uint32_t e1 = lut[src.hi >> (32 - kLutBits)];
-    if (e1) {
-      gap = e1 & 0xFFu;
-      src.drop(e1 >> 8);
-      used += e1 >> 8;
-    } else {
-      if (!src.elias(gap, used)) { err = QSGD_DEV_OVERRUN; break; }
-      src.refill();
-    }
-    neg = src.hi >> 31;
-    const uint32_t e2 = lut[(src.hi << 1) >> (32 - kLutBits)];
-    if (e2) {
-      level = e2 & 0xFFu;
-      src.drop((e2 >> 8) + 1u);
-      used += (e2 >> 8) + 1u;
-    } else {
-      src.drop(1);
-      used += 1;
-      if (!src.elias(level, used)) { err = QSGD_DEV_OVERRUN; break; }
-    }
-    at += gap;
-    if (at >= db || level - 1u >= s || used > total) {     // one rarely taken branch for all three checks
-      err = at >= db ? QSGD_DEV_POSITION : 0u;
-      err |= level - 1u >= s ? QSGD_DEV_LEVEL : 0u;
-      err |= used > total ? QSGD_DEV_OVERRUN : 0u;
-      break;
-    }
-    row[(at * LB) >> 5] |= level << ((at * LB) & 31);
-    srow[at >> 5] |= neg << (at & 31);
+  Window in;
+  in.open(ref.words, ref.lo);
+  const uint32_t end = in.bp + 32u + ref.total;
+  *A_out = __uint_as_float(in.peek());
+  in.drop_even(32u, end);
+  uint8_t* levels = reinterpret_cast<uint8_t*>(row);
+  uint32_t* signs = row + (d >> 2);
+  uint32_t bad = 0, at = 0xFFFFFFFFu;               // position of the previous nonzero (-1)
+  uint32_t gathered = 0, block = 0;                 // signs of the coordinates 32 * block ..
+  while (in.bp < end) {
+    const uint32_t w = in.peek();
+    const uint2 c = code[w >> 25];
+    const uint32_t body = code_body(c), y = in.peek_at(body), z = y << 2;
+    const uint2 e = code[z >> 25];
+    const uint32_t level = code_value(z, e), lb = code_body(e);
+    at += code_value(w, c);
+    bad |= y | (z << lb);                           // the two closing bits
+    if (at >= db || level > s) return at >= db ? QSGD_DEV_POSITION : QSGD_DEV_LEVEL;
+    levels[at] = (uint8_t)level;
+    if (at >> 5 != block) { signs[block] = gathered; gathered = 0u; block = at >> 5; }
+    gathered |= ((y >> 30) & 1u) << (at & 31u);
+    uint32_t bits = body + lb + 3u;
+    if (bits > 32u) { in.drop_even(body, end); bits -= body; }
+    in.drop_even(bits, end);
   }
-  return err;
+  signs[block] = gathered;
+  return bad >> 31 || in.bp != end ? QSGD_DEV_OVERRUN : 0u;
 }
 
 template <bool FUSED>
 __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_constant__ FieldParams p) {
   constexpr int LB = 8;
   extern __shared__ __align__(16) uint32_t fsm[];
-  __shared__ uint16_t elias_lut[1u << kLutBits];
+  __shared__ uint2 code[kCodeEntries];
   chain_wait();                                   // the messages come from the kernels ahead
   if (p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-  fill_elias_lut(elias_lut);
+  for (uint32_t i = tid; i < kCodeEntries; i += blockDim.x) code[i] = code_entry(i);
   __syncthreads();
   const LevelQuotient lq = level_quotient(p.s, p.minus_zero);
 
@@ -158,7 +143,7 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
       uint32_t* bucket = mine + pg * p.bucket_words;
       const uint32_t db = (uint32_t)min((uint64_t)p.d, p.n - (b0 + pg) * p.d);
       float A;
-      const uint32_t st = parse_to_fields<LB>(p.peers, pk, b0 + pg, p.B, db, p.d, p.s, elias_lut,
+      const uint32_t st = parse_to_fields(p.peers, pk, b0 + pg, p.B, db, p.d, p.s, code,
                                               bucket + pk * p.row_words, &A);
       reinterpret_cast<float*>(bucket + p.K * p.row_words)[pk] = A;
       if (st) atomicOr(p.status, st);
@@ -216,7 +201,7 @@ int launch_fields(FieldParams& p, bool fused, cudaStream_t stream) {
   const size_t per_warp = (size_t)G * p.bucket_words * 4;
   // Warps per CTA: the count that leaves the most warps resident on an SM. The code table is
   // per CTA, the fields per warp; the parse is latency-bound, so warps are what counts.
-  const size_t per_cta = 8192 + 1024, budget = (size_t)max_smem - per_cta;
+  const size_t per_cta = 2048, budget = (size_t)max_smem - per_cta;
   const size_t per_sm = 227u << 10;
   int warps = 1, best = 0;
   for (int w = 1; w <= 10; ++w) {

@@ -101,14 +101,6 @@ __device__ __forceinline__ uint32_t dense_symbol(const uint2* code, uint32_t w, 
   return code_value(x, c) - 1u;
 }
 
-// Window::drop without a branch: lanes cross into a new word at different times.
-__device__ __forceinline__ void drop_even(Window& in, uint32_t bits, uint32_t end) {
-  in.bp += bits;
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ge.u32 p, %5, %4;\n\tsetp.lt.and.u32 p, %5, %6, p;\n\t@p mov.u32 %0, %1;\n\t@p mov.u32 %1, %2;\n\t"
-               "@p ld.u32 %2, [%3];\n\t@p add.u64 %3, %3, 4;\n\t@p add.u32 %4, %4, 32;\n\t}"
-               : "+r"(in.w0), "+r"(in.w1), "+r"(in.w2), "+l"(in.wp), "+r"(in.edge) : "r"(in.bp), "r"(end) : "memory");
-}
-
 // Reads symbols from bit `from` to the first one that starts at or behind bit `until` (both counted from
 // bit 0 of words[0]; `end`: first bit behind the string). Returns where that is; *sum: the gaps or, in the
 // dense code, the symbols passed. What is no symbol (the reader is out of step, or the string is
@@ -134,13 +126,13 @@ __device__ __forceinline__ uint32_t walk(const Tables<DENSE>& tab, const uint32_
       uint32_t e = e01 + look(w);
       // long symbols: what the window does not hold is left for the next
       if ((e01 & 0xFFu) > 32u - kDenseBits || (e & 0xFFu) > 31u) e = (e01 & 0xFFu) > 31u ? e0 : e01;
-      drop_even(in, e & 31u, last);
+      in.drop_even(e & 31u, last);
       n += e >> 20;
     }
     while (in.bp < stop) {                        // the symbols that start in front of it
       const uint32_t e = look(in.peek()), room = stop - in.bp;
       const uint32_t one = (e >> 8) & 15u, two = (e >> 12) & 15u;
-      drop_even(in, one >= room ? one : two >= room ? two : e & 31u, last);
+      in.drop_even(one >= room ? one : two >= room ? two : e & 31u, last);
       n += one >= room ? 1u : two >= room ? 2u : e >> 20;
     }
   } else {
@@ -206,7 +198,7 @@ __device__ __forceinline__ uint32_t emit_dense(const Tables<true>& tab, const ui
     if (level > s) return (uint32_t)QSGD_DEV_LEVEL;
     if (q >= full) return (uint32_t)QSGD_DEV_OVERRUN;                        // more symbols than coordinates
     gather(level | (level ? (w >> 31) << CodeOf<WIDTH>::kSignShift : 0u), kBits);
-    drop_even(in, bits, last);
+    in.drop_even(bits, last);
     return 0u;
   };
   if (!few) {
@@ -219,7 +211,7 @@ __device__ __forceinline__ uint32_t emit_dense(const Tables<true>& tab, const ui
         bits += e & 15u;
         entry(e);
       }
-      drop_even(in, bits, last);
+      in.drop_even(bits, last);
       if (e == 0u) {
         const uint32_t err = single(in.peek());
         if (err) return err;
@@ -235,7 +227,7 @@ __device__ __forceinline__ uint32_t emit_dense(const Tables<true>& tab, const ui
       if (err) return err;
     } else {
       entry(e);
-      drop_even(in, e & 15u, last);
+      in.drop_even(e & 15u, last);
     }
   }
   if ((q & 31u) != 0u && q > mine) asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(codes) : "memory");
