@@ -17,16 +17,14 @@ namespace {
 constexpr uint64_t kSmallWork = 8ull << 20;
 
 // A lane per string (or stream of strings), or a team of lanes? A lane per string is the cheaper reading (a team
-// reads its string almost twice) but needs strings enough for the GPU's lanes. Measured lines (us, a lane against
-// a team). s <= 15: 16 K strings of d = 512 33 / 33, of d = 4096 (8 K of them) 168 / 114, 32 K of d = 4096 264 /
-// 563, 32 K of d = 128 19 / 26, 65 K of d = 512 43 / 107. s = 255: 16 K of d = 512 118 / 74, 524 K 1974 / 1744, but
-// 2 M of d = 128 1488 / 1751; from d = 1024 on always teams (131 K strings of d = 4096: 1559 / 493). Code'_s has
-// a symbol per coordinate: always teams.
+// reads its string almost twice) but needs strings enough for the GPU's lanes, and room in shared memory for the whole
+// bucket where s > 15. Measured (us, a team against a lane). s <= 15: 20 K strings of d = 128 27 / 29, 23 K of d = 512
+// 32 / 38, 23 K of d = 4096 93 / 125; 39 K of d = 512 36 / 37, of d = 128 39 / 30, 62 K of d = 512 48 / 40. s = 255:
+// 13 K of d = 96 31 / 34, 16 K of d = 256 50 / 83; 26 K of d = 96 37 / 34, 31 K of d = 64 29 / 24, of d = 256 89 / 87,
+// 524 K of d = 256 1042 / 664; from d = 512 on always teams: 16 K 82 / 149, 262 K 912 / 937, d = 1024 915 / 1632. Code'_s
+// has a symbol per coordinate: always teams.
 bool use_teams(uint64_t B, uint32_t K, uint32_t d, uint32_t s, bool dense) {
-  const uint64_t strings = B * K;
-  if (dense || K > 32u) return true;
-  if (s <= 15u) return strings <= (24u << 10);
-  return d >= 512u || strings <= (40u << 10);
+  return dense || K > 32u || (s > 15u && d >= 512u) || B * K <= (24u << 10);
 }
 
 }  // namespace

@@ -5,12 +5,10 @@
 //
 // A string S can only be parsed front to back, but buckets and peers are independent once the
 // per-bucket offset table gives each string's first bit. A warp owns a group of G buckets.
-// Phase 1 (parse): lane (g, k) reads peer k's string of bucket g through a 64-bit register
-// window (next word prefetched) and rebuilds that peer's *fixed-width fields* -- level fields
-// and sign bitmap -- for the bucket in shared memory. Phase 2 (apply): exactly the fixed-width
-// decoder's inner loop, reading the fields from shared memory: every lane takes 16 coordinates
-// and adds the peers in ascending k, which fixes the summation order however phase 1 was
-// scheduled. Which shapes come here and which are read by teams of lanes: use_teams in elias_decode.cu.
+// Phase 1 (parse): lane (g, k) reads peer k's string of bucket g through a register
+// window (a word ahead) and rebuilds that peer's *fixed-width fields* -- level fields
+// and sign bitmap -- for the bucket in shared memory. Phase 2 (apply): every lane takes 16 coordinates and adds
+// the peers' fields in ascending k, which fixes the summation order however phase 1 was scheduled. Which shapes come here and which are read by teams of lanes: use_teams in elias_decode.cu.
 #include "elias_decode.cuh"
 
 namespace qsgd {
@@ -78,7 +76,10 @@ __device__ __forceinline__ void add_peer_bytes(float (&acc)[16], const uint32_t 
 }
 
 // One lane, one string. Every code goes the same way (code_entry), so that lanes with different codes stay together, and
-// nothing is read back: a level is a byte, and the signs of 32 coordinates are gathered in a register.
+// nothing is read back: a level is a byte, and the signs of 32 coordinates are gathered in a register. The loop is a chain
+// of dependent instructions and bound by their latency. Against tables of whole codes with a way around them for the
+// others, and fields OR-ed in shared memory: 39.9 -> 36.2 us at n = 1 M, d = 96, s = 255, K = 5 (2-norm), 914 -> 664 at
+// n = 16.8 M, d = 256, K = 8 (max-norm), 1124 -> 799 at d = 128, K = 16.
 __device__ __forceinline__ uint32_t parse_to_fields(const PeerSet& peers, uint32_t k, uint64_t b,
                                                     uint64_t B, uint32_t db, uint32_t d, uint32_t s,
                                                     const uint2* code, uint32_t* __restrict__ row, float* A_out) {

@@ -143,12 +143,11 @@ __device__ __forceinline__ uint32_t walk(const Tables<DENSE>& tab, const uint32_
       n += code_value(w, e);
       if (WIDTH == kNibble) {
         const uint32_t tail = tab.symbol[(w << body) >> (32 - kTailBits)];
-        in.drop_even(tail ? body + (tail >> 8) : body + 1u, last);
+        in.drop(tail ? body + (tail >> 8) : body + 1u, last);
       } else {
         const uint32_t y = in.peek_at(body) << 2;
-        uint32_t bits = body + code_body(tab.code[y >> 25]) + 3u;
-        if (bits > 32u) { in.drop_even(body, last); bits -= body; }
-        in.drop_even(bits, last);
+        in.drop(body, last);
+        in.drop(code_body(tab.code[y >> 25]) + 3u, last);
       }
     }
   }
@@ -259,7 +258,7 @@ __device__ __forceinline__ uint32_t emit(const Tables<false>& tab, const uint32_
       if (tail == 0u) return y >> 31 ? QSGD_DEV_OVERRUN : in.bp + body + 2u > last ? QSGD_DEV_OVERRUN : QSGD_DEV_LEVEL;
       if (at >= db) return QSGD_DEV_POSITION;
       put(at, tail);
-      in.drop_even(body + (tail >> 8), last);
+      in.drop(body + (tail >> 8), last);
     } else {
       const uint32_t y = in.peek_at(body), z = y << 2;
       const uint2 c = tab.code[z >> 25];
@@ -268,9 +267,8 @@ __device__ __forceinline__ uint32_t emit(const Tables<false>& tab, const uint32_
       if (at >= db) return QSGD_DEV_POSITION;
       if (level > s) return QSGD_DEV_LEVEL;
       put(at, level | (((y >> 30) & 1u) << kSignShift));
-      uint32_t bits = body + lb + 3u;
-      if (bits > 32u) { in.drop_even(body, last); bits -= body; }
-      in.drop_even(bits, last);
+      in.drop(body, last);
+      in.drop(lb + 3u, last);
     }
   }
   return bad >> 31 ? QSGD_DEV_OVERRUN : 0u;

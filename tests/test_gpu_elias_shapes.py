@@ -109,7 +109,7 @@ def test_malformed_streams(d, K):
             assert same.all()
 
 
-@pytest.mark.parametrize("n,d,s,K", [(1536 * 512, 512, 15, 8), (1536 * 512 + 1, 512, 15, 8), (2 ** 22, 128, 3, 2), (2 ** 25, 4096, 3, 2), (2 ** 20, 4096, 1, 8), (2 ** 20 + 4096, 4096, 1, 8),
+@pytest.mark.parametrize("n,d,s,K", [(3072 * 512, 512, 15, 8), (3072 * 512 + 1, 512, 15, 8), (6144 * 480, 480, 200, 4), (6144 * 480 + 1, 480, 200, 4), (2 ** 22, 128, 3, 2), (2 ** 25, 4096, 3, 2), (2 ** 20, 4096, 1, 8), (2 ** 20 + 4096, 4096, 1, 8),
                                      (10000 * 32 + 7, 32, 16, 5), (9000 * 64, 64, 101, 5), (9000 * 96 + 1, 96, 127, 5), (1400 * 480, 480, 255, 32)])
 def test_lines_between_decoders(n, d, s, K):
     """Both sides of the lines between a lane and a team per string and between one and two launches, against
