@@ -14,8 +14,9 @@
 // The stream is read by table: the next kBits bits index an entry that says how far to go (up to two whole
 // entries of the string, or one and the next gap, or a gap alone), which two bytes to store and where. A bit of
 // state tells whether a gap or, after a gap alone, its sign and level come next. Nothing in the loop depends
-// on what was read but data: lanes with different codes stay together. What no table entry covers -- a gap
-// of 64 or more, a malformed code -- is read by the definition's decoder (slow_entry).
+// on what was read but data: lanes with different codes stay together. A gap
+// that no table entry covers (64 or more) is decoded by all lanes that have come to one together, whatever else there is
+// (a malformed code) by the definition's decoder with every check (slow_entry).
 #include "elias_decode.cuh"
 
 namespace qsgd {
@@ -311,28 +312,45 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
       }
       ask();
       // the burst: all lanes together, until none that can go on is short of the goal
-      int32_t until = (int32_t)(consumed + kRing - kMostAdvance);           // of `at`: room for an entry
+      const int32_t room = (int32_t)(consumed + kRing - kMostAdvance);      // of `at`: room for an entry
+      int32_t until = room;
       const uint32_t last = ready ? min(end, ready - (uint32_t)kAhead + 1u) : 0u;        // first bit to stop at
+      bool hard = false;
       for (;;) {
-        const bool go = (int32_t)at < until && (int32_t)(last - bp) > 0;
-        if (!__any_sync(0xffffffffu, go && (int32_t)at < (int32_t)goal - 1)) break;
-        // (a lane that does not go on finds an entry for nothing)
-        // bits behind the string's end read as ones: no code is complete with them
-        const uint32_t w = __funnelshift_l(w1, w0, bp) | __funnelshift_rc(0xFFFFFFFFu, 0u, end - bp);
-        uint32_t e = table_entry(tab, w, state);
-        e = go ? e : state;
-        store_byte_if(e & kFirst, (__dp4a(e, 0x00010000u, at) & (kRing - 1u)) ^ cell, e >> 4);
-        at += e >> 26;
-        store_byte_if(e & kSecond, (at & (kRing - 1u)) ^ cell, e >> 9);
-        state = e & kStateBit;
-        uint32_t f = table_entry(tab, w << (e & 15u), state);
-        f = go && (int32_t)at < until ? f : state;
-        store_byte_if(f & kFirst, (__dp4a(f, 0x00010000u, at) & (kRing - 1u)) ^ cell, f >> 4);
-        at += f >> 26;
-        store_byte_if(f & kSecond, (at & (kRing - 1u)) ^ cell, f >> 9);
-        until = f & 15u ? until : INT32_MIN;      // nothing for the table here, or far enough
-        state = f & kStateBit;
-        drop((e & 15u) + (f & 15u));
+        for (;;) {
+          const bool go = (int32_t)at < until && (int32_t)(last - bp) > 0;
+          if (!__any_sync(0xffffffffu, go && (int32_t)at < (int32_t)goal - 1)) break;
+          // (a lane that does not go on finds an entry for nothing)
+          // bits behind the string's end read as ones: no code is complete with them
+          const uint32_t w = __funnelshift_l(w1, w0, bp) | __funnelshift_rc(0xFFFFFFFFu, 0u, end - bp);
+          uint32_t e = table_entry(tab, w, state);
+          e = go ? e : state;
+          store_byte_if(e & kFirst, (__dp4a(e, 0x00010000u, at) & (kRing - 1u)) ^ cell, e >> 4);
+          at += e >> 26;
+          store_byte_if(e & kSecond, (at & (kRing - 1u)) ^ cell, e >> 9);
+          state = e & kStateBit;
+          uint32_t f = table_entry(tab, w << (e & 15u), state);
+          f = go && (int32_t)at < until ? f : state;
+          store_byte_if(f & kFirst, (__dp4a(f, 0x00010000u, at) & (kRing - 1u)) ^ cell, f >> 4);
+          at += f >> 26;
+          store_byte_if(f & kSecond, (at & (kRing - 1u)) ^ cell, f >> 9);
+          until = f & 15u ? until : INT32_MIN;      // nothing for the table here, or far enough
+          state = f & kStateBit;
+          drop((e & 15u) + (f & 15u));
+        }
+        // a gap that is too long for the table, in all lanes that have come to one
+        const bool gap = until == INT32_MIN && !hard && state == 0u && (int32_t)at < room && (int32_t)(last - bp) > 0;
+        if (!__any_sync(0xffffffffu, gap && (int32_t)at < (int32_t)goal - 1)) break;
+        if (gap) {
+          uint32_t v, len;
+          hard = !elias_from_window(__funnelshift_l(w1, w0, bp), v, len) || len > end - bp || v > stop - 1u - at;
+          if (!hard) {
+            at += v - 1u;
+            state = kStateBit;
+            until = room;
+            drop(len);
+          }
+        }
       }
       stuck = until == INT32_MIN;
       if (!__any_sync(0xffffffffu, ((live || b < nb) && (int32_t)at < (int32_t)goal - 1) ||
