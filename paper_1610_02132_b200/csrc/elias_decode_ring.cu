@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
       const int32_t room = (int32_t)(consumed + kRing - kMostAdvance);      // of `at`: room for an entry
       int32_t until = room;
       const uint32_t last = ready ? min(end, ready - (uint32_t)kAhead + 1u) : 0u;        // first bit to stop at
-      bool hard = false;
+      bool hard = false, done;
       for (;;) {
         for (;;) {
           const bool go = (int32_t)at < until && (int32_t)(last - bp) > 0;
@@ -338,6 +338,9 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
           state = f & kStateBit;
           drop((e & 15u) + (f & 15u));
         }
+        done = !__any_sync(0xffffffffu, ((live || b < nb) && (int32_t)at < (int32_t)goal - 1) ||
+                                            (live && (int32_t)(at + (state ? 1u : 0u) - stop) >= 0));
+        if (done) break;
         // a gap that is too long for the table, in all lanes that have come to one
         const bool gap = until == INT32_MIN && !hard && state == 0u && (int32_t)at < room && (int32_t)(last - bp) > 0;
         if (!__any_sync(0xffffffffu, gap && (int32_t)at < (int32_t)goal - 1)) break;
@@ -352,10 +355,8 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
           }
         }
       }
+      if (done) break;
       stuck = until == INT32_MIN;
-      if (!__any_sync(0xffffffffu, ((live || b < nb) && (int32_t)at < (int32_t)goal - 1) ||
-                                       (live && (int32_t)(at + (state ? 1u : 0u) - stop) >= 0)))
-        break;
     }
     ask();                                        // they come while the warp adds up
     __syncwarp();
