@@ -341,7 +341,8 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
         done = !__any_sync(0xffffffffu, ((live || b < nb) && (int32_t)at < (int32_t)goal - 1) ||
                                             (live && (int32_t)(at + (state ? 1u : 0u) - stop) >= 0));
         if (done) break;
-        // a gap that is too long for the table, in all lanes that have come to one
+        // a gap that is too long for the table, in all lanes that have come to one (478 -> 467 us against leaving it to
+        // slow_entry at n = 60 M, d = 512, s = 15, K = 16, a mixture of two scales; 161 -> 155 at s = 3, d = 256)
         const bool gap = until == INT32_MIN && !hard && state == 0u && (int32_t)at < room && (int32_t)(last - bp) > 0;
         if (!__any_sync(0xffffffffu, gap && (int32_t)at < (int32_t)goal - 1)) break;
         if (gap) {
