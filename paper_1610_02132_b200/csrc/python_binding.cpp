@@ -29,33 +29,59 @@ const at::Tensor& cuda_tensor(PyObject* o, const char* name) {
   throw Fail{};
 }
 
-// Address of a tensor, a raw device address given as an int, or null for None.
-void* address(PyObject* o) {
-  if (o == Py_None) return nullptr;
-  if (THPVariable_Check(o)) return THPVariable_Unpack(o).data_ptr();
-  const unsigned long long v = PyLong_AsUnsignedLongLongMask(o);
-  if (v == ~0ull && PyErr_Occurred()) throw Fail{};
-  return reinterpret_cast<void*>(v);
-}
+PyObject* g_ctypes_number = nullptr;   // ctypes' c_uint64, c_float and the like
 
-uint64_t u64(PyObject* o) {
-  const unsigned long long v = PyLong_AsUnsignedLongLongMask(o);
-  if (v == ~0ull && PyErr_Occurred()) throw Fail{};
-  return v;
+// A number, also one of ctypes' own.
+struct Number {
+  PyObject* o;
+  explicit Number(PyObject* v) : o(Py_NewRef(v)) {
+    if (PyIndex_Check(v) || PyFloat_Check(v)) return;
+    const int mine = g_ctypes_number ? PyObject_IsInstance(v, g_ctypes_number) : 0;
+    if (mine) Py_SETREF(o, mine > 0 ? PyObject_GetAttrString(v, "value") : nullptr);
+    if (!o) throw Fail{};
+  }
+  Number(const Number&) = delete;
+  ~Number() { Py_XDECREF(o); }
+};
+
+uint64_t u64(PyObject* v) {
+  const Number n(v);
+  const unsigned long long u = PyLong_AsUnsignedLongLongMask(n.o);
+  if (u == ~0ull && PyErr_Occurred()) throw Fail{};
+  return u;
 }
 uint32_t u32(PyObject* o) { return static_cast<uint32_t>(u64(o)); }
 int i32(PyObject* o) { return static_cast<int>(u64(o)); }
 
 float f32(PyObject* o) {
-  const double v = PyFloat_AsDouble(o);
+  const Number n(o);
+  const double v = PyFloat_AsDouble(n.o);
   if (v == -1.0 && PyErr_Occurred()) throw Fail{};
   return static_cast<float>(v);
+}
+
+// Where a tensor, or whatever else has a data_ptr(), lies.
+void* data_of(PyObject* o) {
+  if (THPVariable_Check(o)) return THPVariable_Unpack(o).data_ptr();
+  PyObject* p = PyObject_CallMethod(o, "data_ptr", nullptr);
+  if (!p) throw Fail{};
+  const unsigned long long v = PyLong_AsUnsignedLongLongMask(p);
+  Py_DECREF(p);
+  if (v == ~0ull && PyErr_Occurred()) throw Fail{};
+  return reinterpret_cast<void*>(v);
+}
+void* data_or_null(PyObject* o) { return o == Py_None ? nullptr : data_of(o); }
+
+// The same, or a raw device address given as an integer.
+void* address(PyObject* o) {
+  return !THPVariable_Check(o) && PyIndex_Check(o) ? reinterpret_cast<void*>(u64(o)) : data_of(o);
 }
 
 qsgd_stream_t stream_of(PyObject* o) {
   if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
   PyObject* v = PyObject_GetAttrString(o, "cuda_stream");
   if (!v) throw Fail{};
+  if (v == Py_None) { Py_DECREF(v); return nullptr; }
   const unsigned long long s = PyLong_AsUnsignedLongLongMask(v);
   Py_DECREF(v);
   if (s == ~0ull && PyErr_Occurred()) throw Fail{};
@@ -136,6 +162,7 @@ PyObject* unlocked(F&& call) {
 PyObject* encode(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   QSGD_ARGS(14)
   QSGD_TRY
+  void* ws = data_or_null(a[11]);
   const at::Tensor& g = cuda_tensor(a[0], "g");
   const at::Tensor& out = cuda_tensor(a[9], "out");
   const at::Tensor& info = cuda_tensor(a[10], "out_bits");
@@ -144,7 +171,6 @@ PyObject* encode(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   const uint32_t bucket = u32(a[2]), s = u32(a[3]), step = u32(a[7]), worker = u32(a[8]);
   const int norm = i32(a[4]), code = i32(a[5]);
   const uint64_t seed = u64(a[6]);
-  void* ws = address(a[11]);
   const qsgd_stream_t stream = stream_of(a[13]);
   return unlocked([&] {
     return qsgd_encode(static_cast<const float*>(g.data_ptr()), n, bucket, s, norm, code, seed, step, worker,
@@ -180,6 +206,7 @@ PyObject* encode_static(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
 PyObject* policy_encode(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   QSGD_ARGS(14)
   QSGD_TRY
+  void* ws = data_or_null(a[11]);
   const at::Tensor& g = cuda_tensor(a[0], "g");
   const at::Tensor& out = cuda_tensor(a[9], "out");
   const at::Tensor& info = cuda_tensor(a[10], "out_bits");
@@ -188,7 +215,6 @@ PyObject* policy_encode(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   const uint32_t bucket = u32(a[2]), s = u32(a[3]), step = u32(a[7]), worker = u32(a[8]);
   const int norm = i32(a[4]), code = i32(a[5]);
   const uint64_t seed = u64(a[6]);
-  void* ws = address(a[11]);
   const qsgd_stream_t stream = stream_of(a[13]);
   return unlocked([&] {
     return qsgd_policy_encode(static_cast<const float*>(g.data_ptr()), plan, bucket, s, norm, code, seed, step, worker,
@@ -204,7 +230,7 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   QSGD_ARGS(12)
   QSGD_TRY
   const bool packed = a[0] == Py_True, fused = a[9] != Py_None;
-  float* out = static_cast<float*>(cuda_tensor(a[8], fused ? "x" : "acc").data_ptr());
+  uint32_t* status = static_cast<uint32_t*>(data_of(a[10]));
   Peers msgs, tables;
   uint64_t count[QSGD_MAX_PEERS] = {};
   peers(a[1], &msgs);
@@ -213,11 +239,11 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   const uint64_t n = u64(a[4]);
   const uint32_t bucket = u32(a[5]), s = u32(a[6]);
   const int code = i32(a[7]);
-  uint32_t* status = static_cast<uint32_t*>(address(a[10]));
+  const float eta = fused ? f32(a[9]) : 0.f;
+  float* out = static_cast<float*>(cuda_tensor(a[8], fused ? "x" : "acc").data_ptr());
   const qsgd_stream_t stream = stream_of(a[11]);
   const void* const* mp = msgs.as<void>();
   const uint64_t* const* tp = tables.as<uint64_t>();
-  const float eta = fused ? f32(a[9]) : 0.f;
   return unlocked([&] {
     if (fused)
       return (packed ? qsgd_decode_sgd_step_packed : qsgd_decode_sgd_step)(mp, tp, bytes, msgs.K, n, bucket, s, code,
@@ -233,7 +259,7 @@ PyObject* policy_decode(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   QSGD_ARGS(11)
   QSGD_TRY
   const bool fused = a[8] != Py_None;
-  float* out = static_cast<float*>(cuda_tensor(a[7], fused ? "x" : "acc").data_ptr());
+  uint32_t* status = static_cast<uint32_t*>(data_of(a[9]));
   Peers msgs, tables;
   uint64_t count[QSGD_MAX_PEERS] = {};
   peers(a[0], &msgs);
@@ -242,11 +268,11 @@ PyObject* policy_decode(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   const qsgd_policy* plan = static_cast<const qsgd_policy*>(address(a[3]));
   const uint32_t bucket = u32(a[4]), s = u32(a[5]);
   const int code = i32(a[6]);
-  uint32_t* status = static_cast<uint32_t*>(address(a[9]));
+  const float eta = fused ? f32(a[8]) : 0.f;
+  float* out = static_cast<float*>(cuda_tensor(a[7], fused ? "x" : "acc").data_ptr());
   const qsgd_stream_t stream = stream_of(a[10]);
   const void* const* mp = msgs.as<void>();
   const uint64_t* const* tp = tables.as<uint64_t>();
-  const float eta = fused ? f32(a[8]) : 0.f;
   return unlocked([&] {
     return fused ? qsgd_policy_decode_sgd_step(mp, tp, bytes, msgs.K, plan, bucket, s, code, out, eta, status, stream)
                  : qsgd_policy_decode_accumulate(mp, tp, bytes, msgs.K, plan, bucket, s, code, out, status, stream);
@@ -285,4 +311,10 @@ PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_qsgd_native", nullptr, -1, kMeth
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__qsgd_native(void) { return PyModule_Create(&kModule); }
+PyMODINIT_FUNC PyInit__qsgd_native(void) {
+  PyObject* ctypes = PyImport_ImportModule("_ctypes");
+  if (!ctypes) return nullptr;
+  g_ctypes_number = PyObject_GetAttrString(ctypes, "_SimpleCData");
+  Py_DECREF(ctypes);
+  return g_ctypes_number ? PyModule_Create(&kModule) : nullptr;
+}
