@@ -98,8 +98,10 @@ struct Peers {
 };
 
 struct Sequence {                 // borrowed items of a list or tuple (or of a copy of any other sequence)
-  PyObject* fast;
-  explicit Sequence(PyObject* o) : fast(PySequence_Fast(o, "a sequence is required")) {
+  PyObject* fast = nullptr;
+  explicit Sequence(PyObject* o) {
+    // what has no length (a generator) could be gone through only once
+    if (PyObject_Size(o) >= 0) fast = PySequence_Fast(o, "a sequence is required");
     if (!fast) throw Fail{};
   }
   ~Sequence() { Py_DECREF(fast); }
@@ -108,7 +110,7 @@ struct Sequence {                 // borrowed items of a list or tuple (or of a 
 };
 
 void peers(PyObject* o, Peers* out) {
-  if (o == Py_None) return;
+  if (o == Py_None) return;                       // the library says where that is allowed
   const Sequence s(o);
   out->given = true;
   out->K = s.size();

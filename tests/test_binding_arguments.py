@@ -50,3 +50,14 @@ def test_numbers_of_ctypes_are_taken():
     for n in (1.5, "64", None):
         with pytest.raises(TypeError):
             native.decode(False, [4096], [4096], None, n, 32, 15, 1, X, 0.5, STATUS, None)
+
+
+def test_lists_of_messages_have_a_length():
+    """A generator would be used up by the first of its two readings: the packed form then took every message for
+    empty."""
+    for bad in ((m for m in [BYTES]), iter([BYTES]), 7):
+        with pytest.raises(TypeError):
+            decode(msgs=bad, packed=True)
+    for good in ([BYTES], (BYTES,), {0: 4096}.values()):
+        with pytest.raises(Q.QsgdError, match=NOT_ON_GPU):
+            decode(msgs=good, payload_bytes=[256], packed=True)
