@@ -117,10 +117,19 @@ void peers(PyObject* o, Peers* out) {
   for (uint32_t k = 0; k < out->K && k < QSGD_MAX_PEERS; ++k) out->p[k] = address(s[k]);
 }
 
+// Fewer tables or byte counts than messages: what is missing would read as "none given", and the payload's bound
+// would be gone. (Fixed-width messages have neither: nothing is looked at.)
+void at_least(uint32_t have, const Peers& msgs, int code, const char* name) {
+  if (have >= msgs.K || (code != QSGD_CODE_ELIAS && code != QSGD_CODE_ELIAS_DENSE)) return;
+  PyErr_Format(g_error ? g_error : PyExc_RuntimeError, "%u %s given for %u messages", have, name, msgs.K);
+  throw Fail{};
+}
+
 // Byte counts of the messages: the given list, or (sizes_of_msgs) the sizes of the message tensors.
-const uint64_t* byte_counts(PyObject* o, PyObject* msgs, bool sizes_of_msgs, uint64_t* out) {
+const uint64_t* byte_counts(PyObject* o, PyObject* msgs, const Peers& read, int code, bool sizes_of_msgs, uint64_t* out) {
   if (o == Py_None && !sizes_of_msgs) return nullptr;
   const Sequence s(o == Py_None ? msgs : o);
+  at_least(s.size(), read, code, "byte counts");
   for (uint32_t k = 0; k < s.size() && k < QSGD_MAX_PEERS; ++k) {
     if (o != Py_None) {
       PyObject* v = PyNumber_Long(s[k]);
@@ -237,10 +246,11 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   uint64_t count[QSGD_MAX_PEERS] = {};
   peers(a[1], &msgs);
   peers(a[2], &tables);
-  const uint64_t* bytes = byte_counts(a[3], a[1], packed, count);
+  const int code = i32(a[7]);
+  if (tables.given) at_least(tables.K, msgs, code, packed ? "info words" : "tables");
+  const uint64_t* bytes = byte_counts(a[3], a[1], msgs, code, packed, count);
   const uint64_t n = u64(a[4]);
   const uint32_t bucket = u32(a[5]), s = u32(a[6]);
-  const int code = i32(a[7]);
   const float eta = fused ? f32(a[9]) : 0.f;
   float* out = static_cast<float*>(cuda_tensor(a[8], fused ? "x" : "acc").data_ptr());
   const qsgd_stream_t stream = stream_of(a[11]);
@@ -266,10 +276,11 @@ PyObject* policy_decode(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   uint64_t count[QSGD_MAX_PEERS] = {};
   peers(a[0], &msgs);
   peers(a[1], &tables);
-  const uint64_t* bytes = byte_counts(a[2], a[0], false, count);
   const qsgd_policy* plan = static_cast<const qsgd_policy*>(address(a[3]));
   const uint32_t bucket = u32(a[4]), s = u32(a[5]);
-  const int code = i32(a[6]);
+  const int code = i32(a[6]), lists = plan && !plan->n_buckets ? QSGD_CODE_FIXED : code;      // raw tensors alone: no tables
+  if (tables.given) at_least(tables.K, msgs, lists, "tables");
+  const uint64_t* bytes = byte_counts(a[2], a[0], msgs, lists, false, count);
   const float eta = fused ? f32(a[8]) : 0.f;
   float* out = static_cast<float*>(cuda_tensor(a[7], fused ? "x" : "acc").data_ptr());
   const qsgd_stream_t stream = stream_of(a[10]);

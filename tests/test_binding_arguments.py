@@ -42,8 +42,6 @@ def test_storages_and_other_holders_of_a_data_ptr_are_taken():
 
 def test_numbers_of_ctypes_are_taken():
     native = Q.binding._native
-    native.encode                                          # loads the module
-    native = Q.binding._native
     for n, eta in ((ctypes.c_uint64(64), ctypes.c_float(0.5)), (64, 1)):
         with pytest.raises(Q.QsgdError, match="x " + NOT_ON_GPU):
             native.decode(False, [4096], [4096], None, n, 32, 15, 1, X, eta, STATUS, None)
@@ -61,3 +59,30 @@ def test_lists_of_messages_have_a_length():
     for good in ([BYTES], (BYTES,), {0: 4096}.values()):
         with pytest.raises(Q.QsgdError, match=NOT_ON_GPU):
             decode(msgs=good, payload_bytes=[256], packed=True)
+
+
+@pytest.mark.parametrize("packed", [False, True])
+def test_too_few_tables_or_byte_counts(packed):
+    """What is missing read as a bound that was not given, and the payloads were then read without one."""
+    two = [4096, 8192]
+    for kw in (dict(tables=[4096], payload_bytes=[64, 64]), dict(tables=two, payload_bytes=[64]),
+               dict(tables=two, payload_bytes=[])):
+        with pytest.raises(Q.QsgdError, match="given for 2 messages"):
+            decode(msgs=two, packed=packed, **kw)
+    decoded = dict(msgs=two, tables=two + [16], payload_bytes=[64, 64, 64], packed=packed)      # more are no harm
+    with pytest.raises(Q.QsgdError, match=NOT_ON_GPU):
+        decode(**decoded)
+    native = Q.binding._native
+    for code in (Q.CODE_FIXED, 9):                         # no tables there (9: the library refuses it)
+        with pytest.raises(Q.QsgdError, match=NOT_ON_GPU):
+            native.decode(packed, two, [], [], 64, 32, 15, code, X, None, STATUS, None)
+
+
+def test_too_few_tables_or_byte_counts_under_policy():
+    native, two = Q.binding._native, [4096, 8192]
+    for n_buckets, refused in ((2, True), (0, False)):     # raw tensors alone have no tables
+        plan = Q.binding.PolicyStruct(16, 16, n_buckets, 16, 16, 1, 8, 72, 1)
+        for tables, counts in (([4096], None), (two, [64])):
+            with pytest.raises(Q.QsgdError, match="given for 2 messages" if refused else NOT_ON_GPU):
+                native.policy_decode(two, tables, counts, ctypes.addressof(plan), 32, 15, Q.CODE_ELIAS, X, None, STATUS,
+                                     None)
