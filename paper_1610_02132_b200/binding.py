@@ -271,7 +271,6 @@ class Policy:
         self.struct = PolicyStruct(self.dev["bucket_src"].data_ptr(), self.dev["bucket_len"].data_ptr(), nb,
                                    self.dev["raw_src"].data_ptr(), self.dev["raw_start"].data_ptr(), ns, nr,
                                    self.n, quads.value)
-        self.address = C.addressof(self.struct)
 
 
 def qsgd_policy_message_capacity(plan, s, code_kind):
@@ -292,21 +291,21 @@ def _covered(t, name, plan):
 def qsgd_policy_encode(g, plan, s, norm_kind, code_kind, seed, step, worker, out, out_bits, workspace=None,
                        status_dev=None, stream=None):
     _covered(g, "g", plan)
-    _check(_native.policy_encode(g, plan.address, plan.bucket, s, norm_kind, code_kind, seed, step, worker, out,
+    _check(_native.policy_encode(g, C.addressof(plan.struct), plan.bucket, s, norm_kind, code_kind, seed, step, worker, out,
                                  out_bits, workspace, status_dev, stream))
 
 
 def qsgd_policy_decode_accumulate(msgs, tables, plan, s, code_kind, acc, status_dev, stream=None,
                                   payload_bytes=None):
     _covered(acc, "acc", plan)
-    _check(_native.policy_decode(msgs, tables, payload_bytes, plan.address, plan.bucket, s, code_kind, acc, None,
+    _check(_native.policy_decode(msgs, tables, payload_bytes, C.addressof(plan.struct), plan.bucket, s, code_kind, acc, None,
                                  status_dev, stream))
 
 
 def qsgd_policy_decode_sgd_step(msgs, tables, plan, s, code_kind, x, eta, status_dev, stream=None,
                                 payload_bytes=None):
     _covered(x, "x", plan)
-    _check(_native.policy_decode(msgs, tables, payload_bytes, plan.address, plan.bucket, s, code_kind, x, eta,
+    _check(_native.policy_decode(msgs, tables, payload_bytes, C.addressof(plan.struct), plan.bucket, s, code_kind, x, eta,
                                  status_dev, stream))
 
 

@@ -86,3 +86,16 @@ def test_too_few_tables_or_byte_counts_under_policy():
             with pytest.raises(Q.QsgdError, match="given for 2 messages" if refused else NOT_ON_GPU):
                 native.policy_decode(two, tables, counts, ctypes.addressof(plan), 32, 15, Q.CODE_ELIAS, X, None, STATUS,
                                      None)
+
+
+def test_policy_calls_hand_over_the_struct_that_the_plan_has_now(monkeypatch):
+    seen = []
+    native = types.SimpleNamespace(policy_decode=lambda *a: seen.append(a[3]) or 0)
+    monkeypatch.setattr(Q.binding, "_native", native)
+    monkeypatch.setattr(Q.binding, "_covered", lambda *a: None)
+    plan = types.SimpleNamespace(bucket=32, n=64)
+    structs = [Q.binding.PolicyStruct() for _ in range(2)]
+    for plan.struct in structs:
+        Q.qsgd_policy_decode_accumulate([4096], None, plan, 15, Q.CODE_FIXED, X, STATUS)
+        Q.qsgd_policy_decode_sgd_step([4096], None, plan, 15, Q.CODE_FIXED, X, 0.5, STATUS)
+    assert seen == [ctypes.addressof(s) for s in structs for _ in range(2)]
