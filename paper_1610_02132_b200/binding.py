@@ -13,7 +13,6 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_HERE, "libqsgd.so")
-_NATIVE_PATH = os.path.join(_HERE, "_qsgd_native.so")
 
 NORM_L2, NORM_MAX = 0, 1
 CODE_FIXED, CODE_ELIAS, CODE_ELIAS_DENSE = 0, 1, 2
@@ -124,10 +123,12 @@ class _Native:
 
     def __getattr__(self, name):
         global _native
-        if not os.path.exists(_NATIVE_PATH):
-            raise QsgdError("_qsgd_native.so is not built; run paper_1610_02132_b200.build.build()")
+        from . import build
+        path = build.native_path()
+        if not os.path.exists(path):
+            raise QsgdError("%s is not built; run paper_1610_02132_b200.build.build()" % os.path.basename(path))
         lib()                                             # the library it is linked against: its own message if missing
-        loader = importlib.machinery.ExtensionFileLoader("_qsgd_native", _NATIVE_PATH)
+        loader = importlib.machinery.ExtensionFileLoader("_qsgd_native", path)
         module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_qsgd_native", loader))
         loader.exec_module(module)
         module.set_error(QsgdError)

@@ -1,14 +1,14 @@
-"""Builds libqsgd.so (the C-ABI library with the sm_100a kernels, nvcc) and _qsgd_native.so (its Python
+"""Builds libqsgd.so (the C-ABI library with the sm_100a kernels, nvcc) and _qsgd_native.*.so (its Python
 binding, g++ against the torch headers) in-tree."""
 import glob
 import os
+import re
 import subprocess
 import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libqsgd.so")
-NATIVE = os.path.join(_HERE, "_qsgd_native.so")
 NATIVE_SRC = os.path.join(CSRC, "python_binding.cpp")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -41,12 +41,23 @@ def build_library(force=False, verbose=False):
     return LIB
 
 
+def native_path():
+    """File of the Python binding for the running Python and torch, whose C++ headers it is compiled against: under
+    another of either there is no such file, and it is built instead of an old one being loaded."""
+    import torch
+    key = "torch%s-%d%s" % (torch.__version__, int(torch._C._GLIBCXX_USE_CXX11_ABI), sysconfig.get_config_var("EXT_SUFFIX"))
+    return os.path.join(_HERE, "_qsgd_native." + re.sub(r"[^\w.-]", "_", key))
+
+
 def build_native(force=False):
     """Compile the Python binding; it finds libqsgd.so beside itself and torch's libraries by rpath."""
-    if force or _stale(NATIVE, [NATIVE_SRC] + _headers()):
+    native = native_path()
+    if force or _stale(native, [NATIVE_SRC] + _headers()):
         import torch
         from torch.utils import cpp_extension
-        tmp = NATIVE + ".tmp%d" % os.getpid()
+        for old in glob.glob(os.path.join(_HERE, "_qsgd_native.*so")):      # of another torch or Python
+            os.remove(old)
+        tmp = native + ".tmp%d" % os.getpid()
         inc = cpp_extension.include_paths("cuda") + [sysconfig.get_paths()["include"]]
         libdirs = cpp_extension.library_paths("cuda")
         cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
@@ -56,8 +67,8 @@ def build_native(force=False):
         cmd += ["-L" + p for p in libdirs] + ["-Wl,-rpath," + libdirs[0]]
         cmd += ["-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
         subprocess.check_call(cmd)
-        os.replace(tmp, NATIVE)
-    return NATIVE
+        os.replace(tmp, native)
+    return native
 
 
 def build(force=False, verbose=False):

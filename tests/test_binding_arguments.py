@@ -1,6 +1,7 @@
 """What the Python entry points take for an argument, as far as it shows without a GPU: every call here is refused
 before the library is entered (the parameters are CPU tensors)."""
 import ctypes
+import os
 import types
 
 import pytest
@@ -99,3 +100,18 @@ def test_policy_calls_hand_over_the_struct_that_the_plan_has_now(monkeypatch):
         Q.qsgd_policy_decode_accumulate([4096], None, plan, 15, Q.CODE_FIXED, X, STATUS)
         Q.qsgd_policy_decode_sgd_step([4096], None, plan, 15, Q.CODE_FIXED, X, 0.5, STATUS)
     assert seen == [ctypes.addressof(s) for s in structs for _ in range(2)]
+
+
+def test_native_module_belongs_to_the_torch_and_python_that_run(monkeypatch):
+    """It reads torch's objects directly: one compiled against another torch or Python must not be loaded."""
+    from paper_1610_02132_b200 import build
+    build.build()
+    mine = build.native_path()
+    assert os.path.exists(mine)
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    assert build.native_path() != mine
+    with pytest.raises(Q.QsgdError, match="not built"):
+        Q.binding._Native().encode
+    monkeypatch.undo()
+    monkeypatch.setattr("sysconfig.get_config_var", lambda name: ".cpython-30.so")
+    assert build.native_path() != mine
