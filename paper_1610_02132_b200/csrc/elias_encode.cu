@@ -247,7 +247,7 @@ int run_pipeline(BucketParams& bp, const EliasWs& w, uint32_t s, uint8_t* out, s
     {
       ScopedKernel sk(kKernEliasLength, stream);
       const cudaError_t e = launch_chained(elias_tile_length_kernel<LB, DENSE>, (uint32_t)ctas, kThreads, 0, stream, bp,
-                                           w.cta_sums, sa);
+                                           w.tile_sums, sa);
       if (e != cudaSuccess) return (int)e;
     }
     return launch_tile_scatter(bp, w, s, DENSE, out, stream);

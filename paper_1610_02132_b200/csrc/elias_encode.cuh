@@ -39,6 +39,7 @@ struct EliasWs {
   uint32_t* len;              // L_b
   uint32_t* lane_rec;         // per lane of every bucket team: its bits | (previous nonzero + 1) << 16
   uint64_t* cta_sums;         // per scatter CTA: sum of its buckets' lengths, then exclusive prefix
+  uint64_t* tile_sums;        // the same per tile, where len and lane_rec, which tiles do without, would be
   Ctrl* ctrl;
   size_t bytes;
 };
@@ -72,9 +73,9 @@ inline EliasWs carve(uint8_t* ws, uint64_t n, uint32_t d, uint32_t s) {
   w.fixed = ws + o; o += align16(L.total);
   w.len = reinterpret_cast<uint32_t*>(ws + o); o += align16(4 * L.B);
   w.lane_rec = reinterpret_cast<uint32_t*>(ws + o); o += align16(4 * L.B * tm.lpb);
-  const uint32_t run = tm.nbc < tile_buckets(d) ? tm.nbc : tile_buckets(d);    // buckets per CTA of either kind
-  const uint64_t ctas = (L.B + run - 1) / run;
+  const uint64_t ctas = (L.B + tm.nbc - 1) / tm.nbc;
   w.cta_sums = reinterpret_cast<uint64_t*>(ws + o); o += align16(8 * (ctas + 1));
+  w.tile_sums = reinterpret_cast<uint64_t*>(w.len);     // tiles + 1 <= B + 1 of them: 4 B bytes of len, at least 4 B of lane_rec, 16 of cta_sums
   w.ctrl = reinterpret_cast<Ctrl*>(ws + o); o += align16(sizeof(Ctrl));
   w.bytes = o;
   return w;

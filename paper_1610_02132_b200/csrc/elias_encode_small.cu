@@ -290,7 +290,7 @@ namespace elias {
 
 int launch_tile_scatter(const BucketParams& bp, const EliasWs& w, uint32_t s, bool dense, uint8_t* out, cudaStream_t stream) {
   TileScatterArgs a;
-  a.bp = bp; a.sums = w.cta_sums; a.ctrl = w.ctrl; a.ctas = (uint32_t)((bp.B + bp.nbc - 1) / bp.nbc); a.out = out;
+  a.bp = bp; a.sums = w.tile_sums; a.ctrl = w.ctrl; a.ctas = (uint32_t)((bp.B + bp.nbc - 1) / bp.nbc); a.out = out;
   a.out_capacity = 0; a.out_bits = nullptr; a.status_dev = nullptr;
   return scatter_any(a, s, dense, stream);
 }
@@ -314,7 +314,7 @@ int launch_elias_encode_small(const float* g, uint64_t n, uint32_t d, uint32_t s
   p.log2d = 32;
   if ((d & (d - 1u)) == 0)
     for (p.log2d = 0; (1u << p.log2d) < d; ++p.log2d) {}
-  p.cta_sums = w.cta_sums;
+  p.cta_sums = w.tile_sums;
   p.out = out; p.out_capacity = out_capacity; p.out_bits = out_bits; p.status_dev = status_dev;
   const uint32_t ctas = (uint32_t)((L.B + p.bp.nbc - 1) / p.bp.nbc);
   int st;
@@ -326,7 +326,7 @@ int launch_elias_encode_small(const float* g, uint64_t n, uint32_t d, uint32_t s
   }
   if (st || ctas == 1u) return st;
   TileScatterArgs a;
-  a.bp = p.bp; a.sums = w.cta_sums; a.ctrl = nullptr; a.ctas = ctas; a.out = out;
+  a.bp = p.bp; a.sums = w.tile_sums; a.ctrl = nullptr; a.ctas = ctas; a.out = out;
   a.out_capacity = out_capacity; a.out_bits = out_bits; a.status_dev = status_dev;
   return scatter_any(a, s, dense, stream);
 }
