@@ -107,11 +107,13 @@ constexpr float kTwo125 = 4.253529586511730793292182592897102643e+37f;
 // sign bit into `sw`. `um` is the bit pattern m = top 24 Philox bits read as an fp32, i.e. m * 2^-149.
 // RAW_SIGN: push the sign bit of v as it is; the caller clears the signs of zero levels afterwards
 // with a mask derived from the packed level words (cheaper than two more operations per coordinate
-// when a word holds many fields).
-template <bool RAW_SIGN, bool CLAMP>
+// when a word holds many fields). NAN_ZERO: a t that is no number (a NaN coordinate, or an infinite one in its own
+// infinite scale) gives level 0 instead of s.
+template <bool RAW_SIGN, bool CLAMP, bool NAN_ZERO = false>
 __device__ __forceinline__ uint32_t quantize_one(float v, float r, float sf, float cap, float um,
                                                  uint32_t& sw) {
-  const float t = __fmul_rn(__fmul_rn(sf, fabsf(v)), r);
+  float t = __fmul_rn(__fmul_rn(sf, fabsf(v)), r);
+  if (NAN_ZERO) t = fmaxf(t, 0.0f);
   const float c = fma_rn(um, kTwo125, t);                    // t + m * 2^-24, one rounding
   float fl = __fadd_rd(c, kTwo23);                           // 2^23 + floor(c)
   if (CLAMP) fl = fminf(fl, cap);                            // 2^23 + min(floor(c), s)
@@ -339,7 +341,7 @@ __device__ __forceinline__ void quantize_generic_tile(const QuantizeParams& p, u
     uint32_t sb = 0, lo = 0, hi = 0;             // fields of coordinates 0 .. 3 and 4 .. 7 (LB = 8), else of all in lo
 #pragma unroll
     for (int e = 7; e >= 0; --e) {
-      const uint32_t bits = quantize_one<false, true>(v[j][e], r, sf, kTwo23 + sf, __uint_as_float(rnd[e] >> 8), sb);
+      const uint32_t bits = quantize_one<false, true, true>(v[j][e], r, sf, kTwo23 + sf, __uint_as_float(rnd[e] >> 8), sb);
       if (LB == 8 && e >= 4) hi = hi * 256u + bits;
       else lo = lo * (1u << LB) + bits;
     }
