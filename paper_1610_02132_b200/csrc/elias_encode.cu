@@ -267,9 +267,11 @@ int run_pipeline(BucketParams& bp, const EliasWs& w, uint32_t s, uint8_t* out, s
   {
     const size_t smem = stage_bytes<DENSE>(tm.nbc, bp.d, s);
     auto kern = elias_scatter_kernel<LB, DENSE>;
-    if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return (int)e;
+    if (smem > 48 * 1024) {                        // the opt-in is raised only: threads with other s share it
+      static KernelSite site;
+      int sms = 0, occ = 0;
+      const int st = site.lookup_dynamic(kern, kThreads, smem, &sms, &occ);
+      if (st) return st;
     }
     ScopedKernel sk(kKernEliasScatter, stream);
     return (int)launch_chained(kern, (uint32_t)ctas, kThreads, smem, stream, bp, w.len, w.lane_rec, w.cta_sums, w.ctrl, out);

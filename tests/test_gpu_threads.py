@@ -57,3 +57,36 @@ def test_threads_on_their_own_streams():
         st2, acc = O.decode_accumulate([m], tabs, n, d, s, code_kind)
         assert st2 == 0
         assert np.array_equal(x.view(np.uint32), O.sgd_step(np.zeros(n, np.float32), acc, -1.0, 1).view(np.uint32))
+
+
+def test_threads_whose_kernels_share_an_opt_in():
+    """Two threads whose scatter kernel is the same one with different amounts of shared memory above 48 KB (about 66
+    and 53 KB): neither may lower the other's limit between its request and its launch."""
+    n, d = 6 * 2 ** 20 + 4 * 4096, 4096                   # beyond the problems that go by tiles
+    g = I.gaussian_device(n, 1.0, seed=5)
+    first, errors = {}, []
+
+    def work(s):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                cap = Q.qsgd_message_capacity(n, d, s, O.CODE_ELIAS)
+                out, bits = torch.zeros(cap, dtype=torch.uint8, device="cuda"), torch.zeros(4, dtype=torch.int64, device="cuda")
+                ws = torch.empty(Q.qsgd_workspace_bytes(n, d, s, O.CODE_ELIAS), dtype=torch.uint8, device="cuda")
+                status = Q.new_status()
+                for rep in range(200):
+                    Q.qsgd_encode(g, d, s, O.NORM_MAX, O.CODE_ELIAS, 7, 0, 0, out, bits, ws, status)
+                    if rep == 0:
+                        first[s] = out.clone()
+                stream.synchronize()
+                assert int(status.item()) == 0 and torch.equal(out, first[s])
+        except Exception as e:                         # pragma: no cover
+            errors.append(repr(e))
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(s,)) for s in (255, 16)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not errors, errors
