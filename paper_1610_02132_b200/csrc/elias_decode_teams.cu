@@ -531,6 +531,12 @@ int launch_elias_teams(const FieldParams& f, bool dense, bool fused, cudaStream_
   p.buckets = 1;
   while (p.buckets * 2u * p.Kc * p.T <= kThreads && p.buckets * 2u <= p.B && bytes(p.buckets * 2u, p.Kc) <= (64u << 10)) p.buckets *= 2u;
   while (p.T < 32u && p.buckets * p.Kc * p.T * 2u <= kThreads) p.T <<= 1;
+  // Many peers: fewer lanes per string and one pass over the strings, not several with each its own latency, unless the
+  // strings are long enough for the lanes' work to count (K = 17 to 48, s > 3, d >= 1024: up to a quarter slower). Small
+  // problems of Code_s, s = 1, several passes against one (us): n = 57 K, d = 1024, K = 17 31.5 / 9.1, n = 118 K, d = 1024, K = 32
+  // 45.0 / 10.2.
+  if (p.d < 1024u || p.K <= 16u || p.s <= 3u)
+    while (p.T > 4u && p.buckets * p.Kc * p.T > kThreads) p.T >>= 1;
   const size_t smem = align16(bytes(p.buckets, p.Kc));
 #define QSGD_RUN(D, W) launch_width<D, W>(p, fused, smem, stream)
   if (dense) return width == kNibble ? QSGD_RUN(true, kNibble) : width == kByte ? QSGD_RUN(true, kByte) : QSGD_RUN(true, kWide);

@@ -60,3 +60,12 @@ def test_fewer_bits_do_not_take_longer_in_the_dense_code():
     few, many = time_of(small, large)
     assert few < 1.2 * many
     assert int(small.status.item()) == int(large.status.item()) == 0
+
+
+def test_many_peers_of_a_small_problem_are_read_in_one_pass():
+    """32 short strings a bucket against 8: more to add up, but no more latencies in a row."""
+    n, d = 16 * 1024, 1024
+    make = lambda w: I.gaussian_mixture_device(n, seed=w)
+    eight, all32 = (decode(n, d, 1, O.NORM_L2, O.CODE_ELIAS, K, make) for K in (8, 32))
+    few, many = time_of(eight, all32)
+    assert many < 2.0 * few
