@@ -52,13 +52,15 @@ inline uint32_t tile_buckets(uint32_t d) { return kTileCoords / d; }
 constexpr uint32_t kSmallTiles = 1000;
 
 // By teams (a lane walks 64 coordinates or more: less work per coordinate) or by tiles (a thread has 16: done
-// sooner)? Whole encodes measured both ways on two input families, teams against tiles (us). Tiles in two kernels:
+// sooner)? Whole encodes measured both ways on three input families, teams against tiles (us). Tiles in two kernels:
 // 20.4 / 8.8 at n = 2^20, 18.5 to 26.4 / 17.5 to 21.9 at 3 * 2^20, 20.2 to 28.0 / 20.6 to 26.5 at 1000 tiles
-// (d = 512, s = 15); tiles in three kernels, s = 255: 49 / 47 at 6 * 2^20; Code'_s with d = 512 36 / 39 at
-// 6 * 2^20, with d = 4096 (128 coordinates a lane) 56 / 49 at 2^23, 173 / 176 at 2^25.
+// (d = 512, s = 15); beyond 1000 tiles, where they take three kernels, only for levels above 15: Code_s up to
+// 6 * 2^20 coordinates 0.43 to 1.17 of the time by teams, Code'_s with d > 1024 (128 coordinates a lane) up to 20 * 2^20
+// 0.66 to 1.15. Code'_s with smaller levels, whose symbols cost a lane little, 0.87 to 1.34 from there on (n = 19 M,
+// d = 4096, s = 1: 74 / 98).
 inline bool use_tiles(uint64_t n, uint32_t d, uint32_t s, bool dense) {
   if (n <= kSmallTiles * 4096ull) return true;
-  const uint64_t m = dense ? (d > 1024u ? 20u : 4u) : s > 15u ? 6u : 2u;
+  const uint64_t m = s <= 15u ? 0u : !dense ? 6u : d > 1024u ? 20u : 0u;
   return n <= m << 20;
 }
 inline bool use_small(uint64_t n, uint32_t d, const BucketMap& map) {

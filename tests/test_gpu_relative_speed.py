@@ -1,4 +1,4 @@
-"""Decodes that must not fall behind others of the same size: ratios of times of one and the same run, with room for
+"""Calls that must not fall behind others of the same size: ratios of times of one and the same run, with room for
 noise. What is compared is device time (a graph of several calls, replayed; the shortest replay)."""
 import pytest
 import torch
@@ -69,3 +69,17 @@ def test_many_peers_of_a_small_problem_are_read_in_one_pass():
     eight, all32 = (decode(n, d, 1, O.NORM_L2, O.CODE_ELIAS, K, make) for K in (8, 32))
     few, many = time_of(eight, all32)
     assert many < 2.0 * few
+
+
+def encode(n, d, s, norm, code):
+    g, status = I.gaussian_device(n, 1.0, seed=3), Q.new_status()
+    out = torch.empty(Q.qsgd_message_capacity(n, d, s, code), dtype=torch.uint8, device="cuda")
+    info = torch.zeros(4, dtype=torch.int64, device="cuda")
+    ws = torch.empty(Q.qsgd_workspace_bytes(n, d, s, code), dtype=torch.uint8, device="cuda")
+    return lambda: Q.qsgd_encode(g, d, s, norm, code, 7, 0, 0, out, info, ws, status)
+
+
+def test_dense_encode_grows_no_faster_than_its_length():
+    """Small levels: 18 M coordinates against 24 M, which no rule sends through kernels meant for few."""
+    less, more = time_of(*(encode(n, 4096, 1, O.NORM_L2, O.CODE_ELIAS_DENSE) for n in (18 * 2 ** 20, 24 * 2 ** 20)))
+    assert less < 0.88 * more                              # 0.75 by length alone; 1.0 by tiles
