@@ -309,6 +309,9 @@ class HotPath:
         return float(np.mean(self.info[code][:, 0].astype(np.float64))) / self.n
 
 
+ELIAS_DECODERS = ("decode_elias", "decode_elias_sparse", "decode_elias_teams", "decode_elias_fields")
+
+
 def kernel_algorithmic_bytes(hp, code_name):
     """Bytes each kernel must move per launch (the method's own inputs and outputs)."""
     d, s, K, B = hp.d, hp.s, hp.K, hp.B
@@ -322,8 +325,8 @@ def kernel_algorithmic_bytes(hp, code_name):
         info = hp.info[elias_code]
         msg = float(np.mean(info[:, 2].astype(np.float64))) - hp.prefix
         pay = float(np.mean(info[:, 1].astype(np.float64))) - hp.prefix
-        out.update({"decode_elias": K * msg + 8 * n, "decode_elias_sparse": K * msg + 8 * n,
-                    "elias_scatter": MF + pay + 8 * (B + 1),
+        out.update({name: K * msg + 8 * n for name in ELIAS_DECODERS})
+        out.update({"elias_scatter": MF + pay + 8 * (B + 1),
                     "elias_length": MF - 4 * ((n + 31) // 32) + 4 * B})
         break
     return out
@@ -461,15 +464,14 @@ def run_cuda(args):
     alg = kernel_algorithmic_bytes(hp, None)
     kern_tab = {k: {"ms_total": v[0], "launches": v[1], "avg_us": 1e3 * v[0] / v[1]} for k, v in kern.items()}
     tot = sum(v[0] for v in kern.values()) or 1.0
-    # In the packed form both Elias decoders are launched and one of them returns after reading the
-    # payload lengths: that one moved no message bytes and gets no bandwidth figure.
-    stood_down = None
-    if "decode_elias" in kern_tab and "decode_elias_sparse" in kern_tab:
-        stood_down = min(("decode_elias", "decode_elias_sparse"), key=lambda k: kern_tab[k]["avg_us"])
-        kern_tab[stood_down]["stood_down"] = True
+    # In the packed form several Elias decoders are launched and all but one of them return after reading the
+    # payload lengths: those moved no message bytes and get no bandwidth figure.
+    stood_down = sorted((k for k in kern_tab if k in ELIAS_DECODERS), key=lambda k: kern_tab[k]["avg_us"])[:-1]
+    for k in stood_down:
+        kern_tab[k]["stood_down"] = True
     for k in kern_tab:
         kern_tab[k]["share"] = kern_tab[k]["ms_total"] / tot
-        if k in alg and k != stood_down:
+        if k in alg and k not in stood_down:
             kern_tab[k]["alg_GBps"] = alg[k] / (kern_tab[k]["avg_us"] * 1e-6) / 1e9
             kern_tab[k]["frac_of_%s_hbm" % peak_src] = kern_tab[k]["alg_GBps"] / hbm_peak
     dom = max(kern, key=lambda k: kern[k][0])

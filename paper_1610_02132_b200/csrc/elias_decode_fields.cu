@@ -218,7 +218,7 @@ int launch_fields(FieldParams& p, bool fused, cudaStream_t stream) {
   const uint64_t groups = (p.B + G - 1) / G;
   const uint64_t want = (groups + warps - 1) / warps;
   const uint64_t cap = (uint64_t)sms * occ;
-  ScopedKernel sk(kKernDecodeElias, stream);
+  ScopedKernel sk(kKernDecodeEliasFields, stream);
   return (int)launch_chained(kern, (uint32_t)(want < cap ? want : cap), warps * 32, smem, stream, p);
 }
 

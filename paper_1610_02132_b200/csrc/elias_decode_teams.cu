@@ -499,7 +499,7 @@ int launch_width(TeamParams& p, bool fused, size_t smem, cudaStream_t stream) {
   const int st = site[fused ? 1 : 0].lookup_dynamic(kern, kThreads, smem, &sms, &occ);
   if (st) return st;
   const uint64_t groups = (p.B + p.buckets - 1) / p.buckets, cap = (uint64_t)sms * occ;
-  ScopedKernel sk(kKernDecodeElias, stream);
+  ScopedKernel sk(kKernDecodeEliasTeams, stream);
   return (int)launch_chained(kern, (uint32_t)(groups < cap ? groups : cap), kThreads, smem, stream, p);
 }
 

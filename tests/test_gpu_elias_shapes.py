@@ -1,8 +1,8 @@
 """Elias Encode and Decode at the edges of their dispatch rules: problems read by teams of lanes (parts of a
 string shorter and longer than a lane's least part, peers in several passes, codes on which a reader that
-starts out of step stays out of step), streams read by table (buckets shorter and longer than a ring, gaps that
-the table does not hold, malformed strings inside a stream) and encoded in tiles (tiles of whole buckets, sizes around a tile, both
-sides of the line to the team kernels). Bit for bit against the oracle."""
+starts out of step stays out of step; long gaps, empty buckets and malformed strings among many strings) and encoded in
+tiles (tiles of whole buckets, sizes around a tile, both sides of the line to the team kernels). Bit for bit against the
+oracle. The decoders with a lane per string have their shapes in test_gpu_elias_decoders.py."""
 import numpy as np
 import pytest
 import torch
@@ -62,7 +62,8 @@ def test_teams_out_of_step(code, s, value):
     (1600 * 256 + 9, 256, 15, MAX, 8), (800 * 512 + 3, 512, 15, L2, 17), (500 * 1024 + 7, 1024, 1, MAX, 32), (1600 * 2048 + 2047, 2048, 15, L2, 9),
 ])
 def test_streams(n, d, s, norm, K):
-    """A lane per (run of buckets, peer). Every other peer's strings have long gaps and empty buckets."""
+    """Many strings, up to half of those that get a lane each. Every other peer's strings have long gaps and empty
+    buckets."""
     def make(w):
         if w % 2 == 0:
             return I.gaussian(n, 1.0, seed=50 + w)
@@ -75,7 +76,7 @@ def test_streams(n, d, s, norm, K):
 
 @pytest.mark.parametrize("d,K", [(32, 1), (512, 16), (1024, 24)])
 def test_malformed_streams(d, K):
-    """Streams with noise, strings cut short and offsets out of order in one peer's message: flagged, nothing
+    """Noise, strings cut short and offsets out of order in one peer's message: flagged, nothing
     written out of bounds, and where only one string is bad the buckets of the others come out right."""
     import paper_1610_02132_b200 as Q
     B = 13000 // K + 1

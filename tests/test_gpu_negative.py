@@ -11,12 +11,12 @@ from paper_1610_02132_b200 import inputs as I
 
 pytestmark = pytest.mark.gpu
 
-# (n, d, s, input): one shape per Elias decoder -- whole-bucket fields (d < 1024), fields by ranges
-# (d >= 1024), and the entry-list decoder of the sparse regime (short strings)
+# (n, d, s, input): short and long buckets and short strings. All are small problems, which go to the teams of lanes;
+# test_gpu_elias_decoders.py has malformed messages for every Elias decoder.
 SHAPES = [(4096 + 300, 512, 3, "gauss"), (2 * 4096 + 300, 4096, 3, "gauss"), (3 * 4096 + 300, 4096, 1, "sparse")]
 
 
-@pytest.fixture(params=SHAPES, ids=["fields", "ranged", "sparse"])
+@pytest.fixture(params=SHAPES, ids=["short_buckets", "long_buckets", "short_strings"])
 def shape(request):
     return request.param
 

@@ -216,16 +216,17 @@ def sparse_regime_bits(K, d):
     return 32 + d // 4
 
 
-# Short strings (Section 3.1, sparse regime) take the entry-list decoder; these cases sit on
-# that side of its switch, which is decided on the device from the payload lengths.
+# Short strings (Section 3.1, sparse regime): the larger ones of these cases take the entry-list decoder, on the side of
+# its switch which they are on (decided on the device from the payload lengths); small ones are read by teams.
 @pytest.mark.parametrize("n,d,s,K,zeros", [(5 * 4096 + 123, 4096, 1, 8, 0.3), (9 * 1024 + 77, 1024, 1, 5, 0.3),
                                            (11 * 3008 + 5, 3008, 1, 3, 0.3), (4 * 2048, 2048, 1, 32, 0.3),
                                            (3 * 4096 + 1, 4096, 1, 1, 0.3), (70 * 64 + 9, 64, 3, 16, 0.98),
                                            # enough buckets that a warp takes its full share of them
                                            (7200 * 64 + 5, 64, 1, 8, 0.98), (14300 * 128 + 3, 128, 1, 3, 0.95),
                                            (57000 * 32 + 31, 32, 1, 1, 0.98),
-                                           # few buckets of a size that is no power of two, one or two peers:
-                                           # one bucket per warp, lists of 928 / 32 = 29 and 608 / 32 = 19 entries
+                                           # few buckets of a size that is no power of two, one or two peers (lists of
+                                           # 29 and 19 entries: in test_gpu_elias_decoders.py, with buckets enough for
+                                           # the entry-list decoder to be asked)
                                            (46 * 928, 928, 1, 1, 0.3), (30 * 608 - 3, 608, 1, 2, 0.7)])
 @pytest.mark.parametrize("eta", [0.1, -0.25])
 def test_elias_sparse_regime(n, d, s, K, zeros, eta):
