@@ -11,10 +11,16 @@ namespace qsgd {
 
 namespace {
 
-// Coordinates x peers up to which the sparse-regime decoder is not considered beside the teams: one launch
-// less, and a string's latency decides (n = 2^20, d = 4096, s = 1, K = 8: 16.7 against 31.4 us; at 2^22 41.0
-// against 33.9).
+// Coordinates x peers up to which the sparse-regime decoder is not launched beside the teams (one launch less, and a
+// string's latency decides: n = 2^20, d = 4096, s = 1, K = 8 in the packed form 15.5 against 27.3 us; at 2^22 41.0 against
+// 33.9), and has to itself only what sparse_though_small gives it.
 constexpr uint64_t kSmallWork = 8ull << 20;
+
+// Strings of a small problem that are known to be short, `mean` bits behind the scale: a lane reads one as fast as a team
+// does, and the sums of a bucket are spread over the warps better. 482 such problems measured, sparse-regime decoder
+// against teams: up to 300 bits, with at most 8 peers or more than 2 M coordinates x peers, 0.42 to 1.36 of the time
+// (n = 54 K, d = 1024, s = 1, K = 4 8.0 / 12.3 us); the others 0.68 to 2.7 (n = 57 K, d = 1024, s = 1, K = 17 10.4 / 9.1).
+bool sparse_though_small(uint64_t mean, uint32_t K, uint64_t work) { return mean < 300u && (K <= 8u || work > (2ull << 20)); }
 
 // A lane per string (or stream of strings), or a team of lanes? A lane per string is the cheaper reading (a team
 // reads its string almost twice) but needs strings enough for the GPU's lanes, and room in shared memory for the whole
@@ -52,8 +58,9 @@ int launch_decode_elias(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
   f.peers = peers; f.K = K; f.n = n; f.d = d; f.s = s; f.B = B;
   f.out = acc_or_x; f.c = eta / (float)K; f.minus_zero = -0.f; f.status = status_dev; f.map = map;
   const bool teams = use_teams(B, K, d, s, dense);
+  const bool small = teams && n * K <= kSmallWork;
   bool sparse = false;
-  if (!dense && (host_sparse || !sizes_known) && !(teams && n * K <= kSmallWork)) {
+  if (!dense && (host_sparse ? !small || sparse_though_small(payload_bits / (K * B) - 32u, K, n * K) : !sizes_known && !small)) {
     const int st = launch_elias_sparse(peers, K, n, d, s, acc_or_x, fused, f.c, status_dev, !sizes_known, map, stream, &sparse);
     if (st) return st;
     if (sparse && sizes_known) return 0;                    // the host chose the sparse-regime kernel

@@ -32,10 +32,14 @@ SHAPES = [
 
 
 def worker(call):
-    """The Elias decoder that did the work of a call: the others only stand down."""
+    """The Elias decoder that did the work of a call: the others only stand down. The call's launches queue up behind
+    other work, so that their times hold no time of the host."""
+    other = torch.empty(2 ** 28, device="cuda")
     Q.qsgd_profile_enable(True)
     try:
         Q.qsgd_profile_collect()
+        for _ in range(4):
+            other.zero_()
         call()
         torch.cuda.synchronize()
     finally:
@@ -107,3 +111,17 @@ def test_malformed_messages(name, B, missing, d, s, norm, K, long_gaps):
             if only >= 0:
                 same[only * d: (only + 1) * d] = True
             assert same.all()
+
+
+@pytest.mark.parametrize("n,d,s,K,name", [(54272, 1024, 1, 4, "decode_elias_sparse"), (431883, 4096, 1, 1, "decode_elias_sparse"),
+                                          (13345 * 480, 480, 1, 1, "decode_elias_sparse"), (57037, 1024, 1, 17, "decode_elias_teams")])
+def test_short_strings_of_small_problems(n, d, s, K, name):
+    """The sizes read off the pointers (a table right behind its payload) choose, in one launch."""
+    sent = [encode_parity(I.gaussian_mixture(n, seed=w), d, s, L2, ELIAS, 7, 3, w) for w in range(min(K, 3))]
+    msgs, infos = [sent[k % 3][0] for k in range(K)], [sent[k % 3][1] for k in range(K)]
+    decode_parity(msgs, infos, n, d, s, ELIAS, eta=0.05)
+    B = O.n_buckets(n, d)
+    tables = [m[i[1]: i[1] + 8 * (B + 1)].view(torch.int64) for m, i in zip(msgs, infos)]
+    acc, status, before = torch.empty(n, device="cuda"), Q.new_status(), Q.qsgd_launch_count()
+    assert worker(lambda: Q.qsgd_decode_accumulate(msgs, tables, n, d, s, ELIAS, acc, status)) == name
+    assert Q.qsgd_launch_count() == before + 1
