@@ -309,7 +309,8 @@ class HotPath:
         return float(np.mean(self.info[code][:, 0].astype(np.float64))) / self.n
 
 
-ELIAS_DECODERS = ("decode_elias", "decode_elias_sparse", "decode_elias_teams", "decode_elias_fields")
+ELIAS_DECODERS = ("decode_elias", "decode_elias_sparse", "decode_elias_teams", "decode_elias_fields",
+                  "decode_elias_bytes")
 
 
 def kernel_algorithmic_bytes(hp, code_name):

@@ -86,13 +86,19 @@ __device__ __forceinline__ StringRef string_ref(const PeerSet& ps, uint32_t k, u
   return r;
 }
 
-// Strings short enough for the entry-list decoder? True when the K payloads average less than a
-// quarter of a bit per coordinate beyond the scales: an entry of a sparse bucket costs 11 to 14
-// bits, so a list with room for one entry per 32 positions then fills to about 60 % on average and
-// rarely overflows. Called by every thread of a CTA (it holds CTA barriers): K threads read the K
-// payload lengths side by side and add them up in shared memory, so a kernel that only has to stand
-// down costs one round of loads per CTA. Same answer in every kernel that asks.
-__device__ __forceinline__ bool sparse_regime(const PeerSet& peers, uint32_t K, uint64_t B, uint32_t d) {
+// Which of several decoders launched one after the other does the work? The one in whose regime the mean length of a
+// string lies, in bits behind the scale: lo <= mean < hi. Any decoder is right on any input, the choice is about speed
+// only. lo = 0 and hi = kNoBound: not asked.
+constexpr uint32_t kNoBound = 0xFFFFFFFFu;
+struct Regime {
+  uint32_t lo, hi;
+};
+
+// Mean below `line`? Called by every thread of a CTA (it holds CTA barriers): K threads read the K payload lengths side by
+// side and add them up in shared memory, so that a kernel that only has to stand down costs one round of loads per CTA.
+// Same answer in every kernel that asks. Messages whose table is in a bad place are not short: the kernel for the long
+// ones reports them.
+__device__ __forceinline__ bool mean_below(uint32_t line, const PeerSet& peers, uint32_t K, uint64_t B) {
   __shared__ unsigned long long total_bits;
   __shared__ uint32_t bad_place;
   if (threadIdx.x == 0) { total_bits = 0ull; bad_place = 0u; }
@@ -100,11 +106,11 @@ __device__ __forceinline__ bool sparse_regime(const PeerSet& peers, uint32_t K, 
   // thread k reads peer k's payload length: the K pairs of dependent loads run side by side
   for (uint32_t k = threadIdx.x; k < K; k += blockDim.x) {
     PeerTable pt;
-    if (!peer_table(peers, k, B, &pt)) atomicOr(&bad_place, 1u);     // the field decoders report the bad place
+    if (!peer_table(peers, k, B, &pt)) atomicOr(&bad_place, 1u);
     else atomicAdd(&total_bits, (unsigned long long)__ldg(pt.table + B));
   }
   __syncthreads();
-  return K <= 32u && bad_place == 0u && total_bits < (uint64_t)K * B * (32ull + d / 4u);
+  return bad_place == 0u && total_bits < (uint64_t)K * B * (32ull + line);
 }
 
 struct FieldParams {
@@ -122,7 +128,7 @@ struct FieldParams {
   uint32_t row_words;   // per peer row: d * lb / 32 level words, then d / 32 sign words (padded to 4)
   uint32_t bucket_words;  // K rows + K scales, padded to 4
   float minus_zero;       // -0 (LevelQuotient)
-  uint32_t defer_sparse;  // a sparse-regime kernel was launched beside this one
+  Regime when;
   BucketMap map;          // where the buckets live in `out` (per-tensor policy), or no map
 };
 
@@ -179,7 +185,7 @@ struct SparseParams {
   uint32_t* status;
   uint32_t warp_words;   // shared-memory words per warp: G * R sums, 64 of scales and counts, 32 lists
   uint32_t quad_shift;   // log2(R / 4) when R is a power of two, else 32
-  uint32_t check_regime; // 0: the host already knows that this kernel is the one to run
+  Regime when;
   BucketMap map;         // where the buckets live in `out` (per-tensor policy), or no map
 };
 
@@ -332,12 +338,11 @@ __device__ __forceinline__ uint32_t advance(LaneParse& st, uint32_t rend, uint32
   return n;
 }
 
-// Launchers of the decoders; 0 or a cudaError_t. `launched`: whether the sparse-regime kernel takes the shape.
+// Launchers of the decoders; 0 or a cudaError_t.
 int launch_elias_ring(const FieldParams& p, bool fused, cudaStream_t stream);     // Code_s, s <= 15, at most 32 peers
-int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream);         // Code_s, s > 15, at most 32 peers
+int launch_elias_bytes(const FieldParams& p, bool fused, cudaStream_t stream);    // the same
+int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream);         // Code_s, s > 15, d < 512, at most 32 peers
+int launch_elias_sparse(const FieldParams& p, bool fused, cudaStream_t stream);   // Code_s, at most 32 peers
 int launch_elias_teams(const FieldParams& p, bool dense, bool fused, cudaStream_t stream);
-int launch_elias_sparse(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d, uint32_t s, float* out, bool fused,
-                        float c, uint32_t* status, bool check_regime, const BucketMap& map, cudaStream_t stream,
-                        bool* launched);
 
 }  // namespace qsgd

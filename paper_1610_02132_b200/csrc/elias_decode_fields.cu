@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
   extern __shared__ __align__(16) uint32_t fsm[];
   __shared__ uint2 code[kCodeEntries];
   chain_wait();                                   // the messages come from the kernels ahead
-  if (p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
+  if (p.when.lo && mean_below(p.when.lo, p.peers, p.K, p.B)) return;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   for (uint32_t i = tid; i < kCodeEntries; i += blockDim.x) code[i] = code_entry(i);
   __syncthreads();

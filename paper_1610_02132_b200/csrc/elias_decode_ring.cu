@@ -88,7 +88,7 @@ struct RingParams {
   uint32_t run;           // buckets per run
   uint32_t slots;         // scales kept per lane, a power of two: the buckets that a ring can touch
   uint32_t warp_bytes;
-  uint32_t defer_sparse;  // a sparse-regime kernel was launched beside this one
+  Regime when;
   BucketMap map;
 };
 
@@ -152,9 +152,9 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
   extern __shared__ __align__(16) uint8_t ring_shared[];
   __shared__ uint32_t tab[2u * kTabWords];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-  if (p.defer_sparse) {                           // standing down should cost little: before the table is made
+  if (p.when.lo) {                                // standing down should cost little: before the table is made
     chain_wait();
-    if (sparse_regime(p.peers, p.K, p.B, p.d)) return;
+    if (mean_below(p.when.lo, p.peers, p.K, p.B)) return;
   }
   for (uint32_t i = tid; i < 2u * kTabWords; i += blockDim.x) tab[i] = ring_entry(i & (kTabWords - 1u), i >= kTabWords, p.s);
   const uint32_t G = 32u / p.Kpad, g = lane / p.Kpad, k = lane % p.Kpad, rows = G * p.K;
@@ -437,7 +437,7 @@ int launch_elias_ring(const FieldParams& f, bool fused, cudaStream_t stream) {
   static KernelSite site[4];
   RingParams p;
   p.peers = f.peers; p.K = f.K; p.n = f.n; p.d = f.d; p.s = f.s; p.B = f.B; p.out = f.out; p.c = f.c;
-  p.status = f.status; p.map = f.map; p.defer_sparse = f.defer_sparse;
+  p.status = f.status; p.map = f.map; p.when = f.when;
   p.Kpad = 1;
   while (p.Kpad < p.K) p.Kpad <<= 1;
   const uint32_t G = 32u / p.Kpad;

@@ -8,9 +8,9 @@
 // turn in the k order, adding straight into the tile. In the fused step, groups of four
 // coordinates whose sums are all +0 are left untouched: for c >= 0, x - c * (+0) is x bit for bit.
 //
-// Who runs: when the host can read the payload sizes off the pointers it launches this kernel alone
-// (check_regime = 0). Otherwise this kernel and a field-rebuilding kernel are launched back to back,
-// each evaluates the same predicate on the payload lengths, and exactly one of them does the work.
+// Who runs: when the host can read the payload sizes off the pointers it launches one kernel. Otherwise this one and
+// one or two others are launched back to back, and on the device the mean length of the strings says which one does the
+// work (Regime).
 #include "elias_decode.cuh"
 
 namespace qsgd {
@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(256, 2) decode_elias_sparse_kernel(const __gri
   extern __shared__ __align__(16) uint32_t ssm[];
   __shared__ float xi[256];
   chain_wait();                                   // the messages come from the kernels ahead
-  if (p.check_regime && !sparse_regime(p.peers, p.K, p.B, p.d)) return;
+  if (p.when.hi != kNoBound && !mean_below(p.when.hi, p.peers, p.K, p.B)) return;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   const uint32_t G = p.sh.G, Kpad = p.sh.Kpad, R = p.sh.R, C = p.sh.C;
   for (uint32_t i = tid; i < 256; i += blockDim.x) xi[i] = __fdiv_rn((float)i, (float)p.s);
@@ -212,22 +212,15 @@ __global__ void __launch_bounds__(256, 2) decode_elias_sparse_kernel(const __gri
 
 }  // namespace
 
-// Launches the sparse-regime kernel when the configuration allows one (K <= 32, Code_s); the
-// caller then tells the other decoders to stand down when the predicate holds.
-int launch_elias_sparse(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d, uint32_t s, float* out, bool fused,
-                        float c, uint32_t* status, bool check_regime, const BucketMap& map, cudaStream_t stream,
-                        bool* launched) {
-  *launched = false;
-  if (K > 32u) return 0;
+int launch_elias_sparse(const FieldParams& f, bool fused, cudaStream_t stream) {
   static KernelSite site[2];
   int sms = 0;
   const int st0 = device_sms(&sms);
   if (st0) return st0;
   SparseParams p;
-  p.peers = peers; p.K = K; p.n = n; p.d = d; p.s = s;
-  p.B = (n + d - 1) / d;
-  p.sh = sparse_shape(K, d, p.B, (uint32_t)sms);
-  p.out = out; p.c = c; p.status = status; p.check_regime = check_regime ? 1u : 0u; p.map = map;
+  p.peers = f.peers; p.K = f.K; p.n = f.n; p.d = f.d; p.s = f.s; p.B = f.B;
+  p.sh = sparse_shape(p.K, p.d, p.B, (uint32_t)sms);
+  p.out = f.out; p.c = f.c; p.status = f.status; p.when = f.when; p.map = f.map;
   p.warp_words = p.sh.G * p.sh.R + 64u + p.sh.G * p.sh.Kpad * p.sh.C;
   p.quad_shift = 32;
   const uint32_t tile_quads = p.sh.R >> 2;
@@ -255,13 +248,8 @@ int launch_elias_sparse(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
   const uint64_t want = (groups + warps - 1) / warps;
   const uint64_t cap = (uint64_t)sms * occ;
   const uint32_t grid = (uint32_t)(want < cap ? want : cap);
-  {
-    ScopedKernel sk(kKernDecodeEliasSparse, stream);
-    const cudaError_t le = launch_chained(kern, grid, warps * 32, smem, stream, p);
-    if (le != cudaSuccess) return (int)le;
-  }
-  *launched = true;
-  return 0;
+  ScopedKernel sk(kKernDecodeEliasSparse, stream);
+  return (int)launch_chained(kern, grid, warps * 32, smem, stream, p);
 }
 
 }  // namespace qsgd

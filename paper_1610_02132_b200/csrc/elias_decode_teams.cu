@@ -63,7 +63,7 @@ struct TeamParams {
   uint32_t T;             // lanes per string, a power of two
   uint32_t buckets;       // per CTA and pass
   uint32_t row_bytes;
-  uint32_t defer_sparse;  // a sparse-regime kernel was launched beside this one
+  Regime when;
   BucketMap map;
 };
 
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
   const uint32_t T = p.T, t = lane & (T - 1u), team = tid / T, teams = kThreads / T;
   const uint64_t groups = (p.B + p.buckets - 1) / p.buckets;
   chain_wait();                                         // the messages come from the kernels ahead
-  if (!DENSE && p.defer_sparse && sparse_regime(p.peers, p.K, p.B, p.d)) return;
+  if (!DENSE && p.when.lo && mean_below(p.when.lo, p.peers, p.K, p.B)) return;
 
   for (uint64_t grp = blockIdx.x; grp < groups; grp += gridDim.x) {
     const uint64_t b0 = grp * p.buckets;
@@ -508,7 +508,7 @@ int launch_width(TeamParams& p, bool fused, size_t smem, cudaStream_t stream) {
 int launch_elias_teams(const FieldParams& f, bool dense, bool fused, cudaStream_t stream) {
   TeamParams p;
   p.peers = f.peers; p.K = f.K; p.n = f.n; p.d = f.d; p.s = f.s; p.B = f.B; p.out = f.out; p.c = f.c;
-  p.status = f.status; p.map = f.map; p.defer_sparse = f.defer_sparse;
+  p.status = f.status; p.map = f.map; p.when = f.when;
   const int width = f.s <= 15u ? kNibble : f.s <= 127u ? kByte : kWide;
   p.row_bytes = ((p.d * (width == kWide ? 2u : 1u) + 127u) & ~127u) + kRowPad;
   auto bytes = [&](uint32_t buckets, uint32_t peers) {

@@ -17,11 +17,17 @@ L2, MAX, ELIAS = O.NORM_L2, O.NORM_MAX, O.CODE_ELIAS
 
 # more than 24 K strings for a lane each; (decoder, buckets, coordinates missing in the last, d, s, norm, K, long gaps in every other peer)
 SHAPES = [
-    ("decode_elias", 132000, 27, 32, 15, MAX, 1, True), ("decode_elias", 44000, 1, 96, 3, MAX, 2, True),
-    ("decode_elias", 6500, 0, 160, 15, L2, 4, True), ("decode_elias", 3200, 223, 224, 7, MAX, 8, True),
+    ("decode_elias", 15000, 27, 32, 15, MAX, 9, True), ("decode_elias", 2700, 1, 96, 3, MAX, 17, True),
+    ("decode_elias", 6700, 0, 160, 15, L2, 4, True), ("decode_elias", 3200, 223, 224, 7, MAX, 8, True),
     ("decode_elias", 3100, 247, 256, 15, MAX, 8, True), ("decode_elias", 1500, 509, 512, 15, L2, 17, True),
     ("decode_elias", 800, 1017, 1024, 1, MAX, 32, False), ("decode_elias", 2800, 1, 2048, 15, L2, 9, True),
     ("decode_elias", 1030, 5, 512, 15, MAX, 24, True), ("decode_elias", 1600, 3, 4096, 15, MAX, 16, False),
+    ("decode_elias_bytes", 40000, 27, 32, 15, MAX, 1, True), ("decode_elias_bytes", 1000, 1, 32, 3, L2, 30, False),
+    ("decode_elias_bytes", 13000, 63, 64, 15, MAX, 2, True), ("decode_elias_bytes", 5200, 0, 96, 7, MAX, 5, True),
+    ("decode_elias_bytes", 1600, 13, 160, 3, MAX, 17, False),
+    # decided by the strings: 0.25 to 0.7 bits per coordinate behind the scale, ranges shorter and longer than a bucket
+    ("decode_elias_bytes", 16600, 0, 256, 1, L2, 16, False), ("decode_elias_bytes", 19000, 99, 224, 1, L2, 16, False),
+    ("decode_elias_bytes", 14700, 250, 288, 1, L2, 16, False),
     ("decode_elias_fields", 25000, 95, 96, 255, L2, 1, False), ("decode_elias_fields", 5000, 3, 480, 16, MAX, 5, False),
     ("decode_elias_fields", 800, 31, 32, 255, MAX, 32, False), ("decode_elias_fields", 3200, 0, 256, 255, L2, 8, False),
     ("decode_elias_teams", 3, 7, 4096, 255, MAX, 5, False), ("decode_elias_teams", 1000, 0, 64, 3, L2, 24, True),
