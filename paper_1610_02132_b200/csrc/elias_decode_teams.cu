@@ -9,7 +9,8 @@
 // it, then reads its part through, counting positions. Its start is right when it is where lane t - 1
 // ended; where it is not, the lane reads its part again from there, and so on until all agree. Lane 0 is
 // right from the start and every round makes at least one more lane right, so T rounds always suffice
-// (the time of reading the string by one lane); two or three are the rule. A scan of the counts gives
+// (the time of reading the string by one lane); two or three are the rule. (A lane keeps two readings, so that a lane in
+// front of it that turns out wrong costs it no third one.) A scan of the counts gives
 // every lane the position its part starts at, and a last reading writes one code per coordinate (level,
 // sign) into the string's row in shared memory. Then all threads add the rows in ascending k.
 //
@@ -407,13 +408,53 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
         } else if (j < rows && t == 0u) {
           scales[j] = 0.f;
         }
-        for (;;) {
-          const uint32_t before = __shfl_up_sync(0xffffffffu, m.pos[kMarks - 1u], 1, (int)T);
-          const bool again = t != 0u && before != start;
-          if (!__any_sync(0xffffffffu, again)) break;
-          if (again) {
-            start = before;
-            read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, true, m);
+        if constexpr (!DENSE) {
+          for (;;) {
+            const uint32_t before = __shfl_up_sync(0xffffffffu, m.pos[kMarks - 1u], 1, (int)T);
+            const bool again = t != 0u && before != start;
+            if (!__any_sync(0xffffffffu, again)) break;
+            if (again) {
+              start = before;
+              read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, true, m);
+            }
+          }
+        } else {
+          // Short symbols again: one of an odd length, where they are rare, puts all lanes behind it out of step, each of
+          // which would find out a round after the one in front of it. So where a lane that had to start elsewhere ended
+          // elsewhere too, all lanes of the string read their parts from a bit further on, and keep both readings (K = 4,
+          // n = 67 M, a mixture, s = 15: 1258 -> 583 us at d = 4096, 922 -> 651 at d = 2048).
+          uint32_t other = start;                         // where the other reading started
+          Marks<DENSE> o = m;
+          uint32_t rounds = reads && ref.total < 3u * db ? 1u : 0u;         // until then; 0: never
+          for (;;) {
+            uint32_t before;
+            bool again;
+            for (;;) {
+              before = __shfl_up_sync(0xffffffffu, m.pos[kMarks - 1u], 1, (int)T);
+              again = t != 0u && before != start;
+              const bool had = again && before == other;
+              if (!__any_sync(0xffffffffu, had)) break;
+              if (had) {
+                const Marks<DENSE> q = m;
+                m = o; o = q;
+                other = start; start = before;
+              }
+            }
+            const uint32_t wrong = __ballot_sync(0xffffffffu, again);
+            if (wrong == 0u) break;
+            const bool astray = rounds != 0u && (wrong & (0xFFFFFFFFu >> (32u - T) << (lane & ~(T - 1u)))) != 0u;
+            const bool now = astray && rounds == 2u;
+            if (astray) rounds = now ? 0u : 2u;
+            if (now && t != 0u && start < hi && other == start) {
+              other = start + 1u;
+              read_part<DENSE, WIDTH>(tab, words, other, lo, hi, end, true, o);
+            }
+            if (__any_sync(0xffffffffu, now)) continue;
+            if (again) {
+              o = m; other = start;
+              start = before;
+              read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, true, m);
+            }
           }
         }
         const uint32_t sum = m.sum[kMarks - 1u], stop = m.pos[kMarks - 1u];

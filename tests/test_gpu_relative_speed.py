@@ -62,6 +62,16 @@ def test_fewer_bits_do_not_take_longer_in_the_dense_code():
     assert int(small.status.item()) == int(large.status.item()) == 0
 
 
+def test_rare_odd_symbols_do_not_take_longer_in_the_dense_code():
+    """The same with a few levels of 3 and more among them: symbols of 7 bits, each of which shifts the rest."""
+    n, d, K = 2 ** 22, 4096, 4
+    rare = decode(n, d, 15, O.NORM_L2, O.CODE_ELIAS_DENSE, K, lambda w: I.gaussian_mixture_device(n, seed=w))
+    large = decode(n, d, 15, O.NORM_MAX, O.CODE_ELIAS_DENSE, K)
+    assert rare.bits < 0.6 * large.bits
+    few, many = time_of(rare, large)
+    assert few < 1.3 * many
+
+
 def test_many_peers_of_a_small_problem_are_read_in_one_pass():
     """32 short strings a bucket against 8: more to add up, but no more latencies in a row."""
     n, d = 16 * 1024, 1024
