@@ -289,8 +289,7 @@ int launch_elias_encode(const float* g, uint64_t n, uint32_t d, uint32_t s, int 
                         size_t out_capacity, uint64_t* out_bits, uint8_t* workspace,
                         uint32_t* status_dev, const BucketMap& map, cudaStream_t stream) {
   const EliasWs w = carve(workspace, n, d, s);
-  // (the kernels for small problems wait for nothing: while the test hook bounds the waits, the ones that do take all sizes)
-  if (!quantize_polls_bounded() && use_small(n, d, map))
+  if (use_small(n, d, map))
     return launch_elias_encode_small(g, n, d, s, norm_kind, dense, seed, step, worker, out, out_capacity, out_bits, w, status_dev, stream);
   int st = launch_quantize_fixed(g, n, d, s, norm_kind, seed, step, worker, w.fixed, status_dev, nullptr,
                                  &w.ctrl->arrived, map, stream);

@@ -199,7 +199,6 @@ struct KernelSite {
 // Test hook: bound (in polls) of the waits inside the streaming encoder's main loop.
 void set_quantize_poll_limit(uint32_t polls);
 uint32_t default_quantize_poll_limit();
-bool quantize_polls_bounded();           // set to something else than the default
 
 // Programmatic dependent launch. Every kernel of the library is launched with programmatic stream
 // serialization, so the launch of the next kernel is prepared while the one ahead still runs and its

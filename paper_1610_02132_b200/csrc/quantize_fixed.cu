@@ -866,6 +866,5 @@ int launch_quantize_fixed(const float* g, uint64_t n, uint32_t d, uint32_t s, in
 
 void set_quantize_poll_limit(uint32_t polls) { g_poll_limit.store(polls, std::memory_order_relaxed); }
 uint32_t default_quantize_poll_limit() { return kDrainPolls; }
-bool quantize_polls_bounded() { return g_poll_limit.load(std::memory_order_relaxed) != kDrainPolls; }
 
 }  // namespace qsgd

@@ -31,7 +31,8 @@ def zero_polls():
                                                    (4096, O.CODE_FIXED, O.NORM_MAX), (2048, O.CODE_ELIAS, O.NORM_MAX),
                                                    (512, O.CODE_ELIAS, O.NORM_L2)])
 def test_wait_gives_up_and_kernel_returns(zero_polls, d, code_kind, norm_kind):
-    n, s = 40 * 4096 + 77, 15
+    # Elias: beyond the 1000 tiles up to which an encode takes kernels that wait for nothing
+    n, s = (40 if code_kind == O.CODE_FIXED else 1001) * 4096 + 77, 15
     g = torch.from_numpy(I.gaussian(n, 0.01, seed=3)).cuda()
     cap = Q.qsgd_message_capacity(n, d, s, code_kind)
     big = torch.full((cap + 4096,), CANARY, dtype=torch.uint8, device="cuda")
@@ -62,3 +63,11 @@ def test_wait_gives_up_under_policy(zero_polls, bucket):
     torch.cuda.synchronize()
     assert int(status.item()) & Q.binding.DEV_TIMEOUT
     assert bool((big[cap:] == CANARY).all())
+
+
+@pytest.mark.parametrize("d,code_kind", [(512, O.CODE_ELIAS), (2048, O.CODE_ELIAS_DENSE)])
+def test_small_encodes_take_the_same_way_while_waits_are_bounded(zero_polls, d, code_kind):
+    """Nothing waits in them, so nothing may change: two launches and the exact message."""
+    before = Q.qsgd_launch_count()
+    encode_parity(I.gaussian(40 * 4096 + 77, 0.01, seed=3), d, 15, O.NORM_MAX, code_kind, seed=7, step=0, worker=0)
+    assert Q.qsgd_launch_count() == before + 2 * 2                # encode_parity encodes twice
