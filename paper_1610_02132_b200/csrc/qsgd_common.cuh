@@ -6,7 +6,6 @@
 #include <utility>
 #include <stdint.h>
 
-#include <map>
 #include <mutex>
 
 #include "../../include/qsgd.h"
@@ -132,7 +131,10 @@ constexpr int kMaxDevices = 64;
 
 struct KernelSite {
   std::mutex mu;
-  std::map<uint64_t, int> occ_by_smem[kMaxDevices];   // lookup_dynamic: threads << 32 | bytes -> resident CTAs
+  struct Kept { uint64_t key; int occ; };                // lookup_dynamic: threads << 32 | bytes, resident CTAs
+  static constexpr uint32_t kKept = 32;
+  Kept kept[kMaxDevices][kKept] = {};                    // (fixed: a container could throw through the C entry points)
+  uint32_t oldest[kMaxDevices] = {};
   bool ready[kMaxDevices] = {};
   int sms[kMaxDevices] = {};
   int occ[kMaxDevices] = {};
@@ -164,7 +166,7 @@ struct KernelSite {
   }
 
   // The same for a kernel whose shared memory depends on the problem: the opt-in is raised as needed and
-  // the residency of every size met so far is kept (a few dozen at most: sizes follow K and d).
+  // the residency of the sizes met last is kept (sizes follow K and d).
   template <class Kernel>
   int lookup_dynamic(Kernel kern, int threads, size_t smem, int* sms_out, int* occ_out) {
     int dev = 0;
@@ -173,8 +175,10 @@ struct KernelSite {
     if (dev < 0 || dev >= kMaxDevices) return (int)cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(mu);
     const uint64_t key = (uint64_t)threads << 32 | smem;
-    auto it = occ_by_smem[dev].find(key);
-    if (it == occ_by_smem[dev].end()) {
+    int o = 0;
+    for (const Kept& k : kept[dev])
+      if (k.key == key) o = k.occ;
+    if (o == 0) {
       if (!sms[dev]) {
         e = cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return (int)e;
@@ -184,14 +188,13 @@ struct KernelSite {
         if (e != cudaSuccess) return (int)e;
         opted[dev] = (int)smem;
       }
-      int o = 0;
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, threads, smem);
       if (e != cudaSuccess) return (int)e;
-      if (occ_by_smem[dev].size() > 512) occ_by_smem[dev].clear();
-      it = occ_by_smem[dev].emplace(key, o > 0 ? o : 1).first;
+      if (o < 1) o = 1;
+      kept[dev][oldest[dev]++ % kKept] = Kept{key, o};
     }
     *sms_out = sms[dev];
-    *occ_out = it->second;
+    *occ_out = o;
     return 0;
   }
 };
