@@ -135,8 +135,8 @@ int qsgd_encode(const float* g, uint64_t n, uint32_t bucket, uint32_t s, int nor
  *   tables  host array of K device pointers to the offset tables (Elias kinds; msgs[k] +
  *           out_bits[1]); NULL for fixed-width. With the table directly behind the payload the
  *           library reads the payload sizes off the pointers and chooses between its decoders on
- *           the host; with tables kept elsewhere it decides on the device (two launches, one of
- *           which returns at once). Results are the same either way.
+ *           the host; with tables kept elsewhere it decides on the device (up to three launches, all
+ *           but one of which return at once). Results are the same either way.
  *   payload_bytes  host array of K payload lengths in bytes (the padded payload, = out_bits[1]
  *           of each message), or NULL. The decoders read no payload bit at or beyond
  *           8 * payload_bytes[k]: a table whose last entry claims more is refused with
@@ -174,7 +174,7 @@ int qsgd_decode_sgd_step(const void* const* msgs, const uint64_t* const* tables,
  * The kernels take table k at msgs[k] + infos[k][1]; that place must be 16-byte aligned with all
  * 8 * (B + 1) table bytes inside msg_bytes[k], and infos[k][1] bounds the payload, else
  * QSGD_DEV_TABLE is raised and nothing of that message is read. The choice among the Elias
- * decoders is made on the device (two launches, one returns at once). For QSGD_CODE_FIXED infos
+ * decoders is made on the device (up to three launches, all but one return at once). For QSGD_CODE_FIXED infos
  * and msg_bytes are ignored (may be NULL). Results are bit-identical to the calls above.
  */
 int qsgd_decode_accumulate_packed(const void* const* msgs, const uint64_t* const* infos,

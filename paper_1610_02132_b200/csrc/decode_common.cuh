@@ -1,5 +1,5 @@
-// Reconstruction of +-A * (level / s) from fixed-width fields, shared by the fixed-width decoder
-// (fields read from the message) and the Elias decoder (fields rebuilt in shared memory).
+// What the decoders share: reconstruction of +-A * (level / s) from the fields of a fixed-width message, the places of
+// coordinates in the output, stores of sums and of the step.
 #pragma once
 
 #include "qsgd_common.cuh"

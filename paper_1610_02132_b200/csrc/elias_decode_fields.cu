@@ -185,7 +185,9 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
   }
 }
 
-int launch_fields(FieldParams& p, bool fused, cudaStream_t stream) {
+}  // namespace
+
+int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream) {
   static KernelSite site[2];
   int max_smem = 0;
   const int st0 = device_shared_memory(&max_smem);
@@ -221,9 +223,5 @@ int launch_fields(FieldParams& p, bool fused, cudaStream_t stream) {
   ScopedKernel sk(kKernDecodeEliasFields, stream);
   return (int)launch_chained(kern, (uint32_t)(want < cap ? want : cap), warps * 32, smem, stream, p);
 }
-
-}  // namespace
-
-int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream) { return launch_fields(p, fused, stream); }
 
 }  // namespace qsgd
