@@ -10,26 +10,54 @@ __device__ __forceinline__ float shfl_f(float v, uint32_t src) {
   return __shfl_sync(0xffffffffu, v, (int)src);
 }
 
-// Adds peer k's 16 values to acc[]. SINGLE: the whole chunk lies in one bucket and `lut` is
-// already scaled by A; otherwise `lut` holds +-(level / s) and A is this lane's bucket scale.
-template <int LB, bool SINGLE>
-__device__ __forceinline__ void add_peer_lut(float (&acc)[16], const uint32_t (&w)[4], uint32_t sb,
-                                             float lut, float A) {
+// Two floats in a register pair, and the operations on both at once: one issue slot for two.
+typedef unsigned long long float2p;
+__device__ __forceinline__ float2p pair2(float a, float b) {
+  float2p r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpair2(float2p v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ float2p fma2(float2p a, float2p b, float2p c) {
+  float2p r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ float2p add2(float2p a, float2p b) {
+  float2p r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// acc + RN(A * v). The product is an fma with -0 that the compiler cannot see (a kernel parameter), because ptxas contracts a
+// mul.rn.f32x2 in front of an add.rn.f32x2.
+__device__ __forceinline__ float2p add_product2(float2p acc, float A, float v0, float v1, float minus_zero) {
+  return add2(acc, fma2(pair2(A, A), pair2(v0, v1), pair2(minus_zero, minus_zero)));
+}
+
+// Adds peer k's 16 values to acc[] (coordinates 2 j and 2 j + 1 in acc[j]). SINGLE: the whole chunk lies in one bucket and
+// `lut` is already scaled by A; otherwise `lut` holds +-(level / s) and A is this lane's bucket scale.
+template <bool SINGLE>
+__device__ __forceinline__ float2p add_pair_lut(float2p acc, uint32_t i0, uint32_t i1, float lut, float A, float minus_zero) {
+  const float a = shfl_f(lut, i0), b = shfl_f(lut, i1);
+  return SINGLE ? add2(acc, pair2(a, b)) : add_product2(acc, A, a, b, minus_zero);
+}
+
+template <int LB, bool SINGLE, int W>
+__device__ __forceinline__ void add_peer_lut(float2p (&acc)[8], const uint32_t (&w)[W], uint32_t sb,
+                                             float lut, float A, float minus_zero) {
   if (LB == 4) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const uint32_t word = w[h], s8 = sb >> (8 * h);
+      const uint32_t word = w[h % W], s8 = sb >> (8 * h);
       const uint32_t ev = word & 0x0F0F0F0Fu, od = (word >> 4) & 0x0F0F0F0Fu;
       const uint32_t ie = (((s8 & 0x55u) * 0x00410410u) & 0x10101010u) | ev;   // coords 0,2,4,6
       const uint32_t io = (((s8 & 0xAAu) * 0x00208208u) & 0x10101010u) | od;   // coords 1,3,5,7
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float a = shfl_f(lut, ie >> (8 * j));
-        float b = shfl_f(lut, io >> (8 * j));
-        if (!SINGLE) { a = __fmul_rn(A, a); b = __fmul_rn(A, b); }
-        acc[8 * h + 2 * j] = __fadd_rn(acc[8 * h + 2 * j], a);
-        acc[8 * h + 2 * j + 1] = __fadd_rn(acc[8 * h + 2 * j + 1], b);
-      }
+      for (int j = 0; j < 4; ++j) acc[4 * h + j] = add_pair_lut<SINGLE>(acc[4 * h + j], ie >> (8 * j), io >> (8 * j), lut, A, minus_zero);
     }
   } else if (LB == 2) {
     // 16 two-bit levels in w[0]. Per half (8 coordinates) spread the levels to nibble spacing
@@ -47,11 +75,7 @@ __device__ __forceinline__ void add_peer_lut(float (&acc)[16], const uint32_t (&
       y = (y | (y << 3)) & 0x11111111u;
       const uint32_t z = x | (y << 2);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        float a = shfl_f(lut, z >> (4 * j));
-        if (!SINGLE) a = __fmul_rn(A, a);
-        acc[8 * h + j] = __fadd_rn(acc[8 * h + j], a);
-      }
+      for (int j = 0; j < 4; ++j) acc[4 * h + j] = add_pair_lut<SINGLE>(acc[4 * h + j], z >> (8 * j), z >> (8 * j + 4), lut, A, minus_zero);
     }
   } else {
     // LB = 1: interleave the 16 level bits (even positions) with the 16 sign bits (odd); the
@@ -63,29 +87,30 @@ __device__ __forceinline__ void add_peer_lut(float (&acc)[16], const uint32_t (&
     x = (x | (x << 1)) & 0x55555555u; y = (y | (y << 1)) & 0x55555555u;
     const uint32_t z = x | (y << 1);
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-      float a = shfl_f(lut, z >> (2 * e));
-      if (!SINGLE) a = __fmul_rn(A, a);
-      acc[e] = __fadd_rn(acc[e], a);
-    }
+    for (int j = 0; j < 8; ++j) acc[j] = add_pair_lut<SINGLE>(acc[j], z >> (4 * j), z >> (4 * j + 2), lut, A, minus_zero);
   }
 }
 
-// LB = 8: table lookup of level / s in shared memory (entry l of lane t at word l * 32 + t).
-__device__ __forceinline__ void add_peer_tab(float (&acc)[16], const uint32_t (&w)[4], uint32_t sb,
-                                             const uint8_t* tab_lane, float A) {
+// LB = 8: table lookup of +-(level / s) in shared memory: level l, sign g of lane t at byte 256 l + 128 g + 4 t behind the
+// address 65536, so that lanes never meet in a bank and one byte permute makes an address: of the level's byte, a byte that
+// holds 128 g + 4 t, and the base.
+template <int W>
+__device__ __forceinline__ void add_peer_tab(float2p (&acc)[8], const uint32_t (&w)[W], uint32_t sb, uint32_t lane, float A,
+                                             float minus_zero) {
 #pragma unroll
   for (int h = 0; h < 4; ++h) {
+    // the signs of four coordinates into the highest bits of four bytes: bit j times 2^(7 + 7 j) (no two products meet)
+    const uint32_t four = h & 1 ? ((sb >> (4 * (h & 2))) & 0xF0u) * 0x01020408u : ((sb >> (4 * (h & 2))) & 0x0Fu) * 0x10204080u;
+    const uint32_t t = (four & 0x80808080u) | lane * 0x04040404u;
+    const uint32_t t01 = __byte_perm(t, 1u, 0x5410u), t23 = __byte_perm(t, 1u, 0x5432u);
+    float v[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t off = (j == 0 ? (w[h] << 7) : (w[h] >> (8 * j - 7))) & 0x7F80u;
-      const float xi = *reinterpret_cast<const float*>(tab_lane + off);
-      const uint32_t m = __float_as_uint(__fmul_rn(A, xi)) ^ ((sb << (31 - (4 * h + j))) & 0x80000000u);
-      acc[4 * h + j] = __fadd_rn(acc[4 * h + j], __uint_as_float(m));
-    }
+    for (uint32_t j = 0; j < 4; ++j)
+      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[j]) : "r"(__byte_perm(w[h % W], j < 2 ? t01 : t23, 0x7600u | j << 4 | (4u + (j & 1u)))));
+#pragma unroll
+    for (int j = 0; j < 2; ++j) acc[2 * h + j] = add_product2(acc[2 * h + j], A, v[2 * j], v[2 * j + 1], minus_zero);
   }
 }
-
 
 // Writes 16 accumulated values of one lane: acc as it is, or the SGD step x <- x - c * acc.
 template <bool FUSED>
@@ -162,6 +187,63 @@ __device__ __forceinline__ void store_span8(const OutSpan& sp, const float (&acc
 #pragma unroll
     for (int e = 0; e < 8; ++e)
       if ((uint32_t)e < sp.valid) sp.ptr[e] = FUSED ? __fsub_rn(sp.ptr[e], __fmul_rn(c, acc[e])) : acc[e];
+  }
+}
+
+// A warp's chunk of 512 sums, 16 consecutive ones a lane: acc as it is, or the SGD step. Where the chunk is whole and in one
+// piece, the lanes pass their quads through `turn` (2 KB of the warp's shared memory), so that accesses to `out` are to 512
+// consecutive bytes: with 16 bytes out of every 64 they were a quarter of the fixed-width decoder's L1 wavefronts. SINGLE: the
+// chunk lies in one bucket.
+template <bool FUSED, bool SINGLE>
+__device__ __forceinline__ void store_chunk16(float* out, const BucketMap& map, const float2p (&acc)[8], uint32_t turn, uint32_t ch,
+                                              uint32_t log2_chunks_per_bucket, uint32_t d, uint64_t n, float c, uint32_t lane) {
+  const uint64_t i0 = (uint64_t)ch * 512u, i = i0 + lane * 16u;
+  OutSpan whole;                                  // the chunk, where it is in one piece
+  whole.ptr = out; whole.valid = 0u;
+  if (!map.src) {
+    whole.ptr = out + i0;
+    whole.valid = i0 + 512u <= n ? 512u : 0u;
+  } else if (SINGLE) {
+    const uint32_t b = ch >> log2_chunks_per_bucket;
+    whole = out_span(out, map, b, (ch - (b << log2_chunks_per_bucket)) * 512u, d, n, 512u);
+  }
+  if (whole.valid == 512u && (reinterpret_cast<uintptr_t>(whole.ptr) & 15u) == 0) {
+    // quad j of lane l at 4 l + (j ^ (l / 2 & 3)): eight lanes at a time in eight groups of banks, both ways
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j) {
+      const float2 a = unpair2(acc[2 * j]), b = unpair2(acc[2 * j + 1]);
+      asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(turn + (lane * 4u + (j ^ ((lane >> 1) & 3u))) * 16u),
+                   "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y) : "memory");
+    }
+    float4* o = reinterpret_cast<float4*>(whole.ptr) + lane;
+    const uint32_t from = turn + (lane ^ ((lane >> 3) & 3u)) * 16u;       // quad 32 j + lane
+    float4 x[4];
+    if (FUSED)
+#pragma unroll
+      for (uint32_t j = 0; j < 4; ++j) x[j] = o[j * 32u];
+    __syncwarp();
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j) {
+      float4 r;
+      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "r"(from + j * 512u) : "memory");
+      if (FUSED) {
+        r.x = __fsub_rn(x[j].x, __fmul_rn(c, r.x)); r.y = __fsub_rn(x[j].y, __fmul_rn(c, r.y));
+        r.z = __fsub_rn(x[j].z, __fmul_rn(c, r.z)); r.w = __fsub_rn(x[j].w, __fmul_rn(c, r.w));
+      }
+      o[j * 32u] = r;
+    }
+    __syncwarp();                                 // before the next chunk's quads
+    return;
+  }
+  if (i >= n) return;
+  float v[16];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) { const float2 a = unpair2(acc[j]); v[2 * j] = a.x; v[2 * j + 1] = a.y; }
+  if (map.src) {                                  // per-tensor policy: buckets live elsewhere
+    const uint64_t b = i / d;
+    store_span16<FUSED>(out_span(out, map, b, (uint32_t)(i - b * d), d, n, 16u), v, c);
+  } else {
+    store_lane16<FUSED>(out + i, v, i, n, c);
   }
 }
 

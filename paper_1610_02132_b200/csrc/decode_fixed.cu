@@ -8,8 +8,16 @@
 //   * s <= 15: the 2 * (s + 1) possible values +-A * (level / s) of one (peer, bucket) live one
 //     per lane and are fetched with a warp shuffle indexed by "sign | level"; the sign bits are
 //     spread next to the level nibbles with one multiply per four coordinates;
-//   * s >= 16: level / s (correctly rounded) comes from a shared-memory table replicated per
-//     lane (bank-conflict free), followed by the multiply with A and a sign flip.
+//   * s >= 16: +-(level / s) (correctly rounded) comes from a shared-memory table replicated per
+//     lane (bank-conflict free), at an address that one byte permute makes of level and sign.
+//
+// What bounds it (n = 60 M, d = 512, K = 16): at s = 15 the L1 data path (one shuffle per coordinate and peer: 256 of 400
+// wavefronts per chunk) and the latency of the loads, 221 us; at s = 255 HBM, 88 % of the copy rate. Sums in pairs, one scale
+// read by all lanes instead of shuffled, places in 32 bits, `out` accessed in whole lines and the table with signs took 1489 to
+// 1272 warp instructions per chunk (s = 15) and 1900 to 1488 (s = 255): 251 -> 221 and 340 -> 262 us. Four messages are read
+// at a time (2: 252, 3: 236, 8 with 80 registers: 234 us at s = 15). More bytes in flight did not help: the next group read
+// while this one is added 252 to 270 (spills, or fewer warps), fields copied to shared memory a group ahead 235 (their
+// wavefronts), a ring of bulk copies per CTA 310 (warps that wait for the slowest), the next chunk prefetched to L2 240.
 #include "decode_common.cuh"
 
 namespace qsgd {
@@ -17,7 +25,6 @@ namespace qsgd {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
 constexpr int kChunk = 512;            // coordinates per warp iteration
 
 struct DecodeParams {
@@ -27,77 +34,96 @@ struct DecodeParams {
   uint64_t n;
   uint32_t d;
   uint32_t s;
-  uint32_t log2_chunks_per_bucket;   // valid when single_scale
+  uint32_t log2_chunks_per_bucket;   // SINGLE
   float* out;      // acc (overwritten) or x (updated in place)
   float c;         // eta / K (fused only)
-  uint64_t chunks;
+  float minus_zero;   // -0 that the compiler cannot see (add_product2)
+  uint32_t chunks;
   BucketMap map;
 };
 
-// Peers per unrolled group of the k loop: enough loads in flight to cover their latency, few
-// enough that the 16 running sums and the group's words stay in registers (measured per width).
-template <int LB> struct PeerUnroll { static constexpr int value = LB == 1 ? 3 : 4; };
+template <int LB> struct Shape {                     // 64 registers a thread
+  static constexpr int kMostThreads = LB == 8 ? 1024 : 256, kCtas = LB == 8 ? 1 : 4;
+};
+// LB = 8: the table of level / s, and its place in the window of shared memory (a multiple of 64 KB: add_peer_tab)
+constexpr uint32_t kTableBytes = 65536u, kTableAt = 65536u;
+constexpr uint32_t kTurn = kChunk * 4u;              // bytes per warp to turn sums round
+constexpr uint32_t kGroup = 4;                       // messages read at a time
+
+// What a lane has of one message for its 16 coordinates.
+template <int LB> struct Fields {
+  static constexpr int kWords = LB == 8 ? 4 : LB == 4 ? 2 : 1;
+  uint32_t w[kWords];
+  uint32_t sb;
+  float A;
+};
 
 template <int LB, bool FUSED, bool SINGLE>
-__global__ void __launch_bounds__(kThreads, 4) decode_fixed_kernel(const __grid_constant__ DecodeParams p) {
-  __shared__ __align__(16) float xi_tab[LB == 8 ? 256 * 32 : 32];
-  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float sf = (float)p.s;
+__global__ void __launch_bounds__(Shape<LB>::kMostThreads, Shape<LB>::kCtas) decode_fixed_kernel(const __grid_constant__ DecodeParams p) {
+  extern __shared__ __align__(128) uint8_t fixed_shared[];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
+  const uint32_t turn = (LB == 8 ? kTableAt + kTableBytes : (uint32_t)__cvta_generic_to_shared(fixed_shared)) + warp * kTurn;
   float lut0 = 0.f;                                  // this lane's +-(level / s)
+  const float sf = (float)p.s;
   if (LB == 8) {
-    for (uint32_t i = tid; i < 256 * 32; i += kThreads) xi_tab[i] = __fdiv_rn((float)(i >> 5), sf);
-    __syncthreads();
+    for (uint32_t i = warp; i < 256u; i += warps) {
+      const float q = __fdiv_rn((float)i, sf);
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(kTableAt + i * 256u + lane * 4u), "f"(q) : "memory");
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(kTableAt + i * 256u + 128u + lane * 4u), "f"(-q) : "memory");
+    }
   } else {
     const uint32_t level = lane & ((1u << LB) - 1u), neg = (lane >> LB) & 1u;
     const float q = __fdiv_rn((float)level, sf);
     lut0 = neg ? -q : q;
   }
-  const uint8_t* tab_lane = reinterpret_cast<const uint8_t*>(xi_tab) + 4 * lane;
+  if (LB == 8) __syncthreads();
   chain_wait();                                      // the messages come from the kernels ahead
 
-  for (uint64_t ch = (uint64_t)blockIdx.x * kWarps + warp; ch < p.chunks; ch += (uint64_t)gridDim.x * kWarps) {
-    const uint64_t i0 = ch * kChunk + (uint64_t)lane * 16;       // first coordinate of this lane
-    const bool live = i0 < p.n;                                   // lanes past n only help shuffles
-    const uint64_t b = SINGLE ? (ch >> p.log2_chunks_per_bucket) : (live ? i0 / p.d : 0);
-    float acc[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) acc[e] = 0.f;
-
-    // byte offsets of this lane's scale, 16 sign bits and 16 level fields inside any message
-    const uint64_t slot = i0 >> 4;
-    const uint64_t off_a = 4ull * b, off_s = p.off_sign + 2ull * slot, off_l = p.off_level + (uint64_t)(2 * LB) * slot;
-#pragma unroll PeerUnroll<LB>::value
-    for (uint32_t k = 0; k < p.K; ++k) {
-      uint32_t w[4] = {0u, 0u, 0u, 0u};
-      uint32_t sb = 0;
-      float A = 0.f;
-      if (live) {
-        const uint8_t* m = p.msg[k];
-        A = __ldg(reinterpret_cast<const float*>(m + off_a));
-        sb = __ldg(reinterpret_cast<const uint16_t*>(m + off_s));
-        if (LB == 8) {
-          const uint4 t = __ldg(reinterpret_cast<const uint4*>(m + off_l));
-          w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
-        } else if (LB == 4) {
-          const uint2 t = __ldg(reinterpret_cast<const uint2*>(m + off_l));
-          w[0] = t.x; w[1] = t.y;
-        } else if (LB == 2) {
-          w[0] = __ldg(reinterpret_cast<const uint32_t*>(m + off_l));
-        } else {
-          w[0] = __ldg(reinterpret_cast<const uint16_t*>(m + off_l));
-        }
+  const uint32_t stride = gridDim.x * warps, last_slot = (uint32_t)((p.n - 1) >> 4);
+  for (uint32_t ch = blockIdx.x * warps + warp; ch < p.chunks; ch += stride) {
+    // places of this lane's fields in any message (lanes past n read the last fields again)
+    const uint32_t slot = min(ch * (kChunk / 16) + lane, last_slot);
+    const uint32_t b = SINGLE ? ch >> p.log2_chunks_per_bucket : (uint32_t)(((uint64_t)slot * 16u) / p.d);
+    const uint32_t off_a = 4u * b, off_s = 2u * slot, off_l = (uint32_t)(2 * LB) * slot;       // n <= 2^32: below 2^32
+    auto read = [&](Fields<LB>& to, uint32_t k) {
+      const uint8_t* m = p.msg[k];
+      to.A = __ldg(reinterpret_cast<const float*>(m + off_a));
+      to.sb = __ldg(reinterpret_cast<const uint16_t*>(m + p.off_sign + off_s));
+      const uint8_t* l = m + p.off_level + off_l;
+      constexpr int W = Fields<LB>::kWords;
+      if (LB == 8) {
+        const uint4 t = __ldg(reinterpret_cast<const uint4*>(l));
+        to.w[0] = t.x; to.w[1 % W] = t.y; to.w[2 % W] = t.z; to.w[3 % W] = t.w;
+      } else if (LB == 4) {
+        const uint2 t = __ldg(reinterpret_cast<const uint2*>(l));
+        to.w[0] = t.x; to.w[1 % W] = t.y;
+      } else if (LB == 2) {
+        to.w[0] = __ldg(reinterpret_cast<const uint32_t*>(l));
+      } else {
+        to.w[0] = __ldg(reinterpret_cast<const uint16_t*>(l));
       }
-      if (LB == 8) add_peer_tab(acc, w, sb, tab_lane, A);
-      else if (SINGLE) add_peer_lut<LB, true>(acc, w, sb, __fmul_rn(__shfl_sync(0xffffffffu, A, 0), lut0), A);
-      else add_peer_lut<LB, false>(acc, w, sb, lut0, A);
+    };
+    float2p acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = 0ull;
+    auto add = [&](const Fields<LB>& f) {
+      if (LB == 8) add_peer_tab(acc, f.w, f.sb, lane, f.A, p.minus_zero);
+      else add_peer_lut<LB, SINGLE>(acc, f.w, f.sb, SINGLE ? __fmul_rn(f.A, lut0) : lut0, f.A, p.minus_zero);
+    };
+    uint32_t k = 0;
+    for (; k + kGroup <= p.K; k += kGroup) {
+      Fields<LB> f[kGroup];
+#pragma unroll
+      for (uint32_t u = 0; u < kGroup; ++u) read(f[u], k + u);
+#pragma unroll
+      for (uint32_t u = 0; u < kGroup; ++u) add(f[u]);
     }
-
-    if (!live) continue;
-    if (p.map.src) {                                              // per-tensor policy: buckets live elsewhere
-      store_span16<FUSED>(out_span(p.out, p.map, b, (uint32_t)(i0 - b * p.d), p.d, p.n, 16u), acc, p.c);
-    } else {
-      store_lane16<FUSED>(p.out + i0, acc, i0, p.n, p.c);
+    for (; k < p.K; ++k) {
+      Fields<LB> f;
+      read(f, k);
+      add(f);
     }
+    store_chunk16<FUSED, SINGLE>(p.out, p.map, acc, turn, ch, p.log2_chunks_per_bucket, p.d, p.n, p.c, lane);
   }
 }
 
@@ -124,17 +150,16 @@ int launch_one(const DecodeParams& p, cudaStream_t stream) {
   static KernelSite site;
   auto kern = decode_fixed_kernel<LB, FUSED, SINGLE>;
   int sms = 0, occ = 0;
-  const int st = site.lookup(kern, kThreads, 0, &sms, &occ);
+  int st = device_sms(&sms);
   if (st) return st;
-  const uint64_t want = (p.chunks + kWarps - 1) / kWarps;
-  const uint64_t cap = (uint64_t)sms * occ;
-  const uint32_t grid = (uint32_t)(want < cap ? want : cap);
-  {
-    ScopedKernel sk(kKernDecodeFixed, stream);
-    const cudaError_t e = launch_chained(kern, grid, kThreads, 0, stream, p);
-    if (e != cudaSuccess) return (int)e;
-  }
-  return (int)cudaGetLastError();
+  uint32_t warps = 8;
+  if (LB == 8) while (warps < Shape<LB>::kMostThreads / 32 && p.chunks > warps * (uint32_t)sms) warps *= 2;
+  const size_t smem = (LB == 8 ? kTableAt + kTableBytes : 0u) + warps * kTurn;
+  st = site.lookup_dynamic(kern, (int)warps * 32, smem, &sms, &occ);
+  if (st) return st;
+  const uint32_t want = (p.chunks + warps - 1) / warps, cap = (uint32_t)(sms * occ);
+  ScopedKernel sk(kKernDecodeFixed, stream);
+  return (int)launch_chained(kern, want < cap ? want : cap, warps * 32u, smem, stream, p);
 }
 
 template <int LB>
@@ -153,7 +178,8 @@ int launch_decode_fixed(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
   p.off_sign = L.off_sign; p.off_level = L.off_level;
   p.K = K; p.n = n; p.d = d; p.s = s; p.out = acc_or_x; p.map = map;
   p.c = eta / (float)K;
-  p.chunks = (n + kChunk - 1) / kChunk;
+  p.minus_zero = -0.f;
+  p.chunks = (uint32_t)((n + kChunk - 1) / kChunk);
   // one scale per chunk when the bucket size is 512 * 2^j
   const bool single = d >= (uint32_t)kChunk && (d & (d - 1)) == 0;
   p.log2_chunks_per_bucket = 0;
@@ -162,7 +188,7 @@ int launch_decode_fixed(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
     case 1: return launch_lb<1>(p, fused, single, stream);
     case 2: return launch_lb<2>(p, fused, single, stream);
     case 4: return launch_lb<4>(p, fused, single, stream);
-    default: return launch_lb<8>(p, fused, false, stream);
+    default: return launch_lb<8>(p, fused, single, stream);
   }
 }
 

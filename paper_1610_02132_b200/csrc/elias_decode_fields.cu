@@ -25,22 +25,6 @@ struct LevelQuotient {
   unsigned long long hi, lo, klo, m23, m0;      // 1 / s; its rest; -2^23 * rest; -2^23; -0
 };
 
-__device__ __forceinline__ unsigned long long pair2(float a, float b) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-  unsigned long long r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-
 // `minus_zero` is -0 that the compiler cannot see (a kernel parameter): the product with A is an fma with it, because
 // ptxas contracts a mul.rn.f32x2 in front of an add.rn.f32x2.
 __device__ __forceinline__ LevelQuotient level_quotient(uint32_t s, float minus_zero) {
