@@ -168,7 +168,7 @@ int qsgd_encode(const float* g, uint64_t n, uint32_t bucket, uint32_t s, int nor
     const FixedLayout L = make_fixed_layout(n, bucket, s);
     if (out_capacity < L.total) return QSGD_ERR_CAPACITY;
     return launch_quantize_fixed(g, n, bucket, s, norm_kind, seed, step, worker,
-                                 static_cast<uint8_t*>(out), status_dev, out_bits, nullptr, no_map(), cs);
+                                 static_cast<uint8_t*>(out), status_dev, out_bits, ClearWords{nullptr, 0}, no_map(), cs);
   }
   if (!workspace) return QSGD_ERR_NULL;
   if (!aligned16(workspace)) return QSGD_ERR_ALIGN;
@@ -321,7 +321,7 @@ int qsgd_policy_encode(const float* g, const qsgd_policy* plan, uint32_t bucket,
     if (code_kind == QSGD_CODE_FIXED) {
       if (cap < make_fixed_layout(nc, bucket, s).total) return QSGD_ERR_CAPACITY;
       st = launch_quantize_fixed(g, nc, bucket, s, norm_kind, seed, step, worker, body, status_dev, out_bits,
-                                 nullptr, map_of(plan), cs);
+                                 ClearWords{nullptr, 0}, map_of(plan), cs);
     } else {
       if (!workspace) return QSGD_ERR_NULL;
       if (!aligned16(workspace)) return QSGD_ERR_ALIGN;

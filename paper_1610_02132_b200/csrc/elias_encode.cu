@@ -1,19 +1,24 @@
 // Encode, Elias path (Section 3.1 "Efficient Coding of Gradients", string S; Appendix A.3 for
 // the dense variant). Pipeline on one stream:
 //   1. quantize into the fixed-width layout held in the workspace (quantize_fixed.cu);
-//   2. string length L_b of every bucket, and the sum of the lengths of each CTA's run of
-//      consecutive buckets (elias_length_kernel);
-//   3. the CTA of the length kernel that publishes its sum last (an arrival counter, no waiting)
-//      scans the per-CTA sums, fixes the message geometry and checks the capacity;
-//   4. each CTA of the scatter kernel derives the bit offsets of its own buckets, writes their
+//   2. string length L_b of every bucket, the sum of the lengths of each CTA's run of consecutive
+//      buckets, and by atomic additions the sum of each group of kSumGroup CTAs (elias_length_kernel);
+//   3. each CTA of the scatter kernel adds up the sums in front of its run (find_start), derives the
+//      bit offsets of its own buckets, writes their
 //      offset-table entries, assembles its run of strings in shared memory (lanes own
 //      consecutive sub-ranges of a bucket; bits of neighbouring lanes and buckets meet inside
 //      words and are merged with shared-memory atomics) and flushes whole words to the payload
 //      with coalesced stores (flush_run).
 // A bucket is handled by a team of d / 64 lanes (at most a warp, at least one lane), so that the
-// sequential walk over a lane's nonzeros is long enough to amortise the team's scans. Small problems go
-// by tiles instead (use_tiles), and the smaller ones of those are quantized and measured in one kernel
-// (elias_encode_small.cu).
+// sequential walk over a lane's nonzeros is long enough to amortise the team's scans. Levels above 15 in
+// longer buckets go by tiles, a thread with 16 coordinates, instead (use_tiles), and small problems are quantized and
+// measured in one kernel (elias_encode_small.cu).
+//
+// What bounds them (n = 34 M, d = 512, s = 15, a mixture of two scales): both the integer pipe, 79 % (length, 16.5 us) and 65 %
+// (scatter, 31 us, of which half is the walk over the nonzeros of the lane that has most). Without a scan by the CTA that draws
+// the last ticket, for which every CTA waited at its end: length 20.7 -> 16.5. Code words from bit 31 down with their length
+// beside them, sign included, level words where a lane can index them: scatter 361 -> 303 warp instructions per bucket,
+// 34.3 -> 30.8; whole encode at 60 M 152 -> 137, at 17 M, d = 4096, s = 64, dense code, 85 -> 60.
 #include <mutex>
 
 #include "elias_encode.cuh"
@@ -24,16 +29,17 @@ namespace {
 
 using namespace elias;
 
-// ---- 2. string length per bucket, sum per CTA ------------------------------------------------------
+// ---- 2. string length per bucket, sums per CTA and per group of CTAs ------------------------------------
 template <int LB, bool DENSE>
 __global__ void __launch_bounds__(kThreads) elias_length_kernel(const BucketParams p,
                                                                 uint32_t* __restrict__ len,
                                                                 uint32_t* __restrict__ lane_rec,
-                                                                uint64_t* cta_sums, const ScanArgs sa) {
+                                                                uint32_t* __restrict__ cta_sums, uint64_t* group_sums) {
   __shared__ uint32_t warp_sum[kWarps];
-  __shared__ uint32_t is_last;
   __shared__ uint32_t tab[17];
+  __shared__ SymbolLengths<DENSE ? LB : 1> lengths;
   fill_code_table(tab);
+  if (DENSE) fill_symbol_lengths<DENSE ? LB : 1>(lengths);
   __syncthreads();
   chain_wait();                                    // the fields come from the kernel ahead
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -45,47 +51,48 @@ __global__ void __launch_bounds__(kThreads) elias_length_kernel(const BucketPara
   const uint32_t c_lo = min(tl * p.seg, db), c_hi = min(c_lo + p.seg, db);
   const uint32_t* lwb = p.level + ((base * LB) >> 5);            // the bucket's first level word
   int32_t prev;
-  const uint32_t bits = lane_bits<LB, DENSE>(tab, lwb, p.lpb, c_lo, c_hi, tl, live, &prev);
+  const uint32_t bits = lane_bits<LB, DENSE>(tab, lengths, lwb, p.lpb, c_lo, c_hi, tl, live, &prev);
   if (live) lane_rec[b * p.lpb + tl] = bits | ((uint32_t)(prev + 1) << 16);   // reused by the scatter
   const uint32_t L = team_sum(bits, p.lpb);
   if (live && tl == 0) len[b] = L;
-  uint32_t w = (tl == 0) ? L : 0u;                 // one contribution per bucket
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+  const uint32_t w = __reduce_add_sync(0xffffffffu, tl == 0 ? L : 0u);        // one contribution per bucket
   if (lane == 0) warp_sum[warp] = w;
   __syncthreads();
   if (threadIdx.x == 0) {
-    uint64_t s = 0;
+    uint32_t s = 0;
 #pragma unroll
     for (int i = 0; i < kWarps; ++i) s += warp_sum[i];
     cta_sums[blockIdx.x] = s;
-    // publish, then take a ticket: whoever draws the last one sees every CTA's sum
-    __threadfence();
-    is_last = atomicAdd(&sa.ctrl->arrived, 1u) == gridDim.x - 1u ? 1u : 0u;
-  }
-  __syncthreads();
-  if (is_last) {
-    __threadfence();
-    scan_cta_sums(cta_sums, sa.ctas, p.B, sa.out_capacity, sa.ctrl, sa.out_bits, sa.status_dev);
+    atomicAdd(reinterpret_cast<unsigned long long*>(group_sums) + blockIdx.x / kSumGroup, (unsigned long long)s);
   }
 }
 
-// ---- 4. scatter ----------------------------------------------------------------------------------
+// ---- 3. scatter ----------------------------------------------------------------------------------
+struct ScatterArgs {
+  BucketParams p;
+  const uint32_t* len;
+  const uint32_t* lane_rec;
+  const uint32_t* cta_sums;
+  const uint64_t* group_sums;
+  uint8_t* out;
+  size_t out_capacity;
+  uint64_t* out_bits;
+  uint32_t* status_dev;
+};
+
 template <int LB, bool DENSE>
-__global__ void __launch_bounds__(kThreads) elias_scatter_kernel(const BucketParams p,
-                                                                 const uint32_t* __restrict__ len,
-                                                                 const uint32_t* __restrict__ lane_rec,
-                                                                 const uint64_t* __restrict__ cta_start,
-                                                                 const Ctrl* __restrict__ ctrl,
-                                                                 uint8_t* __restrict__ out) {
+__global__ void __launch_bounds__(kThreads) elias_scatter_kernel(const __grid_constant__ ScatterArgs a) {
+  constexpr uint32_t kFields = 32u / LB, kMask = (1u << LB) - 1u, kWords = 2u * LB;      // of a block of 64 coordinates
   extern __shared__ uint32_t stage[];
   __shared__ uint32_t warp_sum[kWarps];
+  __shared__ uint64_t start_s, total_s;
   __shared__ uint32_t tab[17];
-  __shared__ CodeWords<LB> words;
+  __shared__ CodeWords<LB, DENSE> words;
+  __shared__ uint32_t column[DENSE || LB == 1 ? 1 : kWords * kThreads];       // a block's level words, for each thread its own
+  const BucketParams& p = a.p;
   fill_code_table(tab);
-  if (!DENSE) fill_code_words<LB>(words);
-  chain_wait();                                    // ctrl, lengths and sums come from the kernel ahead
-  if (!ctrl->ok) return;
+  fill_code_words(words);
+  chain_wait();                                    // lengths and sums come from the kernel ahead
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t tl = lane & (p.lpb - 1), team = lane / p.lpb, bpw = 32 / p.lpb;
   const uint64_t b = (uint64_t)blockIdx.x * p.nbc + warp * bpw + team;
@@ -94,14 +101,12 @@ __global__ void __launch_bounds__(kThreads) elias_scatter_kernel(const BucketPar
   const uint32_t db = live ? (uint32_t)min((uint64_t)p.d, p.n - base) : 0;
   const uint32_t c_lo = min(tl * p.seg, db), c_hi = min(c_lo + p.seg, db);
 
-  const uint64_t start = __ldg(cta_start + blockIdx.x), stop = __ldg(cta_start + blockIdx.x + 1);
-  const uint32_t lead = (uint32_t)(start & 31);                     // bits of the first word owned by the previous CTA
-  const uint32_t span = (uint32_t)(stop - start);                   // bits of this CTA's run
-  const uint32_t nwords = (lead + span + 31) >> 5;
-  for (uint32_t j = threadIdx.x; j < nwords; j += kThreads) stage[j] = 0u;
+  const uint32_t span = __ldg(a.cta_sums + blockIdx.x);             // bits of this CTA's run
+  if (warp == 0) find_start(a.cta_sums, a.group_sums, &start_s, &total_s);
+  for (uint32_t j = threadIdx.x; j < (span + 62u) >> 5; j += kThreads) stage[j] = 0u;
 
   // bit offset of every bucket inside the CTA's run: scan of the bucket lengths
-  const uint32_t L = (live && tl == 0) ? __ldg(len + b) : 0u;
+  const uint32_t L = (live && tl == 0) ? __ldg(a.len + b) : 0u;
   uint32_t inc = L;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -109,27 +114,28 @@ __global__ void __launch_bounds__(kThreads) elias_scatter_kernel(const BucketPar
     if (lane >= (uint32_t)o) inc += t;
   }
   if (lane == 31) warp_sum[warp] = inc;
-  __syncthreads();                                                  // staging zeroed, warp sums visible
+  __syncthreads();                                                  // staging zeroed, sums and tables there
+  const uint64_t start = start_s;
+  const uint32_t lead = (uint32_t)(start & 31);                     // bits of the first word owned by the previous CTA
+  uint64_t payload_bytes;
+  if (!fix_geometry(total_s, p.B, a.out_capacity, a.out_bits, a.status_dev, blockIdx.x == 0, &payload_bytes)) return;
   uint32_t before = 0;
 #pragma unroll
   for (int w = 0; w < kWarps; ++w) if ((uint32_t)w < warp) before += warp_sum[w];
   uint32_t bucket_off = before + inc - L;                           // valid in team lane 0
   bucket_off = __shfl_sync(0xffffffffu, bucket_off, (int)(lane - tl));
-  const uint32_t Lb = __shfl_sync(0xffffffffu, L, (int)(lane - tl));
   if (live && tl == 0) {
-    uint64_t* table = reinterpret_cast<uint64_t*>(out + ctrl->payload_bytes);
+    uint64_t* table = reinterpret_cast<uint64_t*>(a.out + payload_bytes);
     table[b] = start + bucket_off;
-    if (b == p.B - 1) table[p.B] = start + bucket_off + Lb;
+    if (b == p.B - 1) table[p.B] = start + bucket_off + L;
   }
 
   // this lane's first bit inside its bucket: scan of the lane lengths over the team
-  int32_t prev;
   const uint32_t* lwb = p.level + ((base * LB) >> 5);            // the bucket's first level word
   const uint32_t* swb = p.sign + (base >> 5);                    // ... and first sign word
   // this lane's share of the string and the nonzero before it were counted by the length kernel
-  const uint32_t rec = live ? __ldg(lane_rec + b * p.lpb + tl) : 0u;
+  const uint32_t rec = live ? __ldg(a.lane_rec + b * p.lpb + tl) : 0u;
   const uint32_t bits = rec & 0xFFFFu;
-  prev = (int32_t)(rec >> 16) - 1;
   uint32_t linc = bits;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -139,65 +145,51 @@ __global__ void __launch_bounds__(kThreads) elias_scatter_kernel(const BucketPar
   if (bits != 0) {
     StageWriter bw;
     bw.begin(stage, lead + bucket_off + (linc - bits));
-    if (tl == 0) bw.put(__float_as_uint(__ldg(p.A + b)), 32);
-    if (DENSE) {
-      // ranges of whole 64-coordinate blocks: sign and level words are loaded once per block and word
-      constexpr uint32_t kFields = 32u / LB, kMask = (1u << LB) - 1u;
-      for (uint32_t c0 = c_lo; c0 < c_hi; c0 += 64u) {
-        const uint32_t* wp = lwb + ((c0 * LB) >> 5);
-        const uint32_t s0 = __ldg(swb + (c0 >> 5)), s1 = (c0 + 32u < c_hi) ? __ldg(swb + (c0 >> 5) + 1) : 0u;
-        const unsigned long long signs = (unsigned long long)s0 | ((unsigned long long)s1 << 32);
+    if (tl == 0) bw.put_word(__float_as_uint(__ldg(p.A + b)));
+    uint32_t prev = (rec >> 16) - 1u;
+    for (uint32_t c0 = c_lo; c0 < c_hi; c0 += 64u) {             // blocks of 64 coordinates
+      const uint32_t* wp = lwb + ((c0 * LB) >> 5);
+      uint32_t w[kWords];
 #pragma unroll
-        for (uint32_t j = 0; j < 2u * LB; ++j) {
-          const uint32_t off = j * kFields;                   // first coordinate of this word in the block
-          if (c0 + off >= c_hi) break;
-          const uint32_t w = __ldg(wp + j);
-          const uint32_t cnt = min(kFields, c_hi - (c0 + off));
-          for (uint32_t f = 0; f < cnt; ++f) {
-            uint32_t ln;
-            const uint32_t code = tab_code(tab, ((w >> (f * LB)) & kMask) + 1u, &ln);
-            bw.put((((uint32_t)(signs >> (off + f)) & 1u) << ln) | code, ln + 1);
+      for (uint32_t j = 0; j < kWords; ++j) w[j] = c0 + j * kFields < c_hi ? __ldg(wp + j) : 0u;
+      uint32_t s0 = __ldg(swb + (c0 >> 5)), s1 = (c0 + 32u < c_hi) ? __ldg(swb + (c0 >> 5) + 1) : 0u;
+      if constexpr (DENSE) {
+        const uint32_t left = c_hi - c0;
+#pragma unroll
+        for (uint32_t j = 0; j < kWords; ++j) {
+          const uint32_t sg = (j * kFields) & 32u ? s1 : s0;
+#pragma unroll
+          for (uint32_t f = 0; f < kFields; ++f) {
+            const uint32_t at = j * kFields + f;
+            const uint32_t e = at < left ? words.level[((w[j] >> (f * LB)) & kMask) | ((sg >> (at & 31u)) & 1u) << LB] : 0u;
+            bw.put_even(e & ~31u, e & 31u);
           }
         }
-      }
-    } else {
-      // ranges of whole 64-coordinate blocks: the block's nonzero mask
-      // and sign bits sit in registers, code words come whole from the two tables.
-      constexpr uint32_t kFields = 32u / LB, kMask = (1u << LB) - 1u;
-      for (uint32_t c0 = c_lo; c0 < c_hi; c0 += 64u) {
-        const uint32_t* wp = lwb + ((c0 * LB) >> 5);
-        unsigned long long m = 0ull;
+      } else {
+        // the block's nonzero masks and signs sit in registers, its level words where they can be indexed
+        uint32_t m0 = 0u, m1 = 0u;
 #pragma unroll
-        for (uint32_t j = 0; j < 2u * LB; ++j) {
-          const uint32_t w = (c0 + j * kFields < c_hi) ? __ldg(wp + j) : 0u;
-          m |= (unsigned long long)nonzero_mask<LB>(w) << (j * kFields);
+        for (uint32_t j = 0; j < kWords; ++j) {
+          const uint32_t m = nonzero_mask<LB>(w[j]);
+          if (j * kFields < 32u) m0 |= m << (j * kFields & 31u);
+          else m1 |= m << (j * kFields & 31u);
+          if (LB != 1) column[j * kThreads + threadIdx.x] = w[j];
         }
-        const uint32_t s0 = __ldg(swb + (c0 >> 5)), s1 = (c0 + 32u < c_hi) ? __ldg(swb + (c0 >> 5) + 1) : 0u;
-        const unsigned long long signs = (unsigned long long)s0 | ((unsigned long long)s1 << 32);
-        while (m) {
-          const uint32_t off = (uint32_t)__ffsll((long long)m) - 1u;
-          m &= m - 1ull;
-          const uint32_t pos = c0 + off, bit = off * LB;
-          const uint32_t level = (__ldg(wp + (bit >> 5)) >> (bit & 31u)) & kMask;
-          const uint32_t gap = pos - (uint32_t)prev;
-          uint32_t gcode, gl;
-          if (gap < 64u) {
-            const uint32_t e = words.gap[gap];
-            gcode = e & 0xFFFFu;
-            gl = e >> 16;
-          } else {
-            gcode = tab_code(tab, gap, &gl);
+        uint32_t half = c0;                                      // first coordinate of the half at hand
+        const uint32_t* mine = column + threadIdx.x;
+        while (m0 | m1) {
+          if (m0 == 0u) {
+            m0 = m1; m1 = 0u; s0 = s1;
+            half = c0 + 32u;
+            if (LB != 1) mine = column + threadIdx.x + LB * kThreads;
           }
-          const uint32_t e = words.level[level];
-          const uint32_t ll = e >> 16;
-          const uint32_t lcode = (e & 0xFFFFu) | ((uint32_t)((signs >> off) & 1ull) << ll);
-          if (gl + ll + 1u <= 32u) {                     // gap, sign and level in one piece (the rule)
-            bw.put((gcode << (ll + 1u)) | lcode, gl + ll + 1u);
-          } else {
-            bw.put(gcode, gl);
-            bw.put(lcode, ll + 1u);
-          }
-          prev = (int32_t)pos;
+          const uint32_t off = (uint32_t)__ffs((int)m0) - 1u, pos = half + off;
+          m0 &= m0 - 1u;
+          uint32_t idx = 1u;
+          if (LB != 1) idx = __funnelshift_r(mine[off / kFields * kThreads], 0u, off * LB) & kMask;
+          idx |= ((s0 >> off) & 1u) << LB;
+          put_entry<LB>(bw, tab, words, pos - prev, idx);
+          prev = pos;
         }
       }
     }
@@ -205,33 +197,32 @@ __global__ void __launch_bounds__(kThreads) elias_scatter_kernel(const BucketPar
   }
   __syncthreads();
   const uint64_t next = (uint64_t)(blockIdx.x + 1u) * p.nbc;       // the next CTA's first bucket
-  flush_run(reinterpret_cast<uint32_t*>(out) + (start >> 5), stage, lead, span, next >= p.B, p.A + next,
-            (uint32_t)(ctrl->payload_bytes / 4 - (start >> 5)));
+  flush_run(reinterpret_cast<uint32_t*>(a.out) + (start >> 5), stage, lead, span, next >= p.B, p.A + next,
+            (uint32_t)(payload_bytes / 4 - (start >> 5)));
 }
 
 // ---- 2. for tiles ----------------------------------------------------------------------------------
 template <int LB, bool DENSE>
-__global__ void __launch_bounds__(kThreads) elias_tile_length_kernel(const BucketParams p, uint64_t* cta_sums, const ScanArgs sa) {
+__global__ void __launch_bounds__(kThreads) elias_tile_length_kernel(const BucketParams p, uint32_t* tile_sums, uint64_t* group_sums) {
   __shared__ uint32_t slots[2][kWarps];
-  __shared__ uint32_t is_last;
   __shared__ uint32_t tab[17];
+  __shared__ SymbolLengths<DENSE ? LB : 1> lengths;
   fill_code_table(tab);
+  if (DENSE) fill_symbol_lengths<DENSE ? LB : 1>(lengths);
   __syncthreads();
   chain_wait();                                    // the fields come from the kernel ahead
   const Piece<LB> q = load_piece<LB>(p);
   const uint32_t mask = DENSE ? 0u : piece_mask<LB>(q);
   const int32_t prev = DENSE ? -1 : nonzero_before<LB>(q, mask, slots[0]);
-  uint32_t total;
-  cta_sum_before(piece_bits<LB, DENSE>(tab, q, mask, prev), slots[1], &total);
-  if (threadIdx.x == 0) {
-    cta_sums[blockIdx.x] = total;
-    __threadfence();
-    is_last = atomicAdd(&sa.ctrl->arrived, 1u) == gridDim.x - 1u ? 1u : 0u;
-  }
+  const uint32_t mine = __reduce_add_sync(0xffffffffu, piece_bits<LB, DENSE>(tab, lengths, q, mask, prev));
+  if ((threadIdx.x & 31) == 0) slots[1][threadIdx.x >> 5] = mine;
   __syncthreads();
-  if (is_last) {
-    __threadfence();
-    scan_cta_sums(cta_sums, sa.ctas, p.B, sa.out_capacity, sa.ctrl, sa.out_bits, sa.status_dev);
+  if (threadIdx.x == 0) {
+    uint32_t s = 0;
+#pragma unroll
+    for (int i = 0; i < kWarps; ++i) s += slots[1][i];
+    tile_sums[blockIdx.x] = s;
+    atomicAdd(reinterpret_cast<unsigned long long*>(group_sums) + blockIdx.x / kSumGroup, (unsigned long long)s);
   }
 }
 
@@ -240,42 +231,34 @@ int run_pipeline(BucketParams& bp, const EliasWs& w, uint32_t s, uint8_t* out, s
                  uint64_t* out_bits, uint32_t* status_dev, cudaStream_t stream) {
   if (use_tiles(bp.n, bp.d, s, DENSE)) {
     bp.lpb = 0; bp.seg = 16; bp.nbc = tile_buckets(bp.d);
-    const uint64_t ctas = (bp.B + bp.nbc - 1) / bp.nbc;
-    ScanArgs sa;
-    sa.ctas = ctas; sa.out_capacity = out_capacity; sa.ctrl = w.ctrl; sa.out_bits = out_bits;
-    sa.status_dev = status_dev;
+    const uint32_t tiles = (uint32_t)((bp.B + bp.nbc - 1) / bp.nbc);
     {
       ScopedKernel sk(kKernEliasLength, stream);
-      const cudaError_t e = launch_chained(elias_tile_length_kernel<LB, DENSE>, (uint32_t)ctas, kThreads, 0, stream, bp,
-                                           w.tile_sums, sa);
+      const cudaError_t e = launch_chained(elias_tile_length_kernel<LB, DENSE>, tiles, kThreads, 0, stream, bp, w.tile_sums, w.tile_groups);
       if (e != cudaSuccess) return (int)e;
     }
-    return launch_tile_scatter(bp, w, s, DENSE, out, stream);
+    return launch_tile_scatter(bp, w, s, DENSE, out, out_capacity, out_bits, status_dev, stream);
   }
   const Teams tm = make_teams(bp.d);
   bp.lpb = tm.lpb; bp.seg = tm.seg; bp.nbc = tm.nbc;
   const uint64_t ctas = (bp.B + tm.nbc - 1) / tm.nbc;
   {
-    ScanArgs sa;
-    sa.ctas = ctas; sa.out_capacity = out_capacity; sa.ctrl = w.ctrl; sa.out_bits = out_bits;
-    sa.status_dev = status_dev;
     ScopedKernel sk(kKernEliasLength, stream);
     const cudaError_t e = launch_chained(elias_length_kernel<LB, DENSE>, (uint32_t)ctas, kThreads, 0, stream, bp, w.len,
-                                         w.lane_rec, w.cta_sums, sa);
+                                         w.lane_rec, w.cta_sums, w.group_sums);
     if (e != cudaSuccess) return (int)e;
   }
-  {
-    const size_t smem = stage_bytes<DENSE>(tm.nbc, bp.d, s);
-    auto kern = elias_scatter_kernel<LB, DENSE>;
-    if (smem > 48 * 1024) {                        // the opt-in is raised only: threads with other s share it
-      static KernelSite site;
-      int sms = 0, occ = 0;
-      const int st = site.lookup_dynamic(kern, kThreads, smem, &sms, &occ);
-      if (st) return st;
-    }
-    ScopedKernel sk(kKernEliasScatter, stream);
-    return (int)launch_chained(kern, (uint32_t)ctas, kThreads, smem, stream, bp, w.len, w.lane_rec, w.cta_sums, w.ctrl, out);
-  }
+  const size_t smem = stage_bytes<DENSE>(tm.nbc, bp.d, s);
+  auto kern = elias_scatter_kernel<LB, DENSE>;
+  static KernelSite site;                          // (the opt-in is raised only: threads with other s share it)
+  int sms = 0, occ = 0;
+  const int st = site.lookup_dynamic(kern, kThreads, smem, &sms, &occ);
+  if (st) return st;
+  ScatterArgs a;
+  a.p = bp; a.len = w.len; a.lane_rec = w.lane_rec; a.cta_sums = w.cta_sums; a.group_sums = w.group_sums;
+  a.out = out; a.out_capacity = out_capacity; a.out_bits = out_bits; a.status_dev = status_dev;
+  ScopedKernel sk(kKernEliasScatter, stream);
+  return (int)launch_chained(kern, (uint32_t)ctas, kThreads, smem, stream, a);
 }
 
 }  // namespace
@@ -291,8 +274,10 @@ int launch_elias_encode(const float* g, uint64_t n, uint32_t d, uint32_t s, int 
   const EliasWs w = carve(workspace, n, d, s);
   if (use_small(n, d, map))
     return launch_elias_encode_small(g, n, d, s, norm_kind, dense, seed, step, worker, out, out_capacity, out_bits, w, status_dev, stream);
+  const uint64_t per_cta = use_tiles(n, d, s, dense) ? tile_buckets(d) : make_teams(d).nbc, B = (n + d - 1) / d;
+  const uint64_t groups = ((B + per_cta - 1) / per_cta + kSumGroup - 1) / kSumGroup;
   int st = launch_quantize_fixed(g, n, d, s, norm_kind, seed, step, worker, w.fixed, status_dev, nullptr,
-                                 &w.ctrl->arrived, map, stream);
+                                 ClearWords{use_tiles(n, d, s, dense) ? w.tile_groups : w.group_sums, (uint32_t)groups}, map, stream);
   if (st) return st;
   const FixedLayout L = make_fixed_layout(n, d, s);
   BucketParams bp;

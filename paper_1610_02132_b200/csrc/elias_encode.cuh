@@ -1,5 +1,5 @@
 // What the encoders of Elias messages share (elias_encode.cu: the general pipeline, elias_encode_small.cu: problems
-// of a few tiles): the workspace, code lengths and code words, the scan of the CTAs' lengths, bit writers.
+// of a few tiles): the workspace, code lengths and code words, where a CTA's run of strings begins, bit writers.
 #pragma once
 
 #include "elias_common.cuh"
@@ -10,12 +10,9 @@ namespace elias {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 
-struct Ctrl {                 // control block at the end of the workspace
-  uint64_t total_bits;
-  uint64_t payload_bytes;
-  uint32_t ok;                // 1 when the message fits out_capacity
-  uint32_t arrived;           // CTAs of the length kernel that have published their sum
-};
+// CTAs of the length kernel whose sums are also added up together, so that a CTA of the scatter kernel finds its run's start
+// and the payload's length by at most one load per group and per CTA of its own group.
+constexpr uint32_t kSumGroup = 64;
 
 struct Teams {
   uint32_t lpb;               // lanes per bucket (power of two, <= 32)
@@ -38,9 +35,10 @@ struct EliasWs {
   uint8_t* fixed;             // fixed-width intermediate
   uint32_t* len;              // L_b
   uint32_t* lane_rec;         // per lane of every bucket team: its bits | (previous nonzero + 1) << 16
-  uint64_t* cta_sums;         // per scatter CTA: sum of its buckets' lengths, then exclusive prefix
-  uint64_t* tile_sums;        // the same per tile, where len and lane_rec, which tiles do without, would be
-  Ctrl* ctrl;
+  uint32_t* cta_sums;         // per scatter CTA: sum of its buckets' lengths
+  uint64_t* group_sums;       // the same per kSumGroup CTAs
+  uint32_t* tile_sums;        // the same per tile, and per kSumGroup tiles: where len, lane_rec and the sums of the CTAs, which
+  uint64_t* tile_groups;      // tiles do without, would be
   size_t bytes;
 };
 
@@ -51,17 +49,14 @@ inline uint32_t tile_buckets(uint32_t d) { return kTileCoords / d; }
 // adds up.
 constexpr uint32_t kSmallTiles = 1000;
 
-// By teams (a lane walks 64 coordinates or more: less work per coordinate) or by tiles (a thread has 16: done
-// sooner)? Whole encodes measured both ways on three input families, teams against tiles (us). Tiles in two kernels:
-// 20.4 / 8.8 at n = 2^20, 18.5 to 26.4 / 17.5 to 21.9 at 3 * 2^20, 20.2 to 28.0 / 20.6 to 26.5 at 1000 tiles
-// (d = 512, s = 15); beyond 1000 tiles, where they take three kernels, only for levels above 15: Code_s up to
-// 6 * 2^20 coordinates 0.43 to 1.17 of the time by teams, Code'_s with d > 1024 (128 coordinates a lane) up to 20 * 2^20
-// 0.66 to 1.15. Code'_s with smaller levels, whose symbols cost a lane little, 0.87 to 1.34 from there on (n = 19 M,
-// d = 4096, s = 1: 74 / 98).
+// Beyond them, and with a bucket map: by teams (a lane walks 64 coordinates or more: less work per coordinate) or by tiles (a thread has 16: shorter
+// walks, less staging per CTA, so more of them resident)? Whole encodes measured both ways, teams against tiles (us). Levels
+// above 15, where a symbol costs most: Code'_s 97 / 70 at n = 17 M, d = 4096, s = 64, 58 / 44 at 8 M, s = 255; Code_s 124 / 103
+// at 17 M, d = 4096, 42 / 40 at 5 M, d = 512, but 89 / 102 at 17 M, d = 128. Levels up to 15: Code'_s 191 / 239 at 67 M,
+// d = 1024, s = 3 and 60 / 69 at 17 M, d = 128, s = 15; Code_s 142 / 204 at 60 M, d = 512, s = 15. Up to 1000 tiles always by
+// tiles: teams do not fill the GPU.
 inline bool use_tiles(uint64_t n, uint32_t d, uint32_t s, bool dense) {
-  if (n <= kSmallTiles * 4096ull) return true;
-  const uint64_t m = s <= 15u ? 0u : !dense ? 6u : d > 1024u ? 20u : 0u;
-  return n <= m << 20;
+  return n <= kSmallTiles * 4096ull || (s > 15u && (dense || d >= 512u));
 }
 inline bool use_small(uint64_t n, uint32_t d, const BucketMap& map) {
   return !map.src && n <= kSmallTiles * (uint64_t)(tile_buckets(d) * d);
@@ -76,9 +71,11 @@ inline EliasWs carve(uint8_t* ws, uint64_t n, uint32_t d, uint32_t s) {
   w.len = reinterpret_cast<uint32_t*>(ws + o); o += align16(4 * L.B);
   w.lane_rec = reinterpret_cast<uint32_t*>(ws + o); o += align16(4 * L.B * tm.lpb);
   const uint64_t ctas = (L.B + tm.nbc - 1) / tm.nbc;
-  w.cta_sums = reinterpret_cast<uint64_t*>(ws + o); o += align16(8 * (ctas + 1));
-  w.tile_sums = reinterpret_cast<uint64_t*>(w.len);     // tiles + 1 <= B + 1 of them: 4 B bytes of len, at least 4 B of lane_rec, 16 of cta_sums
-  w.ctrl = reinterpret_cast<Ctrl*>(ws + o); o += align16(sizeof(Ctrl));
+  w.cta_sums = reinterpret_cast<uint32_t*>(ws + o);
+  w.group_sums = reinterpret_cast<uint64_t*>(ws + o + ((4 * ctas + 7) & ~7ull)); o += align16(8 * (ctas + 1));
+  w.tile_sums = w.len;        // at most B of them
+  w.tile_groups = reinterpret_cast<uint64_t*>(w.cta_sums);     // at most 8 tiles to a scatter CTA: fewer groups than CTAs
+  o += 32;                    // (the size that callers reckon with)
   w.bytes = o;
   return w;
 }
@@ -145,16 +142,16 @@ struct LaneSummary {
   int32_t last;       // last nonzero position, -1 if none
 };
 
-// Sum over the nonzero fields of one level word of 1 + |Elias(level)| (sign bit and level code),
+// `bits` plus the sum over the nonzero fields of one level word of 1 + |Elias(level)| (sign bit and level code),
 // without a loop: |Elias(level)| grows by 1, 2, 3, 1, 4, 1, 1, 1 when the level reaches 1, 2, 4, 8,
 // 16, 32, 64, 128 (Appendix A.2 lengths 1, 3, 6, 7, 11, 12, 13, 14), so the per-field sum is a weighted
 // count of "level >= 2^j" masks, added up across the fields of the word.
 template <int LB>
-__device__ __forceinline__ uint32_t level_code_bits(uint32_t w) {
-  if (LB == 1) return 2u * (uint32_t)__popc(w);
+__device__ __forceinline__ uint32_t add_level_code_bits(uint32_t w, uint32_t bits) {
+  if (LB == 1) return bits + 2u * (uint32_t)__popc(w);
   if (LB == 2) {
     const uint32_t b1 = (w >> 1) & 0x55555555u;
-    return 2u * (uint32_t)(__popc(b1 | (w & 0x55555555u)) + __popc(b1));
+    return bits + 2u * (uint32_t)(__popc(b1 | (w & 0x55555555u)) + __popc(b1));
   }
   if (LB == 4) {
     const uint32_t t3 = w >> 3;
@@ -163,8 +160,7 @@ __device__ __forceinline__ uint32_t level_code_bits(uint32_t w) {
     const uint32_t ge2 = (ge4 | (w >> 1)) & 0x11111111u;
     const uint32_t ge1 = (ge2 | w) & 0x11111111u;
     const uint32_t x = ge8 + 3u * ge4 + 2u * (ge1 + ge2);              // at most 8 per nibble
-    const uint32_t y = (x & 0x0F0F0F0Fu) + ((x >> 4) & 0x0F0F0F0Fu);
-    return (y * 0x01010101u) >> 24;
+    return __dp4a((x & 0x0F0F0F0Fu) + ((x >> 4) & 0x0F0F0F0Fu), 0x01010101u, bits);
   }
   const uint32_t ge128 = (w >> 7) & 0x01010101u;
   const uint32_t ge64 = (ge128 | (w >> 6)) & 0x01010101u;
@@ -174,8 +170,33 @@ __device__ __forceinline__ uint32_t level_code_bits(uint32_t w) {
   const uint32_t ge4 = (ge8 | (w >> 2)) & 0x01010101u;
   const uint32_t ge2 = (ge4 | (w >> 1)) & 0x01010101u;
   const uint32_t ge1 = (ge2 | w) & 0x01010101u;
-  const uint32_t x = 2u * (ge1 + ge2) + 3u * ge4 + ge8 + 4u * ge16 + ge32 + ge64 + ge128;   // at most 15 per byte
-  return (x * 0x01010101u) >> 24;
+  return __dp4a(2u * (ge1 + ge2) + 3u * ge4 + ge8 + 4u * ge16 + ge32 + ge64 + ge128, 0x01010101u, bits);   // at most 15 per byte
+}
+
+// 1 + |Elias(level + 1)| of the dense code's symbols.
+template <int LB> struct SymbolLengths { uint8_t of[1u << LB]; };
+template <int LB>
+__device__ __forceinline__ void fill_symbol_lengths(SymbolLengths<LB>& t) {
+  for (uint32_t l = threadIdx.x; l < (1u << LB); l += kThreads) {
+    const uint32_t m = 32u - (uint32_t)__clz((int)(l + 1u));
+    t.of[l] = (uint8_t)(m <= 1u ? 2u : m + 2u + elias_prefix_len(m));
+  }
+}
+// ... summed over the fields of one level word.
+template <int LB>
+__device__ __forceinline__ uint32_t symbol_bits(const SymbolLengths<LB>& t, uint32_t w, uint32_t count) {
+  constexpr uint32_t kFields = 32u / LB, kMask = (1u << LB) - 1u;
+  uint32_t bits = 0;
+  if constexpr (LB == 1) {                                // two bits, or four
+    const uint32_t there = count >= 32u ? 0xFFFFFFFFu : (1u << count) - 1u;
+    return 2u * min(count, 32u) + 2u * (uint32_t)__popc(w & there);
+  }
+#pragma unroll
+  for (uint32_t f = 0; f < kFields; ++f) {
+    const uint32_t l = t.of[(w >> (f * LB)) & kMask];
+    bits += f < count ? l : 0u;
+  }
+  return bits;
 }
 
 // Sum of |Elias(gap)| over the set bits of a 64-coordinate block except the lowest, gap = distance to
@@ -227,7 +248,7 @@ __device__ __forceinline__ LaneSummary summarize_sparse(const uint32_t* tab, con
     for (uint32_t j = 0; j < 2u * LB; ++j) {
       const uint32_t w = (c0 + j * kFields < c_hi) ? __ldg(wp + j) : 0u;
       m |= (unsigned long long)nonzero_mask<LB>(w) << (j * kFields);
-      bits += level_code_bits<LB>(w);
+      bits = add_level_code_bits<LB>(w, bits);
     }
     if (m) {
       const int32_t lowest = (int32_t)c0 + __ffsll((long long)m) - 1;
@@ -240,27 +261,24 @@ __device__ __forceinline__ LaneSummary summarize_sparse(const uint32_t* tab, con
   return s;
 }
 
-// Whole level words are loaded once and their fields taken from the register (fields past the end of the
-// vector are zero in the fixed-width layout but are not coordinates: the count stops at c_hi).
+// Fields past the end of the vector are zero in the fixed-width layout but are not coordinates: the count stops at c_hi.
 template <int LB>
-__device__ __forceinline__ uint32_t summarize_dense(const uint32_t* tab, const uint32_t* __restrict__ lwb,
+__device__ __forceinline__ uint32_t summarize_dense(const SymbolLengths<LB>& lengths, const uint32_t* __restrict__ lwb,
                                                     uint32_t c_lo, uint32_t c_hi) {
   uint32_t bits = 0;
-  constexpr uint32_t kFields = 32u / LB, kMask = (1u << LB) - 1u;
+  constexpr uint32_t kFields = 32u / LB;
   for (uint32_t c0 = c_lo; c0 < c_hi; c0 += 64u) {
     const uint32_t* wp = lwb + ((c0 * LB) >> 5);
+    uint32_t w[2u * LB];
 #pragma unroll
-    for (uint32_t j = 0; j < 2u * LB; ++j) {
-      const uint32_t cw = c0 + j * kFields;                 // first coordinate of this word
-      if (cw >= c_hi) break;
-      const uint32_t w = __ldg(wp + j);
-      const uint32_t cnt = min(kFields, c_hi - cw);
-      if (cnt == kFields) {
+    for (uint32_t j = 0; j < 2u * LB; ++j) w[j] = c0 + j * kFields < c_hi ? __ldg(wp + j) : 0u;
+    const uint32_t left = c_hi - c0;
+    if (left >= 64u) {
 #pragma unroll
-        for (uint32_t f = 0; f < kFields; ++f) bits += 1u + tab_len(tab, ((w >> (f * LB)) & kMask) + 1u);
-      } else {
-        for (uint32_t f = 0; f < cnt; ++f) bits += 1u + tab_len(tab, ((w >> (f * LB)) & kMask) + 1u);
-      }
+      for (uint32_t j = 0; j < 2u * LB; ++j) bits += symbol_bits<LB>(lengths, w[j], kFields);
+    } else {
+#pragma unroll
+      for (uint32_t j = 0; j < 2u * LB; ++j) bits += symbol_bits<LB>(lengths, w[j], left > j * kFields ? left - j * kFields : 0u);
     }
   }
   return bits;
@@ -278,14 +296,6 @@ __device__ __forceinline__ int32_t prev_nonzero_before_lane(int32_t last, uint32
   return tl == 0 ? -1 : excl;
 }
 
-struct ScanArgs {              // what the last CTA of the length kernel needs for the scan
-  uint64_t ctas;
-  size_t out_capacity;
-  Ctrl* ctrl;
-  uint64_t* out_bits;
-  uint32_t* status_dev;
-};
-
 struct BucketParams {
   const float* A;
   const uint32_t* sign;
@@ -297,14 +307,14 @@ struct BucketParams {
 };
 
 // Bits of this lane's part of its bucket's string (the scale's 32 bits go with team lane 0).
-template <int LB, bool DENSE>
-__device__ __forceinline__ uint32_t lane_bits(const uint32_t* tab, const uint32_t* __restrict__ lwb, uint32_t lpb,
+template <int LB, bool DENSE, class Lengths>
+__device__ __forceinline__ uint32_t lane_bits(const uint32_t* tab, const Lengths& lengths, const uint32_t* __restrict__ lwb, uint32_t lpb,
                                               uint32_t c_lo, uint32_t c_hi, uint32_t tl, bool live,
                                               int32_t* prev_out) {
   uint32_t bits = 0;
   int32_t prev = -1;
-  if (DENSE) {
-    if (live) bits = summarize_dense<LB>(tab, lwb, c_lo, c_hi);
+  if constexpr (DENSE) {
+    if (live) bits = summarize_dense<LB>(lengths, lwb, c_lo, c_hi);
   } else {
     LaneSummary s{0u, -1, -1};
     if (live) s = summarize_sparse<LB>(tab, lwb, c_lo, c_hi);
@@ -326,97 +336,105 @@ __device__ __forceinline__ uint32_t team_sum(uint32_t v, uint32_t lpb) {
   return v;
 }
 
-// ---- scan of the per-CTA sums, run by the CTA of the length kernel that finishes last ------------
-__device__ __forceinline__ uint64_t block_exclusive_scan(uint64_t v, uint64_t* total) {
-  __shared__ uint64_t warp_sums[32];
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  uint64_t inc = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint64_t t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= (uint32_t)o) inc += t;
-  }
-  if (lane == 31) warp_sums[warp] = inc;
-  __syncthreads();
-  uint64_t before = 0, all = 0;
-  for (uint32_t w = 0; w < nwarps; ++w) {
-    const uint64_t t = warp_sums[w];
-    if (w < warp) before += t;
-    all += t;
-  }
-  __syncthreads();
-  *total = all;
-  return before + inc - v;
-}
-
-// In place: cta_sums[c] becomes the first payload bit of CTA c's run, cta_sums[ctas] the payload
-// length. Also: message geometry and capacity check. Called by all threads of one CTA.
-__device__ __forceinline__ void scan_cta_sums(uint64_t* cta_sums, uint64_t ctas, uint64_t B, size_t out_capacity,
-                                              Ctrl* ctrl, uint64_t* out_bits, uint32_t* status_dev) {
-  // every thread owns a contiguous chunk of the sums: one block-wide scan in total
-  const uint64_t chunk = (ctas + blockDim.x - 1) / blockDim.x;
-  const uint64_t lo = min((uint64_t)threadIdx.x * chunk, ctas), hi = min(lo + chunk, ctas);
-  uint64_t mine = 0;
-#pragma unroll 8
-  for (uint64_t i = lo; i < hi; ++i) mine += __ldcg(cta_sums + i);
-  uint64_t total;
-  uint64_t run = block_exclusive_scan(mine, &total);
-  if (threadIdx.x == 0) {
-    const uint64_t pay = align16((total + 7) / 8);
-    const uint64_t total_bytes = pay + 8 * (B + 1);
-    const bool ok = total_bytes <= out_capacity;
-    ctrl->total_bits = total;
-    ctrl->payload_bytes = pay;
-    ctrl->ok = ok ? 1u : 0u;
-    out_bits[0] = total; out_bits[1] = pay; out_bits[2] = total_bytes; out_bits[3] = 0;
+// Sizes of the whole message: the info words, the capacity check. False: it does not fit, nothing is written.
+__device__ __forceinline__ bool fix_geometry(uint64_t total, uint64_t B, size_t out_capacity, uint64_t* out_bits,
+                                             uint32_t* status_dev, bool report, uint64_t* payload_bytes) {
+  const uint64_t pay = align16((total + 7) / 8), bytes = pay + 8 * (B + 1);
+  const bool ok = bytes <= out_capacity;
+  if (report && threadIdx.x == 0) {
+    out_bits[0] = total; out_bits[1] = pay; out_bits[2] = bytes; out_bits[3] = 0;
     if (!ok) atomicOr(status_dev, QSGD_DEV_CAPACITY);
-    cta_sums[ctas] = total;
   }
-#pragma unroll 8
-  for (uint64_t i = lo; i < hi; ++i) {
-    const uint64_t v = __ldcg(cta_sums + i);
-    cta_sums[i] = run;
-    run += v;
-  }
+  *payload_bytes = pay;
+  return ok;
 }
 
-// Whole code words (code | length << 16) of the integers met most: every level, and gaps below 64.
-template <int LB>
+// By one warp: the first payload bit of this CTA's run, and the payload's length.
+__device__ __forceinline__ void find_start(const uint32_t* sums, const uint64_t* groups, uint64_t* start, uint64_t* all) {
+  const uint32_t lane = threadIdx.x & 31, count = (gridDim.x + kSumGroup - 1u) / kSumGroup, mine = blockIdx.x / kSumGroup;
+  uint64_t before = 0, total = 0;
+  for (uint32_t i = lane; i < count; i += 32u) {
+    const uint64_t v = __ldg(groups + i);
+    total += v;
+    before += i < mine ? v : 0ull;
+  }
+  for (uint32_t i = mine * kSumGroup + lane; i < blockIdx.x; i += 32u) before += __ldg(sums + i);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    before += __shfl_xor_sync(0xffffffffu, before, o);
+    total += __shfl_xor_sync(0xffffffffu, total, o);
+  }
+  if (lane == 0) { *start = before; *all = total; }
+}
+
+// Whole code words of what is met most, their bits from bit 31 down and their length in bits 0 .. 4: sign and level (entry
+// level | negative << LB), and gaps below 64. At most 27 bits together.
+template <int LB, bool DENSE>
 struct CodeWords {
-  uint32_t level[1u << LB];
-  uint32_t gap[64];
+  uint32_t level[2u << LB];
+  uint32_t gap[DENSE ? 1 : 64];
 };
-template <int LB>
-__device__ __forceinline__ void fill_code_words(CodeWords<LB>& words) {
-  for (uint32_t k = threadIdx.x; k < (1u << LB) + 64u; k += kThreads) {
-    const uint32_t v = k < (1u << LB) ? k : k - (1u << LB);
-    uint32_t ln = 0;
-    const uint32_t code = v ? elias_code(v, &ln) : 0u;
-    (k < (1u << LB) ? words.level[v] : words.gap[v]) = code | (ln << 16);
+template <int LB, bool DENSE>
+__device__ __forceinline__ void fill_code_words(CodeWords<LB, DENSE>& words) {
+  constexpr uint32_t kLevels = 2u << LB, kMask = (1u << LB) - 1u;
+  for (uint32_t k = threadIdx.x; k < kLevels + (DENSE ? 0u : 64u); k += kThreads) {
+    const bool is_level = k < kLevels;
+    const uint32_t v = is_level ? (k & kMask) + (DENSE ? 1u : 0u) : k - kLevels;
+    uint32_t ln = 0, code = v ? elias_code(v, &ln) : 0u;
+    if (is_level && v) { code |= (k >> LB) << ln; ++ln; }
+    const uint32_t e = v ? code << (32u - ln) | ln : 0u;
+    if (is_level) words.level[k] = e;
+    else words.gap[k - kLevels] = e;
   }
 }
 
-// Lane-private writer into the CTA's staging words in shared memory.
+// Lane-private writer into the CTA's staging words in shared memory: the bits of the word at `at` gather in `acc`.
 struct StageWriter {
-  uint32_t* words;
-  uint32_t widx;
-  uint64_t buf;
-  uint32_t nbuf;
-  __device__ __forceinline__ void begin(uint32_t* w, uint32_t start_bit) {
-    words = w; widx = start_bit >> 5; buf = 0; nbuf = start_bit & 31;
+  uint32_t at, acc, n;
+  __device__ __forceinline__ void begin(uint32_t* words, uint32_t start_bit) {
+    at = (uint32_t)__cvta_generic_to_shared(words) + (start_bit >> 5) * 4u; acc = 0u; n = start_bit & 31u;
   }
-  __device__ __forceinline__ void put(uint32_t code, uint32_t len) {   // len in [1, 32]
-    buf |= (uint64_t)code << (64 - nbuf - len);
-    nbuf += len;
-    if (nbuf >= 32) {
-      atomicOr(words + widx, (uint32_t)(buf >> 32));
-      ++widx; buf <<= 32; nbuf -= 32;
+  // `len` <= 31 bits from bit 31 of c down; below them c is zero
+  __device__ __forceinline__ void put(uint32_t c, uint32_t len) {
+    acc |= c >> n;
+    n += len;
+    if (n >= 32u) {
+      asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(at), "r"(acc) : "memory");
+      at += 4u;
+      n -= 32u;
+      acc = c << (len - n);
     }
   }
+  // The same without a branch, for lanes that put one symbol after the other and come to a word's end at different times.
+  __device__ __forceinline__ void put_even(uint32_t c, uint32_t len) {
+    acc |= c >> n;
+    n += len;
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .u32 t;\n\tsetp.ge.u32 p, %2, 32;\n\t@p red.shared.or.b32 [%0], %1;\n\t@p add.u32 %0, %0, 4;\n\t"
+                 "and.b32 %2, %2, 31;\n\tsub.u32 t, %4, %2;\n\t@p shl.b32 %1, %3, t;\n\t}"
+                 : "+r"(at), "+r"(acc), "+r"(n) : "r"(c), "r"(len) : "memory");
+  }
+  __device__ __forceinline__ void put_word(uint32_t c) {
+    asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(at), "r"(acc | c >> n) : "memory");
+    at += 4u;
+    acc = __funnelshift_l(0u, c, 32u - n) & (n ? 0xFFFFFFFFu : 0u);
+  }
   __device__ __forceinline__ void finish() {
-    if (nbuf) atomicOr(words + widx, (uint32_t)(buf >> 32));
+    if (n) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(at), "r"(acc) : "memory");
   }
 };
+
+// One nonzero: gap, then sign and level (entry `idx` of words.level), in one piece but for gaps from 64 on, whose code goes ahead.
+template <int LB>
+__device__ __forceinline__ void put_entry(StageWriter& bw, const uint32_t* tab, const CodeWords<LB, false>& words, uint32_t gap, uint32_t idx) {
+  if (gap >= 64u) {
+    uint32_t gl;
+    const uint32_t gcode = tab_code(tab, gap, &gl);
+    bw.put(gcode << (32u - gl), gl);
+    gap = 0u;                                            // nothing of it is left
+  }
+  const uint32_t l = words.level[idx], g = words.gap[gap];
+  bw.put((g & ~31u) | __funnelshift_r(l & ~31u, 0u, g), (g + l) & 31u);
+}
 
 inline uint32_t host_elias_len(uint32_t k) {
   uint32_t len = 1;
@@ -429,10 +447,11 @@ inline uint32_t host_elias_len(uint32_t k) {
   return len;
 }
 
-// Staging: the longest legal strings of a CTA's buckets, plus the shared lead-in word.
+// Staging: the longest strings that the fields of a CTA's buckets can make, plus the shared lead-in word.
 template <bool DENSE>
 inline size_t stage_bytes(uint32_t buckets, uint32_t d, uint32_t s) {
-  const uint32_t per = DENSE ? 1 + host_elias_len(s + 1) : 2 + host_elias_len(s);
+  const uint32_t most = (1u << level_bits_for(s)) - 1u;
+  const uint32_t per = DENSE ? 1 + host_elias_len(most + 1) : 2 + host_elias_len(most);
   const size_t run_bits = (size_t)buckets * (32 + (size_t)d * per);
   return ((run_bits + 31) / 32 + 4) * 4;
 }
@@ -550,18 +569,19 @@ __device__ __forceinline__ int32_t nonzero_before(const Piece<LB>& q, uint32_t m
 }
 
 // Bits of the piece's part of its bucket's string (with the scale's 32 where the bucket starts).
-template <int LB, bool DENSE>
-__device__ __forceinline__ uint32_t piece_bits(const uint32_t* tab, const Piece<LB>& q, uint32_t mask, int32_t prev) {
+template <int LB, bool DENSE, class Lengths>
+__device__ __forceinline__ uint32_t piece_bits(const uint32_t* tab, const Lengths& lengths, const Piece<LB>& q, uint32_t mask, int32_t prev) {
   uint32_t bits = q.count && q.c0 == 0u ? 32u : 0u;
-  if (DENSE) {
+  if constexpr (DENSE) {
+    constexpr uint32_t kFields = LB == 1 ? 16u : 32u / LB;
 #pragma unroll
-    for (uint32_t j = 0; j < 16; ++j)
-      if (j < q.count) bits += 1u + tab_len(tab, piece_level<LB>(q, j) + 1u);
+    for (uint32_t j = 0; j < Piece<LB>::kWords; ++j)
+      bits += symbol_bits<LB>(lengths, q.level[j], q.count > j * kFields ? q.count - j * kFields : 0u);
     return bits;
   }
   if (mask) {
 #pragma unroll
-    for (int j = 0; j < Piece<LB>::kWords; ++j) bits += level_code_bits<LB>(q.level[j]);
+    for (int j = 0; j < Piece<LB>::kWords; ++j) bits = add_level_code_bits<LB>(q.level[j], bits);
     bits += gap_code_bits16(mask);
     bits += tab_len(tab, q.c0 + (uint32_t)__ffs((int)mask) - 1u - (uint32_t)prev);
   }
@@ -570,49 +590,32 @@ __device__ __forceinline__ uint32_t piece_bits(const uint32_t* tab, const Piece<
 
 // Assembles the piece's codes at bit `bit` of the CTA's staging words.
 template <int LB, bool DENSE>
-__device__ __forceinline__ void emit_piece(const uint32_t* tab, const CodeWords<LB>& words, uint32_t* stage, uint32_t bit,
+__device__ __forceinline__ void emit_piece(const uint32_t* tab, const CodeWords<LB, DENSE>& words, uint32_t* stage, uint32_t bit,
                                            const Piece<LB>& q, uint32_t mask, int32_t prev, float A) {
+  constexpr uint32_t kMask = (1u << LB) - 1u;
   StageWriter bw;
   bw.begin(stage, bit);
-  if (q.c0 == 0u) bw.put(__float_as_uint(A), 32);
-  if (DENSE) {
+  if (q.c0 == 0u) bw.put_word(__float_as_uint(A));
+  if constexpr (DENSE) {
 #pragma unroll
     for (uint32_t j = 0; j < 16; ++j) {
-      if (j >= q.count) break;
-      uint32_t ln;
-      const uint32_t code = tab_code(tab, piece_level<LB>(q, j) + 1u, &ln);
-      bw.put((((q.sign >> j) & 1u) << ln) | code, ln + 1u);
+      const uint32_t e = j < q.count ? words.level[piece_level<LB>(q, j) | ((q.sign >> j) & 1u) << LB] : 0u;
+      bw.put_even(e & ~31u, e & 31u);
     }
   } else {
     while (mask) {                                 // once per nonzero of the busiest lane
       const uint32_t j = (uint32_t)__ffs((int)mask) - 1u;
       mask &= mask - 1u;
-      const uint32_t pos = q.c0 + j, gap = pos - (uint32_t)prev;
-      uint32_t level, gcode, gl;
+      const uint32_t pos = q.c0 + j;
+      uint32_t w = q.level[0];
       if (LB == 8) {
         const uint32_t lo = j & 4u ? q.level[1 % Piece<LB>::kWords] : q.level[0];
         const uint32_t hi = j & 4u ? q.level[3 % Piece<LB>::kWords] : q.level[2 % Piece<LB>::kWords];
-        level = ((j & 8u ? hi : lo) >> (8u * (j & 3u))) & 0xFFu;
+        w = j & 8u ? hi : lo;
       } else if (LB == 4) {
-        level = (q.level[j >> 3 ? 1 % Piece<LB>::kWords : 0] >> (4u * (j & 7u))) & 15u;
-      } else {
-        level = (q.level[0] >> (LB * j)) & ((1u << LB) - 1u);
+        w = j & 8u ? q.level[1 % Piece<LB>::kWords] : q.level[0];
       }
-      if (gap < 64u) {
-        const uint32_t e = words.gap[gap];
-        gcode = e & 0xFFFFu;
-        gl = e >> 16;
-      } else {
-        gcode = tab_code(tab, gap, &gl);
-      }
-      const uint32_t e = words.level[level], ll = e >> 16;
-      const uint32_t lcode = (e & 0xFFFFu) | (((q.sign >> j) & 1u) << ll);
-      if (gl + ll + 1u <= 32u) {                   // gap, sign and level in one piece (the rule)
-        bw.put((gcode << (ll + 1u)) | lcode, gl + ll + 1u);
-      } else {
-        bw.put(gcode, gl);
-        bw.put(lcode, ll + 1u);
-      }
+      put_entry<LB>(bw, tab, words, pos - (uint32_t)prev, (__funnelshift_r(w, 0u, LB * j) & kMask) | ((q.sign >> j) & 1u) << LB);
       prev = (int32_t)pos;
     }
   }
@@ -636,7 +639,8 @@ __device__ __forceinline__ void flush_run(uint32_t* __restrict__ gw, const uint3
 }
 
 // elias_encode_small.cu
-int launch_tile_scatter(const BucketParams& bp, const EliasWs& w, uint32_t s, bool dense, uint8_t* out, cudaStream_t stream);
+int launch_tile_scatter(const BucketParams& bp, const EliasWs& w, uint32_t s, bool dense, uint8_t* out, size_t out_capacity,
+                        uint64_t* out_bits, uint32_t* status_dev, cudaStream_t stream);
 int launch_elias_encode_small(const float* g, uint64_t n, uint32_t d, uint32_t s, int norm_kind, bool dense, uint64_t seed,
                               uint32_t step, uint32_t worker, uint8_t* out, size_t out_capacity, uint64_t* out_bits,
                               const EliasWs& w, uint32_t* status_dev, cudaStream_t stream);

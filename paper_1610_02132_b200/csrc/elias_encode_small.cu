@@ -21,7 +21,7 @@ struct SmallParams {
   QuantizeParams q;           // what quantizing needs; its regions are those of bp
   BucketParams bp;
   uint32_t log2d;             // of a power-of-two bucket size, else 32
-  uint64_t* cta_sums;         // bits of every tile
+  uint32_t* cta_sums;         // bits of every tile
   // one tile:
   uint8_t* out;
   size_t out_capacity;
@@ -29,22 +29,9 @@ struct SmallParams {
   uint32_t* status_dev;
 };
 
-// Sizes of the whole message: the info words, the capacity check. False: it does not fit, nothing is written.
-__device__ __forceinline__ bool fix_geometry(uint64_t total, uint64_t B, size_t out_capacity, uint64_t* out_bits,
-                                             uint32_t* status_dev, bool report, uint64_t* payload_bytes) {
-  const uint64_t pay = align16((total + 7) / 8), bytes = pay + 8 * (B + 1);
-  const bool ok = bytes <= out_capacity;
-  if (report && threadIdx.x == 0) {
-    out_bits[0] = total; out_bits[1] = pay; out_bits[2] = bytes; out_bits[3] = 0;
-    if (!ok) atomicOr(status_dev, QSGD_DEV_CAPACITY);
-  }
-  *payload_bytes = pay;
-  return ok;
-}
-
 // Writes one tile's run of strings: table entries, codes into `stage` (zeroed), the flush.
 template <int LB, bool DENSE>
-__device__ __forceinline__ void write_tile(const uint32_t* tab, const CodeWords<LB>& words, uint32_t* stage, const BucketParams& p,
+__device__ __forceinline__ void write_tile(const uint32_t* tab, const CodeWords<LB, DENSE>& words, uint32_t* stage, const BucketParams& p,
                                            const Piece<LB>& q, uint32_t mask, int32_t prev, uint32_t bits, uint32_t before,
                                            float A, uint64_t start, uint32_t span, uint64_t payload_bytes, uint8_t* out) {
   const uint32_t lead = (uint32_t)(start & 31);    // bits of the first word that belong to the tile before
@@ -144,9 +131,11 @@ __global__ void __launch_bounds__(kThreads) elias_quantize_length_kernel(const _
   __shared__ float s_rcp[kMaxBucketsPerTile];
   __shared__ uint32_t slots[2][kWarps];
   __shared__ uint32_t tab[17];
-  __shared__ CodeWords<ONE ? LB : 1> words;
+  __shared__ CodeWords<ONE ? LB : 1, DENSE> words;
+  __shared__ SymbolLengths<DENSE ? LB : 1> lengths;
   fill_code_table(tab);
-  if (ONE && !DENSE) fill_code_words<ONE ? LB : 1>(words);
+  if (DENSE) fill_symbol_lengths<DENSE ? LB : 1>(lengths);
+  if (ONE) fill_code_words(words);
   chain_wait();
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   Piece<LB> q;
@@ -173,7 +162,7 @@ __global__ void __launch_bounds__(kThreads) elias_quantize_length_kernel(const _
   __syncthreads();                                  // the code tables are there
   const uint32_t mask = DENSE ? 0u : piece_mask<LB>(q);
   const int32_t prev = DENSE ? -1 : nonzero_before<LB>(q, mask, slots[0]);
-  const uint32_t bits = piece_bits<LB, DENSE>(tab, q, mask, prev);
+  const uint32_t bits = piece_bits<LB, DENSE>(tab, lengths, q, mask, prev);
   uint32_t total;
   const uint32_t before = cta_sum_before(bits, slots[1], &total);
   if constexpr (!ONE) {
@@ -187,12 +176,12 @@ __global__ void __launch_bounds__(kThreads) elias_quantize_length_kernel(const _
   }
 }
 
-// Where a tile's run of strings begins and how long the payload is: from the scan that the length kernel left
-// (ctrl), or by adding up the lengths of all tiles here.
+// Where a tile's run of strings begins and how long the payload is: by sums over groups of tiles, or, in small problems, where
+// nothing has cleared those, every CTA adds up the lengths of all tiles.
 struct TileScatterArgs {
   BucketParams bp;
-  const uint64_t* sums;       // starts of the runs, or lengths
-  const Ctrl* ctrl;           // null: lengths
+  const uint32_t* sums;       // bits of every tile
+  const uint64_t* groups;     // of every kSumGroup tiles, or null
   uint32_t ctas;
   uint8_t* out;
   size_t out_capacity;
@@ -206,26 +195,29 @@ __global__ void __launch_bounds__(kThreads) elias_tile_scatter_kernel(const __gr
   __shared__ uint32_t slots[2][kWarps];
   __shared__ uint64_t before_s[kWarps], total_s[kWarps];
   __shared__ uint32_t tab[17];
-  __shared__ CodeWords<LB> words;
+  __shared__ CodeWords<LB, DENSE> words;
+  __shared__ SymbolLengths<DENSE ? LB : 1> lengths;
   fill_code_table(tab);
-  if (!DENSE) fill_code_words<LB>(words);
+  fill_code_words(words);
+  if (DENSE) fill_symbol_lengths<DENSE ? LB : 1>(lengths);
   chain_wait();                                    // fields and sums come from the kernel ahead
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const Piece<LB> q = load_piece<LB>(a.bp);
   const float A = q.count && q.c0 == 0u ? a.bp.A[(uint64_t)blockIdx.x * a.bp.nbc + q.bucket] : 0.f;
-  uint64_t start, pay;
-  uint32_t span;
-  if (a.ctrl) {
-    if (!a.ctrl->ok) return;
-    start = a.sums[blockIdx.x];
-    span = (uint32_t)(a.sums[blockIdx.x + 1] - start);
-    pay = a.ctrl->payload_bytes;
+  uint64_t start, tot;
+  const uint32_t span = a.sums[blockIdx.x];
+  if (a.groups) {
+    if (warp == 0) find_start(a.sums, a.groups, &before_s[0], &total_s[0]);
+    __syncthreads();
+    start = before_s[0];
+    tot = total_s[0];
   } else {
-    uint64_t bef = 0, tot = 0;
+    uint64_t bef = 0;
+    tot = 0;
     for (uint32_t i = tid; i < a.ctas; i += kThreads) {
-      const uint64_t v = a.sums[i];
+      const uint32_t v = a.sums[i];
       tot += v;
-      bef += i < blockIdx.x ? v : 0ull;
+      bef += i < blockIdx.x ? v : 0u;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -238,15 +230,15 @@ __global__ void __launch_bounds__(kThreads) elias_tile_scatter_kernel(const __gr
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) { bef += before_s[w]; tot += total_s[w]; }
     start = bef;
-    span = (uint32_t)a.sums[blockIdx.x];
-    if (!fix_geometry(tot, a.bp.B, a.out_capacity, a.out_bits, a.status_dev, blockIdx.x == 0, &pay)) return;
   }
+  uint64_t pay;
+  if (!fix_geometry(tot, a.bp.B, a.out_capacity, a.out_bits, a.status_dev, blockIdx.x == 0, &pay)) return;
   const uint32_t nwords = ((uint32_t)(start & 31) + span + 31u) >> 5;
   for (uint32_t j = tid; j < nwords; j += kThreads) stage[j] = 0u;
   __syncthreads();                                 // staging zeroed, tables there
   const uint32_t mask = DENSE ? 0u : piece_mask<LB>(q);
   const int32_t prev = DENSE ? -1 : nonzero_before<LB>(q, mask, slots[0]);
-  const uint32_t bits = piece_bits<LB, DENSE>(tab, q, mask, prev);
+  const uint32_t bits = piece_bits<LB, DENSE>(tab, lengths, q, mask, prev);
   uint32_t total;
   const uint32_t before = cta_sum_before(bits, slots[1], &total);
   write_tile<LB, DENSE>(tab, words, stage, a.bp, q, mask, prev, bits, before, A, start, span, pay, a.out);
@@ -288,10 +280,11 @@ int quantize_lb(const SmallParams& p, int norm_kind, bool dense, uint32_t ctas, 
 
 namespace elias {
 
-int launch_tile_scatter(const BucketParams& bp, const EliasWs& w, uint32_t s, bool dense, uint8_t* out, cudaStream_t stream) {
+int launch_tile_scatter(const BucketParams& bp, const EliasWs& w, uint32_t s, bool dense, uint8_t* out, size_t out_capacity,
+                        uint64_t* out_bits, uint32_t* status_dev, cudaStream_t stream) {
   TileScatterArgs a;
-  a.bp = bp; a.sums = w.tile_sums; a.ctrl = w.ctrl; a.ctas = (uint32_t)((bp.B + bp.nbc - 1) / bp.nbc); a.out = out;
-  a.out_capacity = 0; a.out_bits = nullptr; a.status_dev = nullptr;
+  a.bp = bp; a.sums = w.tile_sums; a.groups = w.tile_groups; a.ctas = (uint32_t)((bp.B + bp.nbc - 1) / bp.nbc); a.out = out;
+  a.out_capacity = out_capacity; a.out_bits = out_bits; a.status_dev = status_dev;
   return scatter_any(a, s, dense, stream);
 }
 
@@ -308,7 +301,7 @@ int launch_elias_encode_small(const float* g, uint64_t n, uint32_t d, uint32_t s
   p.q.sign_out = reinterpret_cast<uint32_t*>(w.fixed + L.off_sign);
   p.q.level_out = reinterpret_cast<uint32_t*>(w.fixed + L.off_level);
   p.q.B = L.B; p.q.sign_words = L.sign_words; p.q.level_words = L.level_words;
-  p.q.tiles = 0; p.q.status = status_dev; p.q.info = nullptr; p.q.total_bytes = L.total; p.q.clear_word = nullptr;
+  p.q.tiles = 0; p.q.status = status_dev; p.q.info = nullptr; p.q.total_bytes = L.total; p.q.clear = ClearWords{nullptr, 0};
   p.bp.A = p.q.A_out; p.bp.sign = p.q.sign_out; p.bp.level = p.q.level_out;
   p.bp.n = n; p.bp.d = d; p.bp.B = L.B; p.bp.lpb = 0; p.bp.seg = 16; p.bp.nbc = tile_buckets(d);
   p.log2d = 32;
@@ -326,7 +319,7 @@ int launch_elias_encode_small(const float* g, uint64_t n, uint32_t d, uint32_t s
   }
   if (st || ctas == 1u) return st;
   TileScatterArgs a;
-  a.bp = p.bp; a.sums = w.tile_sums; a.ctrl = nullptr; a.ctas = ctas; a.out = out;
+  a.bp = p.bp; a.sums = w.tile_sums; a.groups = nullptr; a.ctas = ctas; a.out = out;
   a.out_capacity = out_capacity; a.out_bits = out_bits; a.status_dev = status_dev;
   return scatter_any(a, s, dense, stream);
 }

@@ -71,9 +71,15 @@ struct BucketMap {
 
 inline BucketMap no_map() { return BucketMap{nullptr, nullptr, 1u}; }
 
+// Words that a quantizing kernel sets to zero for a later kernel (none: count 0).
+struct ClearWords {
+  uint64_t* at;
+  uint32_t count;
+};
+
 int launch_quantize_fixed(const float* g, uint64_t n, uint32_t d, uint32_t s, int norm_kind,
                           uint64_t seed, uint32_t step, uint32_t worker, uint8_t* out,
-                          uint32_t* status_dev, uint64_t* info, uint32_t* clear_word, const BucketMap& map,
+                          uint32_t* status_dev, uint64_t* info, const ClearWords& clear, const BucketMap& map,
                           cudaStream_t stream);
 
 int launch_decode_fixed(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d, uint32_t s,

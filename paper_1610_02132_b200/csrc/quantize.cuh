@@ -37,10 +37,15 @@ struct QuantizeParams {
   uint32_t* status;
   uint64_t* info;         // optional: the four message-info words of a fixed-width message
   uint64_t total_bytes;
-  uint32_t* clear_word;   // optional: a word the kernel sets to zero (arrival counter of a later kernel)
+  ClearWords clear;
   BucketMap map;          // per-tensor policy: where each bucket lives in g, or no map
   PhiloxConsts pc;
 };
+
+// By all threads of one CTA.
+__device__ __forceinline__ void clear_words(const ClearWords& c) {
+  for (uint32_t i = threadIdx.x; i < c.count; i += kQuantizeThreads) c.at[i] = 0ull;
+}
 
 __device__ __forceinline__ float fma_rn(float a, float b, float c) {
   float r;
@@ -223,7 +228,7 @@ __device__ __forceinline__ void quantize_generic_tile(const QuantizeParams& p, u
   if (block == 0 && tid == 0 && p.info) {
     p.info[0] = 8 * p.total_bytes; p.info[1] = 0; p.info[2] = p.total_bytes; p.info[3] = 0;
   }
-  if (block == 0 && tid == 0 && p.clear_word) *p.clear_word = 0u;
+  if (block == 0) clear_words(p.clear);
   const uint64_t left = p.n - t0;
   const uint32_t valid = left < p.tile_coords ? (uint32_t)left : p.tile_coords;
   if (valid == 0) {                            // nothing left to encode: only the padding

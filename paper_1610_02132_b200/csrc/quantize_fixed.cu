@@ -103,7 +103,7 @@ struct FastParams {
   uint32_t* status;
   uint64_t* info;           // optional message-info words, written by CTA 0
   uint64_t total_bytes;
-  uint32_t* clear_word;     // optional word set to zero by CTA 0
+  ClearWords clear;         // set to zero by CTA 0
   PhiloxConsts pc;
   uint32_t main_ctas;       // CTAs that stream complete tiles
   uint32_t poll_limit;      // bound of the main-loop waits (the final drain keeps its own bound)
@@ -183,11 +183,11 @@ quantize_pow2_kernel(const __grid_constant__ FastParams p) {
   }
   chain_wait();                                 // nothing above touches global memory
   __syncthreads();
+  if (blockIdx.x == 0) clear_words(p.clear);
   if (MAPPED ? warp == 0 : tid == 0) {
     if (tid == 0 && blockIdx.x == 0 && p.info) {
       p.info[0] = 8 * p.total_bytes; p.info[1] = 0; p.info[2] = p.total_bytes; p.info[3] = 0;
     }
-    if (tid == 0 && blockIdx.x == 0 && p.clear_word) *p.clear_word = 0u;
     for (int s = 0; s < kStages; ++s) {
       const uint32_t t = blockIdx.x + (uint32_t)s * grid;
       if (t < p.full_tiles) issue_tile<MAPPED>(p, sm.tile[s], &sm.full[s], t, lane);
@@ -421,9 +421,9 @@ quantize_warp_kernel(const __grid_constant__ FastParams p) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   chain_wait();                                 // nothing above touches global memory
-  if (tid == 0 && blockIdx.x == 0) {
-    if (p.info) { p.info[0] = 8 * p.total_bytes; p.info[1] = 0; p.info[2] = p.total_bytes; p.info[3] = 0; }
-    if (p.clear_word) *p.clear_word = 0u;
+  if (blockIdx.x == 0) {
+    if (tid == 0 && p.info) { p.info[0] = 8 * p.total_bytes; p.info[1] = 0; p.info[2] = p.total_bytes; p.info[3] = 0; }
+    clear_words(p.clear);
   }
   __syncwarp();
   for (int s = 0; s < kWarpStages; ++s) {
@@ -603,9 +603,9 @@ quantize_group_kernel(const __grid_constant__ FastParams p) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   chain_wait();                                 // nothing above touches global memory
-  if (tid == 0 && blockIdx.x == 0) {
-    if (p.info) { p.info[0] = 8 * p.total_bytes; p.info[1] = 0; p.info[2] = p.total_bytes; p.info[3] = 0; }
-    if (p.clear_word) *p.clear_word = 0u;
+  if (blockIdx.x == 0) {
+    if (tid == 0 && p.info) { p.info[0] = 8 * p.total_bytes; p.info[1] = 0; p.info[2] = p.total_bytes; p.info[3] = 0; }
+    clear_words(p.clear);
   }
   __syncwarp();
   for (int s = 0; s < kWarpStages; ++s) {
@@ -792,7 +792,7 @@ int launch_one(QuantizeParams& p, cudaStream_t stream) {
     fp.log2d = 0;
     while ((1u << fp.log2d) < d) ++fp.log2d;
     fp.A_out = p.A_out; fp.sign_out = p.sign_out; fp.level_out = p.level_out; fp.status = p.status;
-    fp.info = p.info; fp.total_bytes = p.total_bytes; fp.clear_word = p.clear_word;
+    fp.info = p.info; fp.total_bytes = p.total_bytes; fp.clear = p.clear;
     fp.pc = p.pc;
     fp.map = p.map;
     // the ragged tail (fewer than 4096 coordinates) and the zero padding of the three regions go
@@ -802,7 +802,7 @@ int launch_one(QuantizeParams& p, cudaStream_t stream) {
     const bool with_tail = !(p.n == p.coord_base && ((p.B | p.sign_words | p.level_words) & 3ull) == 0);
     fp.tail = p;
     fp.tail.info = nullptr;
-    fp.tail.clear_word = nullptr;
+    fp.tail.clear.count = 0;
     if (d >= 1024) {
       // measured (n = 60 M, s = 15 / 255): with the 2-norm the per-warp pipelines with group barriers
       // take 83-86 us against the CTA-wide ring's 90-92; with the max-norm (100 against 84) and under a
@@ -839,7 +839,7 @@ int launch_lb(QuantizeParams& p, int norm_kind, cudaStream_t stream) {
 
 int launch_quantize_fixed(const float* g, uint64_t n, uint32_t d, uint32_t s, int norm_kind,
                           uint64_t seed, uint32_t step, uint32_t worker, uint8_t* out,
-                          uint32_t* status_dev, uint64_t* info, uint32_t* clear_word, const BucketMap& map,
+                          uint32_t* status_dev, uint64_t* info, const ClearWords& clear, const BucketMap& map,
                           cudaStream_t stream) {
   const FixedLayout L = make_fixed_layout(n, d, s);
   QuantizeParams p;
@@ -855,7 +855,7 @@ int launch_quantize_fixed(const float* g, uint64_t n, uint32_t d, uint32_t s, in
   p.status = status_dev;
   p.info = info;
   p.total_bytes = L.total;
-  p.clear_word = clear_word;
+  p.clear = clear;
   switch (L.lb) {
     case 1: return launch_lb<1>(p, norm_kind, stream);
     case 2: return launch_lb<2>(p, norm_kind, stream);
