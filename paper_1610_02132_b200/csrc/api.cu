@@ -64,7 +64,8 @@ int device_shared_memory(int* bytes_out) {
 static const char* const kKernelNames[kKernCount] = {
     "quantize_fixed", "quantize_tail", "decode_fixed", "sgd_step", "elias_length",
     "elias_scatter", "decode_elias", "decode_elias_sparse", "raw_gather", "raw_decode",
-    "decode_elias_teams", "decode_elias_fields", "decode_elias_bytes"};
+    "decode_elias_teams", "decode_elias_fields", "decode_elias_bytes",
+    "decode_elias_dense"};
 
 namespace {
 

@@ -6,6 +6,9 @@
 // in elias_decode_teams.cu, the nonzero-driven decoder of the sparse regime in elias_decode_sparse.cu; what they
 // share is in elias_decode.cuh.
 #include "elias_decode.cuh"
+#ifndef DL
+#define DL 8192
+#endif
 
 namespace qsgd {
 
@@ -86,6 +89,7 @@ int launch_decode_elias(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
   f.peers = peers; f.K = K; f.n = n; f.d = d; f.s = s; f.B = B;
   f.out = acc_or_x; f.c = eta / (float)K; f.minus_zero = -0.f; f.status = status_dev; f.map = map;
   f.when = Regime{0u, kNoBound};
+  if (dense && s <= 127u && K <= 32u && B * K > DL) return launch_elias_dense(f, fused, stream);
   if (dense || K > 32u) return launch_elias_teams(f, dense, fused, stream);
 
   const bool teams = use_teams(B, K, d, s), small = teams && work <= kSmallWork;

@@ -49,6 +49,7 @@ struct BytesParams {
   uint64_t B;
   float* out;             // acc (overwritten) or x (updated in place)
   float c;                // eta / K
+  float minus_zero;       // add_product2
   uint32_t* status;
   Regime when;
   BucketMap map;
@@ -165,20 +166,21 @@ __global__ void __launch_bounds__(512) decode_elias_bytes_kernel(const __grid_co
         const uint32_t gg = there ? g : 0u;
         const uint8_t* rows = mine + gg * K * row_bytes + cl;
         const float* sc = scales + gg * Kpad;
-        float acc[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+        float2p sum[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll 4
         for (uint32_t k = 0; k < K; ++k) {
           const uint2 cw = there ? *reinterpret_cast<const uint2*>(rows + k * row_bytes) : make_uint2(0u, 0u);
           const float Ak = sc[k];
           const float lutk = SINGLE ? __fmul_rn(Ak, lut0) : lut0;
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float v = shfl_f(lutk, (e < 4 ? cw.x : cw.y) >> (8 * (e & 3)));
-            acc[e] = __fadd_rn(acc[e], SINGLE ? v : __fmul_rn(Ak, v));
+          for (int e = 0; e < 8; e += 2) {
+            const uint32_t w = (e < 4 ? cw.x : cw.y) >> (8 * (e & 3));
+            sum[e / 2] = add_pair_lut<SINGLE>(sum[e / 2], w, w >> 8, lutk, Ak, p.minus_zero);
           }
         }
+        float acc[8];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { const float2 u = unpair2(sum[e]); acc[2 * e] = u.x; acc[2 * e + 1] = u.y; }
         if (live) store_span8<FUSED>(out_span(p.out, p.map, b, c, p.d, p.n, 8u), acc, p.c);
       }
       __syncwarp();
@@ -195,7 +197,7 @@ int launch_elias_bytes(const FieldParams& f, bool fused, cudaStream_t stream) {
   static KernelSite site[4];
   BytesParams p;
   p.peers = f.peers; p.K = f.K; p.n = f.n; p.d = f.d; p.s = f.s; p.B = f.B; p.out = f.out; p.c = f.c;
-  p.status = f.status; p.when = f.when; p.map = f.map;
+  p.status = f.status; p.when = f.when; p.map = f.map; p.minus_zero = f.minus_zero;
   p.Kpad = 1;
   while (p.Kpad < p.K) p.Kpad <<= 1;
   p.G = 32u / p.Kpad;

@@ -17,7 +17,13 @@
 // on what was read but data: lanes with different codes stay together. A gap
 // that no table entry covers (64 or more) is decoded by all lanes that have come to one together, whatever else there is
 // (a malformed code) by the definition's decoder with every check (slow_entry).
-#include "elias_decode.cuh"
+//
+// What bounds it (n = 34 M, d = 512, s = 15, K = 16, a mixture of two scales): shared memory and the shuffles' data path, 70 % of
+// its wavefronts (416 per step of a warp: 128 shuffles, about 96 byte stores and 48 lookups that meet in banks, 48 rows and
+// scales, 36 copies, 34 zeros, 41 sums written), beside 67 % of the issue slots, with the 15 warps that fit. Sums in pairs: 469
+// -> 461 us at n = 60 M. Without any sum it takes 359. A burst of 53 instead of 64 instructions, 18 warps with half of the
+// stream's bytes in shared memory: no faster (472 and 457; 3265 and 3472 against 3284 at n = 268 M, N(0, 1)).
+#include "elias_stream.cuh"
 
 namespace qsgd {
 
@@ -84,6 +90,7 @@ struct RingParams {
   uint64_t B;
   float* out;             // acc (overwritten) or x (updated in place)
   float c;                // eta / K
+  float minus_zero;       // add_product2
   uint32_t* status;
   uint32_t run;           // buckets per run
   uint32_t slots;         // scales kept per lane, a power of two: the buckets that a ring can touch
@@ -91,36 +98,6 @@ struct RingParams {
   Regime when;
   BucketMap map;
 };
-
-__device__ __forceinline__ uint32_t shared_address(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-// The same and a load where `when` is nonzero, without a branch.
-__device__ __forceinline__ void store_byte_if(uint32_t when, uint32_t addr, uint32_t v) {
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.u8 [%1], %2;\n\t}" ::"r"(when), "r"(addr), "r"(v)
-               : "memory");
-}
-__device__ __forceinline__ void load_word_if(bool when, uint32_t& v, uint32_t addr) {
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p ld.shared.u32 %0, [%2];\n\t}" : "+r"(v) : "r"((uint32_t)when), "r"(addr)
-               : "memory");
-}
-__device__ __forceinline__ void store_byte(uint32_t addr, uint32_t v) {
-  asm volatile("st.shared.u8 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ uint32_t load_word(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ void load_words(uint32_t addr, uint32_t& a, uint32_t& b) {
-  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(addr) : "memory");
-}
-// 16 bytes from global to shared memory, in the background; and the wait for all of this thread's.
-__device__ __forceinline__ void copy16(uint32_t addr, const void* from) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(addr), "l"(from) : "memory");
-}
-__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-__device__ __forceinline__ void zero_quad(uint32_t addr) {
-  asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "r"(0) : "memory");
-}
 
 // One entry (or the rest of one) by the definition's decoder, with every check: the QSGD_DEV_* faults, or the
 // next state, last position passed and bits used. The caller stores a rest's byte.
@@ -386,9 +363,9 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
         for (uint32_t h = 0; h < V / 4; ++h) x[h] = reinterpret_cast<const float4*>(sp.ptr)[h];
       const uint32_t row0 = shared_mine + gq * p.K * kRing, pos = (q & (kRing - 1u)) ^ (gq * p.Kpad * 8u);
       const float* sc = scales + (bq & (p.slots - 1u)) * 32u + gq * p.Kpad;
-      float acc[V];
+      float2p sum[V / 2];
 #pragma unroll
-      for (uint32_t e = 0; e < V; ++e) acc[e] = 0.f;
+      for (uint32_t e = 0; e < V / 2; ++e) sum[e] = 0ull;
 #pragma unroll 4
       for (uint32_t kk = 0; kk < p.K; ++kk) {
         uint32_t w[V / 4];
@@ -397,8 +374,13 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_ring_kernel(co
         else w[0] = load_word(addr);
         const float A = sc[kk];
 #pragma unroll
-        for (uint32_t e = 0; e < V; ++e) acc[e] = __fadd_rn(acc[e], __fmul_rn(A, shfl_f(lut0, w[e >> 2] >> (8u * (e & 3u)))));
+        for (uint32_t e = 0; e < V; e += 2)
+          sum[e / 2] = add_product2(sum[e / 2], A, shfl_f(lut0, w[e >> 2] >> (8u * (e & 3u))), shfl_f(lut0, w[e >> 2] >> (8u * (e & 3u) + 8u)),
+                                    p.minus_zero);
       }
+      float acc[V];
+#pragma unroll
+      for (uint32_t e = 0; e < V / 2; ++e) { const float2 u = unpair2(sum[e]); acc[2 * e] = u.x; acc[2 * e + 1] = u.y; }
       if (whole) {
 #pragma unroll
         for (uint32_t h = 0; h < V / 4; ++h) {
@@ -437,7 +419,7 @@ int launch_elias_ring(const FieldParams& f, bool fused, cudaStream_t stream) {
   static KernelSite site[4];
   RingParams p;
   p.peers = f.peers; p.K = f.K; p.n = f.n; p.d = f.d; p.s = f.s; p.B = f.B; p.out = f.out; p.c = f.c;
-  p.status = f.status; p.map = f.map; p.when = f.when;
+  p.status = f.status; p.map = f.map; p.when = f.when; p.minus_zero = f.minus_zero;
   p.Kpad = 1;
   while (p.Kpad < p.K) p.Kpad <<= 1;
   const uint32_t G = 32u / p.Kpad;

@@ -60,6 +60,7 @@ struct TeamParams {
   uint64_t B;
   float* out;             // acc (overwritten) or x (updated in place)
   float c;                // eta / K
+  float minus_zero;       // add_product2
   uint32_t* status;
   uint32_t T;             // lanes per string, a power of two
   uint32_t buckets;       // per CTA and pass
@@ -277,7 +278,7 @@ __device__ __forceinline__ uint32_t emit(const Tables<false>& tab, const uint32_
 
 // Reads a part in kMarks pieces and keeps where each piece ended, so that a lane that has to read its part
 // again from another bit can stop at the first mark where it falls into step with its first reading.
-template <bool DENSE> constexpr uint32_t kMarksOf = DENSE ? 2u : 4u;
+template <bool DENSE> constexpr uint32_t kMarksOf = DENSE ? 1u : 4u;
 constexpr uint32_t kLeastPiece = 96;      // bits
 template <bool DENSE>
 struct Marks {
@@ -487,13 +488,10 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
         const uint8_t* codes = tsm + (size_t)gg * kc * p.row_bytes + place<DENSE, WIDTH>(cc);
         const float* sc = scales + gg * kc;
         float4* carry = reinterpret_cast<float4*>(sums + gg * p.d + cc);
-        float acc[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+        float2p sum[4] = {0ull, 0ull, 0ull, 0ull};
         if (k0) {                                         // the peers of the passes before, added by this thread
           const float4 u = carry[0], v = carry[1];
-          acc[0] = u.x; acc[1] = u.y; acc[2] = u.z; acc[3] = u.w;
-          acc[4] = v.x; acc[5] = v.y; acc[6] = v.z; acc[7] = v.w;
+          sum[0] = pair2(u.x, u.y); sum[1] = pair2(u.z, u.w); sum[2] = pair2(v.x, v.y); sum[3] = pair2(v.z, v.w);
         }
         if (WIDTH == kWide) {
           for (uint32_t k = 0; k < kc; ++k) {
@@ -501,10 +499,7 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
             const uint32_t w[4] = {q.x, q.y, q.z, q.w};
             const float Ak = sc[k];
 #pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              acc[2 * h] = __fadd_rn(acc[2 * h], __fmul_rn(Ak, xi[w[h] & 0xFFFFu]));
-              acc[2 * h + 1] = __fadd_rn(acc[2 * h + 1], __fmul_rn(Ak, xi[w[h] >> 16]));
-            }
+            for (int h = 0; h < 4; ++h) sum[h] = add_product2(sum[h], Ak, xi[w[h] & 0xFFFFu], xi[w[h] >> 16], p.minus_zero);
           }
         } else {
           const float lut = WIDTH == kNibble ? xi[lane] : 0.f;
@@ -513,12 +508,17 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
             const uint2 q = *reinterpret_cast<const uint2*>(codes + k * p.row_bytes);
             const float Ak = sc[k];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const uint32_t code = (e < 4 ? q.x : q.y) >> (8 * (e & 3));
-              acc[e] = __fadd_rn(acc[e], __fmul_rn(Ak, WIDTH == kNibble ? shfl_f(lut, code) : xi[code & 0xFFu]));
+            for (int e = 0; e < 4; ++e) {
+              const uint32_t two = (e < 2 ? q.x : q.y) >> (16 * (e & 1));
+              const float v0 = WIDTH == kNibble ? shfl_f(lut, two) : xi[two & 0xFFu];
+              const float v1 = WIDTH == kNibble ? shfl_f(lut, two >> 8) : xi[(two >> 8) & 0xFFu];
+              sum[e] = add_product2(sum[e], Ak, v0, v1, p.minus_zero);
             }
           }
         }
+        float acc[8];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { const float2 u = unpair2(sum[e]); acc[2 * e] = u.x; acc[2 * e + 1] = u.y; }
         if (!live) continue;
         if (k0 + kc < p.K) {
           carry[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
@@ -549,7 +549,7 @@ int launch_width(TeamParams& p, bool fused, size_t smem, cudaStream_t stream) {
 int launch_elias_teams(const FieldParams& f, bool dense, bool fused, cudaStream_t stream) {
   TeamParams p;
   p.peers = f.peers; p.K = f.K; p.n = f.n; p.d = f.d; p.s = f.s; p.B = f.B; p.out = f.out; p.c = f.c;
-  p.status = f.status; p.map = f.map; p.when = f.when;
+  p.status = f.status; p.map = f.map; p.when = f.when; p.minus_zero = f.minus_zero;
   const int width = f.s <= 15u ? kNibble : f.s <= 127u ? kByte : kWide;
   p.row_bytes = ((p.d * (width == kWide ? 2u : 1u) + 127u) & ~127u) + kRowPad;
   auto bytes = [&](uint32_t buckets, uint32_t peers) {

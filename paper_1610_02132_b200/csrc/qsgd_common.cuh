@@ -123,7 +123,8 @@ int launch_raw_decode(const float* const* raw_regions, uint32_t K, const RawSegm
 enum KernelId {
   kKernQuantize = 0, kKernQuantizeTail, kKernDecodeFixed, kKernSgdStep, kKernEliasLength,
   kKernEliasScatter, kKernDecodeElias, kKernDecodeEliasSparse, kKernRawGather, kKernRawDecode,
-  kKernDecodeEliasTeams, kKernDecodeEliasFields, kKernDecodeEliasBytes, kKernCount      // (kKernDecodeElias: streams of strings by table)
+  kKernDecodeEliasTeams, kKernDecodeEliasFields, kKernDecodeEliasBytes, kKernDecodeEliasDense,
+  kKernCount      // (kKernDecodeElias: streams of strings by table)
 };
 
 // SM count of the current device, and the most shared memory a CTA can have (looked up once per device).
