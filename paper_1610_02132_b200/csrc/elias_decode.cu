@@ -1,14 +1,12 @@
 // Decode-and-aggregate, Elias path, optionally fused with the SGD step (Section 3.1, end of
 // "Efficient Coding of Gradients": scale first, then the codes of the nonzeros in index order;
 // Appendix A.2 decoder; Algorithm 1 for the sum and the step): the choice among the decoders. The one that
-// reads streams of consecutive strings by table is in elias_decode_ring.cu (s <= 15), the ones with a lane per
+// reads streams of consecutive strings by table is in elias_decode_ring.cu (s <= 15) and, for the dense code,
+// elias_decode_dense.cu (s <= 127), the ones with a lane per
 // string in elias_decode_bytes.cu (s <= 15) and elias_decode_fields.cu (larger s), the one with a team of lanes per string
 // in elias_decode_teams.cu, the nonzero-driven decoder of the sparse regime in elias_decode_sparse.cu; what they
 // share is in elias_decode.cuh.
 #include "elias_decode.cuh"
-#ifndef DL
-#define DL 8192
-#endif
 
 namespace qsgd {
 
@@ -31,9 +29,21 @@ bool sparse_though_small(uint32_t mean, uint32_t K, uint64_t work) { return mean
 // 32 / 38, 23 K of d = 4096 93 / 125; 39 K of d = 512 36 / 37, of d = 128 39 / 30, 62 K of d = 512 48 / 40. s = 255:
 // 13 K of d = 96 31 / 34, 16 K of d = 256 50 / 83; 26 K of d = 96 37 / 34, 31 K of d = 64 29 / 24, of d = 256 89 / 87,
 // 524 K of d = 256 1042 / 664; from d = 512 on always teams: 16 K 82 / 149, 262 K 912 / 937, d = 1024 915 / 1632. Code'_s
-// has a symbol per coordinate: always teams.
+// has a symbol per coordinate: teams, or streams (use_streams).
 bool use_teams(uint64_t B, uint32_t K, uint32_t d, uint32_t s) {
   return (s > 15u && d >= 512u) || B * K <= (24u << 10);
+}
+
+// Code'_s: a lane per stream (a code is a byte: s <= 127), or teams, which read a string several times but with all lanes of the
+// GPU? 49 problems measured both ways; strings, and us by streams / by teams. K >= 8: 16 K 169 / 157 (d = 4096, s = 64), 40 / 38
+// (d = 512, s = 22), 28 / 24 (d = 64, s = 15); 24 K 179 / 218, 40 / 48, 26 / 26; 64 K 243 / 544, 48 / 93, 26 / 36. Fewer peers,
+// whose sums the teams spread better: K = 4 24 K 212 / 173, 32 K 216 / 222, 64 K 265 / 427; K = 2 24 K 38 / 34, 32 K 38 / 42;
+// K = 1 32 K 151 / 126, 64 K 177 / 218. Levels so many that most symbols are too long for the table (s = 100, d = 128,
+// max-norm): 32 K 54 / 40, 64 K 65 / 63.
+bool use_streams(uint64_t B, uint32_t K, uint32_t d, uint32_t s) {
+  if (s > 127u || K > 32u) return false;
+  const uint32_t line = s > 15u && s * s > 4u * d ? 64u : K == 1u ? 48u : K < 8u ? 30u : 22u;
+  return B * K > (uint64_t)line << 10;
 }
 
 // Mean bits of a string behind its scale, where the host can tell: in a message the offset table follows the padded
@@ -89,7 +99,7 @@ int launch_decode_elias(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
   f.peers = peers; f.K = K; f.n = n; f.d = d; f.s = s; f.B = B;
   f.out = acc_or_x; f.c = eta / (float)K; f.minus_zero = -0.f; f.status = status_dev; f.map = map;
   f.when = Regime{0u, kNoBound};
-  if (dense && s <= 127u && K <= 32u && B * K > DL) return launch_elias_dense(f, fused, stream);
+  if (dense && use_streams(B, K, d, s)) return launch_elias_dense(f, fused, stream);
   if (dense || K > 32u) return launch_elias_teams(f, dense, fused, stream);
 
   const bool teams = use_teams(B, K, d, s), small = teams && work <= kSmallWork;
