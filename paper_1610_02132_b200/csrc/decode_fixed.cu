@@ -14,7 +14,7 @@
 // What bounds it (n = 60 M, d = 512, K = 16): at s = 15 the L1 data path (one shuffle per coordinate and peer: 256 of 400
 // wavefronts per chunk) and the latency of the loads, 221 us; at s = 255 HBM, 88 % of the copy rate. Sums in pairs, one scale
 // read by all lanes instead of shuffled, places in 32 bits, `out` accessed in whole lines and the table with signs took 1489 to
-// 1272 warp instructions per chunk (s = 15) and 1900 to 1488 (s = 255): 251 -> 221 and 340 -> 262 us. Four messages are read
+// 1272 warp instructions per chunk (s = 15) and 1900 to 1488 (s = 255): 251 -> 221 and 340 -> 263 us. Four messages are read
 // at a time (2: 252, 3: 236, 8 with 80 registers: 234 us at s = 15). More bytes in flight did not help: the next group read
 // while this one is added 252 to 270 (spills, or fewer warps), fields copied to shared memory a group ahead 235 (their
 // wavefronts), a ring of bulk copies per CTA 310 (warps that wait for the slowest), the next chunk prefetched to L2 240.
