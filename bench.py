@@ -310,7 +310,7 @@ class HotPath:
 
 
 ELIAS_DECODERS = ("decode_elias", "decode_elias_sparse", "decode_elias_teams", "decode_elias_fields",
-                  "decode_elias_bytes")
+                  "decode_elias_bytes", "decode_elias_dense")
 
 
 def kernel_algorithmic_bytes(hp, code_name):

@@ -28,7 +28,7 @@ namespace qsgd {
 
 namespace {
 
-constexpr uint32_t kThreads = 256;
+constexpr uint32_t kThreads = 256, kMostThreads = 1024;       // (the latter where strings are shared by several warps)
 template <bool DENSE> constexpr uint32_t kWarmUp = DENSE ? 96 : 64;      // bits: 75-98 % of the starts are then right
 constexpr uint32_t kLeastPart = 64;               // bits of a string that are worth a lane
 constexpr uint32_t kDenseBits = 10;
@@ -63,6 +63,7 @@ struct TeamParams {
   float minus_zero;       // add_product2
   uint32_t* status;
   uint32_t T;             // lanes per string, a power of two
+  uint32_t split;         // SPLIT: warps per string, of 32 lanes each
   uint32_t buckets;       // per CTA and pass
   uint32_t row_bytes;
   Regime when;
@@ -310,18 +311,20 @@ __device__ __forceinline__ void read_part(const Tables<DENSE>& tab, const uint32
   }
 }
 
-template <bool DENSE, int WIDTH, bool FUSED>
-__global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __grid_constant__ TeamParams p) {
+// SPLIT: a string is shared by several warps of a CTA that has a warp for every part of its strings.
+template <bool DENSE, int WIDTH, bool FUSED, bool SPLIT>
+__global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads) decode_elias_teams_kernel(const __grid_constant__ TeamParams p) {
   using Code = typename CodeOf<WIDTH>::type;
   constexpr uint32_t kLevels = 1u << CodeOf<WIDTH>::kSignShift;
   extern __shared__ __align__(16) uint8_t tsm[];
   __shared__ Tables<DENSE> tab;
   __shared__ float xi[2 * kLevels];                     // +-(level / s) by code
-  const uint32_t tid = threadIdx.x, lane = tid & 31;
+  __shared__ uint32_t warp_end[SPLIT ? kMostThreads / 32 : 1], warp_sum[SPLIT ? kMostThreads / 32 : 1];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, threads = SPLIT ? blockDim.x : kThreads;
   const float sf = (float)p.s;
-  for (uint32_t i = tid; i < kCodeEntries; i += kThreads) tab.code[i] = code_entry(i);
+  for (uint32_t i = tid; i < kCodeEntries; i += threads) tab.code[i] = code_entry(i);
   if (DENSE) {
-    for (uint32_t i = tid; i < (1u << kDenseBits); i += kThreads) {
+    for (uint32_t i = tid; i < (1u << kDenseBits); i += threads) {
       const uint32_t w = i << (32 - kDenseBits);
       uint32_t used = 0, held = 0, ends = 0, codes = 0, small = 0, small_bits = 0;
       while (held < 3u) {
@@ -342,9 +345,9 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
       tab.count[i] = held ? used | ends | (held << 20) : min(code_body(code_entry((w << 1) >> 25)) + 2u, 22u) | (1u << 20);
     }
   } else if (WIDTH == kNibble) {
-    for (uint32_t i = tid; i < kTailEntries; i += kThreads) tab.symbol[i] = tail_entry(i, p.s);
+    for (uint32_t i = tid; i < kTailEntries; i += threads) tab.symbol[i] = tail_entry(i, p.s);
   }
-  for (uint32_t i = tid; i < 2u * kLevels; i += kThreads) {
+  for (uint32_t i = tid; i < 2u * kLevels; i += threads) {
     const float q = __fdiv_rn((float)(i & (kLevels - 1u)), sf);
     xi[i] = i & kLevels ? -q : q;
   }
@@ -353,7 +356,10 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
   const uint32_t most = p.buckets * p.Kc;
   float* sums = reinterpret_cast<float*>(tsm + (size_t)most * p.row_bytes);
   float* scales = sums + (p.Kc < p.K ? p.buckets * p.d : 0u);
-  const uint32_t T = p.T, t = lane & (T - 1u), team = tid / T, teams = kThreads / T;
+  const uint32_t T = SPLIT ? 32u : p.T, t = lane & (T - 1u);
+  const uint32_t warps = SPLIT ? p.split : 1u, warp = tid >> 5, part = SPLIT ? warp % warps : 0u;       // of a string
+  const uint32_t team = SPLIT ? warp / warps : tid / T, teams = SPLIT ? (threads >> 5) / warps : kThreads / T;
+  const uint32_t tt = part * 32u + t, TT = T * warps;                     // this lane among the string's lanes
   const uint64_t groups = (p.B + p.buckets - 1) / p.buckets;
   chain_wait();                                         // the messages come from the kernels ahead
   if (!DENSE && p.when.lo && mean_below(p.when.lo, p.peers, p.K, p.B)) return;
@@ -363,7 +369,7 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
     const uint32_t nb = (uint32_t)min((uint64_t)p.buckets, p.B - b0);
     for (uint32_t k0 = 0; k0 < p.K; k0 += p.Kc) {
       const uint32_t kc = min(p.Kc, p.K - k0), rows = p.buckets * kc;
-      for (uint32_t i = tid; i < rows * (p.row_bytes >> 4); i += kThreads)
+      for (uint32_t i = tid; i < rows * (p.row_bytes >> 4); i += threads)
         reinterpret_cast<uint4*>(tsm)[i] = make_uint4(0u, 0u, 0u, 0u);
       __syncthreads();
 
@@ -388,16 +394,16 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
         // 4 and 4 bits long, and a reader that starts an odd number of bits from the front of a string of such levels is
         // out of step to the end of its part: where the symbols are short, parts have an even length (n = 33.5 M, d = 4096,
         // K = 8, 2-norm: 2361 -> 423 us at s = 15, 1851 -> 371 at s = 1).
-        uint32_t per = max((ref.total + T - 1u) / T, kLeastPart);
+        uint32_t per = max((ref.total + TT - 1u) / TT, kLeastPart);
         if (DENSE && ref.total < 3u * db) per = (per + 1u) & ~1u;
-        const uint32_t lo = min(first + t * per, end), hi = t == T - 1u ? end : min(lo + per, end);
+        const uint32_t lo = min(first + tt * per, end), hi = tt == TT - 1u ? end : min(lo + per, end);
         uint32_t start = lo;
         Marks<DENSE> m;
         constexpr uint32_t kMarks = kMarksOf<DENSE>;
 #pragma unroll
         for (uint32_t q = 0; q < kMarks; ++q) { m.pos[q] = lo; m.sum[q] = 0u; }
         if (reads) {
-          if (t == 0u) {
+          if (tt == 0u) {
             Window in;
             in.open(words, first - 32u);
             scales[j] = __uint_as_float(in.peek());
@@ -406,56 +412,70 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
             start = walk<DENSE, WIDTH>(tab, words, lo - min(kWarmUp<DENSE>, lo - first), lo, end, &skipped);
           }
           read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, false, m);
-        } else if (j < rows && t == 0u) {
+        } else if (j < rows && tt == 0u) {
           scales[j] = 0.f;
         }
-        if constexpr (!DENSE) {
-          for (;;) {
-            const uint32_t before = __shfl_up_sync(0xffffffffu, m.pos[kMarks - 1u], 1, (int)T);
-            const bool again = t != 0u && before != start;
-            if (!__any_sync(0xffffffffu, again)) break;
-            if (again) {
-              start = before;
-              read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, true, m);
-            }
-          }
-        } else {
-          // Short symbols again: one of an odd length, where they are rare, puts all lanes behind it out of step, each of
-          // which would find out a round after the one in front of it. So where a lane that had to start elsewhere ended
-          // elsewhere too, all lanes of the string read their parts from a bit further on, and keep both readings (K = 4,
-          // n = 67 M, a mixture, s = 15: 1258 -> 583 us at d = 4096, 922 -> 651 at d = 2048).
-          uint32_t other = start;                         // where the other reading started
-          Marks<DENSE> o = m;
-          uint32_t rounds = reads && ref.total < 3u * db ? 1u : 0u;         // until then; 0: never
-          for (;;) {
-            uint32_t before;
-            bool again;
+        uint32_t other = start;                           // dense code: where the other reading started (below)
+        Marks<DENSE> o = m;
+        uint32_t rounds = reads && ref.total < 3u * db ? 1u : 0u;           // until all lanes read again; 0: never
+        for (;;) {
+          if constexpr (!DENSE) {
             for (;;) {
-              before = __shfl_up_sync(0xffffffffu, m.pos[kMarks - 1u], 1, (int)T);
-              again = t != 0u && before != start;
-              const bool had = again && before == other;
-              if (!__any_sync(0xffffffffu, had)) break;
-              if (had) {
-                const Marks<DENSE> q = m;
-                m = o; o = q;
-                other = start; start = before;
+              const uint32_t before = __shfl_up_sync(0xffffffffu, m.pos[kMarks - 1u], 1, (int)T);
+              const bool again = t != 0u && before != start;
+              if (!__any_sync(0xffffffffu, again)) break;
+              if (again) {
+                start = before;
+                read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, true, m);
               }
             }
-            const uint32_t wrong = __ballot_sync(0xffffffffu, again);
-            if (wrong == 0u) break;
-            const bool astray = rounds != 0u && (wrong & (0xFFFFFFFFu >> (32u - T) << (lane & ~(T - 1u)))) != 0u;
-            const bool now = astray && rounds == 2u;
-            if (astray) rounds = now ? 0u : 2u;
-            if (now && t != 0u && start < hi && other == start) {
-              other = start + 1u;
-              read_part<DENSE, WIDTH>(tab, words, other, lo, hi, end, true, o);
+          } else {
+            // Short symbols again: one of an odd length, where they are rare, puts all lanes behind it out of step, each of
+            // which would find out a round after the one in front of it. So where a lane that had to start elsewhere ended
+            // elsewhere too, all lanes of the string read their parts from a bit further on, and keep both readings (K = 4,
+            // n = 67 M, a mixture, s = 15: 1258 -> 583 us at d = 4096, 922 -> 651 at d = 2048).
+            for (;;) {
+              uint32_t before;
+              bool again;
+              for (;;) {
+                before = __shfl_up_sync(0xffffffffu, m.pos[kMarks - 1u], 1, (int)T);
+                again = t != 0u && before != start;
+                const bool had = again && before == other;
+                if (!__any_sync(0xffffffffu, had)) break;
+                if (had) {
+                  const Marks<DENSE> q = m;
+                  m = o; o = q;
+                  other = start; start = before;
+                }
+              }
+              const uint32_t wrong = __ballot_sync(0xffffffffu, again);
+              if (wrong == 0u) break;
+              const bool astray = rounds != 0u && (wrong & (0xFFFFFFFFu >> (32u - T) << (lane & ~(T - 1u)))) != 0u;
+              const bool now = astray && rounds == 2u;
+              if (astray) rounds = now ? 0u : 2u;
+              if (now && t != 0u && start < hi && other == start) {
+                other = start + 1u;
+                read_part<DENSE, WIDTH>(tab, words, other, lo, hi, end, true, o);
+              }
+              if (__any_sync(0xffffffffu, now)) continue;
+              if (again) {
+                o = m; other = start;
+                start = before;
+                read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, true, m);
+              }
             }
-            if (__any_sync(0xffffffffu, now)) continue;
-            if (again) {
-              o = m; other = start;
-              start = before;
-              read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, true, m);
-            }
+          }
+          if constexpr (!SPLIT) break;
+          // the warps of a string: the first lane of each begins where the warp in front of it ended
+          if (lane == 31u) warp_end[SPLIT ? warp : 0u] = m.pos[kMarks - 1u];
+          __syncthreads();
+          const uint32_t before = SPLIT && part != 0u ? warp_end[SPLIT ? warp - 1u : 0u] : start;
+          const bool wrong = reads && t == 0u && before != start;
+          if (!__syncthreads_or(wrong ? 1 : 0)) break;
+          if (wrong) {
+            o = m; other = start;
+            start = before;
+            read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, true, m);
           }
         }
         const uint32_t sum = m.sum[kMarks - 1u], stop = m.pos[kMarks - 1u];
@@ -464,13 +484,18 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
           const uint32_t q = __shfl_up_sync(0xffffffffu, upto, o, (int)T);
           if (t >= o) upto += q;
         }
+        if constexpr (SPLIT) {
+          if (lane == 31u) warp_sum[warp] = upto;
+          __syncthreads();
+          for (uint32_t w = warp - part; w < warp; ++w) upto += warp_sum[w];
+        }
         uint32_t err = ref.err;
         if (reads) {
           uint8_t* row = tsm + (size_t)j * p.row_bytes;
           if constexpr (DENSE) err |= emit_dense<WIDTH>(tab, words, start, hi, end, upto - sum, db, p.s, ref.total > kFewBits * db, row);
           else err |= emit<WIDTH>(tab, words, start, hi, end, upto - sum - 1u, db, p.s, row);
           // a string must end exactly where the table says and, in the dense code, hold every coordinate
-          if (t == T - 1u && (stop != end || (DENSE && upto != db))) err |= QSGD_DEV_OVERRUN;
+          if (tt == TT - 1u && (stop != end || (DENSE && upto != db))) err |= QSGD_DEV_OVERRUN;
         }
         if (err) atomicOr(p.status, err);
       }
@@ -478,7 +503,7 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
 
       // ---- ascending-k sum; a thread takes 8 coordinates per pass ------------------------------------
       const uint32_t slots_per_bucket = p.d >> 3, slots = nb * slots_per_bucket;
-      for (uint32_t s0 = 0; s0 < slots; s0 += kThreads) {
+      for (uint32_t s0 = 0; s0 < slots; s0 += threads) {
         const uint32_t slot = s0 + tid;
         const uint32_t g = slot / slots_per_bucket, c = (slot - g * slots_per_bucket) << 3;
         const uint64_t b = b0 + g;
@@ -534,14 +559,18 @@ __global__ void __launch_bounds__(kThreads) decode_elias_teams_kernel(const __gr
 
 template <bool DENSE, int WIDTH>
 int launch_width(TeamParams& p, bool fused, size_t smem, cudaStream_t stream) {
-  static KernelSite site[2];
-  auto kern = fused ? decode_elias_teams_kernel<DENSE, WIDTH, true> : decode_elias_teams_kernel<DENSE, WIDTH, false>;
+  static KernelSite site[4];
+  void (*kern)(TeamParams);
+  const bool split = p.split > 1u;
+  if (split) kern = fused ? decode_elias_teams_kernel<DENSE, WIDTH, true, true> : decode_elias_teams_kernel<DENSE, WIDTH, false, true>;
+  else kern = fused ? decode_elias_teams_kernel<DENSE, WIDTH, true, false> : decode_elias_teams_kernel<DENSE, WIDTH, false, false>;
+  const uint32_t threads = split ? p.buckets * p.Kc * p.split * 32u : kThreads;
   int sms = 0, occ = 0;
-  const int st = site[fused ? 1 : 0].lookup_dynamic(kern, kThreads, smem, &sms, &occ);
+  const int st = site[(split ? 2 : 0) + (fused ? 1 : 0)].lookup_dynamic(kern, (int)threads, smem, &sms, &occ);
   if (st) return st;
   const uint64_t groups = (p.B + p.buckets - 1) / p.buckets, cap = (uint64_t)sms * occ;
   ScopedKernel sk(kKernDecodeEliasTeams, stream);
-  return (int)launch_chained(kern, (uint32_t)(groups < cap ? groups : cap), kThreads, smem, stream, p);
+  return (int)launch_chained(kern, (uint32_t)(groups < cap ? groups : cap), threads, smem, stream, p);
 }
 
 }  // namespace
@@ -578,6 +607,15 @@ int launch_elias_teams(const FieldParams& f, bool dense, bool fused, cudaStream_
   // 45.0 / 10.2.
   if (p.d < 1024u || p.K <= 16u || p.s <= 3u)
     while (p.T > 4u && p.buckets * p.Kc * p.T > kThreads) p.T >>= 1;
+  // So few strings that every CTA has an SM to itself: two warps to a string, where each lane then still has 96 bits or so, or
+  // four with twice as many (less is lost to the bits ahead of a part). One against two, and four (us): n = 40 K, d = 4096,
+  // s = 64, K = 8, dense code 30 / 26, 32; 131 K, d = 2048, s = 15, K = 4 32 / 28, 28; 64 K, d = 4096, s = 255, K = 2 73 / 48, 36.
+  p.split = 1;
+  if (p.T == 32u && p.Kc == p.K && (p.B + p.buckets - 1) / p.buckets <= (uint64_t)sms) {
+    const uint32_t likely = p.d * (width == kNibble ? 3u : width == kByte ? 4u : 9u), strings_of_cta = p.buckets * p.Kc;
+    if (strings_of_cta * 64u <= kMostThreads && likely >= 64u * 96u) p.split = 2;
+    if (strings_of_cta * 128u <= kMostThreads && likely >= 128u * 192u) p.split = 4;
+  }
   const size_t smem = align16(bytes(p.buckets, p.Kc));
 #define QSGD_RUN(D, W) launch_width<D, W>(p, fused, smem, stream)
   if (dense) return width == kNibble ? QSGD_RUN(true, kNibble) : width == kByte ? QSGD_RUN(true, kByte) : QSGD_RUN(true, kWide);
