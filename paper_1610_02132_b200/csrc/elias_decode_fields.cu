@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
   const uint32_t warp_words = p.G * p.bucket_words;
   uint32_t* mine = fsm + (size_t)warp * warp_words;
   const uint32_t level_words = (p.d * LB) >> 5;
-  const uint32_t pg = lane / p.Kpad, pk = lane % p.Kpad;      // parse role: bucket in group, peer
+  const uint32_t pg = lane / p.K, pk = lane % p.K;            // parse role: bucket in group, peer
   const uint32_t slots_per_bucket = p.d >> 4;                 // 16-coordinate lane slots
   const uint32_t total_slots = p.G * slots_per_bucket;
   const uint64_t groups = (p.B + p.G - 1) / p.G;
@@ -179,11 +179,9 @@ int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream) {
   const uint32_t level_words = p.d >> 2, sign_words = p.d >> 5;
   p.row_words = (level_words + sign_words + 3u) & ~3u;
   p.bucket_words = (p.K * p.row_words + p.K + 3u) & ~3u;
-  uint32_t kpad = 1;
-  while (kpad < p.K) kpad <<= 1;
-  p.Kpad = kpad;
-  uint32_t G = 32 / kpad;
-  while (G > 1 && (size_t)G * p.bucket_words * 4 > (16u << 10)) G >>= 1;
+  // As many buckets to a warp as it has lanes for (K = 5, d = 96: 6, where a power of two would leave 12 lanes idle).
+  uint32_t G = 32 / p.K;
+  while (G > 1 && (size_t)G * p.bucket_words * 4 > (16u << 10)) --G;
   p.G = G;
   const size_t per_warp = (size_t)G * p.bucket_words * 4;
   // Warps per CTA: the count that leaves the most warps resident on an SM. The code table is
@@ -196,12 +194,22 @@ int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream) {
     const int resident = (int)(per_sm / ((size_t)w * per_warp + per_cta)) * w;
     if (resident > best) { best = resident; warps = w; }
   }
+  // Where all warps are resident at once, the count that spreads them evenly over the SMs.
+  const uint64_t groups = (p.B + G - 1) / G;
+  int sms = 0, occ = 0;
+  int st = device_sms(&sms);
+  if (st) return st;
+  if (groups <= (uint64_t)sms * best) {
+    uint64_t least = ~0ull;
+    for (int w = warps; w >= 1; --w) {
+      const uint64_t per = ((groups + w - 1) / w + sms - 1) / sms * w;
+      if (per < least && per * per_warp + per / w * per_cta <= per_sm) { least = per; warps = w; }
+    }
+  }
   auto kern = fused ? decode_elias_fields_kernel<true> : decode_elias_fields_kernel<false>;
   const size_t smem = (size_t)warps * per_warp;
-  int sms = 0, occ = 0;
-  const int st = site[fused ? 1 : 0].lookup_dynamic(kern, warps * 32, smem, &sms, &occ);
+  st = site[fused ? 1 : 0].lookup_dynamic(kern, warps * 32, smem, &sms, &occ);
   if (st) return st;
-  const uint64_t groups = (p.B + G - 1) / G;
   const uint64_t want = (groups + warps - 1) / warps;
   const uint64_t cap = (uint64_t)sms * occ;
   ScopedKernel sk(kKernDecodeEliasFields, stream);
