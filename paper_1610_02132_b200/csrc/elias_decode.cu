@@ -2,7 +2,7 @@
 // "Efficient Coding of Gradients": scale first, then the codes of the nonzeros in index order;
 // Appendix A.2 decoder; Algorithm 1 for the sum and the step): the choice among the decoders. The one that
 // reads streams of consecutive strings by table is in elias_decode_ring.cu (s <= 15) and, for the dense code,
-// elias_decode_dense.cu (s <= 127), the ones with a lane per
+// elias_decode_dense.cu, the ones with a lane per
 // string in elias_decode_bytes.cu (s <= 15) and elias_decode_fields.cu (larger s), the one with a team of lanes per string
 // in elias_decode_teams.cu, the nonzero-driven decoder of the sparse regime in elias_decode_sparse.cu; what they
 // share is in elias_decode.cuh.
@@ -34,15 +34,16 @@ bool use_teams(uint64_t B, uint32_t K, uint32_t d, uint32_t s) {
   return (s > 15u && d >= 512u) || B * K <= (24u << 10);
 }
 
-// Code'_s: a lane per stream (a code is a byte: s <= 127), or teams, which read a string several times but with all lanes of the
-// GPU? 49 problems measured both ways; strings, and us by streams / by teams. K >= 8: 16 K 169 / 157 (d = 4096, s = 64), 40 / 38
-// (d = 512, s = 22), 28 / 24 (d = 64, s = 15); 24 K 179 / 218, 40 / 48, 26 / 26; 64 K 243 / 544, 48 / 93, 26 / 36. Fewer peers,
-// whose sums the teams spread better: K = 4 24 K 212 / 173, 32 K 216 / 222, 64 K 265 / 427; K = 2 24 K 38 / 34, 32 K 38 / 42;
-// K = 1 32 K 151 / 126, 64 K 177 / 218. Levels so many that most symbols are too long for the table (s = 100, d = 128,
-// max-norm): 32 K 54 / 40, 64 K 65 / 63.
+// Code'_s: a lane per stream, or teams, which read a string several times but with all lanes of the GPU? 60 problems measured
+// both ways; strings, and us by streams / by teams. K >= 8: 16 K 169 / 157 (d = 4096, s = 64), 40 / 38 (d = 512, s = 22), 28 / 24
+// (d = 64, s = 15); 24 K 179 / 218, 40 / 48, 26 / 26; 64 K 243 / 544, 48 / 93, 26 / 36. Fewer peers, whose sums the teams spread
+// better: K = 4 24 K 212 / 173, 32 K 216 / 222, 64 K 265 / 427; K = 2 24 K 38 / 34, 32 K 38 / 42; K = 1 32 K 151 / 126, 64 K
+// 177 / 218. Symbols of levels above 15, which the streams' table seldom holds, only where the bucket's largest level is likely
+// far above the others: max-norm, n = 17 M, K = 8: d = 512, s = 64 552 / 751, d = 4096 705 / 700, but d = 128 633 / 570, d = 64,
+// s = 48 627 / 574; d = 128, s = 100 718 / 599.
 bool use_streams(uint64_t B, uint32_t K, uint32_t d, uint32_t s) {
-  if (s > 127u || K > 32u) return false;
-  const uint32_t line = s > 15u && s * s > 4u * d ? 64u : K == 1u ? 48u : K < 8u ? 30u : 22u;
+  if (K > 32u || s > (d >= 512u ? 64u : 32u)) return false;
+  const uint32_t line = K == 1u ? 48u : K < 8u ? 30u : 22u;
   return B * K > (uint64_t)line << 10;
 }
 

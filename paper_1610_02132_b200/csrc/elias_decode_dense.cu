@@ -1,4 +1,4 @@
-// Decode-and-aggregate, dense code (Code'_s, s <= 127, at most 32 peers), where strings are many: a lane per (run of
+// Decode-and-aggregate, dense code (Code'_s, s <= 127, at most 32 peers), where strings are many and levels are not: a lane per (run of
 // consecutive buckets, peer). (Appendix A.3 for the code, Appendix A.2 for its integers; Algorithm 1 for the sum and the step.)
 //
 // A symbol for every coordinate: lanes that read at the same rate stay at the same positions, so a lane reads its stream from

@@ -17,8 +17,8 @@ L2, MAX, DENSE = O.NORM_L2, O.NORM_MAX, O.CODE_ELIAS_DENSE
 
 # (buckets, coordinates missing in the last, d, s, norm, K)
 SHAPES = [
-    (9000, 27, 32, 15, MAX, 5), (4200, 1, 96, 127, MAX, 16), (8300, 63, 64, 1, L2, 4), (2100, 255, 256, 64, MAX, 32), (2800, 1, 512, 15, L2, 12),
-    (4200, 0, 160, 3, L2, 8), (2000, 4095, 4096, 64, L2, 17), (50000, 0, 128, 15, MAX, 1), (2100, 2047, 2080, 100, L2, 32), (4200, 5, 480, 7, MAX, 8),
+    (9000, 27, 32, 15, MAX, 5), (4200, 1, 96, 32, MAX, 16), (8300, 63, 64, 1, L2, 4), (2100, 255, 512, 64, MAX, 32), (2800, 1, 512, 15, L2, 12),
+    (4200, 0, 160, 3, L2, 8), (2000, 4095, 4096, 64, L2, 17), (50000, 0, 128, 15, MAX, 1), (1000, 2047, 2080, 64, L2, 32), (4200, 5, 480, 7, MAX, 8),
 ]
 
 
