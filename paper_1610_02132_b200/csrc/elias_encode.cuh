@@ -186,17 +186,18 @@ __device__ __forceinline__ void fill_symbol_lengths(SymbolLengths<LB>& t) {
 template <int LB>
 __device__ __forceinline__ uint32_t symbol_bits(const SymbolLengths<LB>& t, uint32_t w, uint32_t count) {
   constexpr uint32_t kFields = 32u / LB, kMask = (1u << LB) - 1u;
-  uint32_t bits = 0;
   if constexpr (LB == 1) {                                // two bits, or four
     const uint32_t there = count >= 32u ? 0xFFFFFFFFu : (1u << count) - 1u;
     return 2u * min(count, 32u) + 2u * (uint32_t)__popc(w & there);
-  }
+  } else {
+    uint32_t bits = 0;
 #pragma unroll
-  for (uint32_t f = 0; f < kFields; ++f) {
-    const uint32_t l = t.of[(w >> (f * LB)) & kMask];
-    bits += f < count ? l : 0u;
+    for (uint32_t f = 0; f < kFields; ++f) {
+      const uint32_t l = t.of[(w >> (f * LB)) & kMask];
+      bits += f < count ? l : 0u;
+    }
+    return bits;
   }
-  return bits;
 }
 
 // Sum of |Elias(gap)| over the set bits of a 64-coordinate block except the lowest, gap = distance to
