@@ -228,7 +228,6 @@ __device__ __forceinline__ void quantize_generic_tile(const QuantizeParams& p, u
   if (block == 0 && tid == 0 && p.info) {
     p.info[0] = 8 * p.total_bytes; p.info[1] = 0; p.info[2] = p.total_bytes; p.info[3] = 0;
   }
-  if (block == 0) clear_words(p.clear);
   const uint64_t left = p.n - t0;
   const uint32_t valid = left < p.tile_coords ? (uint32_t)left : p.tile_coords;
   if (valid == 0) {                            // nothing left to encode: only the padding

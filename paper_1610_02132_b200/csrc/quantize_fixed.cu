@@ -161,6 +161,15 @@ __device__ __forceinline__ void issue_tile(const FastParams& p, float* tile, uin
 // runs the ragged last tile and the region padding through the generic tile code (its operands alias
 // the tile ring). MAPPED: buckets are fetched through a bucket map (per-tensor policy); a separate
 // instantiation, so that the ordinary kernel carries none of that code.
+// What the first CTA writes beside its share of the message, while its first copies are on their way: in front of them it
+// cost every encode below 2 M coordinates 1 %.
+__device__ __forceinline__ void write_beside(const FastParams& p) {
+  if (threadIdx.x == 0 && p.info) {
+    p.info[0] = 8 * p.total_bytes; p.info[1] = 0; p.info[2] = p.total_bytes; p.info[3] = 0;
+  }
+  if (p.clear.count) clear_words(p.clear);
+}
+
 template <int LB, int NORM, bool MAPPED>
 __global__ void __launch_bounds__(kThreads, 4)
 quantize_pow2_kernel(const __grid_constant__ FastParams p) {
@@ -183,16 +192,13 @@ quantize_pow2_kernel(const __grid_constant__ FastParams p) {
   }
   chain_wait();                                 // nothing above touches global memory
   __syncthreads();
-  if (blockIdx.x == 0) clear_words(p.clear);
   if (MAPPED ? warp == 0 : tid == 0) {
-    if (tid == 0 && blockIdx.x == 0 && p.info) {
-      p.info[0] = 8 * p.total_bytes; p.info[1] = 0; p.info[2] = p.total_bytes; p.info[3] = 0;
-    }
     for (int s = 0; s < kStages; ++s) {
       const uint32_t t = blockIdx.x + (uint32_t)s * grid;
       if (t < p.full_tiles) issue_tile<MAPPED>(p, sm.tile[s], &sm.full[s], t, lane);
     }
   }
+  if (blockIdx.x == 0) write_beside(p);
 
   const float sf = (float)p.s;
   const float cap = kTwo23 + sf;
@@ -421,10 +427,6 @@ quantize_warp_kernel(const __grid_constant__ FastParams p) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   chain_wait();                                 // nothing above touches global memory
-  if (blockIdx.x == 0) {
-    if (tid == 0 && p.info) { p.info[0] = 8 * p.total_bytes; p.info[1] = 0; p.info[2] = p.total_bytes; p.info[3] = 0; }
-    clear_words(p.clear);
-  }
   __syncwarp();
   for (int s = 0; s < kWarpStages; ++s) {
     const uint32_t cs = c + (uint32_t)s * stride;
@@ -435,6 +437,7 @@ quantize_warp_kernel(const __grid_constant__ FastParams p) {
   }
   // the map entries of the next chunk to arm are fetched one round ahead of their use
   MappedBucket ahead = fetch_bucket<MAP>(p, c + (uint32_t)kWarpStages * stride, chunks, lane);
+  if (blockIdx.x == 0) write_beside(p);
 
   const float sf = (float)p.s;
   const float cap = kTwo23 + sf;
@@ -603,10 +606,6 @@ quantize_group_kernel(const __grid_constant__ FastParams p) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   chain_wait();                                 // nothing above touches global memory
-  if (blockIdx.x == 0) {
-    if (tid == 0 && p.info) { p.info[0] = 8 * p.total_bytes; p.info[1] = 0; p.info[2] = p.total_bytes; p.info[3] = 0; }
-    clear_words(p.clear);
-  }
   __syncwarp();
   for (int s = 0; s < kWarpStages; ++s) {
     const uint32_t cs = c + (uint32_t)s * stride;
@@ -616,6 +615,7 @@ quantize_group_kernel(const __grid_constant__ FastParams p) {
     }
   }
   MappedBucket ahead = fetch_piece<MAPPED>(p, c + (uint32_t)kWarpStages * stride, chunks, lane);
+  if (blockIdx.x == 0) write_beside(p);
 
   const float sf = (float)p.s;
   const float cap = kTwo23 + sf;
@@ -728,6 +728,7 @@ __global__ void __launch_bounds__(kThreads, 6) quantize_generic_kernel(const Qua
   __shared__ float s_rcp[kMaxBucketsPerTile];
   chain_wait();
   quantize_generic_tile<LB, NORM, MAPPED>(p, blockIdx.x, gridDim.x, tile, part, s_rcp);
+  if (blockIdx.x == 0) clear_words(p.clear);
 }
 
 std::atomic<uint32_t> g_poll_limit{kDrainPolls};
@@ -802,7 +803,6 @@ int launch_one(QuantizeParams& p, cudaStream_t stream) {
     const bool with_tail = !(p.n == p.coord_base && ((p.B | p.sign_words | p.level_words) & 3ull) == 0);
     fp.tail = p;
     fp.tail.info = nullptr;
-    fp.tail.clear.count = 0;
     if (d >= 1024) {
       // measured (n = 60 M, s = 15 / 255): with the 2-norm the per-warp pipelines with group barriers
       // take 83-86 us against the CTA-wide ring's 90-92; with the max-norm (100 against 84) and under a
