@@ -190,24 +190,25 @@ __device__ __forceinline__ void store_span8(const OutSpan& sp, const float (&acc
   }
 }
 
-// A warp's chunk of 512 sums, 16 consecutive ones a lane: acc as it is, or the SGD step. Where the chunk is whole and in one
-// piece, the lanes pass their quads through `turn` (2 KB of the warp's shared memory), so that accesses to `out` are to 512
-// consecutive bytes: with 16 bytes out of every 64 they were a quarter of the fixed-width decoder's L1 wavefronts. SINGLE: the
-// chunk lies in one bucket.
+// A warp's chunk of 512 sums, 16 consecutive ones a lane: acc as it is, or the SGD step. Where the chunk lies in one piece, the
+// lanes pass their quads through `turn` (2 KB of the warp's shared memory), so that accesses to `out` are to 512 consecutive
+// bytes: with 16 bytes out of every 64 they were a quarter of the fixed-width decoder's L1 wavefronts. The chunk at the end of
+// the vector goes the same way, a quad at a time (by its lanes' 16 sums, with code of its own, a ragged decode of some thousand
+// coordinates took 0.3 to 0.5 us of 3 longer). SINGLE: the chunk lies in one bucket.
 template <bool FUSED, bool SINGLE>
 __device__ __forceinline__ void store_chunk16(float* out, const BucketMap& map, const float2p (&acc)[8], uint32_t turn, uint32_t ch,
                                               uint32_t log2_chunks_per_bucket, uint32_t d, uint64_t n, float c, uint32_t lane) {
   const uint64_t i0 = (uint64_t)ch * 512u, i = i0 + lane * 16u;
-  OutSpan whole;                                  // the chunk, where it is in one piece
-  whole.ptr = out; whole.valid = 0u;
-  if (!map.src) {
-    whole.ptr = out + i0;
-    whole.valid = i0 + 512u <= n ? 512u : 0u;
-  } else if (SINGLE) {
-    const uint32_t b = ch >> log2_chunks_per_bucket;
-    whole = out_span(out, map, b, (ch - (b << log2_chunks_per_bucket)) * 512u, d, n, 512u);
-  }
-  if (whole.valid == 512u && (reinterpret_cast<uintptr_t>(whole.ptr) & 15u) == 0) {
+  if (SINGLE || !map.src) {
+    OutSpan sp;
+    if (map.src) {
+      const uint32_t b = ch >> log2_chunks_per_bucket;
+      sp = out_span(out, map, b, (ch - (b << log2_chunks_per_bucket)) * 512u, d, n, 512u);
+    } else {
+      sp.ptr = out + i0;
+      sp.valid = (uint32_t)min((uint64_t)512u, n - i0);
+    }
+    const bool quads = (reinterpret_cast<uintptr_t>(sp.ptr) & 15u) == 0;
     // quad j of lane l at 4 l + (j ^ (l / 2 & 3)): eight lanes at a time in eight groups of banks, both ways
 #pragma unroll
     for (uint32_t j = 0; j < 4; ++j) {
@@ -215,12 +216,23 @@ __device__ __forceinline__ void store_chunk16(float* out, const BucketMap& map, 
       asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(turn + (lane * 4u + (j ^ ((lane >> 1) & 3u))) * 16u),
                    "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y) : "memory");
     }
-    float4* o = reinterpret_cast<float4*>(whole.ptr) + lane;
-    const uint32_t from = turn + (lane ^ ((lane >> 3) & 3u)) * 16u;       // quad 32 j + lane
+    float* o = sp.ptr + lane * 4u;                                        // quad 32 j + lane: from o + 128 j on
+    const uint32_t from = turn + (lane ^ ((lane >> 3) & 3u)) * 16u;
+    const uint32_t left = sp.valid > lane * 4u ? sp.valid - lane * 4u : 0u;
     float4 x[4];
     if (FUSED)
 #pragma unroll
-      for (uint32_t j = 0; j < 4; ++j) x[j] = o[j * 32u];
+      for (uint32_t j = 0; j < 4; ++j) {
+        if (quads && left >= j * 128u + 4u) {
+          x[j] = *reinterpret_cast<const float4*>(o + j * 128u);
+        } else {
+          x[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (left > j * 128u) x[j].x = o[j * 128u];
+          if (left > j * 128u + 1u) x[j].y = o[j * 128u + 1u];
+          if (left > j * 128u + 2u) x[j].z = o[j * 128u + 2u];
+          if (left > j * 128u + 3u) x[j].w = o[j * 128u + 3u];
+        }
+      }
     __syncwarp();
 #pragma unroll
     for (uint32_t j = 0; j < 4; ++j) {
@@ -230,21 +242,24 @@ __device__ __forceinline__ void store_chunk16(float* out, const BucketMap& map, 
         r.x = __fsub_rn(x[j].x, __fmul_rn(c, r.x)); r.y = __fsub_rn(x[j].y, __fmul_rn(c, r.y));
         r.z = __fsub_rn(x[j].z, __fmul_rn(c, r.z)); r.w = __fsub_rn(x[j].w, __fmul_rn(c, r.w));
       }
-      o[j * 32u] = r;
+      if (quads && left >= j * 128u + 4u) {
+        *reinterpret_cast<float4*>(o + j * 128u) = r;
+      } else {
+        if (left > j * 128u) o[j * 128u] = r.x;
+        if (left > j * 128u + 1u) o[j * 128u + 1u] = r.y;
+        if (left > j * 128u + 2u) o[j * 128u + 2u] = r.z;
+        if (left > j * 128u + 3u) o[j * 128u + 3u] = r.w;
+      }
     }
     __syncwarp();                                 // before the next chunk's quads
     return;
   }
-  if (i >= n) return;
+  if (i >= n) return;                             // per-tensor policy, several buckets to a chunk: each lives elsewhere
   float v[16];
 #pragma unroll
   for (int j = 0; j < 8; ++j) { const float2 a = unpair2(acc[j]); v[2 * j] = a.x; v[2 * j + 1] = a.y; }
-  if (map.src) {                                  // per-tensor policy: buckets live elsewhere
-    const uint64_t b = i / d;
-    store_span16<FUSED>(out_span(out, map, b, (uint32_t)(i - b * d), d, n, 16u), v, c);
-  } else {
-    store_lane16<FUSED>(out + i, v, i, n, c);
-  }
+  const uint64_t b = i / d;
+  store_span16<FUSED>(out_span(out, map, b, (uint32_t)(i - b * d), d, n, 16u), v, c);
 }
 
 }  // namespace qsgd
