@@ -10,8 +10,8 @@
 //      words and are merged with shared-memory atomics) and flushes whole words to the payload
 //      with coalesced stores (flush_run).
 // A bucket is handled by a team of d / 64 lanes (at most a warp, at least one lane), so that the
-// sequential walk over a lane's nonzeros is long enough to amortise the team's scans. Levels above 15 in
-// longer buckets go by tiles, a thread with 16 coordinates, instead (use_tiles), and small problems are quantized and
+// sequential walk over a lane's nonzeros is long enough to amortise the team's scans. Levels above 15 go by tiles, a
+// thread with 16 coordinates, in the dense code and in the longest buckets (use_tiles), and small problems are quantized and
 // measured in one kernel (elias_encode_small.cu).
 //
 // What bounds them (n = 34 M, d = 512, s = 15, a mixture of two scales): both the integer pipe, 79 % (length, 16.5 us) and 65 %

@@ -49,14 +49,15 @@ inline uint32_t tile_buckets(uint32_t d) { return kTileCoords / d; }
 // adds up.
 constexpr uint32_t kSmallTiles = 1000;
 
-// Beyond them, and with a bucket map: by teams (a lane walks 64 coordinates or more: less work per coordinate) or by tiles (a thread has 16: shorter
-// walks, less staging per CTA, so more of them resident)? Whole encodes measured both ways, teams against tiles (us). Levels
-// above 15, where a symbol costs most: Code'_s 97 / 70 at n = 17 M, d = 4096, s = 64, 58 / 44 at 8 M, s = 255; Code_s 124 / 103
-// at 17 M, d = 4096, 42 / 40 at 5 M, d = 512, but 89 / 102 at 17 M, d = 128. Levels up to 15: Code'_s 191 / 239 at 67 M,
-// d = 1024, s = 3 and 60 / 69 at 17 M, d = 128, s = 15; Code_s 142 / 204 at 60 M, d = 512, s = 15. Up to 1000 tiles always by
-// tiles: teams do not fill the GPU.
+// Beyond them, and with a bucket map: by teams (a lane walks 64 coordinates or more: less work per coordinate) or by tiles (a thread
+// has 16: shorter walks, less staging per CTA, so more of them resident)? Whole encodes measured both ways, teams against tiles (us).
+// Levels above 15, where a symbol costs most. Code'_s: 97 / 70 at n = 17 M, d = 4096, s = 64, 58 / 44 at 8 M, s = 255. Code_s, 4200
+// encodes of 3 to 120 M: tiles take 0.8 to 0.99 of the speed of teams on average up to d = 3328 from 8 M on (61 M, d = 512, s = 22, a
+// mixture of two scales 190 / 254; 76 M, d = 1024 248 / 325), 1.02 to 1.37 of it at d = 3584 to 4096, where a lane walks 128
+// coordinates and a tile is nearly full. Levels up to 15: Code'_s 191 / 239 at 67 M, d = 1024, s = 3 and 60 / 69 at 17 M, d = 128,
+// s = 15; Code_s 142 / 204 at 60 M, d = 512, s = 15. Up to 1000 tiles always by tiles: teams do not fill the GPU.
 inline bool use_tiles(uint64_t n, uint32_t d, uint32_t s, bool dense) {
-  return n <= kSmallTiles * 4096ull || (s > 15u && (dense || d >= 512u));
+  return n <= kSmallTiles * 4096ull || (s > 15u && (dense || d >= 3584u));
 }
 inline bool use_small(uint64_t n, uint32_t d, const BucketMap& map) {
   return !map.src && n <= kSmallTiles * (uint64_t)(tile_buckets(d) * d);

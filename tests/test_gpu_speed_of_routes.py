@@ -1,0 +1,28 @@
+"""Calls that a rule of a dispatch, or a kernel's split of the work, must not leave behind others of the same size: ratios of
+times of one and the same run, with room for noise."""
+import pytest
+import torch
+
+import paper_1610_02132_b200 as Q
+from oracle import oracle as O
+from paper_1610_02132_b200 import inputs as I
+from test_gpu_relative_speed import decode, time_of
+
+pytestmark = pytest.mark.gpu
+
+L2, MAX, FIXED, ELIAS, DENSE = O.NORM_L2, O.NORM_MAX, O.CODE_FIXED, O.CODE_ELIAS, O.CODE_ELIAS_DENSE
+
+
+def encode(g, d, s, norm, code):
+    n, status = g.numel(), Q.new_status()
+    out = torch.empty(Q.qsgd_message_capacity(n, d, s, code), dtype=torch.uint8, device="cuda")
+    info = torch.zeros(4, dtype=torch.int64, device="cuda")
+    ws = torch.empty(Q.qsgd_workspace_bytes(n, d, s, code), dtype=torch.uint8, device="cuda")
+    return lambda: Q.qsgd_encode(g, d, s, norm, code, 7, 0, 0, out, info, ws, status)
+
+
+def test_elias_encode_of_mostly_small_values_with_many_levels():
+    """Buckets of 512 against buckets of 480, for which there is only one way."""
+    g = I.gaussian_mixture_device(40 * 2 ** 20, seed=3)
+    here, other = time_of(*(encode(g, d, 22, L2, ELIAS) for d in (512, 480)), repeats=4)
+    assert here < 1.1 * other                              # 0.9; 1.2 by tiles
