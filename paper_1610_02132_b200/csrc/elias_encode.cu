@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kThreads) elias_length_kernel(const BucketPara
 #pragma unroll
     for (int i = 0; i < kWarps; ++i) s += warp_sum[i];
     cta_sums[blockIdx.x] = s;
-    atomicAdd(reinterpret_cast<unsigned long long*>(group_sums) + blockIdx.x / kSumGroup, (unsigned long long)s);
+    add_to_groups(group_sums, s);
   }
 }
 
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kThreads) elias_tile_length_kernel(const Bucke
 #pragma unroll
     for (int i = 0; i < kWarps; ++i) s += slots[1][i];
     tile_sums[blockIdx.x] = s;
-    atomicAdd(reinterpret_cast<unsigned long long*>(group_sums) + blockIdx.x / kSumGroup, (unsigned long long)s);
+    add_to_groups(group_sums, s);
   }
 }
 
@@ -275,9 +275,9 @@ int launch_elias_encode(const float* g, uint64_t n, uint32_t d, uint32_t s, int 
   if (use_small(n, d, map))
     return launch_elias_encode_small(g, n, d, s, norm_kind, dense, seed, step, worker, out, out_capacity, out_bits, w, status_dev, stream);
   const uint64_t per_cta = use_tiles(n, d, s, dense) ? tile_buckets(d) : make_teams(d).nbc, B = (n + d - 1) / d;
-  const uint64_t groups = ((B + per_cta - 1) / per_cta + kSumGroup - 1) / kSumGroup;
+  const uint32_t words = sum_words((uint32_t)((B + per_cta - 1) / per_cta));
   int st = launch_quantize_fixed(g, n, d, s, norm_kind, seed, step, worker, w.fixed, status_dev, nullptr,
-                                 ClearWords{use_tiles(n, d, s, dense) ? w.tile_groups : w.group_sums, (uint32_t)groups}, map, stream);
+                                 ClearWords{use_tiles(n, d, s, dense) ? w.tile_groups : w.group_sums, words}, map, stream);
   if (st) return st;
   const FixedLayout L = make_fixed_layout(n, d, s);
   BucketParams bp;

@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kThreads) elias_quantize_length_kernel(const _
 struct TileScatterArgs {
   BucketParams bp;
   const uint32_t* sums;       // bits of every tile
-  const uint64_t* groups;     // of every kSumGroup tiles, or null
+  const uint64_t* groups;     // of every group of tiles, or null
   uint32_t ctas;
   uint8_t* out;
   size_t out_capacity;

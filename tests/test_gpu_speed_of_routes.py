@@ -26,3 +26,11 @@ def test_elias_encode_of_mostly_small_values_with_many_levels():
     g = I.gaussian_mixture_device(40 * 2 ** 20, seed=3)
     here, other = time_of(*(encode(g, d, 22, L2, ELIAS) for d in (512, 480)), repeats=4)
     assert here < 1.1 * other                              # 0.9; 1.2 by tiles
+
+
+def test_encodes_of_more_ctas_grow_no_faster_than_their_length():
+    """Four times the coordinates, with so many CTAs that what each does to find its place must not grow along."""
+    n, d, s = 2 ** 28, 2080, 16
+    g = I.gaussian_device(4 * n, 1.0, seed=3)
+    less, more = time_of(*(encode(g[:m], d, s, L2, DENSE) for m in (n, 4 * n)), repeats=1, replays=4)
+    assert more < 4.4 * less                               # 4.0; 4.8 where every CTA reads the sums of all groups
