@@ -41,10 +41,25 @@ bool use_teams(uint64_t B, uint32_t K, uint32_t d, uint32_t s) {
 // 177 / 218. Symbols of levels above 15, which the streams' table seldom holds, only where the bucket's largest level is likely
 // far above the others: max-norm, n = 17 M, K = 8: d = 512, s = 64 552 / 751, d = 4096 705 / 700, but d = 128 633 / 570, d = 64,
 // s = 48 627 / 574; d = 128, s = 100 718 / 599.
+// Few levels in short buckets, where opening a bucket is most of a stream's work (5200 problems; speed of streams over that of
+// teams): s <= 7, d = 32 0.74 to 0.99 up to 400 K strings, 1.06 to 1.27 beyond, with one or two peers 0.74 to 1.03 at any number;
+// s <= 3, d = 64 and 96 1.1 to 1.3 up to 80 K, 0.93 to 1.02 from there to 256 K, 1.05 to 1.2 beyond, with one or two peers 0.84 to
+// 1.1; s <= 3 and one peer with d = 128 to 192 0.94 to 0.99 from 100 K to 512 K, with longer ones about 1 from 64 K to 256 K.
 bool use_streams(uint64_t B, uint32_t K, uint32_t d, uint32_t s) {
   if (K > 32u || s > (d >= 512u ? 64u : 32u)) return false;
-  const uint32_t line = K == 1u ? 48u : K < 8u ? 30u : 22u;
-  return B * K > (uint64_t)line << 10;
+  const uint64_t strings = B * K;
+  uint32_t line = K == 1u ? 48u : K < 8u ? 30u : 22u, from = 0, to = 0;       // in 1024 strings; from .. to: teams all the same
+  if (s <= 7u && d < 64u) {
+    if (K <= 2u) return false;
+    line = 400u;
+  } else if (s <= 3u && d < 128u) {
+    from = K == 1u ? 100u : K == 2u ? 64u : 80u;
+    to = K <= 2u ? ~0u : 256u;
+  } else if (s <= 3u && K == 1u) {
+    from = d < 256u ? 100u : 64u;
+    to = d < 256u ? 512u : 256u;
+  }
+  return strings > (uint64_t)line << 10 && (strings <= (uint64_t)from << 10 || strings > (uint64_t)to << 10);
 }
 
 // Mean bits of a string behind its scale, where the host can tell: in a message the offset table follows the padded

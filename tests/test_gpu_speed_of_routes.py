@@ -34,3 +34,4 @@ def test_encodes_of_more_ctas_grow_no_faster_than_their_length():
     g = I.gaussian_device(4 * n, 1.0, seed=3)
     less, more = time_of(*(encode(g[:m], d, s, L2, DENSE) for m in (n, 4 * n)), repeats=1, replays=4)
     assert more < 4.4 * less                               # 4.0; 4.8 where every CTA reads the sums of all groups
+
