@@ -277,43 +277,52 @@ __device__ __forceinline__ uint32_t emit(const Tables<false>& tab, const uint32_
   return bad >> 31 ? QSGD_DEV_OVERRUN : 0u;
 }
 
-// Reads a part in kMarks pieces and keeps where each piece ended, so that a lane that has to read its part
+// Reads a part in MARKS pieces and keeps where each piece ended, so that a lane that has to read its part
 // again from another bit can stop at the first mark where it falls into step with its first reading.
-template <bool DENSE> constexpr uint32_t kMarksOf = DENSE ? 1u : 4u;
 constexpr uint32_t kLeastPiece = 96;      // bits
-template <bool DENSE>
+template <uint32_t MARKS>
 struct Marks {
-  static constexpr uint32_t kMarks = kMarksOf<DENSE>;
-  uint32_t pos[kMarks];       // first symbol at or behind the mark
-  uint32_t sum[kMarks];       // positions from the part's start up to there
+  uint32_t pos[MARKS];        // first symbol at or behind the mark
+  uint32_t sum[MARKS];        // positions from the part's start up to there
 };
 
-template <bool DENSE, int WIDTH>
-__device__ __forceinline__ void read_part(const Tables<DENSE>& tab, const uint32_t* words, uint32_t start, uint32_t lo,
-                                          uint32_t hi, uint32_t end, bool again, Marks<DENSE>& m) {
-  constexpr uint32_t kMarks = kMarksOf<DENSE>;
-  const uint32_t piece = max((hi - lo + kMarks - 1u) / kMarks, kLeastPiece);
+// By the lanes of `mask`, which wait for one another at the marks: left to itself the compiler let them read some of the pieces one
+// lane after the other (Code_s, n = 729 K, d = 4096, s = 15, K = 8, max-norm: 35 -> 53 us).
+template <bool DENSE, int WIDTH, uint32_t MARKS>
+__device__ __forceinline__ void read_part(const Tables<DENSE>& tab, const uint32_t* words, uint32_t start, uint32_t lo, uint32_t hi,
+                                          uint32_t end, bool again, uint32_t mask, Marks<MARKS>& m) {
+  const uint32_t piece = max((hi - lo + MARKS - 1u) / MARKS, kLeastPiece);
   uint32_t pos = start, sum = 0;
+  bool apart = true;                                // not in step with the first reading
 #pragma unroll
-  for (uint32_t q = 0; q < kMarks; ++q) {
-    uint32_t n;
-    pos = walk<DENSE, WIDTH>(tab, words, pos, q == kMarks - 1u ? hi : min(lo + (q + 1u) * piece, hi), end, &n);
-    sum += n;
-    if (again && pos == m.pos[q]) {                 // in step from here on: the rest differs by the count only
-      const uint32_t more = sum - m.sum[q];
+  for (uint32_t q = 0; q < MARKS; ++q) {
+    __syncwarp(mask);
+    if (apart) {
+      uint32_t n;
+      pos = walk<DENSE, WIDTH>(tab, words, pos, q == MARKS - 1u ? hi : min(lo + (q + 1u) * piece, hi), end, &n);
+      sum += n;
+      if (again && pos == m.pos[q]) {               // from here on: the rest differs by the count only
+        const uint32_t more = sum - m.sum[q];
 #pragma unroll
-      for (uint32_t r = 0; r < kMarks; ++r)
-        if (r >= q) m.sum[r] += more;
-      return;
+        for (uint32_t r = 0; r < MARKS; ++r)
+          if (r >= q) m.sum[r] += more;
+        apart = false;
+      } else {
+        m.pos[q] = pos;
+        m.sum[q] = sum;
+      }
     }
-    m.pos[q] = pos;
-    m.sum[q] = sum;
   }
+  __syncwarp(mask);
 }
 
 // SPLIT: a string is shared by several warps of a CTA that has a warp for every part of its strings.
-template <bool DENSE, int WIDTH, bool FUSED, bool SPLIT>
-__global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads) decode_elias_teams_kernel(const __grid_constant__ TeamParams p) {
+// CTAs that an SM has to hold, 0 for the compiler's choice. Code'_s, whose loops hold most, is faster with all registers that they
+// want (s = 255, d = 512, K = 32 27.5 -> 25.8 us), Code_s with levels above 127 with 40 a thread and six CTAs (d = 512, K = 5 41 -> 39).
+template <bool DENSE, int WIDTH, bool SPLIT> constexpr uint32_t kLeastCtas = SPLIT ? 0 : DENSE ? 1 : WIDTH == kWide ? 6 : 0;
+
+template <bool DENSE, int WIDTH, bool FUSED, bool SPLIT, uint32_t MARKS>
+__global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads, kLeastCtas<DENSE, WIDTH, SPLIT>) decode_elias_teams_kernel(const __grid_constant__ TeamParams p) {
   using Code = typename CodeOf<WIDTH>::type;
   constexpr uint32_t kLevels = 1u << CodeOf<WIDTH>::kSignShift;
   extern __shared__ __align__(16) uint8_t tsm[];
@@ -398,10 +407,10 @@ __global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads) decode_elias_
         if (DENSE && ref.total < 3u * db) per = (per + 1u) & ~1u;
         const uint32_t lo = min(first + tt * per, end), hi = tt == TT - 1u ? end : min(lo + per, end);
         uint32_t start = lo;
-        Marks<DENSE> m;
-        constexpr uint32_t kMarks = kMarksOf<DENSE>;
+        Marks<MARKS> m;
 #pragma unroll
-        for (uint32_t q = 0; q < kMarks; ++q) { m.pos[q] = lo; m.sum[q] = 0u; }
+        for (uint32_t q = 0; q < MARKS; ++q) { m.pos[q] = lo; m.sum[q] = 0u; }
+        const uint32_t readers = __ballot_sync(0xffffffffu, reads);
         if (reads) {
           if (tt == 0u) {
             Window in;
@@ -411,22 +420,23 @@ __global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads) decode_elias_
             uint32_t skipped;
             start = walk<DENSE, WIDTH>(tab, words, lo - min(kWarmUp<DENSE>, lo - first), lo, end, &skipped);
           }
-          read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, false, m);
+          read_part<DENSE, WIDTH, MARKS>(tab, words, start, lo, hi, end, false, readers, m);
         } else if (j < rows && tt == 0u) {
           scales[j] = 0.f;
         }
         uint32_t other = start;                           // dense code: where the other reading started (below)
-        Marks<DENSE> o = m;
+        Marks<MARKS> o = m;
         uint32_t rounds = reads && ref.total < 3u * db ? 1u : 0u;           // until all lanes read again; 0: never
         for (;;) {
           if constexpr (!DENSE) {
             for (;;) {
-              const uint32_t before = __shfl_up_sync(0xffffffffu, m.pos[kMarks - 1u], 1, (int)T);
+              const uint32_t before = __shfl_up_sync(0xffffffffu, m.pos[MARKS - 1u], 1, (int)T);
               const bool again = t != 0u && before != start;
-              if (!__any_sync(0xffffffffu, again)) break;
+              const uint32_t who = __ballot_sync(0xffffffffu, again);
+              if (who == 0u) break;
               if (again) {
                 start = before;
-                read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, true, m);
+                read_part<DENSE, WIDTH, MARKS>(tab, words, start, lo, hi, end, true, who, m);
               }
             }
           } else {
@@ -438,12 +448,12 @@ __global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads) decode_elias_
               uint32_t before;
               bool again;
               for (;;) {
-                before = __shfl_up_sync(0xffffffffu, m.pos[kMarks - 1u], 1, (int)T);
+                before = __shfl_up_sync(0xffffffffu, m.pos[MARKS - 1u], 1, (int)T);
                 again = t != 0u && before != start;
                 const bool had = again && before == other;
                 if (!__any_sync(0xffffffffu, had)) break;
                 if (had) {
-                  const Marks<DENSE> q = m;
+                  const Marks<MARKS> q = m;
                   m = o; o = q;
                   other = start; start = before;
                 }
@@ -453,21 +463,23 @@ __global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads) decode_elias_
               const bool astray = rounds != 0u && (wrong & (0xFFFFFFFFu >> (32u - T) << (lane & ~(T - 1u)))) != 0u;
               const bool now = astray && rounds == 2u;
               if (astray) rounds = now ? 0u : 2u;
-              if (now && t != 0u && start < hi && other == start) {
+              const bool further = now && t != 0u && start < hi && other == start;
+              const uint32_t who = __ballot_sync(0xffffffffu, further);
+              if (further) {
                 other = start + 1u;
-                read_part<DENSE, WIDTH>(tab, words, other, lo, hi, end, true, o);
+                read_part<DENSE, WIDTH, MARKS>(tab, words, other, lo, hi, end, true, who, o);
               }
               if (__any_sync(0xffffffffu, now)) continue;
               if (again) {
                 o = m; other = start;
                 start = before;
-                read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, true, m);
+                read_part<DENSE, WIDTH, MARKS>(tab, words, start, lo, hi, end, true, wrong, m);
               }
             }
           }
           if constexpr (!SPLIT) break;
           // the warps of a string: the first lane of each begins where the warp in front of it ended
-          if (lane == 31u) warp_end[SPLIT ? warp : 0u] = m.pos[kMarks - 1u];
+          if (lane == 31u) warp_end[SPLIT ? warp : 0u] = m.pos[MARKS - 1u];
           __syncthreads();
           const uint32_t before = SPLIT && part != 0u ? warp_end[SPLIT ? warp - 1u : 0u] : start;
           const bool wrong = reads && t == 0u && before != start;
@@ -475,10 +487,10 @@ __global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads) decode_elias_
           if (wrong) {
             o = m; other = start;
             start = before;
-            read_part<DENSE, WIDTH>(tab, words, start, lo, hi, end, true, m);
+            read_part<DENSE, WIDTH, MARKS>(tab, words, start, lo, hi, end, true, 1u, m);     // (lane 0)
           }
         }
-        const uint32_t sum = m.sum[kMarks - 1u], stop = m.pos[kMarks - 1u];
+        const uint32_t sum = m.sum[MARKS - 1u], stop = m.pos[MARKS - 1u];
         uint32_t upto = sum;                              // positions passed by the lanes up to this one
         for (uint32_t o = 1; o < T; o <<= 1) {
           const uint32_t q = __shfl_up_sync(0xffffffffu, upto, o, (int)T);
@@ -557,13 +569,14 @@ __global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads) decode_elias_
   }
 }
 
-template <bool DENSE, int WIDTH>
+template <bool DENSE, int WIDTH, uint32_t MARKS>
 int launch_width(TeamParams& p, bool fused, size_t smem, cudaStream_t stream) {
   static KernelSite site[4];
   void (*kern)(TeamParams);
   const bool split = p.split > 1u;
-  if (split) kern = fused ? decode_elias_teams_kernel<DENSE, WIDTH, true, true> : decode_elias_teams_kernel<DENSE, WIDTH, false, true>;
-  else kern = fused ? decode_elias_teams_kernel<DENSE, WIDTH, true, false> : decode_elias_teams_kernel<DENSE, WIDTH, false, false>;
+  if (split) kern = fused ? decode_elias_teams_kernel<DENSE, WIDTH, true, true, DENSE ? 1 : MARKS>
+                          : decode_elias_teams_kernel<DENSE, WIDTH, false, true, DENSE ? 1 : MARKS>;
+  else kern = fused ? decode_elias_teams_kernel<DENSE, WIDTH, true, false, MARKS> : decode_elias_teams_kernel<DENSE, WIDTH, false, false, MARKS>;
   const uint32_t threads = split ? p.buckets * p.Kc * p.split * 32u : kThreads;
   int sms = 0, occ = 0;
   const int st = site[(split ? 2 : 0) + (fused ? 1 : 0)].lookup_dynamic(kern, (int)threads, smem, &sms, &occ);
@@ -617,9 +630,14 @@ int launch_elias_teams(const FieldParams& f, bool dense, bool fused, cudaStream_
     if (strings_of_cta * 128u <= kMostThreads && likely >= 128u * 192u) p.split = 4;
   }
   const size_t smem = align16(bytes(p.buckets, p.Kc));
-#define QSGD_RUN(D, W) launch_width<D, W>(p, fused, smem, stream)
-  if (dense) return width == kNibble ? QSGD_RUN(true, kNibble) : width == kByte ? QSGD_RUN(true, kByte) : QSGD_RUN(true, kWide);
-  return width == kNibble ? QSGD_RUN(false, kNibble) : width == kByte ? QSGD_RUN(false, kByte) : QSGD_RUN(false, kWide);
+  // Marks of a dense string's parts: one is 2 to 4 % less work, two save half of a second reading, which is what long symbols and
+  // many peers (few lanes to a string, long parts) lead to. Two against one (us): s = 3, d = 2048, K = 48 74 / 81; s = 127, d = 2048,
+  // K = 32, max-norm 311 / 345; s = 15, d = 4096, K = 16 37.6 / 36.4.
+  const bool two = dense && (p.K > 16u || (p.s > 15u && p.d >= 256u));
+#define QSGD_RUN(D, W, M) launch_width<D, W, M>(p, fused, smem, stream)
+#define QSGD_WIDTHS(D, M) (width == kNibble ? QSGD_RUN(D, kNibble, M) : width == kByte ? QSGD_RUN(D, kByte, M) : QSGD_RUN(D, kWide, M))
+  return !dense ? QSGD_WIDTHS(false, 4) : two ? QSGD_WIDTHS(true, 2) : QSGD_WIDTHS(true, 1);
+#undef QSGD_WIDTHS
 #undef QSGD_RUN
 }
 

@@ -35,3 +35,11 @@ def test_encodes_of_more_ctas_grow_no_faster_than_their_length():
     less, more = time_of(*(encode(g[:m], d, s, L2, DENSE) for m in (n, 4 * n)), repeats=1, replays=4)
     assert more < 4.4 * less                               # 4.0; 4.8 where every CTA reads the sums of all groups
 
+
+
+@pytest.mark.parametrize("n,d,K", [(729088, 4096, 8), (2668, 512, 64)])
+def test_strings_of_more_bits_in_another_decoder_width(n, d, K):
+    """Teams with 15 levels and with 16, whose codes take a byte: max-norm strings of much the same length."""
+    make = lambda w: I.sparse_laplace_device(n, 1e-3, 0.3, seed=w)
+    fewer, more = time_of(*(decode(n, d, s, MAX, ELIAS, K, make) for s in (15, 16)))
+    assert fewer < 1.1 * more
