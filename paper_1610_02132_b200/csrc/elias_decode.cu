@@ -116,10 +116,10 @@ int launch_decode_elias(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
   f.out = acc_or_x; f.c = eta / (float)K; f.minus_zero = -0.f; f.status = status_dev; f.map = map;
   f.when = Regime{0u, kNoBound};
   if (dense && use_streams(B, K, d, s)) return launch_elias_dense(f, fused, stream);
-  if (dense || K > 32u) return launch_elias_teams(f, dense, fused, stream);
+  const uint32_t mean = mean_bits(peers, K, B, n);
+  if (dense || K > 32u) return launch_elias_teams(f, dense, mean, fused, stream);
 
   const bool teams = use_teams(B, K, d, s), small = teams && work <= kSmallWork;
-  const uint32_t mean = mean_bits(peers, K, B, n);
   if (mean != kNoBound) {
     if (mean < sparse_line(d) && (!small || sparse_though_small(mean, K, work))) return launch_elias_sparse(f, fused, stream);
   } else if (!small) {                            // decided on the device: both are launched, one stands down
@@ -128,7 +128,7 @@ int launch_decode_elias(const PeerSet& peers, uint32_t K, uint64_t n, uint32_t d
     if (st) return st;
     f.when = Regime{sparse_line(d), kNoBound};
   }
-  if (teams) return launch_elias_teams(f, false, fused, stream);
+  if (teams) return launch_elias_teams(f, false, mean, fused, stream);
   if (s > 15u) return launch_elias_fields(f, fused, stream);
   const uint32_t line = bytes_line(K, d, work);
   const bool likely = use_bytes(K, d, s, work) && (d <= 96u || mean == kNoBound);

@@ -31,6 +31,7 @@ namespace {
 constexpr uint32_t kThreads = 256, kMostThreads = 1024;       // (the latter where strings are shared by several warps)
 template <bool DENSE> constexpr uint32_t kWarmUp = DENSE ? 96 : 64;      // bits: 75-98 % of the starts are then right
 constexpr uint32_t kLeastPart = 64;               // bits of a string that are worth a lane
+constexpr uint32_t kSplitBits = 120;              // ... that a lane has where a string is shared by several warps
 constexpr uint32_t kDenseBits = 10;
 constexpr uint32_t kFewBits = 7;                  // bits per symbol of a string from which on a table entry rarely holds one
 constexpr uint32_t kRowPad = 16;                  // bytes between rows: teams at similar positions use other banks
@@ -366,9 +367,11 @@ __global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads, kLeastCtas<DE
   float* sums = reinterpret_cast<float*>(tsm + (size_t)most * p.row_bytes);
   float* scales = sums + (p.Kc < p.K ? p.buckets * p.d : 0u);
   const uint32_t T = SPLIT ? 32u : p.T, t = lane & (T - 1u);
-  const uint32_t warps = SPLIT ? p.split : 1u, warp = tid >> 5, part = SPLIT ? warp % warps : 0u;       // of a string
-  const uint32_t team = SPLIT ? warp / warps : tid / T, teams = SPLIT ? (threads >> 5) / warps : kThreads / T;
-  const uint32_t tt = part * 32u + t, TT = T * warps;                     // this lane among the string's lanes
+  // SPLIT: warp w has part w / strings of string w % strings, so that the first parts, which have work whatever the length,
+  // lie on all of an SM's schedulers; warps beyond that help with the tables and the sums only
+  const uint32_t warp = tid >> 5, part = SPLIT ? warp / most : 0u;
+  const uint32_t team = SPLIT ? warp % most : tid / T, teams = SPLIT ? most : kThreads / T;
+  const uint32_t tt = part * 32u + t, TT = SPLIT ? 32u * p.split : T;     // this lane among the string's lanes
   const uint64_t groups = (p.B + p.buckets - 1) / p.buckets;
   chain_wait();                                         // the messages come from the kernels ahead
   if (!DENSE && p.when.lo && mean_below(p.when.lo, p.peers, p.K, p.B)) return;
@@ -387,7 +390,7 @@ __global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads, kLeastCtas<DE
         const uint32_t j = j0 + team;
         const uint32_t g = j / kc, k = j - g * kc;         // k: in this pass
         const uint64_t b = b0 + g;
-        const bool mine = j < rows && g < nb;
+        const bool mine = j < rows && g < nb && tt < TT;
         StringRef ref;
         ref.words = nullptr; ref.lo = 0; ref.total = 0; ref.err = 0;
         uint32_t db = 0;
@@ -403,7 +406,16 @@ __global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads, kLeastCtas<DE
         // 4 and 4 bits long, and a reader that starts an odd number of bits from the front of a string of such levels is
         // out of step to the end of its part: where the symbols are short, parts have an even length (n = 33.5 M, d = 4096,
         // K = 8, 2-norm: 2361 -> 423 us at s = 15, 1851 -> 371 at s = 1).
-        uint32_t per = max((ref.total + TT - 1u) / TT, kLeastPart);
+        // SPLIT: a string that is shorter than was likely goes by fewer lanes, as without: more of them would start out of step.
+        // So does one of symbols that are 2.75 to 3.25 bits on average, in which a warp that starts out of step often stays so
+        // (n = 14 K, d = 2048, s = 32, K = 5, 3.03 bits: 19 us by 32 lanes, 27 by 64; outside that range
+        // 64 lanes are 5 to 40 % faster).
+        uint32_t of = TT;
+        if (SPLIT) {
+          if (of > 64u && ref.total < 128u * kSplitBits) of = 64u;
+          if (ref.total < 64u * kSplitBits || (DENSE && 4u * ref.total >= 11u * db && 4u * ref.total < 13u * db)) of = 32u;
+        }
+        uint32_t per = max((ref.total + of - 1u) / of, kLeastPart);
         if (DENSE && ref.total < 3u * db) per = (per + 1u) & ~1u;
         const uint32_t lo = min(first + tt * per, end), hi = tt == TT - 1u ? end : min(lo + per, end);
         uint32_t start = lo;
@@ -481,7 +493,7 @@ __global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads, kLeastCtas<DE
           // the warps of a string: the first lane of each begins where the warp in front of it ended
           if (lane == 31u) warp_end[SPLIT ? warp : 0u] = m.pos[MARKS - 1u];
           __syncthreads();
-          const uint32_t before = SPLIT && part != 0u ? warp_end[SPLIT ? warp - 1u : 0u] : start;
+          const uint32_t before = SPLIT && part != 0u ? warp_end[SPLIT ? warp - most : 0u] : start;
           const bool wrong = reads && t == 0u && before != start;
           if (!__syncthreads_or(wrong ? 1 : 0)) break;
           if (wrong) {
@@ -499,7 +511,7 @@ __global__ void __launch_bounds__(SPLIT ? kMostThreads : kThreads, kLeastCtas<DE
         if constexpr (SPLIT) {
           if (lane == 31u) warp_sum[warp] = upto;
           __syncthreads();
-          for (uint32_t w = warp - part; w < warp; ++w) upto += warp_sum[w];
+          for (uint32_t w = team; w < warp; w += most) upto += warp_sum[w];
         }
         uint32_t err = ref.err;
         if (reads) {
@@ -577,7 +589,7 @@ int launch_width(TeamParams& p, bool fused, size_t smem, cudaStream_t stream) {
   if (split) kern = fused ? decode_elias_teams_kernel<DENSE, WIDTH, true, true, DENSE ? 1 : MARKS>
                           : decode_elias_teams_kernel<DENSE, WIDTH, false, true, DENSE ? 1 : MARKS>;
   else kern = fused ? decode_elias_teams_kernel<DENSE, WIDTH, true, false, MARKS> : decode_elias_teams_kernel<DENSE, WIDTH, false, false, MARKS>;
-  const uint32_t threads = split ? p.buckets * p.Kc * p.split * 32u : kThreads;
+  const uint32_t parts = p.buckets * p.Kc * p.split * 32u, threads = split && parts > kThreads ? parts : kThreads;
   int sms = 0, occ = 0;
   const int st = site[(split ? 2 : 0) + (fused ? 1 : 0)].lookup_dynamic(kern, (int)threads, smem, &sms, &occ);
   if (st) return st;
@@ -588,7 +600,7 @@ int launch_width(TeamParams& p, bool fused, size_t smem, cudaStream_t stream) {
 
 }  // namespace
 
-int launch_elias_teams(const FieldParams& f, bool dense, bool fused, cudaStream_t stream) {
+int launch_elias_teams(const FieldParams& f, bool dense, uint32_t mean, bool fused, cudaStream_t stream) {
   TeamParams p;
   p.peers = f.peers; p.K = f.K; p.n = f.n; p.d = f.d; p.s = f.s; p.B = f.B; p.out = f.out; p.c = f.c;
   p.status = f.status; p.map = f.map; p.when = f.when; p.minus_zero = f.minus_zero;
@@ -623,11 +635,16 @@ int launch_elias_teams(const FieldParams& f, bool dense, bool fused, cudaStream_
   // So few strings that every CTA has an SM to itself: two warps to a string, where each lane then still has 96 bits or so, or
   // four with twice as many (less is lost to the bits ahead of a part). One against two, and four (us): n = 40 K, d = 4096,
   // s = 64, K = 8, dense code 30 / 26, 32; 131 K, d = 2048, s = 15, K = 4 32 / 28, 28; 64 K, d = 4096, s = 255, K = 2 73 / 48, 36.
+  // By the strings' mean length where it is known, else by what is usual. Strings that are short all the same (gradients of
+  // mostly small values) then cost up to 1 us of 10: so one level in Code_s, whose strings always are, stays with one warp.
   p.split = 1;
   if (p.T == 32u && p.Kc == p.K && (p.B + p.buckets - 1) / p.buckets <= (uint64_t)sms) {
-    const uint32_t likely = p.d * (width == kNibble ? 3u : width == kByte ? 4u : 9u), strings_of_cta = p.buckets * p.Kc;
-    if (strings_of_cta * 64u <= kMostThreads && likely >= 64u * 96u) p.split = 2;
-    if (strings_of_cta * 128u <= kMostThreads && likely >= 128u * 192u) p.split = 4;
+    const uint32_t strings_of_cta = p.buckets * p.Kc;
+    uint32_t likely = p.d * (width == kNibble ? 3u : width == kByte ? 4u : 9u), two = 64u * 96u, four = 128u * 192u;
+    if (mean != kNoBound) { likely = mean; two = 64u * kSplitBits; four = 128u * kSplitBits; }
+    else if (!dense && (p.s == 1u || p.d < (p.s <= 3u ? 3072u : 1536u))) likely = 0u;
+    if (strings_of_cta * 64u <= kMostThreads && likely >= two) p.split = 2;
+    if (strings_of_cta * 128u <= kMostThreads && likely >= four) p.split = 4;
   }
   const size_t smem = align16(bytes(p.buckets, p.Kc));
   // Marks of a dense string's parts: one is 2 to 4 % less work, two save half of a second reading, which is what long symbols and

@@ -43,3 +43,20 @@ def test_strings_of_more_bits_in_another_decoder_width(n, d, K):
     make = lambda w: I.sparse_laplace_device(n, 1e-3, 0.3, seed=w)
     fewer, more = time_of(*(decode(n, d, s, MAX, ELIAS, K, make) for s in (15, 16)))
     assert fewer < 1.1 * more
+
+
+def test_short_strings_where_long_ones_are_shared_by_warps():
+    """A quarter of the bits: strings of mostly small values against such of N(0, 1)."""
+    n, d, s, K = 15792, 4096, 255, 8
+    short = decode(n, d, s, L2, ELIAS, K, lambda w: I.gaussian_mixture_device(n, seed=w))
+    long = decode(n, d, s, L2, ELIAS, K)
+    assert short.bits < 0.4 * long.bits
+    few, many = time_of(short, long)
+    assert few < 0.9 * many
+
+
+def test_one_peer_against_eight():
+    """A CTA with a single string has its tables to make all the same."""
+    n, d, s = 3871, 4096, 15
+    one, eight = time_of(*(decode(n, d, s, L2, DENSE, K) for K in (1, 8)))
+    assert one < 0.9 * eight
