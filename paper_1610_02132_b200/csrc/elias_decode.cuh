@@ -116,7 +116,6 @@ __device__ __forceinline__ bool mean_below(uint32_t line, const PeerSet& peers, 
 struct FieldParams {
   PeerSet peers;
   uint32_t K;
-  uint32_t Kpad;        // lanes per bucket in the parse phase (power of two, <= 32)
   uint32_t G;           // buckets per warp
   uint64_t n;
   uint32_t d;

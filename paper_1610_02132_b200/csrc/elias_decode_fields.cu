@@ -98,21 +98,16 @@ __device__ __forceinline__ uint32_t read_codes(Window& in, uint32_t end, uint32_
   return bad >> 31 || in.bp != end ? QSGD_DEV_OVERRUN : 0u;
 }
 
-__device__ __forceinline__ uint32_t parse_to_fields(const PeerSet& peers, uint32_t k, uint64_t b,
-                                                    uint64_t B, uint32_t db, uint32_t d, uint32_t s,
-                                                    const uint2* code, uint32_t* __restrict__ row, float* A_out) {
+__device__ __forceinline__ uint32_t parse_to_fields(const StringRef& ref, bool ones, uint32_t db, uint32_t d, uint32_t s, const uint2* code,
+                                                    uint32_t* __restrict__ row, float* A_out) {
   *A_out = 0.f;
-  const StringRef ref = string_ref(peers, k, b, B, db);
   if (ref.err) return ref.err;
   Window in;
   in.open(ref.words, ref.lo);
   const uint32_t end = in.bp + 32u + ref.total;
   *A_out = __uint_as_float(in.peek());
   in.drop_even(32u, end);
-  // More than 9 bits per coordinate in all strings of the warp: nearly all levels are nonzero (37.0 -> 33.7 us at n = 1 M, d = 96,
-  // K = 5, N(0, 1); with one loop for all strings 6 % slower at n = 3 M, d = 96, K = 2, a mixture).
-  if (__all_sync(__activemask(), ref.total > 9u * db)) return read_codes<true>(in, end, db, d, s, code, row);
-  return read_codes<false>(in, end, db, d, s, code, row);
+  return ones ? read_codes<true>(in, end, db, d, s, code, row) : read_codes<false>(in, end, db, d, s, code, row);
 }
 
 template <bool FUSED>
@@ -128,7 +123,7 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
   const LevelQuotient lq = level_quotient(p.s, p.minus_zero);
 
   const uint32_t warp_words = p.G * p.bucket_words;
-  uint32_t* mine = fsm + (size_t)warp * warp_words;
+  uint32_t* words = fsm + (size_t)warp * warp_words;
   const uint32_t level_words = (p.d * LB) >> 5;
   const uint32_t pg = lane / p.K, pk = lane % p.K;            // parse role: bucket in group, peer
   const uint32_t slots_per_bucket = p.d >> 4;                 // 16-coordinate lane slots
@@ -137,15 +132,21 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
 
   for (uint64_t grp = (uint64_t)blockIdx.x * nwarps + warp; grp < groups; grp += (uint64_t)gridDim.x * nwarps) {
     const uint64_t b0 = grp * p.G;
-    for (uint32_t q = lane; q < (warp_words >> 2); q += 32) reinterpret_cast<uint4*>(mine)[q] = make_uint4(0u, 0u, 0u, 0u);
+    for (uint32_t q = lane; q < (warp_words >> 2); q += 32) reinterpret_cast<uint4*>(words)[q] = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
     // ---- phase 1: one lane per (bucket, peer) ------------------------------------------------
-    if (pk < p.K && pg < p.G && b0 + pg < p.B) {
-      uint32_t* bucket = mine + pg * p.bucket_words;
-      const uint32_t db = (uint32_t)min((uint64_t)p.d, p.n - (b0 + pg) * p.d);
+    const bool mine = pg < p.G && b0 + pg < p.B;
+    const uint32_t db = mine ? (uint32_t)min((uint64_t)p.d, p.n - (b0 + pg) * p.d) : 0u;
+    StringRef ref;
+    ref.words = nullptr; ref.lo = 0; ref.total = 0; ref.err = 0;
+    if (mine) ref = string_ref(p.peers, pk, b0 + pg, p.B, db);
+    // More than 9 bits per coordinate in all strings of the warp: nearly all levels are nonzero (37.0 -> 33.7 us at n = 1 M, d = 96,
+    // K = 5, N(0, 1); with one loop for all strings 6 % slower at n = 3 M, d = 96, K = 2, a mixture). All lanes vote.
+    const bool ones = __all_sync(0xffffffffu, !mine || ref.err || ref.total > 9u * db);
+    if (mine) {
+      uint32_t* bucket = words + pg * p.bucket_words;
       float A;
-      const uint32_t st = parse_to_fields(p.peers, pk, b0 + pg, p.B, db, p.d, p.s, code,
-                                              bucket + pk * p.row_words, &A);
+      const uint32_t st = parse_to_fields(ref, ones, db, p.d, p.s, code, bucket + pk * p.row_words, &A);
       reinterpret_cast<float*>(bucket + p.K * p.row_words)[pk] = A;
       if (st) atomicOr(p.status, st);
     }
@@ -157,7 +158,7 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
       const uint64_t b = b0 + g;
       const uint64_t i0 = b * p.d + c;
       const bool live = slot < total_slots && b < p.B && i0 < p.n;
-      const uint32_t* bucket = mine + (live ? g : 0) * p.bucket_words;
+      const uint32_t* bucket = words + (live ? g : 0) * p.bucket_words;
       const float* scales = reinterpret_cast<const float*>(bucket + p.K * p.row_words);
       float acc[16];
 #pragma unroll
