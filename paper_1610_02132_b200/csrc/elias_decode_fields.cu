@@ -140,9 +140,9 @@ __global__ void __launch_bounds__(320) decode_elias_fields_kernel(const __grid_c
     StringRef ref;
     ref.words = nullptr; ref.lo = 0; ref.total = 0; ref.err = 0;
     if (mine) ref = string_ref(p.peers, pk, b0 + pg, p.B, db);
-    // More than 9 bits per coordinate in all strings of the warp: nearly all levels are nonzero (37.0 -> 33.7 us at n = 1 M, d = 96,
-    // K = 5, N(0, 1); with one loop for all strings 6 % slower at n = 3 M, d = 96, K = 2, a mixture). All lanes vote.
-    const bool ones = __all_sync(0xffffffffu, !mine || ref.err || ref.total > 9u * db);
+    // More than 9.5 bits per coordinate in all strings of the warp: nearly all levels are nonzero (n = 33 M, d = 96, K = 5, N(0, 1),
+    // 10 bits 578 -> 528 us; strings of 9 to 9.5 bits that have zeros among their levels lost up to 8 %). All lanes vote.
+    const bool ones = __all_sync(0xffffffffu, !mine || ref.err || 2u * ref.total > 19u * db);
     if (mine) {
       uint32_t* bucket = words + pg * p.bucket_words;
       float A;
@@ -196,41 +196,53 @@ int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream) {
   const uint32_t level_words = p.d >> 2, sign_words = p.d >> 5;
   p.row_words = (level_words + sign_words + 3u) & ~3u;
   p.bucket_words = (p.K * p.row_words + p.K + 3u) & ~3u;
-  // As many buckets to a warp as it has lanes for (K = 5, d = 96: 6, where a power of two would leave 12 lanes idle).
-  uint32_t G = 32 / p.K;
-  while (G > 1 && (size_t)G * p.bucket_words * 4 > (16u << 10)) --G;
-  p.G = G;
-  const size_t per_warp = (size_t)G * p.bucket_words * 4;
-  // Warps per CTA: the count that leaves the most warps resident on an SM. The code table is
-  // per CTA, the fields per warp; the parse is latency-bound, so warps are what counts.
-  const size_t per_cta = 2048, budget = (size_t)max_smem - per_cta;
-  const size_t per_sm = 227u << 10;
-  int warps = 1, best = 0;
-  for (int w = 1; w <= 10; ++w) {
-    if ((size_t)w * per_warp > budget) break;
-    const int resident = (int)(per_sm / ((size_t)w * per_warp + per_cta)) * w;
-    if (resident > best) { best = resident; warps = w; }
-  }
-  // Where all warps are resident at once, the count that spreads them evenly over the SMs.
-  const uint64_t groups = (p.B + G - 1) / G;
+  // CTAs of w warps that an SM holds: the code table and what CUDA reserves are per CTA, the fields per warp; 32 warps by registers.
+  const size_t per_cta = 2112, per_sm = 227u << 10;
+  constexpr uint32_t kResident = 32, kMostWarps = 10;
+  auto ctas_of = [&](uint32_t w, size_t per_warp) {
+    if (w * per_warp + per_cta > (size_t)max_smem) return 0u;
+    const uint32_t by_memory = (uint32_t)(per_sm / (w * per_warp + per_cta)), by_registers = kResident / w;
+    return by_memory < by_registers ? by_memory : by_registers;
+  };
+  // Warps per CTA: the count that leaves the most resident, since the parse is latency-bound; from four on, so that all schedulers
+  // of an SM have some.
+  auto most_resident = [&](size_t per_warp, uint32_t* warps) {
+    uint32_t best = 0;
+    for (uint32_t w = 4; w <= kMostWarps; ++w)
+      if (ctas_of(w, per_warp) * w > best) { best = ctas_of(w, per_warp) * w; *warps = w; }
+    for (uint32_t w = 3; best == 0u && w >= 1u; --w)
+      if (ctas_of(w, per_warp)) { best = ctas_of(w, per_warp) * w; *warps = w; }
+    return best;
+  };
   int sms = 0, occ = 0;
   int st = device_sms(&sms);
   if (st) return st;
-  if (groups <= (uint64_t)sms * best) {
+  // Buckets to a warp: a power of two, within 16 KB; or as many as it has lanes for (K = 5, d = 96: 6, where a power of two leaves
+  // 12 lanes idle, n = 33 M 792 -> 530 us), where that leaves room for 32 warps on an SM (n = 12 M, d = 256, K = 5: 6 with 25 warps
+  // 347 us, 4 with 32 286) and at least ten warps with work to each (n = 769 K, d = 256, K = 9: 3 62 us, 2 54).
+  uint32_t G = 32 / p.K, power = 1, warps = 1;
+  while (2u * power <= G && (size_t)(2u * power) * p.bucket_words * 4 <= (16u << 10)) power *= 2u;
+  while (G > power && most_resident((size_t)G * p.bucket_words * 4, &warps) < kResident) --G;
+  if (p.B < 10ull * sms * G) G = power;
+  p.G = G;
+  const size_t per_warp = (size_t)G * p.bucket_words * 4;
+  const uint64_t groups = (p.B + G - 1) / G;
+  if (groups <= (uint64_t)sms * most_resident(per_warp, &warps)) {
+    // all warps are resident at once: the count that spreads them evenly over the SMs
     uint64_t least = ~0ull;
-    for (int w = warps; w >= 1; --w) {
-      const uint64_t per = ((groups + w - 1) / w + sms - 1) / sms * w;
-      if (per < least && per * per_warp + per / w * per_cta <= per_sm) { least = per; warps = w; }
+    for (uint32_t w = kMostWarps; w >= 4u; --w) {
+      const uint64_t ctas = ((groups + w - 1) / w + sms - 1) / sms;
+      if (ctas * w < least && ctas <= ctas_of(w, per_warp)) { least = ctas * w; warps = w; }
     }
   }
   auto kern = fused ? decode_elias_fields_kernel<true> : decode_elias_fields_kernel<false>;
   const size_t smem = (size_t)warps * per_warp;
-  st = site[fused ? 1 : 0].lookup_dynamic(kern, warps * 32, smem, &sms, &occ);
+  st = site[fused ? 1 : 0].lookup_dynamic(kern, (int)warps * 32, smem, &sms, &occ);
   if (st) return st;
   const uint64_t want = (groups + warps - 1) / warps;
   const uint64_t cap = (uint64_t)sms * occ;
   ScopedKernel sk(kKernDecodeEliasFields, stream);
-  return (int)launch_chained(kern, (uint32_t)(want < cap ? want : cap), warps * 32, smem, stream, p);
+  return (int)launch_chained(kern, (uint32_t)(want < cap ? want : cap), warps * 32u, smem, stream, p);
 }
 
 }  // namespace qsgd

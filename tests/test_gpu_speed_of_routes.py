@@ -60,3 +60,10 @@ def test_one_peer_against_eight():
     n, d, s = 3871, 4096, 15
     one, eight = time_of(*(decode(n, d, s, L2, DENSE, K) for K in (1, 8)))
     assert one < 0.9 * eight
+
+
+@pytest.mark.parametrize("n,d,K,other", [(6973756, 480, 4, 512), (2753820, 96, 7, 128)])
+def test_many_levels_in_buckets_of_many_sizes(n, d, K, other):
+    """A lane per string against buckets a little longer, which another decoder reads or another split fits."""
+    here, there = time_of(*(decode(n, m, 255, L2, ELIAS, K) for m in (d, other)))
+    assert here < 1.05 * there
