@@ -173,6 +173,8 @@ int launch_one(const DecodeParams& p, cudaStream_t stream) {
   uint32_t warps = 8;
   if (LB == 8) while (warps < Shape<LB>::kMostThreads / 32 && p.chunks > warps * (uint32_t)sms) warps *= 2;
   const size_t smem = (LB == 8 ? kTableAt + kTableBytes : 0u) + warps * kTurn;
+  if (LB == 8) st = site.dynamic_begins_within(kern, kTableAt);
+  if (st) return st;
   st = site.lookup_dynamic(kern, (int)warps * 32, smem, &sms, &occ);
   if (st) return st;
   const uint32_t want = (p.chunks + warps - 1) / warps, cap = (uint32_t)(sms * occ);

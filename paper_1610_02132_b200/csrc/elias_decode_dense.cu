@@ -46,6 +46,7 @@ struct DenseParams {
   uint32_t run;           // buckets per run
   uint32_t slots;         // scales kept per lane, a power of two: the buckets that a ring can touch
   uint32_t warp_bytes;
+  uint32_t in_front;      // warps whose shared memory lies in front of the tables
   uint32_t work;          // warps of a CTA that have runs; the others help to make the tables
   BucketMap map;
 };
@@ -102,8 +103,8 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) decode_elias_dense_kernel(c
   // per warp: rows of kRing bytes | 32 lanes' pieces of their streams | slots x 32 scales. Position q of lane l's
   // row is byte q ^ 8 l of the row, so that lanes at the same position are in different banks.
   // Warps lie in front of the table and behind it.
-  const uint32_t front = (shared_address(dense_shared) + 255u) & ~255u, in_front = (kTableAt - front) / p.warp_bytes;
-  const uint32_t shared_mine = warp < in_front ? front + warp * p.warp_bytes : kTableEnd + (warp - in_front) * p.warp_bytes;
+  const uint32_t front = (shared_address(dense_shared) + 255u) & ~255u;
+  const uint32_t shared_mine = warp < p.in_front ? front + warp * p.warp_bytes : kTableEnd + (warp - p.in_front) * p.warp_bytes;
   if (warp < p.work)
     for (uint32_t i = lane; i < p.warp_bytes / 16u; i += 32) zero_quad(shared_mine + 16u * i);
   const uint32_t stage = shared_mine + rows * kRing + lane * kStage;
@@ -386,6 +387,7 @@ int launch_elias_dense(const FieldParams& f, bool fused, cudaStream_t stream) {
   if (st) return st;
   constexpr uint32_t kOwn = 3072u;                 // static shared memory, what CUDA reserves, alignment
   const uint32_t in_front = (kTableAt - kOwn) / p.warp_bytes;
+  p.in_front = in_front;
   uint32_t warps = in_front + ((uint32_t)most_shared - kOwn - kTableEnd) / p.warp_bytes;
   if (warps > kMaxWarps) warps = kMaxWarps;
   // one run of consecutive buckets per lane group, all of the same length, in one wave
@@ -405,7 +407,9 @@ int launch_elias_dense(const FieldParams& f, bool fused, cudaStream_t stream) {
     if (byte) kern = fused ? decode_elias_dense_kernel<true, true, 8> : decode_elias_dense_kernel<false, true, 8>;
     else kern = fused ? decode_elias_dense_kernel<true, false, 8> : decode_elias_dense_kernel<false, false, 8>;
   }
-  st = site[(one ? 4 : 0) + (byte ? 2 : 0) + (fused ? 1 : 0)].lookup_dynamic(kern, (int)kMaxWarps * 32, smem, &sms, &occ);
+  KernelSite& here = site[(one ? 4 : 0) + (byte ? 2 : 0) + (fused ? 1 : 0)];
+  st = here.dynamic_begins_within(kern, kOwn - 256u);            // (and up to 256 bytes to the next multiple)
+  if (!st) st = here.lookup_dynamic(kern, (int)kMaxWarps * 32, smem, &sms, &occ);
   if (st) return st;
   ScopedKernel sk(kKernDecodeEliasDense, stream);
   return (int)launch_chained(kern, (uint32_t)((need + warps - 1) / warps), kMaxWarps * 32u, smem, stream, p);

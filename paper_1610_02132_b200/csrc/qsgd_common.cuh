@@ -146,6 +146,7 @@ struct KernelSite {
   int sms[kMaxDevices] = {};
   int occ[kMaxDevices] = {};
   int opted[kMaxDevices] = {};   // dynamic shared memory the kernel may use so far
+  uint32_t front[kMaxDevices] = {};   // 1 + bytes of shared memory in front of the dynamic part
 
   template <class Kernel>
   int lookup(Kernel kern, int threads, size_t smem, int* sms_out, int* occ_out) {
@@ -170,6 +171,26 @@ struct KernelSite {
     *sms_out = sms[dev];
     *occ_out = occ[dev];
     return 0;
+  }
+
+  // For a kernel that puts things at places of its own in the window of shared memory: an error unless its dynamic shared
+  // memory begins within the first `bytes`, behind what CUDA reserves and its static variables. Looked up once per device.
+  template <class Kernel>
+  int dynamic_begins_within(Kernel kern, size_t bytes) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return (int)e;
+    if (dev < 0 || dev >= kMaxDevices) return (int)cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!front[dev]) {
+      cudaFuncAttributes attr;
+      int reserved = 0;
+      e = cudaFuncGetAttributes(&attr, kern);
+      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+      if (e != cudaSuccess) return (int)e;
+      front[dev] = 1u + (uint32_t)reserved + (uint32_t)attr.sharedSizeBytes;
+    }
+    return front[dev] - 1u <= bytes ? 0 : (int)cudaErrorInvalidConfiguration;
   }
 
   // The same for a kernel whose shared memory depends on the problem: the opt-in is raised as needed and
