@@ -167,15 +167,19 @@ template <int LB, bool FUSED, bool SINGLE>
 int launch_one(const DecodeParams& p, cudaStream_t stream) {
   static KernelSite site;
   auto kern = decode_fixed_kernel<LB, FUSED, SINGLE>;
-  int sms = 0, occ = 0;
-  int st = device_sms(&sms);
-  if (st) return st;
+  int sms = 0, occ = 0, st = 0;
   uint32_t warps = 8;
-  if (LB == 8) while (warps < Shape<LB>::kMostThreads / 32 && p.chunks > warps * (uint32_t)sms) warps *= 2;
-  const size_t smem = (LB == 8 ? kTableAt + kTableBytes : 0u) + warps * kTurn;
-  if (LB == 8) st = site.dynamic_begins_within(kern, kTableAt);
-  if (st) return st;
-  st = site.lookup_dynamic(kern, (int)warps * 32, smem, &sms, &occ);
+  size_t smem = warps * kTurn;
+  if constexpr (LB == 8) {
+    st = device_sms(&sms);
+    if (!st) st = site.dynamic_begins_within(kern, kTableAt);
+    if (st) return st;
+    while (warps < Shape<LB>::kMostThreads / 32 && p.chunks > warps * (uint32_t)sms) warps *= 2;
+    smem = kTableAt + kTableBytes + warps * kTurn;
+    st = site.lookup_dynamic(kern, (int)warps * 32, smem, &sms, &occ);
+  } else {
+    st = site.lookup(kern, (int)warps * 32, smem, &sms, &occ);
+  }
   if (st) return st;
   const uint32_t want = (p.chunks + warps - 1) / warps, cap = (uint32_t)(sms * occ);
   ScopedKernel sk(kKernDecodeFixed, stream);
