@@ -342,7 +342,7 @@ int launch_elias_ring(const FieldParams& p, bool fused, cudaStream_t stream);   
 int launch_elias_bytes(const FieldParams& p, bool fused, cudaStream_t stream);    // the same
 int launch_elias_fields(FieldParams& p, bool fused, cudaStream_t stream);         // Code_s, s > 15, d < 512, at most 32 peers
 int launch_elias_sparse(const FieldParams& p, bool fused, cudaStream_t stream);   // Code_s, at most 32 peers
-int launch_elias_dense(const FieldParams& p, bool fused, cudaStream_t stream);    // Code'_s, s <= 127, at most 32 peers
+int launch_elias_dense(const FieldParams& p, bool fused, cudaStream_t stream);    // Code'_s, s <= 64 (use_streams), at most 32 peers
 int launch_elias_teams(const FieldParams& p, bool dense, uint32_t mean, bool fused, cudaStream_t stream);   // mean: of mean_bits
 
 }  // namespace qsgd

@@ -17,8 +17,8 @@ namespace {
 
 // Reconstruction by arithmetic: A * (level / s), the quotient rounded to nearest as the definition has it, without a
 // table. The table took 32 KB of a CTA, so fewer warps fitted, and the parse waits on latency: 42.5 us with it, 39.7 us
-// without (n = 1 M, d = 96, s = 255, K = 5). The fixed-width decoder does nothing else than this, and is faster with its
-// table (335 against 376 us at n = 60 M, K = 16). With 1 / s = hi + lo in two floats, RN(level * hi + RN(level * lo)) is
+// without (n = 1 M, d = 96, s = 255, K = 5). The fixed-width decoder does nothing else than this, and was faster with
+// the table that it had then (335 against 376 us at n = 60 M, K = 16; with signs in the table 263). With 1 / s = hi + lo in two floats, RN(level * hi + RN(level * lo)) is
 // RN(level / s) for every s <= 255 and level <= s (checked exhaustively in rational arithmetic). The level comes as the
 // float 2^23 + level, made by one byte permute. All steps work on pairs (f32x2).
 struct LevelQuotient {

@@ -16,10 +16,10 @@
 //
 // Latency is what counts here: one string of 4096 dense symbols read by one lane is 300 us, whatever else
 // the GPU does. So the strings are read where they are, a word ahead of the need: a copy of them in shared memory costs
-// half of the resident warps (8 workers, n = 16.8 M, s = 64, d = 4096, dense code: 375 us with it, 283 without; Code_s
-// with d = 1024: 693 and 630; only the smallest problems, which leave most of the GPU idle, lose: 17.8 and 18.7 us at
-// n = 100 K). The rest is the number of instructions: the dense code is read three table entries to a window, for 10
-// instructions per symbol against 30 with one entry at a time (412 -> 279 us in all).
+// half of the resident warps (8 workers, n = 16.8 M, s = 64, d = 4096, dense code, which streams read now: 375 us with it,
+// 283 without; Code_s with d = 1024: 693 and 630; only the smallest problems, which leave most of the GPU idle, lose: 17.8 and
+// 18.7 us at n = 100 K). The rest is the number of instructions: the dense code is read three table entries to a window, for 10
+// instructions per symbol against 30 with one entry at a time (412 -> 279 us there).
 #include <type_traits>
 
 #include "elias_decode.cuh"

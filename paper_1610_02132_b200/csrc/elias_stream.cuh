@@ -1,5 +1,6 @@
 // What the decoders with a lane per stream share (elias_decode_ring.cu, elias_decode_dense.cu): accesses to shared memory by
-// address, copies in the background, and the sums of a step written out.
+// address and copies in the background. (The sums of a step are written out in each: they differ by the lookup of a value, and by
+// what the compiler makes of the loop around it.)
 #pragma once
 
 #include "elias_decode.cuh"
@@ -7,7 +8,7 @@
 namespace qsgd {
 
 __device__ __forceinline__ uint32_t shared_address(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-// The same and a load where `when` is nonzero, without a branch.
+// A store and a load that happen where `when` holds, without a branch.
 __device__ __forceinline__ void store_byte_if(uint32_t when, uint32_t addr, uint32_t v) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.u8 [%1], %2;\n\t}" ::"r"(when), "r"(addr), "r"(v)
                : "memory");

@@ -22,10 +22,10 @@ def encode(g, d, s, norm, code):
 
 
 def test_elias_encode_of_mostly_small_values_with_many_levels():
-    """Buckets of 512 against buckets of 480, for which there is only one way."""
+    """22 levels against 15, of which messages are hardly shorter."""
     g = I.gaussian_mixture_device(40 * 2 ** 20, seed=3)
-    here, other = time_of(*(encode(g, d, 22, L2, ELIAS) for d in (512, 480)), repeats=4)
-    assert here < 1.1 * other                              # 0.9; 1.2 by tiles
+    fewer, more = time_of(*(encode(g, 512, s, L2, ELIAS) for s in (15, 22)), repeats=4)
+    assert more < 1.55 * fewer                             # 1.34; 1.76 by tiles
 
 
 def test_encodes_of_more_ctas_grow_no_faster_than_their_length():
@@ -37,22 +37,11 @@ def test_encodes_of_more_ctas_grow_no_faster_than_their_length():
 
 
 
-@pytest.mark.parametrize("n,d,K", [(729088, 4096, 8), (2668, 512, 64)])
-def test_strings_of_more_bits_in_another_decoder_width(n, d, K):
-    """Teams with 15 levels and with 16, whose codes take a byte: max-norm strings of much the same length."""
-    make = lambda w: I.sparse_laplace_device(n, 1e-3, 0.3, seed=w)
-    fewer, more = time_of(*(decode(n, d, s, MAX, ELIAS, K, make) for s in (15, 16)))
-    assert fewer < 1.1 * more
-
-
 def test_short_strings_where_long_ones_are_shared_by_warps():
-    """A quarter of the bits: strings of mostly small values against such of N(0, 1)."""
-    n, d, s, K = 15792, 4096, 255, 8
-    short = decode(n, d, s, L2, ELIAS, K, lambda w: I.gaussian_mixture_device(n, seed=w))
-    long = decode(n, d, s, L2, ELIAS, K)
-    assert short.bits < 0.4 * long.bits
-    few, many = time_of(short, long)
-    assert few < 0.9 * many
+    """Eight peers' strings of mostly small values against seventeen peers', too many to be shared."""
+    n, d, s = 15792, 4096, 255
+    eight, many = time_of(*(decode(n, d, s, L2, ELIAS, K, lambda w: I.gaussian_mixture_device(n, seed=w)) for K in (8, 17)))
+    assert eight < 0.48 * many                             # 0.42; 0.54 where first parts share schedulers
 
 
 def test_one_peer_against_eight():
@@ -67,3 +56,11 @@ def test_many_levels_in_buckets_of_many_sizes(n, d, K, other):
     """A lane per string against buckets a little longer, which another decoder reads or another split fits."""
     here, there = time_of(*(decode(n, m, 255, L2, ELIAS, K) for m in (d, other)))
     assert here < 1.05 * there
+
+
+@pytest.mark.parametrize("d,s,K", [(128, 64, 64), (64, 100, 32)])
+def test_a_few_chunks_more_than_a_round_of_warps(d, s, K):
+    """Fixed-width decode of 8-bit levels: 32 chunks of 512 coordinates on each of 148 SMs, and an eighth more."""
+    n = 512 * 148 * 32
+    round_, more = time_of(*(decode(m, d, s, MAX, FIXED, K) for m in (n, n + n // 8)))
+    assert more < 1.55 * round_                            # 1.3; 1.9 where a few SMs get all of the rest
