@@ -219,6 +219,25 @@ __device__ __forceinline__ void store_chunk16(float* out, const BucketMap& map, 
     float* o = sp.ptr + lane * 4u;                                        // quad 32 j + lane: from o + 128 j on
     const uint32_t from = turn + (lane ^ ((lane >> 3) & 3u)) * 16u;
     const uint32_t left = sp.valid > lane * 4u ? sp.valid - lane * 4u : 0u;
+    if (quads && sp.valid == 512u) {              // nothing to ask for each quad: 1 % of a large decode
+      float4 x[4];
+      if (FUSED)
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) x[j] = *reinterpret_cast<const float4*>(o + j * 128u);
+      __syncwarp();
+#pragma unroll
+      for (uint32_t j = 0; j < 4; ++j) {
+        float4 r;
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "r"(from + j * 512u) : "memory");
+        if (FUSED) {
+          r.x = __fsub_rn(x[j].x, __fmul_rn(c, r.x)); r.y = __fsub_rn(x[j].y, __fmul_rn(c, r.y));
+          r.z = __fsub_rn(x[j].z, __fmul_rn(c, r.z)); r.w = __fsub_rn(x[j].w, __fmul_rn(c, r.w));
+        }
+        *reinterpret_cast<float4*>(o + j * 128u) = r;
+      }
+      __syncwarp();                               // before the next chunk's quads
+      return;
+    }
     float4 x[4];
     if (FUSED)
 #pragma unroll
